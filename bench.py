@@ -59,12 +59,11 @@ def select_workload(name):
     WORKLOAD, N_GAUSS, WIDTH, HEIGHT, PAIR_CAPACITY = name, n, w, h, cap
     return kind
 EVAL_FP32_OPS = 15        # FP32 lane operations per Gaussian-pixel evaluation in Render
-# Kernels of one forward frame: frame parameters 1, preprocess 1, depth sort
-# 4 x (count, count scan, scatter) 12, run scan + pair total 2, slice-0 setup 1,
-# tile pass 1 (count, count scan, scatter) 3, render slice 0 1,
+# Kernels of one forward frame: frame head 1, preprocess 1, depth order (bin
+# scan, bin scatter, window sort with the run scan) 3, tile pass 1 (count, count scan, scatter) 3, render slice 0 1,
 # unfinished-tile table (rows, columns) + compaction (count, scan, scatter) 5,
 # tile pass 1 of slice 1 3, render slice 1 1 (each render derives its column ranges).
-KERNELS_PER_FRAME = 30
+KERNELS_PER_FRAME = 18
 # DRAM bytes (read + write) of one launch from one-pass ncu captures at the
 # heavy 3M-Gaussian 1080p frame: Render (profiles/render_heavy-3M-1080p_traffic.md,
 # its two launches of one frame, 54.8 MB) and the per-tile list pass
@@ -390,11 +389,9 @@ def kernel_bytes(name, n, u, hw):
     return {
         # params (+SH of kept) in; records of kept (64 B), radii/depth, key, box out
         "preprocess": 44 * n + 192 * V + 40 * n + 64 * V,
-        # 4 passes: the first reads the n keys twice and writes the V kept keys +
-        # values; the others count, read and write V keys + values; the last
-        # also gathers and writes the V packed rectangles
-        "depth_pass": 8 * n + 76 * V,
-        "scan_tiles": 8 * V,                       # boxes in depth order in, run offsets out (slice 1 on top)
+        # n keys, ranks and rectangles in, V records of 16 B out and in, and the
+        # order, rectangles and run offsets out
+        "depth_pass": 12 * n + 44 * V,
         "tile_count_columns": None,                # runs of the two depth slices
         "tile_count_scan": 0,                      # 2 x 256 x grid words, L2-resident
         "tile_scatter_columns": None,
@@ -407,8 +404,8 @@ def kernel_bytes(name, n, u, hw):
 
 
 def sort_throughput(ktable, u):
-    """Items per second of the depth sort (Gaussians with tiles over its four
-    passes) and of tile pass 1 (column runs built over its count, count scan
+    """Items per second of the depth sort (Gaussians with tiles over its three
+    kernels, the run scan included) and of tile pass 1 (column runs built over its count, count scan
     and scatter kernels), from the live kernel table."""
     ms = lambda names: sum(ktable[k]["ms_per_frame"] for k in names if k in ktable)
     depth_ms = ms(("depth_pass",))

@@ -138,6 +138,8 @@ adr_status check_params(const float* means, const float* scales, const float* ro
 
 }  // namespace
 
+constexpr int kHostLargestBin = 48;   // word of adr_ctx::host_words
+
 struct adr_ctx {
     int device = 0;
     int max_w = 0, max_h = 0;
@@ -147,7 +149,8 @@ struct adr_ctx {
     bool have_frame = false, have_sort = false, have_render = false;
     cudaStream_t last_stream = nullptr;
     uint32_t* host_words = nullptr;  // pinned: counters + status readback (words 0-31),
-                                     // runs of the last sliced frame (words 40-42)
+                                     // runs of the last sliced frame (words 40-42), the largest
+                                     // depth bin of the last frame to run (word 48)
     // Depth slices pay only when most tiles stop within the nearest Gaussians.
     // After a sliced frame its run counts (all, slice 0, slice 1) come back
     // asynchronously; the next frame slices if the two slices made fewer than
@@ -156,6 +159,7 @@ struct adr_ctx {
     bool slice_probe = false;        // a readback is in flight
     bool slices_pay = true;
     uint32_t frames = 0;
+    uint32_t radix_probe_in = kRadixProbe;   // see next_depth_sort
     int32_t slice_mode = ADR_SLICES_ADAPTIVE;
     int32_t host_reads = ADR_HOST_READ_MAPPED;   // adr_render_host: read mapped host buffers in place
     bool defer_colors = false;   // the next adr_preprocess leaves the SH colours to adr_render
@@ -194,11 +198,11 @@ void free_workspace(Workspace& w) {
         delete w.prof;
         w.prof = nullptr;
     }
-    void* ptrs[] = {w.rec, w.aux, w.depth_key, w.offsets, w.gbox, w.sorted_box, w.gkeys[0],
-                    w.gkeys[1], w.gvals[0], w.gvals[1], w.pruns, w.prows, w.pgauss, w.tcounts, w.ttotals, w.tile_counts,
+    void* ptrs[] = {w.rec, w.aux, w.depth_key, w.offsets, w.gbox, w.sorted_box, w.sortbuf,
+                    w.order, w.win_lo, w.pruns, w.prows, w.pgauss, w.tcounts, w.tile_counts,
                     w.chunk_first, w.ranges, w.last, w.trav, w.tfin, w.lstat, w.g2d, w.load_sums,
                     w.hist, w.counters, w.status, w.lookback, w.d_fp, w.d_stage,
-                    w.slice_counters, w.s_order, w.s_box, w.s_offsets, w.s_chunk_first,
+                    w.s_order, w.s_box, w.s_offsets, w.s_chunk_first,
                     w.surv_cnt, w.surv_flag, w.pst, w.pis, w.tile_done, w.tile_fbase, w.sat};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -211,9 +215,10 @@ size_t workspace_bytes(int64_t max_gaussians, int64_t pair_capacity, int32_t max
     const size_t pixels = (size_t)max_width * max_height;
     const size_t tiles = (size_t)((max_width + kTile - 1) / kTile) * ((max_height + kTile - 1) / kTile);
     const size_t lb = ((N + kSortChunk - 1) / kSortChunk + 2) * kRadix * 8;
-    return N * (kRecFloat4 * 16 + kAuxFloat4 * 16 + 4 * 4 + 8 + 16 + 36 + 12) + P * 14 +
+    return N * (kRecFloat4 * 16 + kAuxFloat4 * 16 + 4 * 4 + 4 + 8 + 16 + 36 + 12) + P * 14 +
            2 * (P / kSortChunk + 2) * 4 + tiles * 20 + pixels * 48 + lb +
-           (size_t)kRadix * (kMaxTileGrid + 2) * 4 + 4096;
+           (size_t)kRadix * kMaxTileGrid * 4 + (kZeroWords + bin_map(max_gaussians).count) * 4 +
+           (N / kWindow + 2) * 4 + 8192;
 }
 
 adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_capacity,
@@ -229,6 +234,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     w.sm_count = sms;
     w.sort_grid = sms * onesweep_blocks_per_sm();
     w.scan_grid = sms * scan_blocks_per_sm();
+    w.window_grid = sms * window_blocks_per_sm();
     w.tile_grid = sms * tile_scatter_blocks_per_sm();
     if (w.tile_grid > kMaxTileGrid) w.tile_grid = kMaxTileGrid;
     const size_t N = (size_t)max_gaussians, P = (size_t)pair_capacity;
@@ -250,16 +256,14 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.offsets, N * sizeof(uint32_t));
     ALLOC(w.gbox, N * sizeof(uint32_t));
     ALLOC(w.sorted_box, N * sizeof(uint32_t));
-    for (int b = 0; b < 2; ++b) {
-        ALLOC(w.gkeys[b], N * sizeof(uint32_t));
-        ALLOC(w.gvals[b], N * sizeof(uint32_t));
-    }
+    ALLOC(w.sortbuf, N * sizeof(uint4));
+    ALLOC(w.order, N * sizeof(uint32_t));
+    ALLOC(w.win_lo, (N / kWindow + 2) * sizeof(uint32_t));
     ALLOC(w.pruns, P * sizeof(uint2));
     ALLOC(w.prows, (P + 8) * sizeof(uint16_t));   // + 16 bytes: Render reads whole 16-byte groups
     ALLOC(w.pgauss, P * sizeof(uint32_t));
     ALLOC(w.tile_counts, (size_t)w.max_tiles * sizeof(uint32_t));
     ALLOC(w.tcounts, (size_t)kRadix * kMaxTileGrid * sizeof(uint32_t));
-    ALLOC(w.ttotals, 2 * kRadix * sizeof(uint32_t));
     ALLOC(w.chunk_first, (P / kSortChunk + 2) * sizeof(uint32_t));
     ALLOC(w.ranges, (size_t)w.max_tiles * sizeof(uint2));
     ALLOC(w.last, pixels * sizeof(int32_t));
@@ -268,7 +272,6 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.lstat, pixels * sizeof(int32_t));
     {
         const size_t tx = (size_t)(max_width + kTile - 1) / kTile, ty = (size_t)(max_height + kTile - 1) / kTile;
-        ALLOC(w.slice_counters, 2 * kCntSlots * sizeof(uint32_t));
         ALLOC(w.s_order, N * sizeof(uint32_t));
         ALLOC(w.s_box, N * sizeof(uint32_t));
         ALLOC(w.s_offsets, N * sizeof(uint32_t));
@@ -284,7 +287,12 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.g2d, N * 9 * sizeof(float));
     ALLOC(w.load_sums, 4 * sizeof(double));
     ALLOC(w.hist, kHistWords * sizeof(uint32_t));
-    ALLOC(w.counters, kCntSlots * sizeof(uint32_t));
+    // the zeroed block; bin counts grow with n, so the largest scene's fit every one
+    const size_t zero_words = kZeroWords + bin_map(max_gaussians).count;
+    ALLOC(w.counters, zero_words * sizeof(uint32_t));
+    w.slice_counters = w.counters + kCntSlots;
+    w.ttotals = w.slice_counters + 2 * kCntSlots;
+    w.bins = w.counters + kZeroWords;
     ALLOC(w.status, sizeof(uint32_t) * 4);
     ALLOC(w.lookback, w.lookback_words * sizeof(unsigned long long));
     ALLOC(w.d_fp, sizeof(FrameParams));
@@ -292,7 +300,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
 #undef ALLOC
     if (cudaMemset(w.lookback, 0, w.lookback_words * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(w.status, 0, sizeof(uint32_t) * 4) != cudaSuccess ||
-        cudaMemset(w.counters, 0, kCntSlots * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMemset(w.counters, 0, zero_words * sizeof(uint32_t)) != cudaSuccess ||
         cudaMemset(w.d_stage, 0, sizeof(uint32_t)) != cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess) {
         free_workspace(w);
@@ -361,6 +369,9 @@ adr_status adr_create(adr_ctx** out, int64_t max_gaussians, int64_t pair_capacit
     }
     cudaError_t e = cudaHostAlloc((void**)&c->host_words, 64 * sizeof(uint32_t), cudaHostAllocDefault);
     if (e != cudaSuccess) { free_ctx(c); return fail(ADR_ERR_CUDA, "cudaHostAlloc: %s", cudaGetErrorString(e)); }
+    c->host_words[kHostLargestBin] = 0;
+    e = cudaHostGetDevicePointer((void**)&c->ws.largest_bin, c->host_words + kHostLargestBin, 0);
+    if (e != cudaSuccess) { free_ctx(c); return fail(ADR_ERR_CUDA, "cudaHostGetDevicePointer: %s", cudaGetErrorString(e)); }
     e = cudaEventCreateWithFlags(&c->slice_ev, cudaEventDisableTiming);
     if (e != cudaSuccess) { free_ctx(c); return fail(ADR_ERR_CUDA, "cudaEventCreate: %s", cudaGetErrorString(e)); }
     *out = c;
@@ -389,6 +400,9 @@ adr_status adr_preprocess(adr_ctx* c, const float* means, const float* scales, c
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     fill_frame_state(c->fs, n, cam, st);
+    // The host word is written by the device and read without waiting.
+    c->fs.depth_sort = next_depth_sort(*static_cast<volatile uint32_t*>(c->host_words + kHostLargestBin),
+                                       c->radix_probe_in);
     enqueue_preprocess(c->ws, c->fs, c->epoch, means, scales, rots, opac, sh, strm, true,
                        c->defer_colors);
     if ((s = check_launch("adr_preprocess")) != ADR_OK) return s;

@@ -131,7 +131,8 @@ enum Counter : int {
     kCntDepthKept = 4,    // Gaussians with tiles, counted by the first depth pass
     kCntScanFailed = 5,   // non-zero: a lookback wait of the run scan gave up (the frame
                           // is then skipped: its pair count reads as saturated)
-                          // words 6-7: unused
+    kCntWindowsDone = 6,  // windows the window sort has finished (bins.cu)
+                          // word 7: unused
     kCntPairs64 = 8,      // words 8-9: P as a 64-bit sum
     kCntSlots = 16
 };
@@ -158,20 +159,23 @@ struct Profiler {
 struct Workspace {
     int64_t max_n = 0, capacity = 0;       // Gaussians, Gaussian-tile pairs
     int max_tiles = 0;
-    int sm_count = 0, sort_grid = 0, scan_grid = 0, tile_grid = 0;
+    int sm_count = 0, sort_grid = 0, scan_grid = 0, tile_grid = 0, window_grid = 0;
     float4* rec = nullptr;                 // [max_n * kRecFloat4]
     float4* aux = nullptr;                 // [max_n * kAuxFloat4]
     uint32_t* depth_key = nullptr;         // [max_n]
     uint32_t* offsets = nullptr;           // [max_n]
     uint32_t* gbox = nullptr;              // [max_n] packed tile rectangle per Gaussian (all ones: none)
     uint32_t* sorted_box = nullptr;        // [max_n] the same per depth-order position
-    uint32_t* gkeys[2] = {nullptr, nullptr};   // [max_n] each
-    uint32_t* gvals[2] = {nullptr, nullptr};   // [max_n] each
+    uint4* sortbuf = nullptr;              // [max_n] (key, index, box) records of the window sort; the
+                                           // radix sort's two buffers of max_n keys and max_n values
+    uint32_t* order = nullptr;             // [max_n] Gaussians by depth
+    uint32_t* win_lo = nullptr;            // [max_n / kWindow + 2] first position of each window
     uint2* pruns = nullptr;                // [capacity] column runs grouped by tile column
     uint16_t* prows = nullptr;             // [capacity] their row intervals y0 | (h - 1) << 8
     uint32_t* pgauss = nullptr;            // [capacity] Gaussian ids of the pairs by (tile, depth)
     uint32_t* tcounts = nullptr;           // [kRadix * kMaxTileGrid] per-(digit, CTA) counts / starts
-    uint32_t* ttotals = nullptr;           // [2 * kRadix] per-digit totals of the two tile passes
+    uint32_t* ttotals = nullptr;           // [kTotalSets * kRadix] per-digit totals of the tile passes
+                                           // (in the zeroed block, see kZeroWords)
     uint32_t* tile_counts = nullptr;       // [max_tiles] pairs per tile
     uint32_t* chunk_first = nullptr;       // [capacity / kSortChunk + 2]
     uint2* ranges = nullptr;               // [max_tiles]
@@ -182,7 +186,10 @@ struct Workspace {
     float* g2d = nullptr;                  // [max_n * 9] backward: dL/d(px, py, conic, sigma, rgb)
     double* load_sums = nullptr;           // [4] load-balancing loss moments
     uint32_t* hist = nullptr;              // [kHistWords]
-    uint32_t* counters = nullptr;          // [kCntSlots]
+    uint32_t* counters = nullptr;          // [kCntSlots], the start of the zeroed block
+    uint32_t* bins = nullptr;              // [kMaxBins or fewer] depth histogram, then bin starts
+                                           // (in the zeroed block)
+    uint32_t* largest_bin = nullptr;       // host word (mapped, may be null): the frame's largest bin
     uint32_t* status = nullptr;            // [4]
     unsigned long long* lookback = nullptr;
     size_t lookback_words = 0;             // (max_n / kSortChunk + 2) * kRadix
@@ -192,6 +199,7 @@ struct Workspace {
     uint32_t* d_stage = nullptr;           // [1] stage counter (see EpochRef)
     // Depth slices of the forward frame (slices.cu); all null: one slice.
     uint32_t* slice_counters = nullptr;    // [2 * kCntSlots] counter blocks of slices 0 and 1
+                                           // (in the zeroed block)
     uint32_t* s_order = nullptr;           // [max_n] slice-1 Gaussians in depth order
     uint32_t* s_box = nullptr;             // [max_n] their packed rectangles
     uint32_t* s_offsets = nullptr;         // [max_n] their run offsets
@@ -205,11 +213,56 @@ struct Workspace {
     uint32_t* sat = nullptr;               // [(tiles_x + 1) * (tiles_y + 1)] at the largest image
 };
 
+// Words that start a frame at zero, one block: counters, the counters of the
+// two depth slices, the tile passes' totals, then the frame's depth bins.
+enum TotalSet : int { kTotalsFirst = 0, kTotalsSlice1 = 1, kTotalsRows = 2, kTotalSets = 3 };
+constexpr int kZeroWords = 3 * kCntSlots + kTotalSets * kRadix;   // + the bins
+static_assert(kZeroWords % 4 == 0, "the bins are read 16 bytes at a time");
+
+// Depth bins (bins.cu): kBinOctaves octaves of depth from the near plane (at
+// least 2^-6) on, each 2^(23 - shift) bins; nearer and farther keys fall into
+// the first and the last bin.
+constexpr int kBinOctaves = 16;
+constexpr int kMaxBins = kBinOctaves << 13;
+struct BinMap {
+    int shift = 0;
+    uint32_t count = 0;
+};
+BinMap bin_map(int64_t n);
+__device__ __forceinline__ uint32_t bin_base(float near_z) {
+    return __float_as_uint(fmaxf(near_z, 0.015625f));
+}
+__device__ __forceinline__ uint32_t bin_of(uint32_t key, uint32_t base, const BinMap& m) {
+    return min((max(key, base) - base) >> m.shift, m.count - 1u);
+}
+// Gaussians of a window of the window sort, not counting what its last bin adds.
+constexpr int kWindow = 1024;
+constexpr uint32_t kRadixBin = 8192;
+constexpr uint32_t kRadixProbe = 64;   // a histogram every 64th radix frame
+
 // hist layout: 4 x 256 per-digit totals of the depth passes.
 constexpr int kHistWords = kMaxPasses * kRadix;
 
 // Contents of the column-run buffer: every Gaussian's runs, or a slice's.
 enum RunsHeld : int { kRunsAll = 0, kRunsSlice0 = 1, kRunsSlice1 = 2 };
+
+// How a frame orders its Gaussians by depth: by bins (bins.cu), or by the
+// radix sort (sort.cu), with or without a depth histogram beside it.  Both give
+// the same order; the radix sort is the faster one when one bin holds more than
+// kRadixBin Gaussians (very many at nearly one depth: the bin is sorted by one
+// CTA and counted by atomics on one address).  A caller learns the last frame's
+// largest bin and picks: next_depth_sort.
+enum DepthSort : int { kSortBins = 0, kSortRadix = 1, kSortRadixProbe = 2 };
+// `probe_in`: radix frames until the next one with a histogram.
+inline DepthSort next_depth_sort(uint32_t largest_bin, uint32_t& probe_in) {
+    if (largest_bin <= kRadixBin) {
+        probe_in = kRadixProbe;
+        return kSortBins;
+    }
+    if (--probe_in > 0) return kSortRadix;
+    probe_in = kRadixProbe;
+    return kSortRadixProbe;
+}
 
 // What one frame's stages hand to the next.
 struct FrameState {
@@ -228,6 +281,8 @@ struct FrameState {
     const uint2* runs = nullptr;             // column runs by (column, depth)
     const uint16_t* rows = nullptr;          // their row intervals
     bool allow_slices = true;                // the caller's choice for the next sort
+    DepthSort depth_sort = kSortBins;
+    bool totals_used[kTotalSets] = {false, false, false};   // written since the frame's head zeroed them
     bool sliced = false;                     // the frame renders in two depth slices
     bool split_last_slice = false;           // slice 1 renders tiles by pixel halves (f2)
     int runs_held = 0;                       // which Gaussians' column runs ws.pruns holds
@@ -247,7 +302,10 @@ void count_stage(std::atomic<uint32_t>& calls, const Workspace& ws, cudaStream_t
 // memory, so the kernels that read them can be captured once in a graph and
 // replayed for other cameras.
 void launch_set_frame_params(const FrameParams& p, FrameParams* d_fp, cudaStream_t stream);
-const void* set_frame_params_kernel();
+// A frame's first kernel: zeroes `words` words (a multiple of 4) and, unless
+// d_fp is null, stores the camera and settings as above.
+void launch_frame_head(const FrameParams& p, FrameParams* d_fp, uint32_t* zero, uint32_t words,
+                       cudaStream_t stream);
 
 // Stage orchestration shared by every entry point (pipeline.cu).
 // set_params = false leaves the camera/settings in ws.d_fp to the caller (a
@@ -296,9 +354,12 @@ struct PreprocessOut {
     float4* aux;
     uint32_t* depth_key;
     uint32_t* gbox;
+    uint32_t* bins;          // depth histogram (zeroed)
+    uint32_t* rank;          // each kept Gaussian's arrival rank in its bin
 };
 struct PreprocessBatch {
     int count = 0;
+    BinMap map;              // count 0: no histogram
     PreprocessOut cam[kMaxBatch];
 };
 // grid = chunks of 256 Gaussians x count, the camera index fastest
@@ -316,6 +377,24 @@ void launch_depth_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
                        uint32_t* vals_out, int64_t n, uint32_t* kept, bool first, int shift,
                        uint32_t* counts, uint32_t* totals, const uint32_t* pay_in,
                        uint32_t* pay_out, uint32_t* status, int grid, cudaStream_t stream);
+
+// The depth order by binning (bins.cu), from the histogram and ranks that
+// Preprocess left.  bin_scan: bins -> starts, windows; *largest (may be null)
+// gets the largest bin's count, counters (with set_counts) the Gaussians with
+// tiles.  bin_scatter: (key, index, box) records grouped by bin.  window_sort:
+// the records in order, with the outputs of launch_scan_tiles and, unless
+// slice0 is null, depth slice 0's counters (it may overwrite the records).
+int window_blocks_per_sm();
+void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, uint32_t* counters,
+                     bool set_counts, uint32_t* largest, cudaStream_t stream);
+void launch_bin_scatter(const uint32_t* keys, const uint32_t* ranks, const uint32_t* boxes,
+                        const uint32_t* bins, const FrameParams* fp, const BinMap& map, int64_t n,
+                        uint4* out, uint32_t* status, cudaStream_t stream);
+void launch_window_sort(uint4* recs, const uint32_t* win_lo, const uint32_t* gbox, int64_t n,
+                        int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
+                        uint32_t* chunk_first, unsigned long long* lookback, EpochRef epoch,
+                        uint32_t* counters, uint32_t* slice0, uint32_t* status, int grid,
+                        cudaStream_t stream);
 
 // SH colours (Sec. 3.2.1, stage 1's view-dependent colour) of the Gaussians
 // ids[0 .. *count) into their render records (rec[3 i + 2].xyz), on demand:
@@ -399,6 +478,11 @@ struct SliceState {
 #define ADR_SLICE_DIV 16
 #endif
 constexpr int kSliceDiv = ADR_SLICE_DIV;
+// Gaussians of slice 0: ceil(V / kSliceDiv), at least one when V > 0.
+__device__ __forceinline__ uint32_t slice0_count(uint32_t visible) {
+    const uint32_t div = kSliceDiv > 0 ? (uint32_t)kSliceDiv : 1u;
+    return visible == 0 ? 0u : max(1u, (visible + div - 1u) / div);
+}
 constexpr uint32_t kSliceProbe = 16;   // a context re-measures the slices every 16 frames
 // One camera's inputs and outputs of a Render launch.
 struct RenderCam {

@@ -1,0 +1,589 @@
+// The view-depth order of the Gaussians with tiles (the depth half of the
+// paper's (tile | depth) sort key, Sec. 3.2.1) by binning, with stage 2, the
+// scan of their column runs, in its last kernel.
+//
+// Preprocess adds every kept Gaussian to a histogram of its depth key (the
+// key's distance from the nearest key in units of 2^shift; a depth octave is
+// 512 to 8192 bins, by the scene's size) and keeps the count it found there,
+// its arrival rank in the bin.  Then
+//   k_bin_scan     turns the histogram into every bin's start (one cluster of 8
+//                  CTAs, block totals exchanged through distributed shared
+//                  memory) and finds where the windows begin: window w holds
+//                  the bins that start at positions [w kWindow, (w + 1) kWindow);
+//   k_bin_scatter  writes each Gaussian's (key, index) at its bin's start plus
+//                  its rank: the Gaussians are grouped by bin, in no order inside;
+//   k_window_sort  sorts one window at a time on chip and scans its run counts.
+// Keys equal in all 32 bits are ordered by Gaussian index, so the result is
+// that of the stable radix sort (sort.cu), whatever order the arrivals took.
+//
+// The radix sort's four passes are twelve launches whose time is the latency
+// of one 4096-key chunk's chain (load, sixteen ranking rounds, prefix,
+// write-out) several times over, whatever the number of keys; here a key is
+// moved once through memory and once through shared memory.  Measured with the
+// run scan that both need, us per frame (10k / 300k / 1.5M Gaussians with
+// tiles): see the table at kWindow.
+#include <cooperative_groups.h>
+
+#include "lookback.cuh"
+
+namespace adr {
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr int kScanCluster = 8;          // CTAs of k_bin_scan
+constexpr int kWinThreads = 256;
+constexpr int kWinItems = 8;
+constexpr int kWinCap = kWinThreads * kWinItems;   // Gaussians of a window sorted on chip
+constexpr int kLargeItems = 4;           // per thread and round of the large windows' radix sort
+constexpr int kSubBits = 12;
+constexpr int kSub = 1 << kSubBits;      // sub-bins of a window's key range
+constexpr int kWinWarps = kWinThreads / 32;
+
+// ---------------------------------------------------------------------------
+// Bin starts and window starts.  Warp w of CTA r holds the 128 kQuads bins from
+// 128 kQuads (r * warps + w) on, 4 consecutive bins a lane and load.
+// ---------------------------------------------------------------------------
+template <int kQuads>
+__global__ void __cluster_dims__(kScanCluster, 1, 1)
+k_bin_scan(uint32_t* __restrict__ bins, uint32_t* __restrict__ win_lo, uint32_t* __restrict__ counters,
+           int set_counts, uint32_t* __restrict__ largest) {
+    pdl_prologue();
+    __shared__ uint32_t s_w[32], s_max[32];
+    __shared__ uint32_t s_total, s_cta_max;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = (int)blockDim.x >> 5;
+    const uint32_t rank = cluster.block_rank();
+    uint4* b4 = reinterpret_cast<uint4*>(bins) + (size_t)(rank * (uint32_t)warps + (uint32_t)warp) * 32 * kQuads + lane;
+    uint4 v[kQuads];
+    uint32_t first[kQuads], sum = 0, big = 0;   // first: the warp's items before this lane's quad
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) v[q] = b4[32 * q];
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) {
+        const uint32_t t = v[q].x + v[q].y + v[q].z + v[q].w;
+        big = max(big, max(max(v[q].x, v[q].y), max(v[q].z, v[q].w)));
+        uint32_t incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        first[q] = sum + incl - t;
+        sum += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    big = __reduce_max_sync(0xffffffffu, big);
+    if (lane == 0) {
+        s_w[warp] = sum;
+        s_max[warp] = big;
+    }
+    __syncthreads();
+    uint32_t before = 0;
+    for (int w = 0; w < warp; ++w) before += s_w[w];
+    if (tid == (int)blockDim.x - 1) {
+        s_total = before + sum;
+        uint32_t m = 0;
+        for (int w = 0; w < warps; ++w) m = max(m, s_max[w]);
+        s_cta_max = m;
+    }
+    cluster.sync();
+    uint32_t total = 0, most = 0;
+#pragma unroll
+    for (uint32_t r = 0; r < (uint32_t)kScanCluster; ++r) {
+        const uint32_t t = *cluster.map_shared_rank(&s_total, r);
+        most = max(most, *cluster.map_shared_rank(&s_cta_max, r));
+        before += r < rank ? t : 0u;
+        total += t;
+    }
+    // A bin [s, e): the windows it starts (s a multiple of kWindow) begin at s;
+    // the windows whose first position falls inside it begin at e.
+    auto place = [&](uint32_t s, uint32_t& c) {
+        const uint32_t e = s + c;
+        uint32_t w = (s + (uint32_t)kWindow - 1u) / (uint32_t)kWindow;
+        if (c != 0u && w * (uint32_t)kWindow < e) {
+            if (w * (uint32_t)kWindow == s) win_lo[w++] = s;
+            for (; w * (uint32_t)kWindow < e; ++w) win_lo[w] = e;
+        }
+        c = s;
+        return e;
+    };
+#pragma unroll
+    for (int q = 0; q < kQuads; ++q) {
+        uint32_t s = before + first[q];
+        s = place(s, v[q].x);
+        s = place(s, v[q].y);
+        s = place(s, v[q].z);
+        place(s, v[q].w);
+        b4[32 * q] = v[q];
+    }
+    if (rank == 0 && tid == 0) {
+        win_lo[(total + (uint32_t)kWindow - 1u) / (uint32_t)kWindow] = total;
+        if (set_counts) {
+            counters[kCntVisible] = total;
+            counters[kCntDepthKept] = total;
+        }
+        if (largest) *largest = most;
+    }
+    cluster.sync();   // no CTA leaves while another reads its totals
+}
+
+// Four consecutive Gaussians per thread, 16-byte loads.
+__global__ void __launch_bounds__(256)
+k_bin_scatter(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ ranks,
+              const uint32_t* __restrict__ boxes, const uint32_t* __restrict__ bins, const FrameParams* __restrict__ fp, BinMap map,
+              int64_t n, uint4* __restrict__ out, uint32_t* __restrict__ status) {
+    pdl_prologue();
+    const uint32_t base = bin_base(fp->cam.near_z);
+    const int64_t i0 = 4 * ((int64_t)blockIdx.x * 256 + threadIdx.x);
+    if (i0 >= n) return;
+    uint32_t k[4], r[4], x[4];
+    if (i0 + 4 <= n) {
+        const uint4 a = *reinterpret_cast<const uint4*>(keys + i0);
+        const uint4 b = *reinterpret_cast<const uint4*>(ranks + i0);
+        const uint4 c = *reinterpret_cast<const uint4*>(boxes + i0);
+        k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
+        r[0] = b.x; r[1] = b.y; r[2] = b.z; r[3] = b.w;
+        x[0] = c.x; x[1] = c.y; x[2] = c.z; x[3] = c.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            k[q] = i0 + q < n ? keys[i0 + q] : 0xFFFFFFFFu;
+            r[q] = i0 + q < n ? ranks[i0 + q] : 0u;
+            x[q] = i0 + q < n ? boxes[i0 + q] : 0u;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (k[q] == 0xFFFFFFFFu) continue;   // no tiles
+        const uint32_t pos = bins[bin_of(k[q], base, map)] + r[q];
+        if ((int64_t)pos < n) out[pos] = make_uint4(k[q], (uint32_t)(i0 + q), x[q], 0u);
+        else atomicOr(status, kErrRange);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Window sort and run scan.
+// ---------------------------------------------------------------------------
+struct alignas(16) WindowShared {
+    union {
+        uint2 rec[kWinCap];                      // (key, index) grouped by sub-bin
+        struct {
+            uint32_t idx[kWinCap];               // the window in depth order
+            uint32_t box[kWinCap];
+        } out;
+        uint32_t warp_cnt[kWinWarps][kRadix];    // large windows: radix ranking
+    } u;
+    union {
+        uint32_t pair[kSub / 2 + 4];             // sub-bin counts, then starts, two 16-bit words each
+        uint32_t off[kWinCap];                   // run offsets from the window's first run
+        uint32_t run[kRadix];                    // large windows: next position of each digit
+    } c;
+    uint32_t w0[kWinWarps], w1[kWinWarps];
+    unsigned long long sums[2];                  // column runs and pairs of the window
+    uint32_t ticket, prefix;
+};
+static_assert(kWinCap * 2 == kSub && kWinCap < (1 << 16), "16-bit starts, thread t scans 16 sub-bins");
+
+__device__ __forceinline__ uint32_t box_runs(uint32_t box) { return ((box >> 16) & 0xFFu) + 1u; }
+__device__ __forceinline__ uint32_t box_rows(uint32_t box) { return (box >> 24) + 1u; }
+
+// Exclusive scan over the block of one value per thread; `total` the sum.
+__device__ __forceinline__ uint32_t win_scan(uint32_t v, uint32_t* s_w, uint32_t& total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    uint32_t base = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < kWinWarps; ++w) {
+        const uint32_t s = s_w[w];
+        base += w < warp ? s : 0u;
+        total += s;
+    }
+    __syncthreads();
+    return base + x - v;
+}
+
+// Window [lo, lo + m), m <= kWinCap, into sm.u.out in depth order.  Its key
+// range is cut into at most kSub sub-bins, filled with shared-memory atomics; a
+// Gaussian's place is its sub-bin's start plus the members before it (a window
+// has about kSub / 4 Gaussians, so most are alone in their sub-bin).
+__device__ __forceinline__ void sort_on_chip(WindowShared& sm, const uint4* __restrict__ recs, uint32_t lo,
+                                             int m) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint4 rec[kWinItems];   // key, index, box, then the place
+    uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        const int s = q * kWinThreads + tid;
+        if (s < m) rec[q] = recs[lo + s];
+    }
+    uint4* c4 = reinterpret_cast<uint4*>(sm.c.pair) + 2 * tid;
+    c4[0] = make_uint4(0u, 0u, 0u, 0u);
+    c4[1] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        if (q * kWinThreads + tid < m) {
+            kmin = min(kmin, rec[q].x);
+            kmax = max(kmax, rec[q].x);
+        }
+    }
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    if (lane == 0) {
+        sm.w0[warp] = kmin;
+        sm.w1[warp] = kmax;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kWinWarps; ++w) {
+        kmin = min(kmin, sm.w0[w]);
+        kmax = max(kmax, sm.w1[w]);
+    }
+    const int bits = 32 - __clz(kmax - kmin);
+    const int shift = bits > kSubBits ? bits - kSubBits : 0;
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        if (q * kWinThreads + tid < m) {   // .w: arrival rank in the sub-bin
+            const uint32_t sub = (rec[q].x - kmin) >> shift, half = 16u * (sub & 1u);
+            rec[q].w = (atomicAdd(&sm.c.pair[sub >> 1], 1u << half) >> half) & 0xFFFFu;
+        }
+    }
+    __syncthreads();
+    {
+        uint4 a = c4[0], b = c4[1];
+        uint32_t* v[8] = {&a.x, &a.y, &a.z, &a.w, &b.x, &b.y, &b.z, &b.w};
+        uint32_t sum = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sum += (*v[j] & 0xFFFFu) + (*v[j] >> 16);
+        uint32_t total;
+        uint32_t run = win_scan(sum, sm.w0, total);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t lo16 = *v[j] & 0xFFFFu, hi16 = *v[j] >> 16;
+            *v[j] = run | ((run + lo16) << 16);
+            run += lo16 + hi16;
+        }
+        c4[0] = a;
+        c4[1] = b;
+        if (tid == 0) sm.c.pair[kSub / 2] = (uint32_t)m;
+    }
+    __syncthreads();
+    const uint16_t* start = reinterpret_cast<const uint16_t*>(sm.c.pair);
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        if (q * kWinThreads + tid < m) {   // .w: slot
+            rec[q].w += start[(rec[q].x - kmin) >> shift];
+            sm.u.rec[rec[q].w] = make_uint2(rec[q].x, rec[q].y);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        if (q * kWinThreads + tid < m) {   // .w: place in the window
+            const uint32_t sub = (rec[q].x - kmin) >> shift;
+            const uint32_t s0 = start[sub], s1 = start[sub + 1];
+            if (s1 - s0 > 1u) {
+                uint32_t place = s0;
+                for (uint32_t j = s0; j < s1; ++j) {
+                    const uint2 r = sm.u.rec[j];
+                    place += (r.x < rec[q].x || (r.x == rec[q].x && r.y < rec[q].y)) ? 1u : 0u;
+                }
+                rec[q].w = place;
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kWinItems; ++q) {
+        if (q * kWinThreads + tid < m) {
+            sm.u.out.idx[rec[q].w] = rec[q].y;
+            sm.u.out.box[rec[q].w] = rec[q].z;
+        }
+    }
+    __syncthreads();
+}
+
+// A window of more than kWinCap Gaussians (one bin that large: very many
+// Gaussians at nearly one depth): a least-significant-digit radix sort by
+// (key, index) of the CTA alone, skipping the digits that all its Gaussians
+// share.  The window's 16-byte records make room for two buffers of (key, index).
+// Returns the one holding the result.
+__device__ const uint2* sort_large(WindowShared& sm, uint4* recs, uint32_t m) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint2 *src = reinterpret_cast<uint2*>(recs), *dst = src + m;
+    const uint4 first = recs[0];
+    uint32_t dk = 0, di = 0;
+    for (uint32_t c0 = 0; c0 < m; c0 += kWinThreads) {   // (key, index) into the first half, in place
+        const uint32_t s = c0 + tid;
+        const uint4 r = s < m ? recs[s] : first;
+        dk |= r.x ^ first.x;
+        di |= r.y ^ first.y;
+        __syncthreads();   // what is overwritten has been read
+        if (s < m) src[s] = make_uint2(r.x, r.y);
+        __syncthreads();
+    }
+    dk = __reduce_or_sync(0xffffffffu, dk);
+    di = __reduce_or_sync(0xffffffffu, di);
+    if (lane == 0) {
+        sm.w0[warp] = dk;
+        sm.w1[warp] = di;
+    }
+    __syncthreads();
+    for (int w = 0; w < kWinWarps; ++w) {
+        dk |= sm.w0[w];
+        di |= sm.w1[w];
+    }
+    uint32_t* run = sm.c.run;
+    for (int pass = 0; pass < 8; ++pass) {
+        const int shift = 8 * (pass & 3);
+        if ((((pass < 4 ? di : dk) >> shift) & 0xFFu) == 0u) continue;
+        auto digit = [&](uint2 r) { return ((pass < 4 ? r.y : r.x) >> shift) & 0xFFu; };
+        __syncthreads();
+        run[tid] = 0u;
+        __syncthreads();
+        for (uint32_t s = tid; s < m; s += kWinThreads) atomicAdd(&run[digit(src[s])], 1u);
+        __syncthreads();
+        uint32_t total;
+        run[tid] = win_scan(run[tid], sm.w0, total);
+        for (uint32_t c0 = 0; c0 < m; c0 += kWinThreads * kLargeItems) {
+            for (int d = lane; d < kRadix; d += 32) sm.u.warp_cnt[warp][d] = 0u;
+            __syncwarp();
+            uint2 rec[kLargeItems];
+            uint32_t at[kLargeItems];
+#pragma unroll
+            for (int q = 0; q < kLargeItems; ++q) {   // warp-striped, so the order is kept
+                const uint32_t s = c0 + warp * (kLargeItems * 32) + q * 32 + lane;
+                const bool in = s < m;
+                rec[q] = in ? src[s] : make_uint2(0u, 0u);
+                const uint32_t d = digit(rec[q]);
+                uint32_t peers = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+                for (int b = 0; b < kRadixBits; ++b) {
+                    const uint32_t ones = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                    peers &= ((d >> b) & 1u) ? ones : ~ones;
+                }
+                const uint32_t had = in ? sm.u.warp_cnt[warp][d] : 0u;
+                at[q] = had + __popc(peers & ((1u << lane) - 1u));
+                __syncwarp();
+                if (in && lane == 31 - __clz(peers)) sm.u.warp_cnt[warp][d] = had + __popc(peers);
+                __syncwarp();
+            }
+            __syncthreads();
+            uint32_t p = run[tid];
+            for (int w = 0; w < kWinWarps; ++w) {
+                const uint32_t c = sm.u.warp_cnt[w][tid];
+                sm.u.warp_cnt[w][tid] = p;
+                p += c;
+            }
+            run[tid] = p;
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < kLargeItems; ++q) {
+                const uint32_t s = c0 + warp * (kLargeItems * 32) + q * 32 + lane;
+                if (s < m) dst[sm.u.warp_cnt[warp][digit(rec[q])] + at[q]] = rec[q];
+            }
+            __syncthreads();
+        }
+        uint2* other = src;
+        src = dst;
+        dst = other;
+    }
+    __syncthreads();
+    return src;
+}
+
+// The parts of k_window_sort for a window that does not fit on chip: its order,
+// boxes and sums, and its run offsets.
+__device__ __noinline__ void order_large(WindowShared& sm, uint4* recs, uint32_t m, const uint32_t* gbox,
+                                         uint32_t* order, uint32_t* sorted_box) {
+    const uint2* sorted = sort_large(sm, recs, m);
+    if (threadIdx.x < 2) sm.sums[threadIdx.x] = 0ull;
+    __syncthreads();
+    unsigned long long runs = 0, pairs = 0;
+    for (uint32_t s = threadIdx.x; s < m; s += kWinThreads) {
+        const uint32_t i = sorted[s].y, box = gbox[i];
+        order[s] = i;
+        sorted_box[s] = box;
+        runs += box_runs(box);
+        pairs += box_runs(box) * box_rows(box);
+    }
+    atomicAdd(&sm.sums[0], runs);
+    atomicAdd(&sm.sums[1], pairs);
+}
+
+__device__ __noinline__ void offsets_large(WindowShared& sm, uint32_t lo, uint32_t m, const uint32_t* sorted_box,
+                                           uint32_t prefix, int64_t capacity, uint32_t* offsets,
+                                           uint32_t* chunk_first) {
+    for (uint32_t p0 = 0; p0 < m; p0 += kWinThreads) {
+        const uint32_t s = p0 + threadIdx.x;
+        const uint32_t t = s < m ? box_runs(sorted_box[lo + s]) : 0u;
+        uint32_t total;
+        const uint32_t run = sat_add(prefix, win_scan(t, sm.w0, total));
+        if (s < m) {
+            offsets[lo + s] = run;
+            mark_chunks(run, t, lo + s, capacity, chunk_first);
+        }
+        prefix = sat_add(prefix, total);
+    }
+}
+
+__global__ void __launch_bounds__(kWinThreads, 5)
+k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* __restrict__ gbox,
+              int64_t n_max, int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
+              uint32_t* __restrict__ chunk_first, unsigned long long* __restrict__ lookback, EpochRef eref,
+              uint32_t* counters, uint32_t* __restrict__ slice0, uint32_t* __restrict__ status,
+              LookbackTest lt) {
+    pdl_prologue();
+    __shared__ WindowShared sm;
+    const uint32_t epoch = (*eref.stage) * 8u + eref.pass;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t V = (uint32_t)min((int64_t)counters[kCntVisible], n_max);
+    const uint32_t windows = (V + (uint32_t)kWindow - 1u) / (uint32_t)kWindow;
+    unsigned long long* pairs64 = reinterpret_cast<unsigned long long*>(counters + kCntPairs64);
+    for (;;) {
+        // Windows are taken in order, so a window's predecessors are done or running.
+        if (tid == 0) sm.ticket = atomicAdd(counters + kCntScanTicket, 1u);
+        __syncthreads();
+        const uint32_t w = sm.ticket;
+        if (w >= windows) return;
+        const uint32_t lo = min(win_lo[w], V), hi = min(max(win_lo[w + 1], lo), V), m = hi - lo;
+        const bool on_chip = m <= (uint32_t)kWinCap;
+        if (on_chip) {
+            sort_on_chip(sm, recs, lo, (int)m);
+            // Thread t's eight consecutive Gaussians: their run offsets from the
+            // window's first run (at most 2048 x 256 runs, 2048 x 65536 pairs).
+            uint32_t runs = 0, pairs = 0, off[kWinItems];
+            const uint4* b4 = reinterpret_cast<const uint4*>(sm.u.out.box) + 2 * tid;
+            const uint4 a = b4[0], b = b4[1];
+            const uint32_t box[kWinItems] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int q = 0; q < kWinItems; ++q) {
+                off[q] = runs;
+                if (kWinItems * tid + q < (int)m) {
+                    runs += box_runs(box[q]);
+                    pairs += box_runs(box[q]) * box_rows(box[q]);
+                }
+            }
+            uint32_t total;
+            const uint32_t before = win_scan(runs, sm.w0, total);
+            uint4* o4 = reinterpret_cast<uint4*>(sm.c.off) + 2 * tid;
+            o4[0] = make_uint4(before + off[0], before + off[1], before + off[2], before + off[3]);
+            o4[1] = make_uint4(before + off[4], before + off[5], before + off[6], before + off[7]);
+            pairs = __reduce_add_sync(0xffffffffu, pairs);
+            if (lane == 0) sm.w1[warp] = pairs;
+            __syncthreads();
+            if (tid == 0) {
+                unsigned long long p = 0;
+                for (int q = 0; q < kWinWarps; ++q) p += sm.w1[q];
+                sm.sums[0] = total;
+                sm.sums[1] = p;
+            }
+        } else {
+            order_large(sm, recs + lo, m, gbox, order + lo, sorted_box + lo);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t total = (uint32_t)min(sm.sums[0], (unsigned long long)kSat);
+            if (lane == 0 && sm.sums[1]) atomicAdd(pairs64, sm.sums[1]);
+            const uint32_t excl = warp_lookback(lookback, w, total, epoch, status, counters, lt);
+            if (lane == 0) {
+                sm.prefix = excl;
+                if (w + 1 == windows) counters[kCntRuns] = sat_add(excl, total);
+            }
+        } else if (on_chip) {   // meanwhile the other warps write the order out
+            for (int s = tid - 32; s < (int)m; s += kWinThreads - 32) {
+                order[lo + s] = sm.u.out.idx[s];
+                sorted_box[lo + s] = sm.u.out.box[s];
+            }
+        }
+        __syncthreads();
+        if (on_chip) {
+            for (int s = tid; s < (int)m; s += kWinThreads) {
+                const uint32_t run = sat_add(sm.prefix, sm.c.off[s]);
+                offsets[lo + s] = run;
+                mark_chunks(run, box_runs(sm.u.out.box[s]), lo + s, capacity, chunk_first);
+            }
+        } else {
+            offsets_large(sm, lo, m, sorted_box, sm.prefix, capacity, offsets, chunk_first);
+        }
+        // The last window to finish closes the frame's counts: the pair total P
+        // (saturated to 31 bits) with the capacity flag, and depth slice 0.  If
+        // a lookback wait gave up, the run offsets are not a valid scan: P reads
+        // as saturated, so every later stage skips its work.
+        __threadfence();
+        __syncthreads();
+        if (tid == 0 && atomicAdd(counters + kCntWindowsDone, 1u) + 1u == windows) {
+            __threadfence();
+            const unsigned long long p = atomicAdd(pairs64, 0ull);
+            const bool failed = atomicAdd(counters + kCntScanFailed, 0u) != 0u;
+            const uint32_t pairs = failed ? kSat : (uint32_t)min(p, (unsigned long long)kSat);
+            counters[kCntPairs] = pairs;
+            if (!failed && p > (unsigned long long)capacity) atomicOr(status, kErrCapacity);
+            if (slice0) {
+                const uint32_t K0 = slice0_count(V);
+                slice0[kCntPairs] = pairs;
+                slice0[kCntVisible] = K0;
+                slice0[kCntRuns] = K0 < V ? __ldcg(offsets + K0) : __ldcg(counters + kCntRuns);
+                slice0[kCntDepthKept] = K0;
+            }
+        }
+    }
+}
+
+}  // namespace
+
+BinMap bin_map(int64_t n) {
+    BinMap m;
+    m.shift = n <= (1 << 15) ? 14 : n <= (1 << 18) ? 13 : n <= (1 << 19) ? 12 : n <= (1 << 20) ? 11 : 10;
+    m.count = (uint32_t)kBinOctaves << (23 - m.shift);
+    return m;
+}
+
+int window_blocks_per_sm() {
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_window_sort, kWinThreads, 0) != cudaSuccess)
+        return 1;
+    return b > 0 ? b : 1;
+}
+
+void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, uint32_t* counters,
+                     bool set_counts, uint32_t* largest, cudaStream_t stream) {
+    // 1, 2 or 4 quads of bins a lane in 256 to 1024 threads, for 2^13 to 2^17 bins
+    const int set = set_counts ? 1 : 0;
+    const uint32_t per_cta = map.count / kScanCluster;
+    if (per_cta <= 1024)
+        launch_pdl(k_bin_scan<1>, kScanCluster, per_cta / 4, 0, stream, bins, win_lo, counters, set, largest);
+    else if (per_cta <= 2048)
+        launch_pdl(k_bin_scan<2>, kScanCluster, per_cta / 8, 0, stream, bins, win_lo, counters, set, largest);
+    else
+        launch_pdl(k_bin_scan<4>, kScanCluster, per_cta / 16, 0, stream, bins, win_lo, counters, set, largest);
+}
+
+void launch_bin_scatter(const uint32_t* keys, const uint32_t* ranks, const uint32_t* boxes,
+                        const uint32_t* bins, const FrameParams* fp, const BinMap& map, int64_t n,
+                        uint4* out, uint32_t* status, cudaStream_t stream) {
+    if (n <= 0) return;
+    launch_pdl(k_bin_scatter, (unsigned)((n + 1023) / 1024), 256, 0, stream, keys, ranks, boxes, bins, fp, map,
+               n, out, status);
+}
+
+void launch_window_sort(uint4* recs, const uint32_t* win_lo, const uint32_t* gbox, int64_t n,
+                        int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
+                        uint32_t* chunk_first, unsigned long long* lookback, EpochRef epoch,
+                        uint32_t* counters, uint32_t* slice0, uint32_t* status, int grid,
+                        cudaStream_t stream) {
+    if (n <= 0) return;
+    const int64_t most = (n + kWindow - 1) / kWindow;
+    launch_pdl(k_window_sort, (unsigned)(most < grid ? most : grid), kWinThreads, 0, stream, recs, win_lo, gbox,
+               n, capacity, order, sorted_box, offsets, chunk_first, lookback, epoch, counters, slice0, status,
+               lookback_test());
+}
+
+}  // namespace adr

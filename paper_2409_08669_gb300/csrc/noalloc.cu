@@ -45,9 +45,10 @@ constexpr size_t kOffDepth = align256(kOffAux + kNaMaxGaussians * kAuxFloat4 * 1
 constexpr size_t kOffOffsets = align256(kOffDepth + kNaMaxGaussians * 4);
 constexpr size_t kOffGBox = align256(kOffOffsets + kNaMaxGaussians * 4);
 constexpr size_t kOffSortedBox = align256(kOffGBox + kNaMaxGaussians * 4);
-constexpr size_t kOffGKeys = align256(kOffSortedBox + kNaMaxGaussians * 4);   // 2 buffers
-constexpr size_t kOffGVals = align256(kOffGKeys + 2 * kNaMaxGaussians * 4);   // 2 buffers
-constexpr size_t kOffPRuns = align256(kOffGVals + 2 * kNaMaxGaussians * 4);
+constexpr size_t kOffSortBuf = align256(kOffSortedBox + kNaMaxGaussians * 4);
+constexpr size_t kOffOrder = align256(kOffSortBuf + kNaMaxGaussians * 16);
+constexpr size_t kOffWinLo = align256(kOffOrder + kNaMaxGaussians * 4);
+constexpr size_t kOffPRuns = align256(kOffWinLo + (kNaMaxGaussians / kWindow + 2) * 4);
 constexpr size_t kOffPRows = align256(kOffPRuns + kNaMaxPairs * 8);
 constexpr size_t kOffPGauss = align256(kOffPRows + (kNaMaxPairs + 8) * 2);
 constexpr size_t kOffChunkFirst = align256(kOffPGauss + kNaMaxPairs * 4);
@@ -57,13 +58,13 @@ constexpr size_t kOffTrav = align256(kOffLast + kPixels * 4);
 constexpr size_t kOffTfin = align256(kOffTrav + kPixels * 4);
 constexpr size_t kOffHist = align256(kOffTfin + kPixels * 4);
 constexpr size_t kOffCounters = align256(kOffHist + kHistWords * 4);
-constexpr size_t kOffStatus = align256(kOffCounters + kCntSlots * 4);
+constexpr size_t kNaZeroWords = kZeroWords + kMaxBins;   // more than bin_map(kNaMaxGaussians) asks for
+constexpr size_t kOffStatus = align256(kOffCounters + kNaZeroWords * 4);
 constexpr size_t kLookbackWords = (kNaMaxGaussians / kSortChunk + 2) * kRadix;
 constexpr size_t kOffFrameParams = align256(kOffStatus + 16);
 constexpr size_t kOffStage = align256(kOffFrameParams + sizeof(FrameParams));
 constexpr size_t kOffTCounts = align256(kOffStage + 16);
-constexpr size_t kOffTTotals = align256(kOffTCounts + (size_t)kRadix * kMaxTileGrid * 4);
-constexpr size_t kOffTileCounts = align256(kOffTTotals + 2 * kRadix * 4);
+constexpr size_t kOffTileCounts = align256(kOffTCounts + (size_t)kRadix * kMaxTileGrid * 4);
 constexpr size_t kOffLookback = align256(kOffTileCounts + kNaMaxTiles * 4);
 constexpr size_t kNaBytes = align256(kOffLookback + kLookbackWords * 8);
 
@@ -102,6 +103,7 @@ adr_status setup(int dev, DeviceState*& out) {
         w.sm_count = sms;
         w.sort_grid = sms * onesweep_blocks_per_sm();
         w.scan_grid = sms * scan_blocks_per_sm();
+        w.window_grid = sms * window_blocks_per_sm();
         w.tile_grid = sms * tile_scatter_blocks_per_sm();
         if (w.tile_grid > kMaxTileGrid) w.tile_grid = kMaxTileGrid;
         w.rec = reinterpret_cast<float4*>(b + kOffRec);
@@ -110,23 +112,23 @@ adr_status setup(int dev, DeviceState*& out) {
         w.offsets = reinterpret_cast<uint32_t*>(b + kOffOffsets);
         w.gbox = reinterpret_cast<uint32_t*>(b + kOffGBox);
         w.sorted_box = reinterpret_cast<uint32_t*>(b + kOffSortedBox);
-        for (int k = 0; k < 2; ++k) {
-            w.gkeys[k] = reinterpret_cast<uint32_t*>(b + kOffGKeys) + k * kNaMaxGaussians;
-            w.gvals[k] = reinterpret_cast<uint32_t*>(b + kOffGVals) + k * kNaMaxGaussians;
-        }
+        w.sortbuf = reinterpret_cast<uint4*>(b + kOffSortBuf);
+        w.order = reinterpret_cast<uint32_t*>(b + kOffOrder);
+        w.win_lo = reinterpret_cast<uint32_t*>(b + kOffWinLo);
         w.pruns = reinterpret_cast<uint2*>(b + kOffPRuns);
         w.prows = reinterpret_cast<uint16_t*>(b + kOffPRows);
         w.pgauss = reinterpret_cast<uint32_t*>(b + kOffPGauss);
         w.tile_counts = reinterpret_cast<uint32_t*>(b + kOffTileCounts);
         w.tcounts = reinterpret_cast<uint32_t*>(b + kOffTCounts);
-        w.ttotals = reinterpret_cast<uint32_t*>(b + kOffTTotals);
         w.chunk_first = reinterpret_cast<uint32_t*>(b + kOffChunkFirst);
         w.ranges = reinterpret_cast<uint2*>(b + kOffRanges);
         w.last = reinterpret_cast<int32_t*>(b + kOffLast);
         w.trav = reinterpret_cast<int32_t*>(b + kOffTrav);
         w.tfin = reinterpret_cast<float*>(b + kOffTfin);
         w.hist = reinterpret_cast<uint32_t*>(b + kOffHist);
-        w.counters = reinterpret_cast<uint32_t*>(b + kOffCounters);
+        w.counters = reinterpret_cast<uint32_t*>(b + kOffCounters);   // the zeroed block, no depth slices
+        w.ttotals = w.counters + 3 * kCntSlots;
+        w.bins = w.counters + kZeroWords;
         w.status = reinterpret_cast<uint32_t*>(b + kOffStatus);
         w.lookback = reinterpret_cast<unsigned long long*>(b + kOffLookback);
         w.d_fp = reinterpret_cast<FrameParams*>(b + kOffFrameParams);

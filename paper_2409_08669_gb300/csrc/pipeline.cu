@@ -42,13 +42,26 @@ void Profiler::end(cudaStream_t s) {
 namespace {
 __global__ void k_set_frame_params(FrameParams p, FrameParams* __restrict__ out) {
     pdl_prologue(); *out = p; }
+
+constexpr int kHeadThreads = 256;
+__global__ void __launch_bounds__(kHeadThreads)
+k_frame_head(FrameParams p, FrameParams* __restrict__ out, uint4* __restrict__ zero, uint32_t quads) {
+    pdl_prologue();
+    const uint32_t i = blockIdx.x * kHeadThreads + threadIdx.x;
+    if (i < quads) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (i == 0 && out) *out = p;
+}
 }  // namespace
 
 void launch_set_frame_params(const FrameParams& p, FrameParams* d_fp, cudaStream_t stream) {
     launch_pdl(k_set_frame_params, 1, 1, 0, stream, p, d_fp);
 }
 
-const void* set_frame_params_kernel() { return reinterpret_cast<const void*>(&k_set_frame_params); }
+void launch_frame_head(const FrameParams& p, FrameParams* d_fp, uint32_t* zero, uint32_t words,
+                       cudaStream_t stream) {
+    launch_pdl(k_frame_head, (words / 4 + kHeadThreads - 1) / kHeadThreads, kHeadThreads, 0, stream, p, d_fp,
+               reinterpret_cast<uint4*>(zero), words / 4);
+}
 
 void count_stage(std::atomic<uint32_t>& calls, const Workspace& ws, cudaStream_t stream) {
     // The device tag is (stage count) * 8 + pass in 32 bits; clear the lookback
@@ -67,44 +80,66 @@ void fill_frame_state(FrameState& fs, int64_t n, const CamDev& cam, const SetDev
     fs.sorted_gauss = nullptr;
 }
 
-// Before Preprocess: the stage tag, the frame parameters and the counters.
+// Before Preprocess: the stage tag, the frame parameters and the zeroed words.
 static void preprocess_head(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& epoch,
                             cudaStream_t stream, bool set_params) {
     count_stage(epoch, ws, stream);
-    if (set_params) launch_set_frame_params(FrameParams{fs.cam, fs.st}, ws.d_fp, stream);
-    cudaMemsetAsync(ws.counters, 0, kCntSlots * sizeof(uint32_t), stream);
-    cudaMemsetAsync(ws.hist, 0, kHistWords * sizeof(uint32_t), stream);
+    launch_frame_head(FrameParams{fs.cam, fs.st}, set_params ? ws.d_fp : nullptr, ws.counters,
+                      kZeroWords + bin_map(fs.n).count, stream);
+    for (bool& used : fs.totals_used) used = false;
+}
+
+static BinMap frame_bins(const FrameState& fs) {
+    return fs.depth_sort == kSortRadix ? BinMap{} : bin_map(fs.n);
 }
 
 static PreprocessOut preprocess_out(const Workspace& ws) {
-    return PreprocessOut{ws.d_fp, ws.d_stage, ws.rec, ws.aux, ws.depth_key, ws.gbox};
+    // the ranks sit in the run offsets' array, which is written after their last use
+    return PreprocessOut{ws.d_fp, ws.d_stage, ws.rec, ws.aux, ws.depth_key, ws.gbox, ws.bins, ws.offsets};
 }
 
-// After Preprocess: the Gaussians by view depth, then the run scan.
+// After Preprocess: the Gaussians by view depth and the scan of their column
+// runs (stage 2, + bookkeeping for stage 3), over the V Gaussians with tiles.
 static void preprocess_tail(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
     const int64_t n = fs.n;
-    // Gaussians by view depth: 4 stable 8-bit passes over the V Gaussians with
-    // tiles (the first pass drops the others, key 0xFFFFFFFF, and counts the
-    // V).  The last pass carries the packed rectangles into depth order.
+    const EpochRef ep{ws.d_stage, (uint32_t)kMaxPasses};
+    const BinMap map = bin_map(n);
+    fs.order = ws.order;
+    if (fs.depth_sort != kSortRadix)
+        TIMED(ws, kKDepthPass, stream,
+              launch_bin_scan(ws.bins, map, ws.win_lo, ws.counters, fs.depth_sort == kSortBins, ws.largest_bin,
+                              stream));
+    if (fs.depth_sort == kSortBins) {
+        TIMED(ws, kKDepthPass, stream,
+              launch_bin_scatter(ws.depth_key, ws.offsets, ws.gbox, ws.bins, ws.d_fp, map, n, ws.sortbuf,
+                                 ws.status, stream));
+        TIMED(ws, kKDepthPass, stream,
+              launch_window_sort(ws.sortbuf, ws.win_lo, ws.gbox, n, ws.capacity, ws.order,
+                                 ws.sorted_box, ws.offsets, ws.chunk_first, ws.lookback, ep, ws.counters,
+                                 ws.slice_counters, ws.status, ws.window_grid, stream));
+        return;
+    }
+    // Very many Gaussians in one bin: 4 stable 8-bit passes (the first drops the
+    // Gaussians without tiles, key 0xFFFFFFFF, and counts the V; the last
+    // carries the packed rectangles into depth order), then the run scan.
+    cudaMemsetAsync(ws.hist, 0, kHistWords * sizeof(uint32_t), stream);
     const uint32_t* kin = ws.depth_key;
     const uint32_t* vin = nullptr;
     for (int p = 0; p < kMaxPasses; ++p) {
+        uint32_t* keys = reinterpret_cast<uint32_t*>(ws.sortbuf) + (size_t)(p & 1) * 2 * ws.max_n;
+        uint32_t* vals = p + 1 == kMaxPasses ? ws.order : keys + ws.max_n;
         TIMED(ws, kKDepthPass, stream,
-              launch_depth_pass(kin, vin, ws.gkeys[p & 1], ws.gvals[p & 1], n,
-                                ws.counters + kCntDepthKept, p == 0, 8 * p, ws.tcounts,
+              launch_depth_pass(kin, vin, keys, vals, n, ws.counters + kCntDepthKept, p == 0, 8 * p, ws.tcounts,
                                 ws.hist + p * kRadix, p + 1 == kMaxPasses ? ws.gbox : nullptr,
                                 p + 1 == kMaxPasses ? ws.sorted_box : nullptr, ws.status,
                                 ws.sort_grid, stream));
-        kin = ws.gkeys[p & 1];
-        vin = ws.gvals[p & 1];
+        kin = keys;
+        vin = vals;
     }
-    fs.order = vin;
-    // Stage 2 (+ bookkeeping for stage 3): scan of tile counts in depth order
-    // over the V Gaussians with tiles.
-    const EpochRef ep{ws.d_stage, (uint32_t)kMaxPasses};
     TIMED(ws, kKScanTiles, stream,
           launch_scan_tiles(ws.sorted_box, n, ws.capacity, ws.offsets, ws.chunk_first, ws.lookback,
                             ep, ws.counters, ws.status, ws.scan_grid, stream));
+    if (ws.slice_counters) launch_slice0_setup(ws.counters, ws.offsets, ws.slice_counters, stream);
 }
 
 void enqueue_preprocess(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& epoch,
@@ -119,6 +154,7 @@ void enqueue_preprocess(const Workspace& ws, FrameState& fs, std::atomic<uint32_
     // deferred to Render) the SH colour.
     PreprocessBatch pb;
     pb.count = 1;
+    pb.map = frame_bins(fs);
     pb.cam[0] = preprocess_out(ws);
     TIMED(ws, kKPreprocess, stream,
           launch_preprocess((int)fs.n, means, scales, rots, opac, defer_colors ? nullptr : sh, pb,
@@ -126,10 +162,19 @@ void enqueue_preprocess(const Workspace& ws, FrameState& fs, std::atomic<uint32_
     preprocess_tail(ws, fs, stream);
 }
 
+// One of the tile passes' total sets, zero: as the frame's head left it, or
+// cleared again for a second pass of the frame.
+static uint32_t* fresh_totals(const Workspace& ws, FrameState& fs, TotalSet which, cudaStream_t stream) {
+    uint32_t* totals = ws.ttotals + (int)which * kRadix;
+    if (fs.totals_used[which]) cudaMemsetAsync(totals, 0, kRadix * sizeof(uint32_t), stream);
+    fs.totals_used[which] = true;
+    return totals;
+}
+
 // Stage 4, pass 2 and stage 5: the pairs of the column runs grouped by tile
 // row (per-tile lists), then every tile's [start, end).
 static void enqueue_tile_pass2(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
-    cudaMemsetAsync(ws.ttotals + kRadix, 0, kRadix * sizeof(uint32_t), stream);
+    uint32_t* totals = fresh_totals(ws, fs, kTotalsRows, stream);
     cudaMemsetAsync(ws.tile_counts, 0, (size_t)fs.num_tiles * sizeof(uint32_t), stream);
     if (fs.n > 0 && fs.order) {
         // The runs' pair counts vary, so the pass uses many small run ranges
@@ -137,10 +182,10 @@ static void enqueue_tile_pass2(const Workspace& ws, FrameState& fs, cudaStream_t
         const int G2 = kMaxTileGrid;
         TIMED(ws, kKTileCountRows, stream,
               launch_tile_count_rows(ws.pruns, ws.counters, ws.capacity, fs.cam.tiles_x, fs.num_tiles,
-                                     ws.tcounts, ws.ttotals + kRadix, ws.tile_counts, ws.status, G2,
+                                     ws.tcounts, totals, ws.tile_counts, ws.status, G2,
                                      stream));
         TIMED(ws, kKTileCountScan, stream,
-              launch_tile_count_scan(ws.tcounts, ws.ttotals + kRadix, G2, stream));
+              launch_tile_count_scan(ws.tcounts, totals, G2, stream));
         TIMED(ws, kKTileScatterRows, stream,
               launch_tile_scatter_rows(ws.pruns, ws.counters, ws.capacity, ws.tcounts, ws.pgauss,
                                        ws.status, G2, fs.cam.tiles_y, stream));
@@ -155,14 +200,14 @@ static void enqueue_tile_pass2(const Workspace& ws, FrameState& fs, cudaStream_t
 // Stage 3-4, pass 1: the column runs of `src`'s Gaussians, generated on chip
 // and grouped by tile column (stage 5, each column's [start, end), is the
 // prefix of the per-column totals, which Render takes itself).
-static void enqueue_pass1(const Workspace& ws, const FrameState& fs, const PairSource& src,
+static void enqueue_pass1(const Workspace& ws, FrameState& fs, const PairSource& src, TotalSet which,
                           cudaStream_t stream) {
     const int G = ws.tile_grid;
-    cudaMemsetAsync(ws.ttotals, 0, kRadix * sizeof(uint32_t), stream);
+    uint32_t* totals = fresh_totals(ws, fs, which, stream);
     if (fs.n > 0 && fs.order) {
         TIMED(ws, kKTileCountColumns, stream,
-              launch_tile_count_columns(src, ws.tcounts, ws.ttotals, ws.status, G, stream));
-        TIMED(ws, kKTileCountScan, stream, launch_tile_count_scan(ws.tcounts, ws.ttotals, G, stream));
+              launch_tile_count_columns(src, ws.tcounts, totals, ws.status, G, stream));
+        TIMED(ws, kKTileCountScan, stream, launch_tile_count_scan(ws.tcounts, totals, G, stream));
         TIMED(ws, kKTileScatterColumns, stream,
               launch_tile_scatter_columns(src, ws.tcounts, ws.pruns, ws.prows, ws.status, G, stream));
     }
@@ -200,12 +245,10 @@ void enqueue_sort(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& ep
     if (fs.sliced) {
         // Slice 0: the nearest Gaussians' runs; Render builds slice 1 from what
         // its pixels still need.
-        cudaMemsetAsync(ws.slice_counters, 0, 2 * kCntSlots * sizeof(uint32_t), stream);
-        launch_slice0_setup(ws.counters, ws.offsets, ws.slice_counters, stream);
-        enqueue_pass1(ws, fs, pair_source(ws, fs, 0), stream);
+        enqueue_pass1(ws, fs, pair_source(ws, fs, 0), kTotalsFirst, stream);
         fs.runs_held = kRunsSlice0;
     } else {
-        enqueue_pass1(ws, fs, pair_source(ws, fs, -1), stream);
+        enqueue_pass1(ws, fs, pair_source(ws, fs, -1), kTotalsFirst, stream);
         fs.runs_held = kRunsAll;
     }
 }
@@ -213,7 +256,7 @@ void enqueue_sort(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& ep
 void enqueue_tile_lists(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
     if (fs.lists == kListsTiles) return;
     if (fs.runs_held != kRunsAll) {   // the column runs of every Gaussian first
-        enqueue_pass1(ws, fs, pair_source(ws, fs, -1), stream);
+        enqueue_pass1(ws, fs, pair_source(ws, fs, -1), kTotalsFirst, stream);
         fs.runs_held = kRunsAll;
     }
     enqueue_tile_pass2(ws, fs, stream);
@@ -238,7 +281,7 @@ static RenderCam render_cam(const Workspace& ws, const FrameState& fs, float* im
     rc.tfin = ws.tfin;
     rc.lstat = ws.lstat;
     rc.trace = ws.tile_trace;
-    rc.ss.col_totals = ws.ttotals;
+    rc.ss.col_totals = ws.ttotals + (phase == 2 ? (int)kTotalsSlice1 : (int)kTotalsFirst) * kRadix;
     rc.ss.capacity = ws.capacity;
     rc.ss.phase = phase;
     rc.ss.col_counters = phase == 0 ? ws.counters
@@ -291,7 +334,7 @@ static void slice1_runs(const Workspace& ws, FrameState& fs, cudaStream_t stream
                            fs.order, ws.counters, surv_grid, ws.surv_cnt, ws.surv_flag, ws.max_n,
                            ws.capacity / kSortChunk + 2, ws.s_order, ws.s_box, ws.s_offsets,
                            ws.s_chunk_first, c1, ws.status, stream));
-    enqueue_pass1(ws, fs, pair_source(ws, fs, 1), stream);
+    enqueue_pass1(ws, fs, pair_source(ws, fs, 1), kTotalsSlice1, stream);
     fs.runs_held = kRunsSlice1;
 }
 
@@ -329,7 +372,7 @@ static void render_items(const BatchItem* items, int count, cudaStream_t stream,
     }
     per_item(items, count, stream, bs, [&](int b, cudaStream_t s) {
         const BatchItem& it = items[b];
-        if (it.fs->runs_held != kRunsSlice0) enqueue_pass1(*it.ws, *it.fs, pair_source(*it.ws, *it.fs, 0), s);
+        if (it.fs->runs_held != kRunsSlice0) enqueue_pass1(*it.ws, *it.fs, pair_source(*it.ws, *it.fs, 0), kTotalsFirst, s);
         it.fs->runs_held = kRunsSlice0;
         enqueue_colors(*it.ws, *it.fs, 1, s);
     });
@@ -353,6 +396,7 @@ void enqueue_frame_batch(const BatchItem* items, int count, const float* means, 
     if (count < 1 || count > kMaxBatch) return;
     PreprocessBatch pb;
     pb.count = count;
+    pb.map = frame_bins(*items[0].fs);
     for (int b = 0; b < count; ++b) {
         const BatchItem& it = items[b];
         preprocess_head(*it.ws, *it.fs, *it.epoch, stream, set_params);

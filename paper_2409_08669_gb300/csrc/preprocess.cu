@@ -189,6 +189,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
     float4* __restrict__ aux = out.aux;
     uint32_t* __restrict__ depth_key = out.depth_key;
     uint32_t* __restrict__ gbox = out.gbox;
+    uint32_t rank = 0;   // arrival rank in the depth bin
 
     const float mx = means[3 * i + 0], my = means[3 * i + 1], mz = means[3 * i + 2];
     // Sort depth: fixed evaluation order, each operation rounded separately.
@@ -296,6 +297,9 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
                 rc = make_ushort4((unsigned short)tx0, (unsigned short)ty0, (unsigned short)tx1,
                                   (unsigned short)ty1);
                 key = __float_as_uint(depth);
+                // The depth histogram (bins.cu); the count comes back while the
+                // SH coefficients are on their way.
+                if (batch.map.count) rank = atomicAdd(out.bins + bin_of(key, bin_base(cam.near_z), batch.map), 1u);
                 // SH colour, d = normalise(X0 - cam_pos); with sh == nullptr
                 // (deferred colours) k_colors fills .xyz in for the Gaussians
                 // a Render launch blends.
@@ -321,6 +325,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
         rec[3 * i + 1] = r1;
         rec[3 * i + 2] = r2;
         aux[2 * i + 0] = a0;
+        out.rank[i] = rank;
     }
     aux[2 * i + 1] = a1;
     depth_key[i] = key;

@@ -48,6 +48,8 @@ struct Scene {
     int64_t n;
     SetDev st;
     double pairs_per_pixel = -1.0;   // learned; < 0 = unknown
+    uint32_t largest_bin = 0;        // of the last completed frame with a depth histogram
+    uint32_t radix_probe_in = kRadixProbe;   // see next_depth_sort
 };
 
 enum ReqState { kQueued, kRunning, kDone };
@@ -74,7 +76,7 @@ struct Slot {
     std::atomic<uint32_t> calls{0};
     cudaStream_t stream = nullptr;     // this camera's sort stages within a batch
     float* img = nullptr;              // slot-owned image the graph renders into
-    uint32_t* host_words = nullptr;    // pinned: status word, pair count
+    uint32_t* host_words = nullptr;    // pinned: status word, pair count, largest depth bin
 };
 
 // max_batch slots that render one batch at a time.
@@ -84,7 +86,7 @@ struct Group {
     cudaEvent_t done = nullptr;
     BatchStreams bs{};
     std::vector<Request*> reqs;        // the batch in flight (empty: free)
-    // key: scene, batch size, then width and height of each camera
+    // key: scene, batch size, depth sort, then width and height of each camera
     std::map<std::vector<int>, GraphEntry> graphs;
 };
 
@@ -175,16 +177,18 @@ adr_status capture_batch(adr_server* s, Group& g, const Scene& sc, GraphEntry& g
 }
 
 adr_status run_batch(adr_server* s, Group& g) {
-    const Scene& sc = s->scenes[g.reqs[0]->scene];
+    Scene& sc = s->scenes[g.reqs[0]->scene];
     const int k = (int)g.reqs.size();
     cudaStream_t strm = g.stream;
+    const DepthSort depth_sort = next_depth_sort(sc.largest_bin, sc.radix_probe_in);
     for (int b = 0; b < k; ++b) {
         Slot& sl = *g.slots[b];
         fill_frame_state(sl.fs, sc.n, g.reqs[b]->cam, sc.st);
+        sl.fs.depth_sort = depth_sort;
         SERVE_CUDA("clearing the status word", cudaMemsetAsync(sl.ws.status, 0, 16, strm));
     }
     if (s->cfg.use_graphs) {
-        std::vector<int> key{g.reqs[0]->scene, k};
+        std::vector<int> key{g.reqs[0]->scene, k, (int)depth_sort};
         for (int b = 0; b < k; ++b) {
             key.push_back(g.reqs[b]->cam.width);
             key.push_back(g.reqs[b]->cam.height);
@@ -230,7 +234,8 @@ adr_status run_batch(adr_server* s, Group& g) {
 
 #undef SERVE_CUDA
 
-void finish_request(adr_server* s, Request* r, uint32_t bits, uint32_t pairs, cudaError_t q) {
+void finish_request(adr_server* s, Request* r, const uint32_t* host_words, cudaError_t q) {
+    const uint32_t bits = host_words[0], pairs = host_words[1];
     r->t_done = now_ms();
     if (q != cudaSuccess) {
         r->result = ADR_ERR_CUDA;
@@ -242,6 +247,7 @@ void finish_request(adr_server* s, Request* r, uint32_t bits, uint32_t pairs, cu
         if (rep.status == ADR_ERR_CUDA) snprintf(s->error, sizeof(s->error), "%s", rep.message);
     }
     Scene& sc = s->scenes[r->scene];
+    if (q == cudaSuccess) sc.largest_bin = host_words[2];
     if (q == cudaSuccess && !(bits & kErrLookback)) {   // a skipped frame's pair count is not a measurement
         const double ppp = (double)pairs / ((double)r->cam.width * r->cam.height);
         sc.pairs_per_pixel = sc.pairs_per_pixel < 0 ? ppp
@@ -266,7 +272,7 @@ void scheduler(adr_server* s) {
             const cudaError_t q = cudaEventQuery(g->done);
             if (q == cudaErrorNotReady) continue;
             for (size_t b = 0; b < g->reqs.size(); ++b)
-                finish_request(s, g->reqs[b], g->slots[b]->host_words[0], g->slots[b]->host_words[1], q);
+                finish_request(s, g->reqs[b], g->slots[b]->host_words, q);
             g->reqs.clear();
             progressed = true;
         }
@@ -384,7 +390,8 @@ adr_status adr_serve_create(adr_server** out, const adr_serve_config* cfg) {
         if (st != ADR_OK ||
             cudaStreamCreateWithFlags(&sl->stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaMalloc((void**)&sl->img, (size_t)3 * cfg->max_width * cfg->max_height * sizeof(float)) != cudaSuccess ||
-            cudaHostAlloc((void**)&sl->host_words, 16, cudaHostAllocDefault) != cudaSuccess) {
+            cudaHostAlloc((void**)&sl->host_words, 16, cudaHostAllocDefault) != cudaSuccess ||
+            cudaHostGetDevicePointer((void**)&sl->ws.largest_bin, sl->host_words + 2, 0) != cudaSuccess) {
             (void)cudaGetLastError();   // an allocation error is not sticky: clear it
             destroy_server(s);
             return report_error(ADR_ERR_CUDA, "adr_serve_create: slot allocation failed");

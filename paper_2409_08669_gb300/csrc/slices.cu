@@ -25,12 +25,6 @@ namespace {
 
 constexpr int kSurvThreads = 256;
 
-// Gaussians of slice 0: ceil(V / kSliceDiv), at least one when V > 0.
-__device__ __forceinline__ uint32_t slice0_count(uint32_t visible) {
-    const uint32_t div = kSliceDiv > 0 ? (uint32_t)kSliceDiv : 1u;
-    return visible == 0 ? 0u : max(1u, (visible + div - 1u) / div);
-}
-
 __global__ void k_slice0_setup(const uint32_t* __restrict__ counters,
                                const uint32_t* __restrict__ offsets, uint32_t* __restrict__ c0) {
     pdl_prologue();
