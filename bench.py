@@ -59,11 +59,12 @@ def select_workload(name):
     WORKLOAD, N_GAUSS, WIDTH, HEIGHT, PAIR_CAPACITY = name, n, w, h, cap
     return kind
 EVAL_FP32_OPS = 15        # FP32 lane operations per Gaussian-pixel evaluation in Render
-# Kernels of one forward frame: frame head 1, preprocess 1, depth order (bin
-# scan, bin scatter, window sort with the run scan) 3, tile pass 1 (count, count scan, scatter) 3, render slice 0 1,
-# unfinished-tile table (rows, columns) + compaction (count, scan, scatter) 5,
+# Kernels of one sliced forward frame: frame head 1, preprocess 1, depth order of
+# slice 0 (bin scan, bin scatter, window sort with the run scan) 3, tile pass 1 (count, count scan, scatter) 3, render slice 0 1,
+# unfinished-tile table (rows, columns) 2, depth order of slice 1 (its selection
+# into bins, bin scan, bin scatter, window sort) 4,
 # tile pass 1 of slice 1 3, render slice 1 1 (each render derives its column ranges).
-KERNELS_PER_FRAME = 18
+KERNELS_PER_FRAME = 19
 # DRAM bytes (read + write) of one launch from one-pass ncu captures at the
 # heavy 3M-Gaussian 1080p frame: Render (profiles/render_heavy-3M-1080p_traffic.md,
 # its two launches of one frame, 54.8 MB) and the per-tile list pass
@@ -389,9 +390,10 @@ def kernel_bytes(name, n, u, hw):
     return {
         # params (+SH of kept) in; records of kept (64 B), radii/depth, key, box out
         "preprocess": 44 * n + 192 * V + 40 * n + 64 * V,
-        # n keys, ranks and rectangles in, V records of 16 B out and in, and the
-        # order, rectangles and run offsets out
-        "depth_pass": 12 * n + 44 * V,
+        # n keys and ranks in; of the Gaussians ordered here (all with tiles, or
+        # depth slice 0 of a sliced frame) a rectangle in, a record of 16 B out
+        # and in, and the order, rectangle and run offset out
+        "depth_pass": 8 * n + 48 * (V // 16 if u.get("sliced") else V),
         "tile_count_columns": None,                # runs of the two depth slices
         "tile_count_scan": 0,                      # 2 x 256 x grid words, L2-resident
         "tile_scatter_columns": None,
@@ -404,8 +406,9 @@ def kernel_bytes(name, n, u, hw):
 
 
 def sort_throughput(ktable, u):
-    """Items per second of the depth sort (Gaussians with tiles over its three
-    kernels, the run scan included) and of tile pass 1 (column runs built over its count, count scan
+    """Items per second of the depth order (Gaussians with tiles over its three
+    kernels, of which a sliced frame sorts the nearest 1/16 only; the run scan
+    included) and of tile pass 1 (column runs built over its count, count scan
     and scatter kernels), from the live kernel table."""
     ms = lambda names: sum(ktable[k]["ms_per_frame"] for k in names if k in ktable)
     depth_ms = ms(("depth_pass",))

@@ -328,10 +328,11 @@ adr_status adr_sync_status(adr_ctx *ctx);
  * their work; adr_sync_status, adr_render_frame_noalloc and adr_serve_poll then
  * return ADR_ERR_TIMEOUT.  This hook makes that happen on purpose, so tests can
  * drive the path without a fault: while withheld_chunk >= 0, the scan's chunk
- * `withheld_chunk` (4096 Gaussians with tiles per chunk, in depth order) never
- * publishes its prefix and every lookback wait gives up after spin_limit
- * (1..2^22) polls, so the next chunk's wait runs out (frames whose Gaussians
- * with tiles fill fewer than withheld_chunk + 2 chunks are unaffected).
+ * `withheld_chunk` (a window of about 1024 Gaussians with tiles per chunk, in
+ * depth order, 4096 after the radix sort; each depth slice is scanned on its
+ * own) never publishes its prefix and every lookback wait gives up after
+ * spin_limit (1..2^22) polls, so the next chunk's wait runs out (scans of fewer
+ * than withheld_chunk + 2 chunks are unaffected).
  * withheld_chunk < 0 restores normal operation (spin_limit ignored).  The
  * setting is process-wide, applies to kernels launched after the call (a CUDA
  * graph captured meanwhile keeps it) and is not thread-safe with respect to

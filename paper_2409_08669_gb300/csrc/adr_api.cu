@@ -199,7 +199,7 @@ void free_workspace(Workspace& w) {
         w.prof = nullptr;
     }
     void* ptrs[] = {w.rec, w.aux, w.depth_key, w.offsets, w.gbox, w.sorted_box, w.sortbuf,
-                    w.order, w.win_lo, w.pruns, w.prows, w.pgauss, w.tcounts, w.tile_counts,
+                    w.order, w.win_lo, w.rank, w.s_win_lo, w.pruns, w.prows, w.pgauss, w.tcounts, w.tile_counts,
                     w.chunk_first, w.ranges, w.last, w.trav, w.tfin, w.lstat, w.g2d, w.load_sums,
                     w.hist, w.counters, w.status, w.lookback, w.d_fp, w.d_stage,
                     w.s_order, w.s_box, w.s_offsets, w.s_chunk_first,
@@ -215,10 +215,10 @@ size_t workspace_bytes(int64_t max_gaussians, int64_t pair_capacity, int32_t max
     const size_t pixels = (size_t)max_width * max_height;
     const size_t tiles = (size_t)((max_width + kTile - 1) / kTile) * ((max_height + kTile - 1) / kTile);
     const size_t lb = ((N + kSortChunk - 1) / kSortChunk + 2) * kRadix * 8;
-    return N * (kRecFloat4 * 16 + kAuxFloat4 * 16 + 4 * 4 + 4 + 8 + 16 + 36 + 12) + P * 14 +
+    return N * (kRecFloat4 * 16 + kAuxFloat4 * 16 + 4 * 4 + 8 + 8 + 16 + 36 + 12) + P * 14 +
            2 * (P / kSortChunk + 2) * 4 + tiles * 20 + pixels * 48 + lb +
-           (size_t)kRadix * kMaxTileGrid * 4 + (kZeroWords + bin_map(max_gaussians).count) * 4 +
-           (N / kWindow + 2) * 4 + 8192;
+           (size_t)kRadix * kMaxTileGrid * 4 + (kZeroWords + 2 * bin_map(max_gaussians).count) * 4 +
+           2 * (N / kWindow + 2) * 4 + 8192;
 }
 
 adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_capacity,
@@ -258,6 +258,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.sorted_box, N * sizeof(uint32_t));
     ALLOC(w.sortbuf, N * sizeof(uint4));
     ALLOC(w.order, N * sizeof(uint32_t));
+    ALLOC(w.rank, N * sizeof(uint32_t));
     ALLOC(w.win_lo, (N / kWindow + 2) * sizeof(uint32_t));
     ALLOC(w.pruns, P * sizeof(uint2));
     ALLOC(w.prows, (P + 8) * sizeof(uint16_t));   // + 16 bytes: Render reads whole 16-byte groups
@@ -272,6 +273,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.lstat, pixels * sizeof(int32_t));
     {
         const size_t tx = (size_t)(max_width + kTile - 1) / kTile, ty = (size_t)(max_height + kTile - 1) / kTile;
+        ALLOC(w.s_win_lo, (N / kWindow + 2) * sizeof(uint32_t));
         ALLOC(w.s_order, N * sizeof(uint32_t));
         ALLOC(w.s_box, N * sizeof(uint32_t));
         ALLOC(w.s_offsets, N * sizeof(uint32_t));
@@ -288,10 +290,11 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.load_sums, 4 * sizeof(double));
     ALLOC(w.hist, kHistWords * sizeof(uint32_t));
     // the zeroed block; bin counts grow with n, so the largest scene's fit every one
-    const size_t zero_words = kZeroWords + bin_map(max_gaussians).count;
+    const size_t zero_words = kZeroWords + 2 * bin_map(max_gaussians).count;
     ALLOC(w.counters, zero_words * sizeof(uint32_t));
     w.slice_counters = w.counters + kCntSlots;
     w.ttotals = w.slice_counters + 2 * kCntSlots;
+    w.sums = reinterpret_cast<unsigned long long*>(w.ttotals + kTotalSets * kRadix);
     w.bins = w.counters + kZeroWords;
     ALLOC(w.status, sizeof(uint32_t) * 4);
     ALLOC(w.lookback, w.lookback_words * sizeof(unsigned long long));
@@ -540,9 +543,11 @@ adr_status adr_read_gaussians(adr_ctx* c, float* geom, int32_t* rect, int32_t* t
     DeviceGuard guard(c->device);
     // A frame computes the SH colours of the Gaussians it blends only; the
     // inspection reports every Gaussian with tiles, from the frame's SH array.
-    if (geom && c->fs.defer_colors && c->fs.sh && c->fs.order && c->fs.n > 0)
+    if (geom && c->fs.defer_colors && c->fs.sh && c->fs.order && c->fs.n > 0) {
+        enqueue_order_all(c->ws, c->fs, (cudaStream_t)stream);
         launch_colors(c->fs.order, c->ws.counters + kCntVisible, c->fs.means, c->fs.sh, c->ws.d_fp,
                       c->ws.rec, c->ws.sm_count, (cudaStream_t)stream);
+    }
     launch_read_gaussians(c->ws.rec, c->ws.aux, c->ws.gbox, (int)c->fs.n, geom, rect,
                           tiles, (cudaStream_t)stream);
     return check_launch("adr_read_gaussians") == ADR_OK ? ok() : ADR_ERR_CUDA;

@@ -131,8 +131,8 @@ enum Counter : int {
     kCntDepthKept = 4,    // Gaussians with tiles, counted by the first depth pass
     kCntScanFailed = 5,   // non-zero: a lookback wait of the run scan gave up (the frame
                           // is then skipped: its pair count reads as saturated)
-    kCntWindowsDone = 6,  // windows the window sort has finished (bins.cu)
-                          // word 7: unused
+    kCntSliceBin = 6,     // binned depth order: depth slice 0 is the bins below this one
+    kCntLargestBin = 7,   // binned depth order: Gaussians in the fullest bin
     kCntPairs64 = 8,      // words 8-9: P as a 64-bit sum
     kCntSlots = 16
 };
@@ -187,8 +187,10 @@ struct Workspace {
     double* load_sums = nullptr;           // [4] load-balancing loss moments
     uint32_t* hist = nullptr;              // [kHistWords]
     uint32_t* counters = nullptr;          // [kCntSlots], the start of the zeroed block
-    uint32_t* bins = nullptr;              // [kMaxBins or fewer] depth histogram, then bin starts
-                                           // (in the zeroed block)
+    unsigned long long* sums = nullptr;    // [kSumSlots * kSumStride] pairs and runs (in the zeroed block)
+    uint32_t* bins = nullptr;              // [kMaxBins or fewer, twice with depth slices] depth histogram,
+                                           // then bin starts (in the zeroed block)
+    uint32_t* rank = nullptr;              // [max_n] arrival rank of each Gaussian in its bin
     uint32_t* largest_bin = nullptr;       // host word (mapped, may be null): the frame's largest bin
     uint32_t* status = nullptr;            // [4]
     unsigned long long* lookback = nullptr;
@@ -204,6 +206,7 @@ struct Workspace {
     uint32_t* s_box = nullptr;             // [max_n] their packed rectangles
     uint32_t* s_offsets = nullptr;         // [max_n] their run offsets
     uint32_t* s_chunk_first = nullptr;     // [capacity / kSortChunk + 2]
+    uint32_t* s_win_lo = nullptr;          // [max_n / kWindow + 2] windows of slice 1
     uint32_t* surv_cnt = nullptr;          // [2 * kMaxTileGrid] per-CTA kept counts and runs
     uint8_t* surv_flag = nullptr;          // [max_n] kept flag per depth-order position
     float4* pst = nullptr;                 // [max pixels] T, C of unfinished tiles
@@ -214,10 +217,15 @@ struct Workspace {
 };
 
 // Words that start a frame at zero, one block: counters, the counters of the
-// two depth slices, the tile passes' totals, then the frame's depth bins.
+// two depth slices, the tile passes' totals, Preprocess's sums, then the depth
+// bins of the frame and (with depth slices) those of slice 1's Gaussians.
 enum TotalSet : int { kTotalsFirst = 0, kTotalsSlice1 = 1, kTotalsRows = 2, kTotalSets = 3 };
-constexpr int kZeroWords = 3 * kCntSlots + kTotalSets * kRadix;   // + the bins
-static_assert(kZeroWords % 4 == 0, "the bins are read 16 bytes at a time");
+constexpr int kSumSlots = 64;    // Preprocess's pair and run sums: 64-bit words 0 and 1 of each slot
+constexpr int kSumStride = 4;    // 64-bit words (32 bytes) a slot
+constexpr int kZeroWords = 3 * kCntSlots + kTotalSets * kRadix + 2 * kSumSlots * kSumStride;   // + the bins
+static_assert(kZeroWords % 4 == 0 && (3 * kCntSlots + kTotalSets * kRadix) % 4 == 0,
+              "the bins are read 16 bytes at a time, the sums are 64-bit words");
+constexpr uint32_t kNoRank = 0xFFFFFFFFu;   // arrival rank of a Gaussian that takes no part
 
 // Depth bins (bins.cu): kBinOctaves octaves of depth from the near plane (at
 // least 2^-6) on, each 2^(23 - shift) bins; nearer and farther keys fall into
@@ -264,6 +272,10 @@ inline DepthSort next_depth_sort(uint32_t largest_bin, uint32_t& probe_in) {
     return kSortRadixProbe;
 }
 
+// Gaussians whose depth order a frame has built so far (a mask).  A sliced frame
+// of the binned order needs slice 0's only.
+enum OrderHeld : int { kOrderSlice0 = 1, kOrderAll = 2 };
+
 // What one frame's stages hand to the next.
 struct FrameState {
     int64_t n = 0;
@@ -282,6 +294,8 @@ struct FrameState {
     const uint16_t* rows = nullptr;          // their row intervals
     bool allow_slices = true;                // the caller's choice for the next sort
     DepthSort depth_sort = kSortBins;
+    bool slice1_bins_used = false;           // slice 1's bins are no longer zero
+    int order_held = 0;                      // which of OrderHeld `order` and its boxes and offsets hold
     bool totals_used[kTotalSets] = {false, false, false};   // written since the frame's head zeroed them
     bool sliced = false;                     // the frame renders in two depth slices
     bool split_last_slice = false;           // slice 1 renders tiles by pixel halves (f2)
@@ -319,6 +333,8 @@ void enqueue_sort(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& ep
 // Builds per-tile lists (from every Gaussian's column runs) if the last sort
 // made column lists; what the backward and the pair inspection read.
 void enqueue_tile_lists(const Workspace& ws, FrameState& fs, cudaStream_t stream);
+// The depth order of every Gaussian with tiles, if the frame has not built it.
+void enqueue_order_all(const Workspace& ws, FrameState& fs, cudaStream_t stream);
 void enqueue_render(const Workspace& ws, FrameState& fs, float* img, float* t_final,
                     int32_t* load, cudaStream_t stream);
 // A batched frame: up to kMaxBatch cameras of one scene (same n, same
@@ -355,7 +371,8 @@ struct PreprocessOut {
     uint32_t* depth_key;
     uint32_t* gbox;
     uint32_t* bins;          // depth histogram (zeroed)
-    uint32_t* rank;          // each kept Gaussian's arrival rank in its bin
+    uint32_t* rank;          // each kept Gaussian's arrival rank in its bin, else kNoRank
+    unsigned long long* sums;   // kSumSlots slots (zeroed): pairs and column runs
 };
 struct PreprocessBatch {
     int count = 0;
@@ -378,23 +395,32 @@ void launch_depth_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
                        uint32_t* counts, uint32_t* totals, const uint32_t* pay_in,
                        uint32_t* pay_out, uint32_t* status, int grid, cudaStream_t stream);
 
-// The depth order by binning (bins.cu), from the histogram and ranks that
-// Preprocess left.  bin_scan: bins -> starts, windows; *largest (may be null)
-// gets the largest bin's count, counters (with set_counts) the Gaussians with
-// tiles.  bin_scatter: (key, index, box) records grouped by bin.  window_sort:
-// the records in order, with the outputs of launch_scan_tiles and, unless
-// slice0 is null, depth slice 0's counters (it may overwrite the records).
+// The depth order by binning (bins.cu), from the histogram, ranks and sums that
+// Preprocess left.
+//   bin_scan:    bins -> starts and windows; what else it closes is `what`.
+//   bin_scatter: (key, index, box) records grouped by bin, of the Gaussians with
+//                a rank, or of those in the bins below *bin_limit.
+//   window_sort: the records of the first block[kCntVisible] Gaussians in order,
+//                with the outputs of launch_scan_tiles (the run total goes to
+//                block, a failed wait to `counters` and the slices' blocks); it
+//                may overwrite the records.
+enum BinScan : int {
+    kScanLargest = 0,   // the largest bin only (beside the radix sort)
+    kScanFrame = 1,     // + the frame's counts (pairs with the capacity flag, runs, Gaussians) and slice 0
+    kScanSlice1 = 2     // + slice 1's counts
+};
 int window_blocks_per_sm();
-void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, uint32_t* counters,
-                     bool set_counts, uint32_t* largest, cudaStream_t stream);
+void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, BinScan what, uint32_t* counters,
+                     uint32_t* slice_counters, const unsigned long long* sums, int64_t capacity,
+                     uint32_t* largest, uint32_t* status, cudaStream_t stream);
 void launch_bin_scatter(const uint32_t* keys, const uint32_t* ranks, const uint32_t* boxes,
-                        const uint32_t* bins, const FrameParams* fp, const BinMap& map, int64_t n,
-                        uint4* out, uint32_t* status, cudaStream_t stream);
+                        const uint32_t* bins, const uint32_t* bin_limit, bool few, const FrameParams* fp,
+                        const BinMap& map, int64_t n, uint4* out, uint32_t* status, cudaStream_t stream);
 void launch_window_sort(uint4* recs, const uint32_t* win_lo, const uint32_t* gbox, int64_t n,
                         int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
                         uint32_t* chunk_first, unsigned long long* lookback, EpochRef epoch,
-                        uint32_t* counters, uint32_t* slice0, uint32_t* status, int grid,
-                        cudaStream_t stream);
+                        uint32_t* block, uint32_t* counters, uint32_t* slice_counters, uint32_t* status,
+                        int grid, cudaStream_t stream);
 
 // SH colours (Sec. 3.2.1, stage 1's view-dependent colour) of the Gaussians
 // ids[0 .. *count) into their render records (rec[3 i + 2].xyz), on demand:
@@ -515,12 +541,18 @@ struct RenderBatch {
 void launch_render(const RenderBatch& batch, cudaStream_t stream);
 void launch_slice0_setup(const uint32_t* counters, const uint32_t* offsets, uint32_t* c0,
                          cudaStream_t stream);
-void launch_survivors(const uint32_t* tile_done, int tiles_x, int tiles_y, uint32_t* sat,
-                      const uint32_t* sorted_box, const uint32_t* order, const uint32_t* counters,
-                      int grid, uint32_t* cnt, uint8_t* keep_flag, int64_t n_max, int64_t chunk_max,
-                      uint32_t* s_order, uint32_t* s_box, uint32_t* s_offsets,
+// The summed-area table of the unfinished tiles, and slice 1's selection with
+// it: over the depth order (radix frames), or over the Gaussians by index,
+// counting the kept ones in depth bins (their arrival rank, else kNoRank).
+void launch_unfinished_table(const uint32_t* tile_done, int tiles_x, int tiles_y, uint32_t* sat,
+                             cudaStream_t stream);
+void launch_survivors(int tiles_x, const uint32_t* sat, const uint32_t* sorted_box, const uint32_t* order,
+                      const uint32_t* counters, int grid, uint32_t* cnt, uint8_t* keep_flag, int64_t n_max,
+                      int64_t chunk_max, uint32_t* s_order, uint32_t* s_box, uint32_t* s_offsets,
                       uint32_t* s_chunk_first, uint32_t* c1, uint32_t* status, cudaStream_t stream);
-
+void launch_survivor_bins(const uint32_t* keys, const uint32_t* boxes, int64_t n, int tiles_x,
+                          const uint32_t* sat, const FrameParams* fp, const BinMap& map,
+                          const uint32_t* counters, uint32_t* bins, uint32_t* rank, cudaStream_t stream);
 
 // Backward (backward.cu).
 void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec,

@@ -46,8 +46,9 @@ constexpr int kWinWarps = kWinThreads / 32;
 // ---------------------------------------------------------------------------
 template <int kQuads>
 __global__ void __cluster_dims__(kScanCluster, 1, 1)
-k_bin_scan(uint32_t* __restrict__ bins, uint32_t* __restrict__ win_lo, uint32_t* __restrict__ counters,
-           int set_counts, uint32_t* __restrict__ largest) {
+k_bin_scan(uint32_t* __restrict__ bins, uint32_t* __restrict__ win_lo, int what, uint32_t* __restrict__ counters,
+           uint32_t* __restrict__ slices, const unsigned long long* __restrict__ sums, int64_t capacity,
+           uint32_t* __restrict__ largest, uint32_t* __restrict__ status) {
     pdl_prologue();
     __shared__ uint32_t s_w[32], s_max[32];
     __shared__ uint32_t s_total, s_cta_max;
@@ -96,67 +97,118 @@ k_bin_scan(uint32_t* __restrict__ bins, uint32_t* __restrict__ win_lo, uint32_t*
         total += t;
     }
     // A bin [s, e): the windows it starts (s a multiple of kWindow) begin at s;
-    // the windows whose first position falls inside it begin at e.
-    auto place = [&](uint32_t s, uint32_t& c) {
+    // the windows whose first position falls inside it begin at e.  Depth slice 0
+    // ends with the bin that holds its last Gaussian.
+    const uint32_t K0 = what == kScanFrame ? slice0_count(total) : 0u;
+    auto place = [&](uint32_t s, uint32_t& c, uint32_t bin) {
         const uint32_t e = s + c;
-        uint32_t w = (s + (uint32_t)kWindow - 1u) / (uint32_t)kWindow;
-        if (c != 0u && w * (uint32_t)kWindow < e) {
+        if (c != 0u) {
+            uint32_t w = (s + (uint32_t)kWindow - 1u) / (uint32_t)kWindow;
             if (w * (uint32_t)kWindow == s) win_lo[w++] = s;
             for (; w * (uint32_t)kWindow < e; ++w) win_lo[w] = e;
+            if (s < K0 && K0 <= e) {
+                counters[kCntSliceBin] = bin + 1u;
+                if (slices) slices[kCntVisible] = slices[kCntDepthKept] = e;
+            }
         }
         c = s;
         return e;
     };
+    auto crosses = [&](uint32_t s, uint32_t e) {   // a window begins in [s, e), or slice 0 ends in (s, e]
+        return (s + (uint32_t)kWindow - 1u) / (uint32_t)kWindow != (e + (uint32_t)kWindow - 1u) / (uint32_t)kWindow ||
+               (s < K0 && K0 <= e);
+    };
 #pragma unroll
     for (int q = 0; q < kQuads; ++q) {
         uint32_t s = before + first[q];
-        s = place(s, v[q].x);
-        s = place(s, v[q].y);
-        s = place(s, v[q].z);
-        place(s, v[q].w);
-        b4[32 * q] = v[q];
-    }
-    if (rank == 0 && tid == 0) {
-        win_lo[(total + (uint32_t)kWindow - 1u) / (uint32_t)kWindow] = total;
-        if (set_counts) {
-            counters[kCntVisible] = total;
-            counters[kCntDepthKept] = total;
+        uint4 c = v[q];
+        const uint32_t bin = (((rank * (uint32_t)warps + (uint32_t)warp) * kQuads + q) * 32u + (uint32_t)lane) * 4u;
+        if (crosses(s, s + c.x + c.y + c.z + c.w)) {
+            s = place(s, c.x, bin);
+            s = place(s, c.y, bin + 1u);
+            s = place(s, c.z, bin + 2u);
+            place(s, c.w, bin + 3u);
+        } else {
+            c = make_uint4(s, s + c.x, s + c.x + c.y, s + c.x + c.y + c.z);
         }
-        if (largest) *largest = most;
+        b4[32 * q] = c;
+    }
+    if (rank == 0 && warp == 0) {
+        if (what == kScanFrame) {   // Preprocess's sums, saturated to 31 bits
+            unsigned long long p = 0, r = 0;
+            for (int k = lane; k < kSumSlots; k += 32) {
+                p += sums[kSumStride * k];
+                r += sums[kSumStride * k + 1];
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                p += __shfl_xor_sync(0xffffffffu, p, o);
+                r += __shfl_xor_sync(0xffffffffu, r, o);
+            }
+            if (lane == 0) {
+                const uint32_t pairs = (uint32_t)min(p, (unsigned long long)kSat);
+                counters[kCntPairs] = pairs;
+                counters[kCntRuns] = (uint32_t)min(r, (unsigned long long)kSat);
+                counters[kCntVisible] = counters[kCntDepthKept] = total;
+                if (slices) slices[kCntPairs] = pairs;
+                if (p > (unsigned long long)capacity) atomicOr(status, kErrCapacity);
+            }
+        } else if (what == kScanSlice1 && lane == 0) {
+            uint32_t* c1 = slices + kCntSlots;
+            c1[kCntVisible] = c1[kCntDepthKept] = total;
+            c1[kCntPairs] = counters[kCntPairs];
+        }
+        if (lane == 0) {
+            win_lo[(total + (uint32_t)kWindow - 1u) / (uint32_t)kWindow] = total;
+            if (what != kScanSlice1) {
+                counters[kCntLargestBin] = most;
+                if (largest) *largest = most;
+            }
+        }
     }
     cluster.sync();   // no CTA leaves while another reads its totals
 }
 
-// Four consecutive Gaussians per thread, 16-byte loads.
+// Four consecutive Gaussians per thread, 16-byte loads.  kFew: most of them take
+// no part (depth slices), so ranks are read first and boxes one by one.  Bound
+// by its scattered accesses, about one clock per lane and SM each: a bin start
+// gathered and a record written per Gaussian that takes part.
+template <bool kFew>
 __global__ void __launch_bounds__(256)
 k_bin_scatter(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ ranks,
-              const uint32_t* __restrict__ boxes, const uint32_t* __restrict__ bins, const FrameParams* __restrict__ fp, BinMap map,
+              const uint32_t* __restrict__ boxes, const uint32_t* __restrict__ bins,
+              const uint32_t* __restrict__ bin_limit, const FrameParams* __restrict__ fp, BinMap map,
               int64_t n, uint4* __restrict__ out, uint32_t* __restrict__ status) {
     pdl_prologue();
-    const uint32_t base = bin_base(fp->cam.near_z);
+    const uint32_t base = bin_base(fp->cam.near_z), limit = bin_limit ? *bin_limit : 0xFFFFFFFFu;
     const int64_t i0 = 4 * ((int64_t)blockIdx.x * 256 + threadIdx.x);
     if (i0 >= n) return;
-    uint32_t k[4], r[4], x[4];
+    uint32_t k[4] = {0u, 0u, 0u, 0u}, r[4], x[4];
     if (i0 + 4 <= n) {
-        const uint4 a = *reinterpret_cast<const uint4*>(keys + i0);
         const uint4 b = *reinterpret_cast<const uint4*>(ranks + i0);
-        const uint4 c = *reinterpret_cast<const uint4*>(boxes + i0);
-        k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
         r[0] = b.x; r[1] = b.y; r[2] = b.z; r[3] = b.w;
-        x[0] = c.x; x[1] = c.y; x[2] = c.z; x[3] = c.w;
+        if (kFew && (r[0] & r[1] & r[2] & r[3]) == kNoRank) return;   // no rank is that large
+        const uint4 a = *reinterpret_cast<const uint4*>(keys + i0);
+        k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
+        if (!kFew) {
+            const uint4 c = *reinterpret_cast<const uint4*>(boxes + i0);
+            x[0] = c.x; x[1] = c.y; x[2] = c.z; x[3] = c.w;
+        }
     } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            k[q] = i0 + q < n ? keys[i0 + q] : 0xFFFFFFFFu;
-            r[q] = i0 + q < n ? ranks[i0 + q] : 0u;
-            x[q] = i0 + q < n ? boxes[i0 + q] : 0u;
+            r[q] = i0 + q < n ? ranks[i0 + q] : kNoRank;
+            if (i0 + q < n) k[q] = keys[i0 + q];
+            if (!kFew && i0 + q < n) x[q] = boxes[i0 + q];
         }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if (k[q] == 0xFFFFFFFFu) continue;   // no tiles
-        const uint32_t pos = bins[bin_of(k[q], base, map)] + r[q];
-        if ((int64_t)pos < n) out[pos] = make_uint4(k[q], (uint32_t)(i0 + q), x[q], 0u);
+        if (r[q] == kNoRank) continue;
+        const uint32_t bin = bin_of(k[q], base, map);
+        if (bin >= limit) continue;
+        const uint32_t pos = bins[bin] + r[q];
+        if ((int64_t)pos < n) out[pos] = make_uint4(k[q], (uint32_t)(i0 + q), kFew ? boxes[i0 + q] : x[q], 0u);
         else atomicOr(status, kErrRange);
     }
 }
@@ -179,13 +231,12 @@ struct alignas(16) WindowShared {
         uint32_t run[kRadix];                    // large windows: next position of each digit
     } c;
     uint32_t w0[kWinWarps], w1[kWinWarps];
-    unsigned long long sums[2];                  // column runs and pairs of the window
-    uint32_t ticket, prefix;
+    unsigned long long sum;                      // large windows: column runs
+    uint32_t ticket, prefix, total;              // total: the window's column runs
 };
 static_assert(kWinCap * 2 == kSub && kWinCap < (1 << 16), "16-bit starts, thread t scans 16 sub-bins");
 
 __device__ __forceinline__ uint32_t box_runs(uint32_t box) { return ((box >> 16) & 0xFFu) + 1u; }
-__device__ __forceinline__ uint32_t box_rows(uint32_t box) { return (box >> 24) + 1u; }
 
 // Exclusive scan over the block of one value per thread; `total` the sum.
 __device__ __forceinline__ uint32_t win_scan(uint32_t v, uint32_t* s_w, uint32_t& total) {
@@ -400,22 +451,22 @@ __device__ const uint2* sort_large(WindowShared& sm, uint4* recs, uint32_t m) {
 }
 
 // The parts of k_window_sort for a window that does not fit on chip: its order,
-// boxes and sums, and its run offsets.
+// boxes and run total, and its run offsets.
 __device__ __noinline__ void order_large(WindowShared& sm, uint4* recs, uint32_t m, const uint32_t* gbox,
                                          uint32_t* order, uint32_t* sorted_box) {
     const uint2* sorted = sort_large(sm, recs, m);
-    if (threadIdx.x < 2) sm.sums[threadIdx.x] = 0ull;
+    if (threadIdx.x == 0) sm.sum = 0ull;
     __syncthreads();
-    unsigned long long runs = 0, pairs = 0;
+    unsigned long long runs = 0;
     for (uint32_t s = threadIdx.x; s < m; s += kWinThreads) {
         const uint32_t i = sorted[s].y, box = gbox[i];
         order[s] = i;
         sorted_box[s] = box;
         runs += box_runs(box);
-        pairs += box_runs(box) * box_rows(box);
     }
-    atomicAdd(&sm.sums[0], runs);
-    atomicAdd(&sm.sums[1], pairs);
+    atomicAdd(&sm.sum, runs);
+    __syncthreads();
+    if (threadIdx.x == 0) sm.total = (uint32_t)min(sm.sum, (unsigned long long)kSat);
 }
 
 __device__ __noinline__ void offsets_large(WindowShared& sm, uint32_t lo, uint32_t m, const uint32_t* sorted_box,
@@ -434,22 +485,21 @@ __device__ __noinline__ void offsets_large(WindowShared& sm, uint32_t lo, uint32
     }
 }
 
-__global__ void __launch_bounds__(kWinThreads, 5)
+__global__ void __launch_bounds__(kWinThreads, 4)
 k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* __restrict__ gbox,
               int64_t n_max, int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
               uint32_t* __restrict__ chunk_first, unsigned long long* __restrict__ lookback, EpochRef eref,
-              uint32_t* counters, uint32_t* __restrict__ slice0, uint32_t* __restrict__ status,
-              LookbackTest lt) {
+              uint32_t* block, uint32_t* __restrict__ counters, uint32_t* __restrict__ slices,
+              uint32_t* __restrict__ status, LookbackTest lt) {
     pdl_prologue();
     __shared__ WindowShared sm;
     const uint32_t epoch = (*eref.stage) * 8u + eref.pass;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t V = (uint32_t)min((int64_t)counters[kCntVisible], n_max);
+    const uint32_t V = (uint32_t)min((int64_t)block[kCntVisible], n_max);
     const uint32_t windows = (V + (uint32_t)kWindow - 1u) / (uint32_t)kWindow;
-    unsigned long long* pairs64 = reinterpret_cast<unsigned long long*>(counters + kCntPairs64);
     for (;;) {
         // Windows are taken in order, so a window's predecessors are done or running.
-        if (tid == 0) sm.ticket = atomicAdd(counters + kCntScanTicket, 1u);
+        if (tid == 0) sm.ticket = atomicAdd(block + kCntScanTicket, 1u);
         __syncthreads();
         const uint32_t w = sm.ticket;
         if (w >= windows) return;
@@ -458,44 +508,37 @@ k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* 
         if (on_chip) {
             sort_on_chip(sm, recs, lo, (int)m);
             // Thread t's eight consecutive Gaussians: their run offsets from the
-            // window's first run (at most 2048 x 256 runs, 2048 x 65536 pairs).
-            uint32_t runs = 0, pairs = 0, off[kWinItems];
+            // window's first run.
+            uint32_t runs = 0, off[kWinItems];
             const uint4* b4 = reinterpret_cast<const uint4*>(sm.u.out.box) + 2 * tid;
             const uint4 a = b4[0], b = b4[1];
             const uint32_t box[kWinItems] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
             for (int q = 0; q < kWinItems; ++q) {
                 off[q] = runs;
-                if (kWinItems * tid + q < (int)m) {
-                    runs += box_runs(box[q]);
-                    pairs += box_runs(box[q]) * box_rows(box[q]);
-                }
+                if (kWinItems * tid + q < (int)m) runs += box_runs(box[q]);
             }
             uint32_t total;
             const uint32_t before = win_scan(runs, sm.w0, total);
             uint4* o4 = reinterpret_cast<uint4*>(sm.c.off) + 2 * tid;
             o4[0] = make_uint4(before + off[0], before + off[1], before + off[2], before + off[3]);
             o4[1] = make_uint4(before + off[4], before + off[5], before + off[6], before + off[7]);
-            pairs = __reduce_add_sync(0xffffffffu, pairs);
-            if (lane == 0) sm.w1[warp] = pairs;
-            __syncthreads();
-            if (tid == 0) {
-                unsigned long long p = 0;
-                for (int q = 0; q < kWinWarps; ++q) p += sm.w1[q];
-                sm.sums[0] = total;
-                sm.sums[1] = p;
-            }
+            if (tid == 0) sm.total = total;
         } else {
             order_large(sm, recs + lo, m, gbox, order + lo, sorted_box + lo);
         }
         __syncthreads();
         if (warp == 0) {
-            const uint32_t total = (uint32_t)min(sm.sums[0], (unsigned long long)kSat);
-            if (lane == 0 && sm.sums[1]) atomicAdd(pairs64, sm.sums[1]);
-            const uint32_t excl = warp_lookback(lookback, w, total, epoch, status, counters, lt);
+            bool gave_up;
+            const uint32_t excl = warp_lookback(lookback, w, sm.total, epoch, status, lt, &gave_up);
             if (lane == 0) {
                 sm.prefix = excl;
-                if (w + 1 == windows) counters[kCntRuns] = sat_add(excl, total);
+                if (w + 1 == windows) block[kCntRuns] = sat_add(excl, sm.total);
+                if (gave_up) {   // not a valid scan: the pair counts read as saturated, so every
+                                 // later stage skips its work
+                    counters[kCntPairs] = kSat;
+                    if (slices) slices[kCntPairs] = slices[kCntSlots + kCntPairs] = kSat;
+                }
             }
         } else if (on_chip) {   // meanwhile the other warps write the order out
             for (int s = tid - 32; s < (int)m; s += kWinThreads - 32) {
@@ -513,27 +556,7 @@ k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* 
         } else {
             offsets_large(sm, lo, m, sorted_box, sm.prefix, capacity, offsets, chunk_first);
         }
-        // The last window to finish closes the frame's counts: the pair total P
-        // (saturated to 31 bits) with the capacity flag, and depth slice 0.  If
-        // a lookback wait gave up, the run offsets are not a valid scan: P reads
-        // as saturated, so every later stage skips its work.
-        __threadfence();
-        __syncthreads();
-        if (tid == 0 && atomicAdd(counters + kCntWindowsDone, 1u) + 1u == windows) {
-            __threadfence();
-            const unsigned long long p = atomicAdd(pairs64, 0ull);
-            const bool failed = atomicAdd(counters + kCntScanFailed, 0u) != 0u;
-            const uint32_t pairs = failed ? kSat : (uint32_t)min(p, (unsigned long long)kSat);
-            counters[kCntPairs] = pairs;
-            if (!failed && p > (unsigned long long)capacity) atomicOr(status, kErrCapacity);
-            if (slice0) {
-                const uint32_t K0 = slice0_count(V);
-                slice0[kCntPairs] = pairs;
-                slice0[kCntVisible] = K0;
-                slice0[kCntRuns] = K0 < V ? __ldcg(offsets + K0) : __ldcg(counters + kCntRuns);
-                slice0[kCntDepthKept] = K0;
-            }
-        }
+        __syncthreads();   // the window is no longer read
     }
 }
 
@@ -553,37 +576,35 @@ int window_blocks_per_sm() {
     return b > 0 ? b : 1;
 }
 
-void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, uint32_t* counters,
-                     bool set_counts, uint32_t* largest, cudaStream_t stream) {
+void launch_bin_scan(uint32_t* bins, const BinMap& map, uint32_t* win_lo, BinScan what, uint32_t* counters,
+                     uint32_t* slice_counters, const unsigned long long* sums, int64_t capacity,
+                     uint32_t* largest, uint32_t* status, cudaStream_t stream) {
     // 1, 2 or 4 quads of bins a lane in 256 to 1024 threads, for 2^13 to 2^17 bins
-    const int set = set_counts ? 1 : 0;
     const uint32_t per_cta = map.count / kScanCluster;
-    if (per_cta <= 1024)
-        launch_pdl(k_bin_scan<1>, kScanCluster, per_cta / 4, 0, stream, bins, win_lo, counters, set, largest);
-    else if (per_cta <= 2048)
-        launch_pdl(k_bin_scan<2>, kScanCluster, per_cta / 8, 0, stream, bins, win_lo, counters, set, largest);
-    else
-        launch_pdl(k_bin_scan<4>, kScanCluster, per_cta / 16, 0, stream, bins, win_lo, counters, set, largest);
+    const int quads = per_cta <= 1024 ? 1 : per_cta <= 2048 ? 2 : 4;
+    auto* kernel = quads == 1 ? k_bin_scan<1> : quads == 2 ? k_bin_scan<2> : k_bin_scan<4>;
+    launch_pdl(kernel, kScanCluster, per_cta / (4 * quads), 0, stream, bins, win_lo, (int)what, counters,
+               slice_counters, sums, capacity, largest, status);
 }
 
 void launch_bin_scatter(const uint32_t* keys, const uint32_t* ranks, const uint32_t* boxes,
-                        const uint32_t* bins, const FrameParams* fp, const BinMap& map, int64_t n,
-                        uint4* out, uint32_t* status, cudaStream_t stream) {
+                        const uint32_t* bins, const uint32_t* bin_limit, bool few, const FrameParams* fp,
+                        const BinMap& map, int64_t n, uint4* out, uint32_t* status, cudaStream_t stream) {
     if (n <= 0) return;
-    launch_pdl(k_bin_scatter, (unsigned)((n + 1023) / 1024), 256, 0, stream, keys, ranks, boxes, bins, fp, map,
-               n, out, status);
+    launch_pdl(few ? k_bin_scatter<true> : k_bin_scatter<false>, (unsigned)((n + 1023) / 1024), 256, 0, stream,
+               keys, ranks, boxes, bins, bin_limit, fp, map, n, out, status);
 }
 
 void launch_window_sort(uint4* recs, const uint32_t* win_lo, const uint32_t* gbox, int64_t n,
                         int64_t capacity, uint32_t* order, uint32_t* sorted_box, uint32_t* offsets,
                         uint32_t* chunk_first, unsigned long long* lookback, EpochRef epoch,
-                        uint32_t* counters, uint32_t* slice0, uint32_t* status, int grid,
-                        cudaStream_t stream) {
+                        uint32_t* block, uint32_t* counters, uint32_t* slice_counters, uint32_t* status,
+                        int grid, cudaStream_t stream) {
     if (n <= 0) return;
     const int64_t most = (n + kWindow - 1) / kWindow;
     launch_pdl(k_window_sort, (unsigned)(most < grid ? most : grid), kWinThreads, 0, stream, recs, win_lo, gbox,
-               n, capacity, order, sorted_box, offsets, chunk_first, lookback, epoch, counters, slice0, status,
-               lookback_test());
+               n, capacity, order, sorted_box, offsets, chunk_first, lookback, epoch, block, counters,
+               slice_counters, status, lookback_test());
 }
 
 }  // namespace adr

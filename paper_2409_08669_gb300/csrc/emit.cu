@@ -90,8 +90,10 @@ k_scan_tiles(const uint32_t* __restrict__ sorted_box, int64_t n_host, int64_t ca
         const uint32_t texcl = wbase + x - tsum;
         if (warp == 0) {
             if (lane == 0 && pairs) atomicAdd(pairs64, (unsigned long long)pairs);
-            const uint32_t excl = warp_lookback(lookback, chunk, total, epoch, status, counters, lt);
+            bool gave_up;
+            const uint32_t excl = warp_lookback(lookback, chunk, total, epoch, status, lt, &gave_up);
             if (lane == 0) {
+                if (gave_up) atomicExch(counters + kCntScanFailed, 1u);
                 s_prefix = excl;
                 if (base + kScanChunk >= n) counters[kCntRuns] = sat_add(excl, total);
             }

@@ -20,11 +20,12 @@ __device__ __forceinline__ uint32_t sat_add(uint32_t a, uint32_t b) {
 // predecessors; the words up to the nearest inclusive prefix are summed.
 // Lane 0 publishes this chunk's aggregate first and its inclusive prefix last
 // (except the chunk the testing hook withholds).  A wait that makes no
-// progress for lt.spin_limit polls gives up: it flags the status word and the
-// frame's counters and returns the partial prefix.
+// progress for lt.spin_limit polls gives up: it flags the status word, sets
+// *gave_up and returns the partial prefix.
 __device__ __forceinline__ uint32_t warp_lookback(unsigned long long* lookback, uint32_t chunk, uint32_t total,
-                                  uint32_t epoch, uint32_t* status, uint32_t* counters,
-                                  LookbackTest lt) {
+                                  uint32_t epoch, uint32_t* status, LookbackTest lt,
+                                  bool* gave_up) {
+    *gave_up = false;
     const int lane = threadIdx.x & 31;
     const unsigned long long tag = (unsigned long long)epoch << 32;
     volatile unsigned long long* lb = lookback;
@@ -56,10 +57,8 @@ __device__ __forceinline__ uint32_t warp_lookback(unsigned long long* lookback, 
         j -= take;
         if (take == 0) {
             if (++spins > lt.spin_limit) {
-                if (lane == 0) {
-                    atomicOr(status, kErrLookback);
-                    atomicExch(counters + kCntScanFailed, 1u);
-                }
+                if (lane == 0) atomicOr(status, kErrLookback);
+                *gave_up = true;
                 break;
             }
             __nanosleep(32);

@@ -47,7 +47,8 @@ constexpr size_t kOffGBox = align256(kOffOffsets + kNaMaxGaussians * 4);
 constexpr size_t kOffSortedBox = align256(kOffGBox + kNaMaxGaussians * 4);
 constexpr size_t kOffSortBuf = align256(kOffSortedBox + kNaMaxGaussians * 4);
 constexpr size_t kOffOrder = align256(kOffSortBuf + kNaMaxGaussians * 16);
-constexpr size_t kOffWinLo = align256(kOffOrder + kNaMaxGaussians * 4);
+constexpr size_t kOffRank = align256(kOffOrder + kNaMaxGaussians * 4);
+constexpr size_t kOffWinLo = align256(kOffRank + kNaMaxGaussians * 4);
 constexpr size_t kOffPRuns = align256(kOffWinLo + (kNaMaxGaussians / kWindow + 2) * 4);
 constexpr size_t kOffPRows = align256(kOffPRuns + kNaMaxPairs * 8);
 constexpr size_t kOffPGauss = align256(kOffPRows + (kNaMaxPairs + 8) * 2);
@@ -58,7 +59,7 @@ constexpr size_t kOffTrav = align256(kOffLast + kPixels * 4);
 constexpr size_t kOffTfin = align256(kOffTrav + kPixels * 4);
 constexpr size_t kOffHist = align256(kOffTfin + kPixels * 4);
 constexpr size_t kOffCounters = align256(kOffHist + kHistWords * 4);
-constexpr size_t kNaZeroWords = kZeroWords + kMaxBins;   // more than bin_map(kNaMaxGaussians) asks for
+constexpr size_t kNaZeroWords = kZeroWords + 8192;   // the bins of bin_map(kNaMaxGaussians)
 constexpr size_t kOffStatus = align256(kOffCounters + kNaZeroWords * 4);
 constexpr size_t kLookbackWords = (kNaMaxGaussians / kSortChunk + 2) * kRadix;
 constexpr size_t kOffFrameParams = align256(kOffStatus + 16);
@@ -76,6 +77,7 @@ struct DeviceState {
     unsigned char* base = nullptr;   // device address of g_na_scratch on this device
     Workspace ws;                    // buffers inside the array
     std::atomic<uint32_t> epoch{0};
+    uint32_t largest_bin = 0, radix_probe_in = kRadixProbe;   // see next_depth_sort
 };
 
 std::mutex g_setup_mutex;
@@ -128,6 +130,8 @@ adr_status setup(int dev, DeviceState*& out) {
         w.hist = reinterpret_cast<uint32_t*>(b + kOffHist);
         w.counters = reinterpret_cast<uint32_t*>(b + kOffCounters);   // the zeroed block, no depth slices
         w.ttotals = w.counters + 3 * kCntSlots;
+        w.sums = reinterpret_cast<unsigned long long*>(w.ttotals + kTotalSets * kRadix);
+        w.rank = reinterpret_cast<uint32_t*>(b + kOffRank);
         w.bins = w.counters + kZeroWords;
         w.status = reinterpret_cast<uint32_t*>(b + kOffStatus);
         w.lookback = reinterpret_cast<unsigned long long*>(b + kOffLookback);
@@ -178,6 +182,7 @@ extern "C" adr_status adr_render_frame_noalloc(const float* means, const float* 
         return report_error(ADR_ERR_CUDA, "adr_render_frame_noalloc: cudaMemsetAsync failed");
     FrameState fs;
     fill_frame_state(fs, n, cam, st);
+    fs.depth_sort = next_depth_sort(ds->largest_bin, ds->radix_probe_in);
     enqueue_preprocess(ws, fs, ds->epoch, means, scales, rots, opac, sh, strm);
     enqueue_sort(ws, fs, ds->epoch, strm);
     enqueue_render(ws, fs, img, t_final, load, strm);
@@ -186,14 +191,15 @@ extern "C" adr_status adr_render_frame_noalloc(const float* means, const float* 
 
     // Report pair overflow and bounded-wait expiry: read the status word and the
     // pair count back (into host stack memory) and wait for the frame.
-    uint32_t words[2] = {0, 0};
+    uint32_t words[1 + kCntLargestBin + 1] = {0};
     if (cudaMemcpyAsync(&words[0], ws.status, 4, cudaMemcpyDeviceToHost, strm) != cudaSuccess ||
-        cudaMemcpyAsync(&words[1], ws.counters + kCntPairs, 4, cudaMemcpyDeviceToHost, strm) != cudaSuccess ||
+        cudaMemcpyAsync(&words[1], ws.counters, 4 * (kCntLargestBin + 1), cudaMemcpyDeviceToHost, strm) != cudaSuccess ||
         cudaStreamSynchronize(strm) != cudaSuccess)
         return report_error(ADR_ERR_CUDA, "adr_render_frame_noalloc: status readback failed");
     // A wait that gave up skips the frame and reads its pair count as
     // saturated, so it is reported before the capacity check.
-    const StatusReport r = status_from_bits(words[0], (int64_t)words[1], kNaMaxPairs);
+    const StatusReport r = status_from_bits(words[0], (int64_t)words[1 + kCntPairs], kNaMaxPairs);
+    if (n > 0 && fs.depth_sort != kSortRadix) ds->largest_bin = words[1 + kCntLargestBin];
     if (r.status == ADR_ERR_CAPACITY)
         return report_error(ADR_ERR_CAPACITY,
                             "adr_render_frame_noalloc: more than 1048576 Gaussian-tile pairs "

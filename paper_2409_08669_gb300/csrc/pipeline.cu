@@ -85,8 +85,10 @@ static void preprocess_head(const Workspace& ws, FrameState& fs, std::atomic<uin
                             cudaStream_t stream, bool set_params) {
     count_stage(epoch, ws, stream);
     launch_frame_head(FrameParams{fs.cam, fs.st}, set_params ? ws.d_fp : nullptr, ws.counters,
-                      kZeroWords + bin_map(fs.n).count, stream);
+                      kZeroWords + (ws.slice_counters ? 2u : 1u) * bin_map(fs.n).count, stream);
     for (bool& used : fs.totals_used) used = false;
+    fs.order_held = 0;
+    fs.slice1_bins_used = false;
 }
 
 static BinMap frame_bins(const FrameState& fs) {
@@ -94,31 +96,42 @@ static BinMap frame_bins(const FrameState& fs) {
 }
 
 static PreprocessOut preprocess_out(const Workspace& ws) {
-    // the ranks sit in the run offsets' array, which is written after their last use
-    return PreprocessOut{ws.d_fp, ws.d_stage, ws.rec, ws.aux, ws.depth_key, ws.gbox, ws.bins, ws.offsets};
+    return PreprocessOut{ws.d_fp, ws.d_stage, ws.rec, ws.aux, ws.depth_key, ws.gbox, ws.bins, ws.rank, ws.sums};
 }
 
-// After Preprocess: the Gaussians by view depth and the scan of their column
-// runs (stage 2, + bookkeeping for stage 3), over the V Gaussians with tiles.
+// The binned depth order of slice 0's Gaussians or of all of them, with the scan
+// of their column runs (stage 2, + bookkeeping for stage 3).
+static void enqueue_order(const Workspace& ws, FrameState& fs, OrderHeld which, cudaStream_t stream) {
+    if (fs.order_held & which) return;
+    const bool slice0 = which == kOrderSlice0;
+    const EpochRef ep{ws.d_stage, (uint32_t)(kMaxPasses + (slice0 ? 1 : 0))};
+    TIMED(ws, kKDepthPass, stream,
+          launch_bin_scatter(ws.depth_key, ws.rank, ws.gbox, ws.bins, slice0 ? ws.counters + kCntSliceBin : nullptr,
+                             slice0, ws.d_fp, bin_map(fs.n), fs.n, ws.sortbuf, ws.status, stream));
+    TIMED(ws, kKDepthPass, stream,
+          launch_window_sort(ws.sortbuf, ws.win_lo, ws.gbox, fs.n, ws.capacity, ws.order, ws.sorted_box,
+                             ws.offsets, ws.chunk_first, ws.lookback, ep,
+                             slice0 ? ws.slice_counters : ws.counters, ws.counters, ws.slice_counters,
+                             ws.status, ws.window_grid, stream));
+    fs.order_held |= which;
+}
+
+void enqueue_order_all(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
+    enqueue_order(ws, fs, kOrderAll, stream);
+}
+
+// After Preprocess: the depth bins' starts and the frame's counts; the order
+// itself follows in the sort stage, of the Gaussians it needs.
 static void preprocess_tail(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
     const int64_t n = fs.n;
-    const EpochRef ep{ws.d_stage, (uint32_t)kMaxPasses};
-    const BinMap map = bin_map(n);
     fs.order = ws.order;
     if (fs.depth_sort != kSortRadix)
         TIMED(ws, kKDepthPass, stream,
-              launch_bin_scan(ws.bins, map, ws.win_lo, ws.counters, fs.depth_sort == kSortBins, ws.largest_bin,
-                              stream));
-    if (fs.depth_sort == kSortBins) {
-        TIMED(ws, kKDepthPass, stream,
-              launch_bin_scatter(ws.depth_key, ws.offsets, ws.gbox, ws.bins, ws.d_fp, map, n, ws.sortbuf,
-                                 ws.status, stream));
-        TIMED(ws, kKDepthPass, stream,
-              launch_window_sort(ws.sortbuf, ws.win_lo, ws.gbox, n, ws.capacity, ws.order,
-                                 ws.sorted_box, ws.offsets, ws.chunk_first, ws.lookback, ep, ws.counters,
-                                 ws.slice_counters, ws.status, ws.window_grid, stream));
-        return;
-    }
+              launch_bin_scan(ws.bins, bin_map(n), ws.win_lo,
+                              fs.depth_sort == kSortBins ? kScanFrame : kScanLargest, ws.counters,
+                              ws.slice_counters, ws.sums, ws.capacity, ws.largest_bin, ws.status, stream));
+    if (fs.depth_sort == kSortBins) return;
+    fs.order_held = kOrderAll | kOrderSlice0;
     // Very many Gaussians in one bin: 4 stable 8-bit passes (the first drops the
     // Gaussians without tiles, key 0xFFFFFFFF, and counts the V; the last
     // carries the packed rectangles into depth order), then the run scan.
@@ -136,6 +149,7 @@ static void preprocess_tail(const Workspace& ws, FrameState& fs, cudaStream_t st
         kin = keys;
         vin = vals;
     }
+    const EpochRef ep{ws.d_stage, (uint32_t)kMaxPasses};
     TIMED(ws, kKScanTiles, stream,
           launch_scan_tiles(ws.sorted_box, n, ws.capacity, ws.offsets, ws.chunk_first, ws.lookback,
                             ep, ws.counters, ws.status, ws.scan_grid, stream));
@@ -245,9 +259,11 @@ void enqueue_sort(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& ep
     if (fs.sliced) {
         // Slice 0: the nearest Gaussians' runs; Render builds slice 1 from what
         // its pixels still need.
+        enqueue_order(ws, fs, kOrderSlice0, stream);
         enqueue_pass1(ws, fs, pair_source(ws, fs, 0), kTotalsFirst, stream);
         fs.runs_held = kRunsSlice0;
     } else {
+        enqueue_order_all(ws, fs, stream);
         enqueue_pass1(ws, fs, pair_source(ws, fs, -1), kTotalsFirst, stream);
         fs.runs_held = kRunsAll;
     }
@@ -256,6 +272,7 @@ void enqueue_sort(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& ep
 void enqueue_tile_lists(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
     if (fs.lists == kListsTiles) return;
     if (fs.runs_held != kRunsAll) {   // the column runs of every Gaussian first
+        enqueue_order_all(ws, fs, stream);
         enqueue_pass1(ws, fs, pair_source(ws, fs, -1), kTotalsFirst, stream);
         fs.runs_held = kRunsAll;
     }
@@ -325,15 +342,41 @@ static void render_launch(const BatchItem* items, int count, int phase, cudaStre
 // unfinished tile, with their run offsets, then their column runs.
 static void slice1_runs(const Workspace& ws, FrameState& fs, cudaStream_t stream) {
     uint32_t* c1 = ws.slice_counters + kCntSlots;
-    // The survivor selection walks the Gaussians behind slice 0 in 256-item steps,
-    // each CTA its own range: ~1024 Gaussians per CTA keeps each CTA's chain of
-    // steps short (2048 CTAs at 3M Gaussians: 1.49 -> 1.52 k frames/s).
-    const int surv_grid = (int)std::min<int64_t>(kMaxTileGrid, std::max<int64_t>(ws.sort_grid, fs.n / 1024));
     TIMED(ws, kKSlice, stream,
-          launch_survivors(ws.tile_done, fs.cam.tiles_x, fs.cam.tiles_y, ws.sat, ws.sorted_box,
-                           fs.order, ws.counters, surv_grid, ws.surv_cnt, ws.surv_flag, ws.max_n,
-                           ws.capacity / kSortChunk + 2, ws.s_order, ws.s_box, ws.s_offsets,
-                           ws.s_chunk_first, c1, ws.status, stream));
+          launch_unfinished_table(ws.tile_done, fs.cam.tiles_x, fs.cam.tiles_y, ws.sat, stream));
+    if (fs.depth_sort == kSortBins) {
+        const BinMap map = bin_map(fs.n);
+        uint32_t* bins = ws.bins + map.count;
+        uint32_t* rank = ws.s_offsets;   // last read before the run offsets are written
+        const EpochRef ep{ws.d_stage, (uint32_t)(kMaxPasses + 2)};
+        if (fs.slice1_bins_used) {   // a second render of the frame
+            cudaMemsetAsync(bins, 0, map.count * sizeof(uint32_t), stream);
+            cudaMemsetAsync(c1, 0, kCntSlots * sizeof(uint32_t), stream);
+        }
+        fs.slice1_bins_used = true;
+        TIMED(ws, kKSlice, stream,
+              launch_survivor_bins(ws.depth_key, ws.gbox, fs.n, fs.cam.tiles_x, ws.sat, ws.d_fp, map,
+                                   ws.counters, bins, rank, stream));
+        TIMED(ws, kKSlice, stream,
+              launch_bin_scan(bins, map, ws.s_win_lo, kScanSlice1, ws.counters, ws.slice_counters, nullptr,
+                              ws.capacity, nullptr, ws.status, stream));
+        TIMED(ws, kKSlice, stream,
+              launch_bin_scatter(ws.depth_key, rank, ws.gbox, bins, nullptr, true, ws.d_fp, map, fs.n,
+                                 ws.sortbuf, ws.status, stream));
+        TIMED(ws, kKSlice, stream,
+              launch_window_sort(ws.sortbuf, ws.s_win_lo, ws.gbox, fs.n, ws.capacity, ws.s_order, ws.s_box,
+                                 ws.s_offsets, ws.s_chunk_first, ws.lookback, ep, c1, ws.counters,
+                                 ws.slice_counters, ws.status, ws.window_grid, stream));
+    } else {
+        // The survivor selection walks the Gaussians behind slice 0 in 256-item steps,
+        // each CTA its own range: ~1024 Gaussians per CTA keeps each CTA's chain of
+        // steps short (2048 CTAs at 3M Gaussians: 1.49 -> 1.52 k frames/s).
+        const int surv_grid = (int)std::min<int64_t>(kMaxTileGrid, std::max<int64_t>(ws.sort_grid, fs.n / 1024));
+        TIMED(ws, kKSlice, stream,
+              launch_survivors(fs.cam.tiles_x, ws.sat, ws.sorted_box, fs.order, ws.counters, surv_grid,
+                               ws.surv_cnt, ws.surv_flag, ws.max_n, ws.capacity / kSortChunk + 2, ws.s_order,
+                               ws.s_box, ws.s_offsets, ws.s_chunk_first, c1, ws.status, stream));
+    }
     enqueue_pass1(ws, fs, pair_source(ws, fs, 1), kTotalsSlice1, stream);
     fs.runs_held = kRunsSlice1;
 }

@@ -189,7 +189,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
     float4* __restrict__ aux = out.aux;
     uint32_t* __restrict__ depth_key = out.depth_key;
     uint32_t* __restrict__ gbox = out.gbox;
-    uint32_t rank = 0;   // arrival rank in the depth bin
+    uint32_t rank = kNoRank;   // arrival rank in the depth bin
 
     const float mx = means[3 * i + 0], my = means[3 * i + 1], mz = means[3 * i + 2];
     // Sort depth: fixed evaluation order, each operation rounded separately.
@@ -325,14 +325,24 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
         rec[3 * i + 1] = r1;
         rec[3 * i + 2] = r2;
         aux[2 * i + 0] = a0;
-        out.rank[i] = rank;
     }
+    out.rank[i] = rank;
     aux[2 * i + 1] = a1;
     depth_key[i] = key;
     // packed rectangle x0 | y0 << 8 | (w-1) << 16 | (h-1) << 24, all ones if no tiles
     gbox[i] = ntiles ? (uint32_t)rc.x | ((uint32_t)rc.y << 8) | ((uint32_t)(rc.z - rc.x - 1) << 16) |
                            ((uint32_t)(rc.w - rc.y - 1) << 24)
                      : 0xFFFFFFFFu;
+    // The frame's pairs and column runs, a warp's lanes together (whichever of
+    // them are here together: the sums add up), over kSumSlots addresses.
+    const unsigned lanes = __activemask();
+    const uint32_t pairs = __reduce_add_sync(lanes, ntiles);
+    const uint32_t runs = __reduce_add_sync(lanes, (uint32_t)(rc.z - rc.x));
+    if ((threadIdx.x & 31) == (unsigned)(__ffs(lanes) - 1) && pairs) {
+        unsigned long long* slot = out.sums + kSumStride * (blockIdx.x / (unsigned)batch.count % kSumSlots);
+        atomicAdd(slot, (unsigned long long)pairs);
+        atomicAdd(slot + 1, (unsigned long long)runs);
+    }
 }
 
 // Stage 1's view-dependent colour, rgb = max(0, sum_k sh_k Y_k(d) + 0.5) with

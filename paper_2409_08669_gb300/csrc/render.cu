@@ -250,7 +250,11 @@ k_render(const RenderBatch batch) {
     int32_t cnt_a = 0, cnt_b = 0, last_a = 0, last_b = 0;
     int2 stop = make_int2(0, 0);
     int32_t fbase = 0;   // position in the tile's own list of this batch's first entry
-    if (batch.cam[cb].ss.phase == 2) {   // last slice: resume the tiles the first slice left unfinished
+    // Last slice: resume the tiles the first slice left unfinished.  A scan that
+    // failed (its pair count reads as saturated) skips the frame instead: every
+    // tile then holds the background, those that slice 0 had finished too.
+    if (batch.cam[cb].ss.phase == 2 &&
+        (int64_t)batch.cam[cb].ss.col_counters[kCntPairs] <= batch.cam[cb].ss.capacity) {
         const SliceState& ss = batch.cam[cb].ss;
         if (ss.tile_done[tile_rm0]) return;
         const size_t pixa = (size_t)ya0 * cam.width + x0;
@@ -468,7 +472,8 @@ k_render_half(const RenderBatch batch) {
     const SetDev st = rc.fp->st;
     const int ty = tile_index % cam.tiles_y, tx = tile_index / cam.tiles_y;
     const int tile_rm = ty * cam.tiles_x + tx;
-    if (ss.tile_done[tile_rm]) return;
+    const bool skipped = (int64_t)ss.col_counters[kCntPairs] > ss.capacity;   // as in k_render
+    if (!skipped && ss.tile_done[tile_rm]) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // warp w: the 8x4 block (w mod 2, w div 2) of the half; lane l: (l mod 8, l div 8)
     const int lx = (warp & 1) * 8 + (lane & 7), ly = half * 8 + (warp >> 1) * 4 + (lane >> 3);
@@ -481,13 +486,13 @@ k_render_half(const RenderBatch batch) {
     bool done = !in_p;
     const float e_low = st.e_low, t_min = st.t_min;
     const size_t pix = in_p ? (size_t)y * cam.width + x : 0;
-    if (in_p) {   // resume the state slice 0 left
+    if (in_p && !skipped) {   // resume the state slice 0 left
         const float4 a = ss.pst[pix];
         const int4 b = ss.pis[pix];
         T = a.x; C0 = a.y; C1 = a.z; C2 = a.w;
         cnt = b.x; last = b.y; done = b.w != 0; stop = done ? b.z : 0;
     }
-    int32_t fbase = ss.tile_fbase[tile_rm];
+    int32_t fbase = skipped ? 0 : ss.tile_fbase[tile_rm];
     column_range(ss, tx, lane, warp, &s_range);
     __syncthreads();
     const uint2 range = s_range;

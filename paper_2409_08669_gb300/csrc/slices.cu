@@ -3,19 +3,23 @@
 // stops within the first ~1-3% of its depth-ordered list, so most column runs
 // are never read.  The frame therefore builds the column runs in two slices
 // of the depth order:
-//   slice 0: the nearest V/16 Gaussians with tiles (all their runs);
+//   slice 0: the nearest V/16 Gaussians with tiles (all their runs; in the
+//            binned depth order, up to the end of a bin);
 //   slice 1: the other Gaussians that touch a tile with a pixel still going
-//            after slice 0 (a stable compaction of the depth order).
+//            after slice 0, in depth order.
 // Render blends slice 0, keeps the state of the unfinished tiles, and blends
 // slice 1 into them.  A tile's list is the concatenation of its slice-0 and
 // slice-1 lists, which is its full list with only Gaussians behind its last
 // pixel's stop left out, so every pixel is the same as from the full list.
 //
-//   k_slice0_setup   counters of slice 0 (its Gaussians, runs, the pair flag)
+//   k_slice0_setup   counters of slice 0 (its Gaussians, runs, the pair flag),
+//                    after the radix sort
 //   k_sat_rows / k_sat_cols
 //                    summed-area table of the unfinished tiles
+//   k_survivor_bins  slice 1's Gaussians for the kernels of bins.cu, which sort
+//                    them and scan their runs
 //   k_surv_count / k_surv_scan / k_surv_scatter
-//                    stable compaction of the Gaussians [K0, V) whose tile
+//                    the same from the radix sort's order: stable compaction of the Gaussians [K0, V) whose tile
 //                    rectangle holds an unfinished tile, with their run
 //                    offsets and chunk starts and slice 1's counters
 #include "adr_internal.cuh"
@@ -106,6 +110,50 @@ __device__ __forceinline__ bool survives(uint32_t box, const uint32_t* __restric
     const uint32_t s = __ldg(sat + (size_t)y1 * W + x1) - __ldg(sat + (size_t)y0 * W + x1) -
                        __ldg(sat + (size_t)y1 * W + x0) + __ldg(sat + (size_t)y0 * W + x0);
     return s != 0u;
+}
+
+// Slice 1 of the binned depth order: the Gaussians in bins of slice 0's limit or
+// beyond whose rectangle holds an unfinished tile, counted in depth bins of
+// their own.  Four consecutive Gaussians per thread, in index order: nothing
+// here needs the order of the farther Gaussians, so a sliced frame never sorts
+// them.  Bound by the 8 B per Gaussian read and 4 written, and by one scattered
+// atomic per kept Gaussian.
+__global__ void __launch_bounds__(kSurvThreads)
+k_survivor_bins(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ boxes, int64_t n, int sat_w,
+                const uint32_t* __restrict__ sat, const FrameParams* __restrict__ fp, BinMap map,
+                const uint32_t* __restrict__ counters, uint32_t* __restrict__ bins,
+                uint32_t* __restrict__ rank) {
+    pdl_prologue();
+    const uint32_t base = bin_base(fp->cam.near_z), limit = counters[kCntSliceBin];
+    const int64_t i0 = 4 * ((int64_t)blockIdx.x * kSurvThreads + threadIdx.x);
+    if (i0 >= n) return;
+    uint32_t k[4], x[4], r[4];
+    const bool full = i0 + 4 <= n;
+    if (full) {
+        const uint4 a = *reinterpret_cast<const uint4*>(keys + i0);
+        const uint4 b = *reinterpret_cast<const uint4*>(boxes + i0);
+        k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
+        x[0] = b.x; x[1] = b.y; x[2] = b.z; x[3] = b.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            k[q] = i0 + q < n ? keys[i0 + q] : 0u;
+            x[q] = i0 + q < n ? boxes[i0 + q] : 0xFFFFFFFFu;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t bin = bin_of(k[q], base, map);
+        r[q] = kNoRank;
+        if (x[q] != 0xFFFFFFFFu && bin >= limit && survives(x[q], sat, sat_w)) r[q] = atomicAdd(bins + bin, 1u);
+    }
+    if (full) {
+        *reinterpret_cast<uint4*>(rank + i0) = make_uint4(r[0], r[1], r[2], r[3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i0 + q < n) rank[i0 + q] = r[q];
+    }
 }
 
 // Positions [K0 + b * per, K0 + (b + 1) * per) of the depth order for CTA b.
@@ -269,21 +317,32 @@ void launch_slice0_setup(const uint32_t* counters, const uint32_t* offsets, uint
     launch_pdl(k_slice0_setup, 1, 1, 0, stream, counters, offsets, c0);
 }
 
-void launch_survivors(const uint32_t* tile_done, int tiles_x, int tiles_y, uint32_t* sat,
-                      const uint32_t* sorted_box, const uint32_t* order, const uint32_t* counters,
-                      int grid, uint32_t* cnt, uint8_t* keep_flag, int64_t n_max, int64_t chunk_max,
-                      uint32_t* s_order, uint32_t* s_box, uint32_t* s_offsets,
-                      uint32_t* s_chunk_first, uint32_t* c1, uint32_t* status, cudaStream_t stream) {
+void launch_unfinished_table(const uint32_t* tile_done, int tiles_x, int tiles_y, uint32_t* sat,
+                             cudaStream_t stream) {
     const int warps = kSurvThreads / 32;
     launch_pdl(k_sat_rows, (tiles_y + 1 + warps - 1) / warps, kSurvThreads, 0, stream, tile_done, tiles_x,
                                                                                tiles_y, sat);
     launch_pdl(k_sat_cols, (tiles_x + 1 + warps - 1) / warps, kSurvThreads, 0, stream, tiles_x, tiles_y, sat);
+}
+
+void launch_survivors(int tiles_x, const uint32_t* sat, const uint32_t* sorted_box, const uint32_t* order,
+                      const uint32_t* counters, int grid, uint32_t* cnt, uint8_t* keep_flag, int64_t n_max,
+                      int64_t chunk_max, uint32_t* s_order, uint32_t* s_box, uint32_t* s_offsets,
+                      uint32_t* s_chunk_first, uint32_t* c1, uint32_t* status, cudaStream_t stream) {
     launch_pdl(k_surv_count, grid, kSurvThreads, 0, stream, sorted_box, counters, sat, tiles_x, grid, cnt,
                                                     keep_flag);
     launch_pdl(k_surv_scan, 1, kMaxTileGrid / 8, 0, stream, cnt, grid, counters, c1);
     launch_pdl(k_surv_scatter, grid, kSurvThreads, 0, stream, sorted_box, order, counters, keep_flag, grid,
                                                       cnt, n_max, chunk_max, s_order, s_box,
                                                       s_offsets, s_chunk_first, status);
+}
+
+void launch_survivor_bins(const uint32_t* keys, const uint32_t* boxes, int64_t n, int tiles_x,
+                          const uint32_t* sat, const FrameParams* fp, const BinMap& map,
+                          const uint32_t* counters, uint32_t* bins, uint32_t* rank, cudaStream_t stream) {
+    if (n <= 0) return;
+    launch_pdl(k_survivor_bins, (unsigned)((n + 4 * kSurvThreads - 1) / (4 * kSurvThreads)), kSurvThreads, 0,
+               stream, keys, boxes, n, tiles_x + 1, sat, fp, map, counters, bins, rank);
 }
 
 }  // namespace adr
