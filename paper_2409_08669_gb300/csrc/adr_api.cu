@@ -287,7 +287,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
         ALLOC(w.sat, (tx + 1) * (ty + 1) * sizeof(uint32_t));
     }
     ALLOC(w.g2d, N * 9 * sizeof(float));
-    ALLOC(w.load_sums, 4 * sizeof(double));
+    ALLOC(w.load_sums, 8 * sizeof(double));
     ALLOC(w.hist, kHistWords * sizeof(uint32_t));
     // the zeroed block; bin counts grow with n, so the largest scene's fit every one
     const size_t zero_words = kZeroWords + 2 * bin_map(max_gaussians).count;

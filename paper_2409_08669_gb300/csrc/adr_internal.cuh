@@ -184,7 +184,7 @@ struct Workspace {
     float* tfin = nullptr;                 // [max pixels] final transmittance of the last render
     int32_t* lstat = nullptr;              // [max pixels] l_i | terminated << 31 of the last render
     float* g2d = nullptr;                  // [max_n * 9] backward: dL/d(px, py, conic, sigma, rgb)
-    double* load_sums = nullptr;           // [4] load-balancing loss moments
+    double* load_sums = nullptr;           // [8] load-balancing loss: mean, std at 2, 3; integer sums from 4
     uint32_t* hist = nullptr;              // [kHistWords]
     uint32_t* counters = nullptr;          // [kCntSlots], the start of the zeroed block
     unsigned long long* sums = nullptr;    // [kSumSlots * kSumStride] pairs and runs (in the zeroed block)
@@ -573,6 +573,37 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// Paired FP32 operations (sm_100+): each half rounds as the scalar one does.
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 fsub2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "sub.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
 }
 
 // The eigen-form quadratic of a Gaussian at a pixel, shared by Render and its
