@@ -183,7 +183,7 @@ struct Workspace {
     int32_t* trav = nullptr;               // [max pixels]
     float* tfin = nullptr;                 // [max pixels] final transmittance of the last render
     int32_t* lstat = nullptr;              // [max pixels] l_i | terminated << 31 of the last render
-    float* g2d = nullptr;                  // [max_n * 9] backward: dL/d(px, py, conic, sigma, rgb)
+    float* g2d = nullptr;                  // [max_n * 9] backward: moments of v (1, x, y, xx, xy, yy), dL/drgb
     double* load_sums = nullptr;           // [8] load-balancing loss: mean, std at 2, 3; integer sums from 4
     uint32_t* hist = nullptr;              // [kHistWords]
     uint32_t* counters = nullptr;          // [kCntSlots], the start of the zeroed block
@@ -556,7 +556,7 @@ void launch_survivor_bins(const uint32_t* keys, const uint32_t* boxes, int64_t n
 
 // Backward (backward.cu).
 void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec,
-                            const float4* aux, const FrameParams* fp, int num_tiles,
+                            const FrameParams* fp, int num_tiles,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
                             cudaStream_t stream);
@@ -572,6 +572,14 @@ void launch_preprocess_backward(int n, const float* means, const float* scales, 
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 1 / x with the hardware's approximate reciprocal (PTX rcp.approx.ftz, relative
+// error ~2^-23).
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -601,6 +609,16 @@ __device__ __forceinline__ float2 fsub2(float2 a, float2 b) {
     asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
         "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
         "sub.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;

@@ -5,10 +5,13 @@
 //
 //   k_render_backward     per tile, walks each pixel's blended Gaussians from
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
-//                         and accumulates dL/d(px, py, conic, sigma, rgb);
-//                         warp-reduced, then atomicAdd into 9 floats per Gaussian.
-//   k_preprocess_backward chain rule from those 2D quantities to means, scales,
-//                         rotations, opacities and SH coefficients.
+//                         and accumulates the moments of v = alpha dL/dalpha about
+//                         the Gaussian's centre (1, x, y, xx, xy, yy) and its
+//                         colour gradient; warp-reduced, then atomicAdd into 9
+//                         floats per Gaussian.
+//   k_preprocess_backward dL/d(px, py, conic, sigma) from the moments, and the
+//                         chain rule to means, scales, rotations, opacities and
+//                         SH coefficients.
 //   k_load_moments / k_load_grad
 //                         L_load = std over pixels of l_i (Eq. 13, population
 //                         form) and dL_load/dl_i = (l_i - mean) / (HW std).
@@ -17,156 +20,192 @@
 namespace adr {
 namespace {
 
-constexpr int kBwdThreads = kTilePixels;
+constexpr int kBwdThreads = kTilePixels / 2;   // two vertically adjacent pixels per thread
+constexpr int kBwdWarps = kBwdThreads / 32;
+constexpr int kBwdStage = 256;                 // list positions staged at a time
 
-// Sum over the warp of nine per-lane values, as a reduce-scatter over 16
-// slots (slots 9-15 zero) by recursive halving: at distance 16, 8, 4, 2 each
-// lane keeps half of its slots (the half bit 4, 3, 2, 1 of its lane selects)
-// and adds its partner's copy of them, then pairs (lane, lane ^ 1) add; 16
-// shuffles instead of 45.  Lanes 2s and 2s + 1 end with the total of slot s.
+// Sum over the warp of nine per-lane values, as a reduce-scatter by recursive
+// halving: at distance 16, 8, 4 and 2 the lanes whose bit is clear keep the first
+// ceil(n / 2) of their n values and the others the rest (5 and 4 of 9, then 3 and
+// 2, 2 and 1, 1), each adding its partner's copy of them, then pairs add: 12
+// shuffles.  Lanes 2 s and 2 s + 1 share one value; reduce_slot says which.
 __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) {
-    float a[16];
+    float a[9];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = i < 9 ? v[i] : 0.f;
+    for (int i = 0; i < 9; ++i) a[i] = v[i];
+    constexpr int kKeep[4] = {5, 3, 2, 1};   // kept by the lower lanes
+    int n = 9;
 #pragma unroll
-    for (int half = 8, dist = 16; half >= 1; half >>= 1, dist >>= 1) {
+    for (int step = 0; step < 4; ++step) {
+        const int dist = 16 >> step, keep = kKeep[step];
         const bool up = (lane & dist) != 0;
 #pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const float send = up ? a[i] : a[i + half];
-            const float keep = up ? a[i + half] : a[i];
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, dist);
+        for (int i = 0; i < keep; ++i) {
+            const float hi = i + keep < n ? a[i + keep] : 0.f;   // none for the odd one
+            const float send = up ? a[i] : hi, own = up ? hi : a[i];
+            a[i] = own + __shfl_xor_sync(0xffffffffu, send, dist);
         }
+        n = keep;
     }
     return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
+// The slot (0..8) whose total a lane ends with; -1 for lanes left without one.
+__device__ __forceinline__ int reduce_slot(int lane) {
+    constexpr int kKeep[4] = {5, 3, 2, 1};
+    int base = 0, n = 9;   // the slots the lane still holds: base .. base + n - 1
+#pragma unroll
+    for (int step = 0; step < 4; ++step) {
+        if (lane & (16 >> step)) {
+            base += kKeep[step];
+            n -= kKeep[step];
+        } else {
+            n = min(n, kKeep[step]);
+        }
+    }
+    return n > 0 ? base : -1;
+}
 
-__global__ void __launch_bounds__(kBwdThreads, 5)   // 5 CTAs per SM: <= 48 registers
+// One CTA of 128 threads per tile, its pixels laid out as in k_render: warp w has
+// the 8x8 quadrant (w mod 2, w div 2), a lane two vertically adjacent pixels.
+// Bound by instruction issue.  What a (warp, Gaussian) costs is mostly the sum
+// over lanes, so a warp covers 64 pixels in a compact square (a Gaussian of a few
+// pixels meets few of them), the pixels' arithmetic is paired FP32, and the nine
+// sums are the ones that need no Gaussian constant: with v = -2 dL/dq (zero where
+// alpha is clamped) the moments of v about the Gaussian's centre and the colour
+// weights.  Both pixels of a thread share dx, so its moments come from three
+// values.  k_preprocess_backward applies the conic and the opacity once per
+// Gaussian.  1M Gaussians at 1280x720: 650 us with a pixel per thread, 16x2-pixel
+// warps and nine finished gradients per pixel (646M warp instructions), 246 us now
+// (187M).
+__global__ void __launch_bounds__(kBwdThreads, 6)   // 80 registers; 5, 7 and 8 CTAs per SM: 249, 252, 256 us
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
-                  const float4* __restrict__ rec, const float4* __restrict__ aux,
+                  const float4* __restrict__ rec,
                   const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
                   const float* __restrict__ t_final, const int32_t* __restrict__ lstat,
                   const float* __restrict__ dl_dimg, const float* __restrict__ dl_dload,
                   float* __restrict__ g2d) {
-    __shared__ float2 s_xy[kBwdThreads];
-    __shared__ float2 s_k[kBwdThreads];       // quad_k of the Gaussian at this tile
-    __shared__ float4 s_w[kBwdThreads];
-    __shared__ float4 s_c[kBwdThreads];
-    __shared__ float4 s_conic[kBwdThreads];   // conic a, b, c, sigma
-    __shared__ uint32_t s_g[kBwdThreads];
+    __shared__ float4 s_kl[kBwdStage];    // quad_k (two), log2(sigma), centre x from the tile origin
+    __shared__ float4 s_nw[kBwdStage];    // -w1x, -w2x, -w1y, -w2y
+    __shared__ float4 s_cy[kBwdStage];    // red, green, blue, centre y
+    __shared__ uint32_t s_g[kBwdStage];
+    __shared__ int s_max[kBwdWarps];
 
-    const CamDev cam = fp->cam;
-    const SetDev st = fp->st;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tiles_x = fp->cam.tiles_x, width = fp->cam.width, height = fp->cam.height;
+    const float e_low = fp->st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
     const int tile = blockIdx.x;
-    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
-    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
+    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int lx = (warp & 1) * 8 + (lane & 7), ly = (warp >> 1) * 8 + 2 * (lane >> 3);
     const int x = tx * kTile + lx, y = ty * kTile + ly;
-    const bool inside = x < cam.width && y < cam.height;
     const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-    const float fx = (float)lx, fy = (float)ly;
-    const size_t hw = (size_t)cam.width * cam.height;
-    const size_t pix = inside ? (size_t)y * cam.width + x : 0;
-
+    const float fx = (float)lx, fya = (float)ly;
+    const size_t hw = (size_t)width * height;
     const uint2 range = ranges[tile];
-    int32_t last = inside ? last_pos[pix] : 0;          // 1-based position of the last blend
-    float T = inside ? t_final[pix] : 1.f;
-    float g0 = 0.f, g1 = 0.f, g2 = 0.f, gl = 0.f;
-    if (inside) {
-        g0 = dl_dimg[pix];
-        g1 = dl_dimg[hw + pix];
-        g2 = dl_dimg[2 * hw + pix];
-        if (dl_dload) gl = dl_dload[pix];
-    }
+    if (range.x >= range.y) return;
+
+    // Pixel a in .x, pixel b in .y.
+    int32_t last_a = 0, last_b = 0;       // 1-based position of the last blend
+    float2 T = make_float2(1.f, 1.f);
+    float2 g0 = make_float2(0.f, 0.f), g1 = g0, g2 = g0, gl = g0, gl_stop = g0;
     // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
     // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
     // that stopped (a more opaque Gaussian makes it stop sooner).
-    float gl_stop = 0.f;
-    if (st.load_grad == ADR_LOAD_GRAD_TERMINATION && inside && gl != 0.f && lstat) {
-        const int32_t ls = lstat[pix];
-        if (ls < 0 && T < 1.f) {
-            gl_stop = gl * -(float)(ls & 0x7FFFFFFF) / -logf(T);
-            gl = 0.f;
+    const bool termination = fp->st.load_grad == ADR_LOAD_GRAD_TERMINATION && lstat;
+    auto pixel = [&](size_t pix, int32_t& last, float& t, float& r, float& g, float& b, float& l, float& l_stop) {
+        last = last_pos[pix];
+        t = t_final[pix];
+        r = dl_dimg[pix];
+        g = dl_dimg[hw + pix];
+        b = dl_dimg[2 * hw + pix];
+        if (!dl_dload) return;
+        l = dl_dload[pix];
+        if (termination && l != 0.f) {
+            const int32_t ls = lstat[pix];
+            if (ls < 0 && t < 1.f) {
+                l_stop = l * -(float)(ls & 0x7FFFFFFF) / -logf(t);
+                l = 0.f;
+            }
         }
-    }
-    float acc0 = st.bg[0], acc1 = st.bg[1], acc2 = st.bg[2];   // colour behind the current Gaussian
-    const float e_low = st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
+    };
+    const size_t pixa = (size_t)y * width + x;
+    if (x < width && y < height) pixel(pixa, last_a, T.x, g0.x, g1.x, g2.x, gl.x, gl_stop.x);
+    if (x < width && y + 1 < height) pixel(pixa + width, last_b, T.y, g0.y, g1.y, g2.y, gl.y, gl_stop.y);
+    float2 acc0 = make_float2(fp->st.bg[0], fp->st.bg[0]);   // colour behind the current Gaussian
+    float2 acc1 = make_float2(fp->st.bg[1], fp->st.bg[1]);
+    float2 acc2 = make_float2(fp->st.bg[2], fp->st.bg[2]);
+    const float2 fx2 = make_float2(fx, fx), fya2 = make_float2(fya, fya), fyb2 = make_float2(fya + 1.f, fya + 1.f);
+    const float2 one2 = make_float2(1.f, 1.f);
+    const int slot = (lane & 1) ? -1 : reduce_slot(lane);
 
-    if (range.x < range.y) {
-        // The longest prefix any pixel of the warp, and of the tile, needs.
-        const int warp_last = __reduce_max_sync(0xffffffffu, last);
-        const int max_last = warp_last;
-        __shared__ int s_max[kBwdThreads / 32];
-        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = max_last;
+    // The longest prefix any pixel of the warp, and of the tile, needs.
+    const int warp_last = __reduce_max_sync(0xffffffffu, max(last_a, last_b));
+    if (lane == 0) s_max[warp] = warp_last;
+    __syncthreads();
+    int tile_last = 0;
+#pragma unroll
+    for (int w = 0; w < kBwdWarps; ++w) tile_last = max(tile_last, s_max[w]);
+    // Batches of list positions, from the back.
+    for (int bend = tile_last; bend > 0; bend -= kBwdStage) {
+        const int bstart = max(0, bend - kBwdStage);
         __syncthreads();
-        int tile_last = 0;
-        for (int w = 0; w < kBwdThreads / 32; ++w) tile_last = max(tile_last, s_max[w]);
-        // Batches of 256 list positions, from the back.
-        for (int bend = tile_last; bend > 0; bend -= kBwdThreads) {
-            const int bstart = max(0, bend - kBwdThreads);
-            __syncthreads();
-            const int pos = bstart + threadIdx.x;
-            if (pos < bend) {
-                const uint32_t g = sorted_gauss[range.x + pos];
-                const float4 r0 = rec[3 * (size_t)g + 0];
-                const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
-                                             __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
-                const float4 w = rec[3 * (size_t)g + 1];
-                s_xy[threadIdx.x] = c;
-                s_k[threadIdx.x] = quad_k(c, w);
-                s_w[threadIdx.x] = w;
-                s_c[threadIdx.x] = rec[3 * (size_t)g + 2];
-                s_conic[threadIdx.x] = aux[2 * (size_t)g + 0];
-                s_g[threadIdx.x] = g;
-            }
-            __syncthreads();
-            // this warp's positions: none of its pixels blended one past warp_last
-            for (int p = min(bend, warp_last) - 1; p >= bstart; --p) {
-                const int j = p - bstart;
-                bool contrib = false;
-                float d_px = 0.f, d_py = 0.f, d_ca = 0.f, d_cb = 0.f, d_cc = 0.f, d_sig = 0.f;
-                float d_r = 0.f, d_g = 0.f, d_b = 0.f;
-                if (p < last) {
-                    // Same evaluation as the forward pass, so the same skip decision.
-                    const float2 c = s_xy[j];
-                    const float4 w = s_w[j];
-                    const float4 col = s_c[j];
-                    const float dx = c.x - fx, dy = c.y - fy;
-                    const float e = quad_exponent(s_k[j], w, col.w, fx, fy);
-                    if (e >= e_low) {
-                        const float raw = ex2_approx(e);
-                        const float alpha = fminf(0.99f, raw);
-                        contrib = true;
-                        const float one_m = 1.f - alpha;
-                        T = T / one_m;                                    // T before this blend
-                        const float wgt = alpha * T;
-                        d_r = wgt * g0;
-                        d_g = wgt * g1;
-                        d_b = wgt * g2;
-                        float dalpha = T * ((col.x - acc0) * g0 + (col.y - acc1) * g1 + (col.z - acc2) * g2);
-                        dalpha += gl + gl_stop / one_m;                   // load term
-                        acc0 = fmaf(col.x, alpha, one_m * acc0);
-                        acc1 = fmaf(col.y, alpha, one_m * acc1);
-                        acc2 = fmaf(col.z, alpha, one_m * acc2);
-                        if (raw < 0.99f) {                                // not clamped
-                            const float4 cn = s_conic[j];
-                            d_sig = dalpha * raw / cn.w;                  // alpha = sigma * G
-                            const float dq = -0.5f * raw * dalpha;        // G = exp(-q/2)
-                            d_px = dq * 2.f * fmaf(cn.x, dx, cn.y * dy);
-                            d_py = dq * 2.f * fmaf(cn.y, dx, cn.z * dy);
-                            d_ca = dq * dx * dx;
-                            d_cb = dq * 2.f * dx * dy;
-                            d_cc = dq * dy * dy;
-                        }
-                    }
-                }
-                if (__any_sync(0xffffffffu, contrib)) {
-                    const int lane = threadIdx.x & 31;
-                    const float v[9] = {d_px, d_py, d_ca, d_cb, d_cc, d_sig, d_r, d_g, d_b};
-                    const float tot = reduce_scatter9(v, lane);
-                    const int slot = (lane >> 1) & 15;   // the slot lane's total belongs to
-                    if (!(lane & 1) && slot < 9) atomicAdd(g2d + (size_t)s_g[j] * 9 + slot, tot);
-                }
-            }
+        for (int j = threadIdx.x; j < bend - bstart; j += kBwdThreads) {
+            const uint32_t g = sorted_gauss[range.x + bstart + j];
+            const float4 r0 = rec[3 * (size_t)g + 0];
+            const float4 w = rec[3 * (size_t)g + 1];
+            const float4 col = rec[3 * (size_t)g + 2];
+            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+            const float2 k = quad_k(c, w);
+            s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
+            s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
+            s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
+            s_g[j] = g;
+        }
+        __syncthreads();
+        // this warp's positions: none of its pixels blended one past warp_last
+#pragma unroll 2
+        for (int j = min(bend, warp_last) - bstart - 1; j >= 0; --j) {
+            const int p = bstart + j;
+            const float4 kl = s_kl[j];
+            const float4 nw = s_nw[j];
+            // Same evaluation as the forward pass, so the same skip decision.
+            const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
+            const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
+            const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
+            const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
+            const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
+            const bool la = ea >= e_low && p < last_a, lb = eb >= e_low && p < last_b;
+            if (!__any_sync(0xffffffffu, la || lb)) continue;
+            const float4 cy = s_cy[j];
+            // A pixel that did not blend this Gaussian has raw = alpha = 0, which
+            // leaves its T and colour as they are and adds nothing to the sums.
+            const float2 raw = make_float2(la ? ex2_approx(ea) : 0.f, lb ? ex2_approx(eb) : 0.f);
+            const float2 alpha = make_float2(fminf(0.99f, raw.x), fminf(0.99f, raw.y));
+            const float2 one_m = fsub2(one2, alpha);
+            // 1 / (1 - alpha): the hardware reciprocal and one Newton step
+            float2 inv = make_float2(rcp_approx(one_m.x), rcp_approx(one_m.y));
+            inv = ffma2(inv, ffma2(make_float2(-one_m.x, -one_m.y), inv, one2), inv);
+            T = fmul2(T, inv);                                   // T before this blend
+            const float2 wgt = fmul2(alpha, T);
+            const float2 d0 = fsub2(make_float2(cy.x, cy.x), acc0), d1 = fsub2(make_float2(cy.y, cy.y), acc1),
+                         d2 = fsub2(make_float2(cy.z, cy.z), acc2);
+            float2 dalpha = fmul2(T, ffma2(d2, g2, ffma2(d1, g1, fmul2(d0, g0))));
+            dalpha = fadd2(dalpha, ffma2(gl_stop, inv, gl));     // load term
+            acc0 = ffma2(alpha, d0, acc0);                       // alpha c + (1 - alpha) acc
+            acc1 = ffma2(alpha, d1, acc1);
+            acc2 = ffma2(alpha, d2, acc2);
+            float2 v = fmul2(raw, dalpha);                       // alpha = sigma G, G = exp(-q / 2)
+            if (!(raw.x < 0.99f)) v.x = 0.f;                     // clamped
+            if (!(raw.y < 0.99f)) v.y = 0.f;
+            const float dx = kl.w - fx, dya = cy.w - fya, dyb = dya - 1.f;
+            const float V = v.x + v.y;
+            const float vya = v.x * dya, vyb = v.y * dyb;
+            const float Vy = vya + vyb, Vyy = fmaf(vyb, dyb, vya * dya), Vx = V * dx;
+            const float sums[9] = {V, Vx, Vy, Vx * dx, Vy * dx, Vyy,
+                                   fmaf(wgt.x, g0.x, wgt.y * g0.y), fmaf(wgt.x, g1.x, wgt.y * g1.y),
+                                   fmaf(wgt.x, g2.x, wgt.y * g2.y)};
+            const float tot = reduce_scatter9(sums, lane);
+            if (slot >= 0) atomicAdd(g2d + (size_t)s_g[j] * 9 + slot, tot);
         }
     }
 }
@@ -232,8 +271,14 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
         for (int j = 0; j < 12; ++j) gsh4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
         const float* G = g2d + (size_t)i * 9;
-        const float gpx = G[0], gpy = G[1], gca = G[2], gcb = G[3], gcc = G[4];
-        go = G[5];
+        // With q = C_a dx^2 + 2 C_b dx dy + C_c dy^2 and v = -2 dL/dq per pixel:
+        // dL/dC from the second moments, dL/dp from C times the first ones, and
+        // dL/dsigma = V / sigma.
+        const float4 cn = aux[2 * (size_t)i];
+        const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
+        const float gpx = -fmaf(Ca, G[1], Cb * G[2]), gpy = -fmaf(Cb, G[1], Cc * G[2]);
+        const float gca = -0.5f * G[3], gcb = -G[4], gcc = -0.5f * G[5];
+        go = G[0] / cn.w;
         const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
         // --- colour: rgb = max(0, sum_k sh_k Y_k(d) + 0.5), d = (X0 - cam) / |X0 - cam|
         float vx = mx - cam.cam_pos[0], vy = my - cam.cam_pos[1], vz = mz - cam.cam_pos[2];
@@ -318,8 +363,6 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
             for (int c = 0; c < 3; ++c) T[r][c] = J[r][0] * V[c] + J[r][1] * V[4 + c] + J[r][2] * V[8 + c];
         // dL/dSigma' = -C G_C C with the conic C (from the forward pass) and the
         // symmetric gradient G_C = [[gca, gcb/2], [gcb/2, gcc]].
-        const float4 cn = aux[2 * (size_t)i];
-        const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
         const float Ga = gca, Gb = 0.5f * gcb, Gc = gcc;
         // X = G_C C
         const float X00 = Ga * Ca + Gb * Cb, X01 = Ga * Cb + Gb * Cc;
@@ -491,13 +534,13 @@ k_load_grad(const int32_t* __restrict__ load, int64_t hw, double* __restrict__ s
 }  // namespace
 
 void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec,
-                            const float4* aux, const FrameParams* fp, int num_tiles,
+                            const FrameParams* fp, int num_tiles,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
                             cudaStream_t stream) {
     const int tiles = num_tiles;
     if (tiles <= 0) return;
-    k_render_backward<<<tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, aux, fp,
+    k_render_backward<<<tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, fp,
                                                          last, t_final, lstat, dl_dimg, dl_dload, g2d);
 }
 
