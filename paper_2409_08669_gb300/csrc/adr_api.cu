@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <vector>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -198,14 +199,7 @@ void free_workspace(Workspace& w) {
         delete w.prof;
         w.prof = nullptr;
     }
-    void* ptrs[] = {w.rec, w.aux, w.depth_key, w.offsets, w.gbox, w.sorted_box, w.sortbuf,
-                    w.order, w.win_lo, w.rank, w.s_win_lo, w.pruns, w.prows, w.pgauss, w.tcounts, w.tile_counts,
-                    w.chunk_first, w.ranges, w.last, w.trav, w.tfin, w.lstat, w.g2d, w.load_sums,
-                    w.hist, w.counters, w.status, w.lookback, w.d_fp, w.d_stage,
-                    w.s_order, w.s_box, w.s_offsets, w.s_chunk_first,
-                    w.surv_cnt, w.surv_flag, w.pst, w.pis, w.tile_done, w.tile_fbase, w.sat};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    if (w.arena) cudaFree(w.arena);
     w = Workspace{};
 }
 
@@ -240,15 +234,18 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     const size_t N = (size_t)max_gaussians, P = (size_t)pair_capacity;
     const size_t pixels = (size_t)max_width * max_height;
     w.lookback_words = ((N + kSortChunk - 1) / kSortChunk + 2) * kRadix;
-#define ALLOC(ptr, bytes)                                                                   \
-    do {                                                                                    \
-        e = cudaMalloc((void**)&(ptr), (bytes));                                           \
-        if (e != cudaSuccess) {                                                             \
-            (void)cudaGetLastError(); /* not sticky: clear it for the next launch check */  \
-            free_workspace(w);                                                              \
-            return fail(ADR_ERR_CUDA, "cudaMalloc(%zu) for %s: %s", (size_t)(bytes), #ptr,  \
-                        cudaGetErrorString(e));                                             \
-        }                                                                                   \
+    // One allocation: a cudaMalloc costs tens of microseconds, and a workspace
+    // has some forty buffers.  Each starts at a 256-byte boundary.
+    struct Piece {
+        void** ptr;
+        size_t at;
+    };
+    std::vector<Piece> pieces;
+    size_t total = 0;
+#define ALLOC(p, bytes)                                                     \
+    do {                                                                    \
+        pieces.push_back({reinterpret_cast<void**>(&(p)), total});          \
+        total += ((size_t)(bytes) + 255) & ~(size_t)255;                    \
     } while (0)
     ALLOC(w.rec, N * kRecFloat4 * sizeof(float4));
     ALLOC(w.aux, N * kAuxFloat4 * sizeof(float4));
@@ -292,15 +289,22 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     // the zeroed block; bin counts grow with n, so the largest scene's fit every one
     const size_t zero_words = kZeroWords + 2 * bin_map(max_gaussians).count;
     ALLOC(w.counters, zero_words * sizeof(uint32_t));
-    w.slice_counters = w.counters + kCntSlots;
-    w.ttotals = w.slice_counters + 2 * kCntSlots;
-    w.sums = reinterpret_cast<unsigned long long*>(w.ttotals + kTotalSets * kRadix);
-    w.bins = w.counters + kZeroWords;
     ALLOC(w.status, sizeof(uint32_t) * 4);
     ALLOC(w.lookback, w.lookback_words * sizeof(unsigned long long));
     ALLOC(w.d_fp, sizeof(FrameParams));
     ALLOC(w.d_stage, sizeof(uint32_t));
 #undef ALLOC
+    e = cudaMalloc(&w.arena, total);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();   // not sticky: clear it for the next launch check
+        w = Workspace{};
+        return fail(ADR_ERR_CUDA, "cudaMalloc(%zu) for the workspace: %s", total, cudaGetErrorString(e));
+    }
+    for (const Piece& p : pieces) *p.ptr = static_cast<unsigned char*>(w.arena) + p.at;
+    w.slice_counters = w.counters + kCntSlots;
+    w.ttotals = w.slice_counters + 2 * kCntSlots;
+    w.sums = reinterpret_cast<unsigned long long*>(w.ttotals + kTotalSets * kRadix);
+    w.bins = w.counters + kZeroWords;
     if (cudaMemset(w.lookback, 0, w.lookback_words * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(w.status, 0, sizeof(uint32_t) * 4) != cudaSuccess ||
         cudaMemset(w.counters, 0, zero_words * sizeof(uint32_t)) != cudaSuccess ||

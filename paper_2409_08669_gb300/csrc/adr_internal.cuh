@@ -157,6 +157,7 @@ struct Profiler {
 // Device buffers one frame needs.  The context path allocates them with
 // cudaMalloc; the allocation-free path carves them out of a static array.
 struct Workspace {
+    void* arena = nullptr;                 // the context path's one allocation (all buffers below)
     int64_t max_n = 0, capacity = 0;       // Gaussians, Gaussian-tile pairs
     int max_tiles = 0;
     int sm_count = 0, sort_grid = 0, scan_grid = 0, tile_grid = 0, window_grid = 0;
