@@ -31,13 +31,32 @@ namespace {
 // pixels, and the blend of the two pixels is one paired sequence without
 // branches (weight alpha T, then T - alpha T, which is T (1 - alpha) of Eq. 3
 // with one rounding fewer): every pixel takes exactly the decisions of
-// quad_exponent's scalar evaluation, which the backward uses too.  The loop
-// is unrolled by four.
+// quad_exponent's scalar evaluation, which the backward uses too.
+//
+// Bound by instruction issue (70 to 75% of the slots while all SMs are busy).  Of
+// the staged Gaussians only a part blends at a pixel of a given quadrant (measured
+// on a CPU walk of 60 tiles each: 22% for 150k large Gaussians at 1001x667, 40% with the plain
+// rectangles, 65% at 1M to 3M and 1080p), so staging tests each against the four
+// quadrants (quadrants_reached, exact up to its rounding margin) and a warp walks
+// its quadrant's own list.  What it walks nearly always blends, so the loop has no
+// skip: two list entries a step, straight-line, with one vote per step for the
+// rare stop.  With one entry a step, every entry evaluated and a vote and a branch
+// for the skip and the stop each, a step was a chain of about 200 clocks where a
+// tile's warp is alone on its scheduler.  Frames before -> after: 150k 1001x667
+// 316 -> 182 us, 600k plain 720p 262 -> 195, 3M 1080p 579 -> 516, 3M 4K 1087 -> 969,
+// 2k 64x48 160 -> 137.  Four entries a step: fewer instructions, but 72 registers
+// and more steps with a stop in them (3M 4K 974, 16 served frames 3305 against
+// 3140).  Staging 128 at a time: 3M 1080p 534.
 constexpr int kRenderThreads = kTilePixels / 2;
 constexpr int kStage = kTilePixels;          // Gaussians staged per batch
 constexpr int kRenderWarps = kRenderThreads / 32;
+static_assert(kStage % kRenderThreads == 0, "whole rounds of staging");
+constexpr int kGroup = 2;                    // list entries blended per step
 constexpr float kInf = __builtin_huge_valf();
 
+__device__ __forceinline__ float4 at_offset(const float4* s, uint32_t bytes) {
+    return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s) + bytes);
+}
 
 // Column tx's run range [start, end) in its pass's column lists (empty after
 // a pair overflow); warp 0 writes it to *out, the caller synchronises.
@@ -127,23 +146,84 @@ __device__ __forceinline__ uint32_t stage_column_batch(uint32_t base, uint32_t e
     return total;
 }
 
+// Which of the tile's 8x8 quadrants a Gaussian can blend in, as bits
+// (quadrant x, y at bit x + 2 y): those with a point where its exponent
+// log2(sigma) - |u|^2 reaches the limit.  |u|^2 is a convex quadratic, so its
+// minimum over a rectangle lies at the centre's nearest x or y edge line, at the
+// other coordinate's minimiser clamped to the rectangle; u is formed from k and
+// w as the pixels form it.  A quadrant is dropped only where the bound holds
+// with every rounding on the wrong side: the errors of k, of u and of the
+// minimiser are a few ulp of `scale` (the largest term that cancels in u), and
+// those of the exponent a few ulp of its own terms.  Comparisons with a NaN keep
+// the quadrant.
+__device__ __forceinline__ uint32_t quadrants_reached(float2 c, float2 k, float4 w, float log2_sigma, float e_lim) {
+    const float thr = log2_sigma - e_lim;
+    if (thr < 0.f) return 0u;   // no pixel reaches the limit: |u|^2 >= 0
+    const float scale = (fabsf(w.x) + fabsf(w.z)) * (fabsf(c.x) + 16.f) + (fabsf(w.y) + fabsf(w.w)) * (fabsf(c.y) + 16.f);
+    const float reach = sqrtf(thr) + fmaf(4e-6f, scale, 1e-5f);
+    const float most = fmaf(reach, reach, fmaf(1e-6f, fabsf(log2_sigma) + fabsf(e_lim), 1e-5f));
+    const float A = fmaf(w.x, w.x, w.z * w.z), B = fmaf(w.x, w.y, w.z * w.w), C = fmaf(w.y, w.y, w.w * w.w);
+    const float slope_y = -B * rcp_approx(C), slope_x = -B * rcp_approx(A);   // the minimiser's drift per pixel off centre
+    float xs[2], ys[2], fy[2], fx[2];
+    float2 ux[2], uy[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float lo = 8.f * (float)h, hi = lo + 7.f;
+        xs[h] = fminf(fmaxf(c.x, lo), hi);
+        ys[h] = fminf(fmaxf(c.y, lo), hi);
+        fy[h] = fmaf(slope_y, xs[h] - c.x, c.y);   // y of the minimum on the line x = xs
+        fx[h] = fmaf(slope_x, ys[h] - c.y, c.x);
+        ux[h] = make_float2(fmaf(-w.x, xs[h], k.x), fmaf(-w.z, xs[h], k.y));
+        uy[h] = make_float2(fmaf(-w.y, ys[h], k.x), fmaf(-w.w, ys[h], k.y));
+    }
+    uint32_t out = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int hx = q & 1, hy = q >> 1;
+        const float y = fminf(fmaxf(fy[hx], 8.f * (float)hy), 8.f * (float)hy + 7.f);
+        const float x = fminf(fmaxf(fx[hy], 8.f * (float)hx), 8.f * (float)hx + 7.f);
+        const float a1 = fmaf(-w.y, y, ux[hx].x), a2 = fmaf(-w.w, y, ux[hx].y);
+        const float b1 = fmaf(-w.x, x, uy[hy].x), b2 = fmaf(-w.z, x, uy[hy].y);
+        const float least = fminf(fmaf(a1, a1, a2 * a2), fmaf(b1, b1, b2 * b2));
+        if (!(least > most)) out |= 1u << q;
+    }
+    return out;
+}
+
 // The m staged Gaussians' terms, the centre taken relative to the tile origin
-// (ox, oy): (hi - origin) is exact, one rounding for lo.  Ends with a barrier.
+// (ox, oy): (hi - origin) is exact, one rounding for lo.  With kLists the
+// Gaussians each quadrant can blend are marked in s_mask[quadrant][slot / 32].
+// Ends with a barrier.
+template <bool kLists>
 __device__ __forceinline__ void stage_records(int m, const uint32_t* s_gid, const float4* __restrict__ rec,
-                                              float ox, float oy, float4* s_kl, float4* s_nw,
-                                              float4* s_rg, float2* s_bb) {
-    for (int sl = threadIdx.x; sl < m; sl += kRenderThreads) {
-        const uint32_t gi = s_gid[sl];
-        const float4 r0 = rec[3 * (size_t)gi + 0];
-        const float4 w = rec[3 * (size_t)gi + 1];
-        const float4 col = rec[3 * (size_t)gi + 2];
-        const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
-                                     __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
-        const float2 k = quad_k(c, w);
-        s_kl[sl] = make_float4(k.x, k.y, col.w, 0.f);   // k1, k2, log2(sigma), -
-        s_nw[sl] = make_float4(-w.x, -w.z, -w.y, -w.w);  // -w1x, -w2x, -w1y, -w2y
-        s_rg[sl] = make_float4(col.x, col.x, col.y, col.y);
-        s_bb[sl] = make_float2(col.z, col.z);
+                                              float ox, float oy, float e_lim, float4* s_kl, float4* s_nw,
+                                              float4* s_rg, uint32_t (*s_mask)[kStage / 32]) {
+    const int lane = threadIdx.x & 31;
+    for (int s0 = 0; s0 < m; s0 += kRenderThreads) {
+        const int sl = s0 + (int)threadIdx.x;
+        uint32_t reached = 0u;
+        if (sl < m) {
+            const uint32_t gi = s_gid[sl];
+            const float4 r0 = rec[3 * (size_t)gi + 0];
+            const float4 w = rec[3 * (size_t)gi + 1];
+            const float4 col = rec[3 * (size_t)gi + 2];
+            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+            const float2 k = quad_k(c, w);
+            s_kl[sl] = make_float4(k.x, k.y, col.w, col.z);   // k1, k2, log2(sigma), blue
+            s_nw[sl] = make_float4(-w.x, -w.z, -w.y, -w.w);   // -w1x, -w2x, -w1y, -w2y
+            s_rg[sl] = make_float4(col.x, col.x, col.y, col.y);
+            if (kLists) reached = quadrants_reached(c, k, w, col.w, e_lim);
+        }
+        if (kLists) {
+            uint32_t mine = 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t b = __ballot_sync(0xffffffffu, (reached >> q) & 1u);
+                if (lane == q) mine = b;
+            }
+            if (lane < 4) s_mask[lane][sl >> 5] = mine;
+        }
     }
     __syncthreads();
 }
@@ -152,20 +232,17 @@ __device__ __forceinline__ void stage_records(int m, const uint32_t* s_gid, cons
 // frames; one camera otherwise): blocks [tile_begin[b], tile_begin[b + 1])
 // are camera b's tiles.
 // The tile's constants, kept in shared memory so that the blend loop holds
-// only its own state in registers: with them, and the pixels' stop positions,
-// out of the registers and the single-camera launch indexing no camera array,
-// the column-run kernel of one camera fits 56 registers without spilling,
-// i.e. 9 CTAs (36 warps) per SM.
+// only its own state in registers.
 struct TileInfo {
     int width, height, tiles_x, tiles_y, tx, ty;
 };
 
-#ifndef ADR_RENDER_CTAS
-#define ADR_RENDER_CTAS 9   // CTAs per SM: 56 registers, no spills (10: 48 with spills)
-#endif
+// CTAs per SM: 64 registers, no spills.  Frame at 4K, 3M Gaussians: 8 CTAs 969 us,
+// 9 (56 registers, small spills) 976, 7 982.
+constexpr int kRenderCtas = 8;
 // kBatched: blocks of several cameras (the serving scheduler's batched frames).
 template <bool kRuns, bool kBatched>
-__global__ void __launch_bounds__(kRenderThreads, ADR_RENDER_CTAS)
+__global__ void __launch_bounds__(kRenderThreads, kRenderCtas)
 k_render(const RenderBatch batch) {
     pdl_prologue();
     int cb = 0;
@@ -175,11 +252,12 @@ k_render(const RenderBatch batch) {
     }
     __shared__ uint32_t s_tstart;
     __shared__ TileInfo s_ti;
-    __shared__ float4 s_kl[kStage];    // k1, k2, log2(sigma), -
-    __shared__ float4 s_nw[kStage];    // -w1x, -w2x, -w1y, -w2y
-    __shared__ float4 s_rg[kStage];    // red, red, green, green
-    __shared__ float2 s_bb[kStage];    // blue, blue
+    __shared__ float4 s_kl[kStage + 1];    // k1, k2, log2(sigma), blue; the last reaches no pixel
+    __shared__ float4 s_nw[kStage + 1];    // -w1x, -w2x, -w1y, -w2y
+    __shared__ float4 s_rg[kStage + 1];    // red, red, green, green
     __shared__ uint32_t s_gid[kStage];
+    __shared__ uint32_t s_mask[kRenderWarps][kStage / 32];      // staged Gaussians each quadrant can blend
+    __shared__ alignas(8) uint32_t s_list[kRenderWarps][kStage + 2 * kGroup];   // the same, as byte offsets in s_kl
     __shared__ int2 s_stop[kRenderThreads];             // each thread's stop positions (0: none)
     __shared__ uint32_t s_wsum[kRenderWarps];           // kept runs per warp
     __shared__ uint32_t s_next;
@@ -207,7 +285,8 @@ k_render(const RenderBatch batch) {
     // Each pixel's limit on the exponent: a Gaussian reaches it iff e >= limit.
     // e_low while the pixel blends; +inf for a pixel outside the image or
     // one that stopped (done), so the skip test needs no separate flag.
-    const float e_low = batch.cam[cb].fp->st.e_low, t_min = batch.cam[cb].fp->st.t_min;
+    // Below 2^-126 the 2^e of the blend is 0 (ftz), which blends nothing.
+    const float e_low = fmaxf(batch.cam[cb].fp->st.e_low, -126.f), t_min = batch.cam[cb].fp->st.t_min;
     float2 elim = make_float2((x0 < cam.width && ya0 < cam.height) ? e_low : kInf,
                               (x0 < cam.width && ya0 + 1 < cam.height) ? e_low : kInf);
     const int tile_rm0 = ty0 * cam.tiles_x + tx0;
@@ -247,6 +326,10 @@ k_render(const RenderBatch batch) {
         fbase = ss.tile_fbase[tile_rm0];
     }
     s_stop[threadIdx.x] = stop;
+    if (threadIdx.x == 0) {
+        s_kl[kStage] = make_float4(0.f, 0.f, -kInf, 0.f);
+        s_nw[kStage] = s_rg[kStage] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     if (kRuns) {   // column tx's runs start after the runs of the columns before it
         column_range(batch.cam[cb].ss, tx0, lane, warp, &s_range);
     }
@@ -277,68 +360,100 @@ k_render(const RenderBatch batch) {
             next = base + total;
         }
         const int m = (int)min(total, (uint32_t)kStage);
-        stage_records(m, s_gid, batch.cam[cb].rec, (float)(tx * kTile), (float)(ty * kTile), s_kl, s_nw,
-                      s_rg, s_bb);
+        stage_records<true>(m, s_gid, batch.cam[cb].rec, (float)(tx * kTile), (float)(ty * kTile), e_low, s_kl, s_nw,
+                            s_rg, s_mask);
         if (!__all_sync(0xffffffffu, fminf(elim.x, elim.y) == kInf)) {   // warp-uniform: the loop votes
+            // The quadrant's own list, padded to a whole group.
+            uint32_t* list = s_list[warp];
+            int n = 0;
+            for (int wd = 0; 32 * wd < m; ++wd) {
+                const uint32_t b = s_mask[warp][wd];
+                if ((b >> lane) & 1u) list[n + __popc(b & ((1u << lane) - 1u))] = (uint32_t)(32 * wd + lane) * 16u;
+                n += __popc(b);
+            }
+            if (lane < 2 * kGroup) list[n + lane] = kStage * 16u;
+            __syncwarp();
             // A pixel becomes done only where it stops (its exponent limit
             // then becomes +inf, so no later Gaussian reaches it), and the
-            // loop leaves there once every pixel of the warp is done.  The batch goes in
-            // windows of 32 positions: bit k of bits_a / bits_b records that
-            // pixel a / b blended position j0 + k, and each window's bits are
+            // loop leaves there once every pixel of the warp is done.  The list goes in
+            // windows of 32 entries: bit k of bits_a / bits_b records that
+            // pixel a / b blended entry i0 + k, and each window's bits are
             // folded into l_i (their count) and the last blended position
             // (their highest bit) when the window ends.
             bool warp_done = false;
+            uint2 ahead = *reinterpret_cast<const uint2*>(list);   // the next group's entries
 #pragma unroll 1
-            for (int j0 = 0; j0 < m && !warp_done; j0 += 32) {
-                const int len = min(32, m - j0);
+            for (int i0 = 0; i0 < n && !warp_done; i0 += 32) {
+                const int len = min(32, n - i0);
                 uint32_t bits_a = 0u, bits_b = 0u;
-#pragma unroll 4
-                for (int k = 0; k < len; ++k) {
-                    const int j = j0 + k;
-                    const float4 kl = s_kl[j];
-                    const float4 nw = s_nw[j];
-                    // u = (k - w_x fx) - w_y fy, the fx-term shared, as quad_exponent
-                    const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
-                    const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
-                    const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
-                    // e = log2(sigma) - q log2(e) / 2; alpha = min(0.99, 2^e) (Eq. 2)
-                    // reaches alpha_low iff e >= e_low
-                    const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
-                    const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
-                    const bool la = ea >= elim.x, lb = eb >= elim.y;
-                    if (!__any_sync(0xffffffffu, la || lb)) continue;   // no pixel of the warp reaches alpha_low
-                    // Front-to-back step (Eq. 3), both pixels at once: a pixel
-                    // that skips has alpha 0 here, so T and C stay as they are.
-                    float2 alpha = make_float2(la ? fminf(0.99f, ex2_approx(ea)) : 0.f,
+#pragma unroll 1
+                for (int k = 0; k < len && !warp_done; k += kGroup) {
+                    const uint32_t off[kGroup] = {ahead.x, ahead.y};
+                    ahead = *reinterpret_cast<const uint2*>(list + i0 + k + kGroup);
+                    float2 alpha[kGroup], wgt[kGroup], now = T;
+                    float blue[kGroup];
+                    uint32_t na = 0u, nb = 0u;
+#pragma unroll
+                    for (int q = 0; q < kGroup; ++q) {
+                        const float4 kl = at_offset(s_kl, off[q]);
+                        const float4 nw = at_offset(s_nw, off[q]);
+                        blue[q] = kl.w;
+                        // u = (k - w_x fx) - w_y fy, the fx-term shared, as quad_exponent
+                        const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
+                        const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
+                        const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
+                        // e = log2(sigma) - q log2(e) / 2; alpha = min(0.99, 2^e) (Eq. 2)
+                        // reaches alpha_low iff e >= e_low
+                        const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
+                        const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
+                        const bool la = ea >= elim.x, lb = eb >= elim.y;
+                        // A pixel that skips has alpha 0, so T and C stay as they are.
+                        alpha[q] = make_float2(la ? fminf(0.99f, ex2_approx(ea)) : 0.f,
                                                lb ? fminf(0.99f, ex2_approx(eb)) : 0.f);
-                    // T (1 - alpha) = T - alpha T
-                    float2 wgt = fmul2(alpha, T);
-                    float2 test_T = fsub2(T, wgt);
-                    // a done pixel keeps T >= t_min, so only a pixel stopping here can vote
-                    if (__any_sync(0xffffffffu, fminf(test_T.x, test_T.y) < t_min)) {
-                        // rare: a pixel stops before this Gaussian, which it does not blend
-                        const int32_t pos = fbase + j + 1;
-                        if (test_T.x < t_min) { alpha.x = wgt.x = 0.f; test_T.x = T.x; s_stop[threadIdx.x].x = pos; elim.x = kInf; }
-                        if (test_T.y < t_min) { alpha.y = wgt.y = 0.f; test_T.y = T.y; s_stop[threadIdx.x].y = pos; elim.y = kInf; }
-                        if (__all_sync(0xffffffffu, fminf(elim.x, elim.y) == kInf)) {   // nothing blends this Gaussian
-                            warp_done = true;
-                            break;
-                        }
+                        if (la) na |= 1u << q;
+                        if (lb) nb |= 1u << q;
                     }
-                    const float4 rg = s_rg[j];
-                    C0 = ffma2(make_float2(rg.x, rg.y), wgt, C0);
-                    C1 = ffma2(make_float2(rg.z, rg.w), wgt, C1);
-                    C2 = ffma2(s_bb[j], wgt, C2);
-                    T = test_T;
-                    const uint32_t bit = 1u << k;
-                    // blended: alpha >= alpha_low (> 0) and the pixel did not stop here
-                    if (alpha.x > 0.f) bits_a |= bit;
-                    if (alpha.y > 0.f) bits_b |= bit;
+                    // Front-to-back steps (Eq. 3), both pixels at once: T (1 - alpha) = T - alpha T
+#pragma unroll
+                    for (int q = 0; q < kGroup; ++q) {
+                        wgt[q] = fmul2(alpha[q], now);
+                        now = fsub2(now, wgt[q]);
+                    }
+                    // T never grows, and a done pixel keeps T >= t_min: some pixel stops
+                    // in this group iff its last T is below t_min.
+                    if (__any_sync(0xffffffffu, fminf(now.x, now.y) < t_min)) {
+                        // The steps again, each pixel up to the Gaussian it stops before,
+                        // which it does not blend.
+                        now = T;
+#pragma unroll
+                        for (int q = 0; q < kGroup; ++q) {
+                            const int32_t pos = fbase + (int32_t)(off[q] / 16u) + 1;
+                            if (elim.x == kInf) alpha[q].x = 0.f;
+                            if (elim.y == kInf) alpha[q].y = 0.f;
+                            wgt[q] = fmul2(alpha[q], now);
+                            float2 t = fsub2(now, wgt[q]);
+                            if (t.x < t_min) { wgt[q].x = 0.f; t.x = now.x; s_stop[threadIdx.x].x = pos; elim.x = kInf; na &= (1u << q) - 1u; }
+                            if (t.y < t_min) { wgt[q].y = 0.f; t.y = now.y; s_stop[threadIdx.x].y = pos; elim.y = kInf; nb &= (1u << q) - 1u; }
+                            now = t;
+                        }
+                        warp_done = __all_sync(0xffffffffu, fminf(elim.x, elim.y) == kInf);
+                    }
+                    T = now;
+#pragma unroll
+                    for (int q = 0; q < kGroup; ++q) {
+                        const float4 rg = at_offset(s_rg, off[q]);
+                        C0 = ffma2(make_float2(rg.x, rg.y), wgt[q], C0);
+                        C1 = ffma2(make_float2(rg.z, rg.w), wgt[q], C1);
+                        C2 = ffma2(make_float2(blue[q], blue[q]), wgt[q], C2);
+                    }
+                    bits_a |= na << k;
+                    bits_b |= nb << k;
                 }
                 cnt_a += __popc(bits_a);
                 cnt_b += __popc(bits_b);
-                if (bits_a) last_a = fbase + j0 + 32 - __clz(bits_a);   // 1-based position of the highest bit
-                if (bits_b) last_b = fbase + j0 + 32 - __clz(bits_b);
+                // 1-based position of the highest bit's Gaussian
+                if (bits_a) last_a = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_a)] / 16u);
+                if (bits_b) last_b = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_b)] / 16u);
             }
         }
         fbase += m;
@@ -432,7 +547,6 @@ k_render_half(const RenderBatch batch) {
     __shared__ float4 s_kl[kStage];
     __shared__ float4 s_nw[kStage];
     __shared__ float4 s_rg[kStage];
-    __shared__ float2 s_bb[kStage];
     __shared__ uint32_t s_gid[kStage];
     __shared__ uint32_t s_wsum[kRenderWarps];
     __shared__ uint32_t s_next;
@@ -454,7 +568,7 @@ k_render_half(const RenderBatch batch) {
     float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
     int32_t cnt = 0, last = 0, stop = 0;
     bool done = !in_p;
-    const float e_low = st.e_low, t_min = st.t_min;
+    const float e_low = fmaxf(st.e_low, -126.f), t_min = st.t_min;   // as in k_render
     const size_t pix = in_p ? (size_t)y * cam.width + x : 0;
     if (in_p && !skipped) {   // resume the state slice 0 left
         const float4 a = ss.pst[pix];
@@ -473,7 +587,7 @@ k_render_half(const RenderBatch batch) {
         const uint32_t total = stage_column_batch(base, range.y, ty, rc.rows, rc.runs, s_gid, s_wsum,
                                                   &s_next, lane, warp, &next);
         const int m = (int)min(total, (uint32_t)kStage);
-        stage_records(m, s_gid, rc.rec, ox, oy, s_kl, s_nw, s_rg, s_bb);
+        stage_records<false>(m, s_gid, rc.rec, ox, oy, 0.f, s_kl, s_nw, s_rg, nullptr);
         if (!__all_sync(0xffffffffu, done)) {
 #pragma unroll 1
             for (int j = 0; j < m; ++j) {
@@ -494,7 +608,7 @@ k_render_half(const RenderBatch batch) {
                 const float4 rg = s_rg[j];
                 C0 = fmaf(rg.x, wgt, C0);
                 C1 = fmaf(rg.z, wgt, C1);
-                C2 = fmaf(s_bb[j].x, wgt, C2);
+                C2 = fmaf(kl.w, wgt, C2);
                 T = test_T;
                 if (l) { ++cnt; last = fbase + j + 1; }
             }
