@@ -556,7 +556,7 @@ void launch_survivor_bins(const uint32_t* keys, const uint32_t* boxes, int64_t n
                           const uint32_t* counters, uint32_t* bins, uint32_t* rank, cudaStream_t stream);
 
 // Backward (backward.cu).
-void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec,
+void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
                             const FrameParams* fp, int num_tiles,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
@@ -638,6 +638,72 @@ __device__ __forceinline__ float quad_exponent(float2 k, float4 w, float log2_si
     const float u1 = fmaf(-w.y, fy, fmaf(-w.x, fx, k.x));
     const float u2 = fmaf(-w.w, fy, fmaf(-w.z, fx, k.y));
     return fmaf(-u1, u1, fmaf(-u2, u2, log2_sigma));
+}
+
+// Which of the four kW x kH pixel rectangles of a tile (row by row) a Gaussian can
+// blend in, as bits: those with a point where its exponent log2(sigma) - |u|^2
+// reaches the limit.  |u|^2 is a convex quadratic, so its minimum over a rectangle
+// lies at the centre's nearest x or y edge line, at the other coordinate's
+// minimiser clamped to the rectangle; u is formed from k and w as the pixels form
+// it.  A rectangle is dropped only where the bound holds with every rounding on
+// the wrong side: the errors of k, of u and of the minimiser are a few ulp of
+// `scale` (the largest term that cancels in u), and those of the exponent a few
+// ulp of its own terms.  Comparisons with a NaN keep the rectangle.
+template <int kW, int kH>
+__device__ __forceinline__ uint32_t rects_reached(float2 c, float2 k, float4 w, float log2_sigma, float e_lim) {
+    constexpr int kNx = kTile / kW, kNy = kTile / kH;
+    static_assert(kNx * kNy == 4 && kNx * kW == kTile && kNy * kH == kTile, "four rectangles cover the tile");
+    const float thr = log2_sigma - e_lim;
+    if (thr < 0.f) return 0u;   // no pixel reaches the limit: |u|^2 >= 0
+    const float scale = (fabsf(w.x) + fabsf(w.z)) * (fabsf(c.x) + 16.f) + (fabsf(w.y) + fabsf(w.w)) * (fabsf(c.y) + 16.f);
+    const float reach = sqrtf(thr) + fmaf(4e-6f, scale, 1e-5f);
+    const float most = fmaf(reach, reach, fmaf(1e-6f, fabsf(log2_sigma) + fabsf(e_lim), 1e-5f));
+    const float A = fmaf(w.x, w.x, w.z * w.z), B = fmaf(w.x, w.y, w.z * w.w), C = fmaf(w.y, w.y, w.w * w.w);
+    const float slope_y = -B * rcp_approx(C), slope_x = -B * rcp_approx(A);   // the minimiser's drift per pixel off centre
+    float2 ux[kNx], uy[kNy];
+    float fy[kNx], fx[kNy];
+#pragma unroll
+    for (int i = 0; i < kNx; ++i) {
+        const float xs = fminf(fmaxf(c.x, (float)(kW * i)), (float)(kW * i + kW - 1));
+        fy[i] = fmaf(slope_y, xs - c.x, c.y);   // y of the minimum on the line x = xs
+        ux[i] = make_float2(fmaf(-w.x, xs, k.x), fmaf(-w.z, xs, k.y));
+    }
+#pragma unroll
+    for (int i = 0; i < kNy; ++i) {
+        const float ys = fminf(fmaxf(c.y, (float)(kH * i)), (float)(kH * i + kH - 1));
+        fx[i] = fmaf(slope_x, ys - c.y, c.x);
+        uy[i] = make_float2(fmaf(-w.y, ys, k.x), fmaf(-w.w, ys, k.y));
+    }
+    uint32_t out = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int hx = q % kNx, hy = q / kNx;
+        const float y = fminf(fmaxf(fy[hx], (float)(kH * hy)), (float)(kH * hy + kH - 1));
+        const float x = fminf(fmaxf(fx[hy], (float)(kW * hx)), (float)(kW * hx + kW - 1));
+        const float a1 = fmaf(-w.y, y, ux[hx].x), a2 = fmaf(-w.w, y, ux[hx].y);
+        const float b1 = fmaf(-w.x, x, uy[hy].x), b2 = fmaf(-w.z, x, uy[hy].y);
+        const float least = fminf(fmaf(a1, a1, a2 * a2), fmaf(b1, b1, b2 * b2));
+        if (!(least > most)) out |= 1u << q;
+    }
+    return out;
+}
+
+// The record at a byte offset of a float4 array in shared memory.
+__device__ __forceinline__ float4 at_offset(const float4* s, uint32_t bytes) {
+    return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s) + bytes);
+}
+
+// A warp's own list of the m staged Gaussians: those marked in `mask` (32 a word),
+// as byte offsets of 16-byte records.  Returns their number; the caller syncs the warp.
+__device__ __forceinline__ int warp_list(const uint32_t* mask, int m, int lane, uint32_t* list) {
+    int n = 0;
+    for (int wd = 0; 32 * wd < m; ++wd) {
+        uint32_t b = mask[wd];
+        if (m - 32 * wd < 32) b &= (1u << (m - 32 * wd)) - 1u;
+        if ((b >> lane) & 1u) list[n + __popc(b & ((1u << lane) - 1u))] = (uint32_t)(32 * wd + lane) * 16u;
+        n += __popc(b);
+    }
+    return n;
 }
 
 // 1-D taps of the SSIM window (the 2-D window is their outer product).

@@ -5,13 +5,13 @@
 //
 //   k_render_backward     per tile, walks each pixel's blended Gaussians from
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
-//                         and accumulates the moments of v = alpha dL/dalpha about
-//                         the Gaussian's centre (1, x, y, xx, xy, yy) and its
-//                         colour gradient; warp-reduced, then atomicAdd into 9
-//                         floats per Gaussian.
-//   k_preprocess_backward dL/d(px, py, conic, sigma) from the moments, and the
-//                         chain rule to means, scales, rotations, opacities and
-//                         SH coefficients.
+//                         and accumulates, with v = alpha dL/dalpha, sum v, dL/d(px,
+//                         py), the second moments of v about the Gaussian's centre
+//                         and its colour gradient; warp-reduced, then atomicAdd
+//                         into 9 floats per Gaussian.
+//   k_preprocess_backward dL/d(conic, sigma) from the moments, and the chain rule
+//                         to means, scales, rotations, opacities and SH
+//                         coefficients.
 //   k_load_moments / k_load_grad
 //                         L_load = std over pixels of l_i (Eq. 13, population
 //                         form) and dL_load/dl_i = (l_i - mean) / (HW std).
@@ -25,10 +25,10 @@ constexpr int kBwdWarps = kBwdThreads / 32;
 constexpr int kBwdStage = 256;                 // list positions staged at a time
 
 // Sum over the warp of nine per-lane values, as a reduce-scatter by recursive
-// halving: at distance 16, 8, 4 and 2 the lanes whose bit is clear keep the first
+// halving: at distance 8, 4, 2 and 1 the lanes whose bit is clear keep the first
 // ceil(n / 2) of their n values and the others the rest (5 and 4 of 9, then 3 and
-// 2, 2 and 1, 1), each adding its partner's copy of them, then pairs add: 12
-// shuffles.  Lanes 2 s and 2 s + 1 share one value; reduce_slot says which.
+// 2, 2 and 1, 1), each adding its partner's copy of them, then the warp's halves
+// add: 12 shuffles.  Lanes s and s + 16 share one value; reduce_slot says which.
 __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) {
     float a[9];
 #pragma unroll
@@ -37,7 +37,7 @@ __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) 
     int n = 9;
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
-        const int dist = 16 >> step, keep = kKeep[step];
+        const int dist = 8 >> step, keep = kKeep[step];
         const bool up = (lane & dist) != 0;
 #pragma unroll
         for (int i = 0; i < keep; ++i) {
@@ -47,7 +47,7 @@ __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) 
         }
         n = keep;
     }
-    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 16);
 }
 // The slot (0..8) whose total a lane ends with; -1 for lanes left without one.
 __device__ __forceinline__ int reduce_slot(int lane) {
@@ -55,7 +55,7 @@ __device__ __forceinline__ int reduce_slot(int lane) {
     int base = 0, n = 9;   // the slots the lane still holds: base .. base + n - 1
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
-        if (lane & (16 >> step)) {
+        if (lane & (8 >> step)) {
             base += kKeep[step];
             n -= kKeep[step];
         } else {
@@ -65,21 +65,24 @@ __device__ __forceinline__ int reduce_slot(int lane) {
     return n > 0 ? base : -1;
 }
 
-// One CTA of 128 threads per tile, its pixels laid out as in k_render: warp w has
-// the 8x8 quadrant (w mod 2, w div 2), a lane two vertically adjacent pixels.
-// Bound by instruction issue.  What a (warp, Gaussian) costs is mostly the sum
-// over lanes, so a warp covers 64 pixels in a compact square (a Gaussian of a few
-// pixels meets few of them), the pixels' arithmetic is paired FP32, and the nine
-// sums are the ones that need no Gaussian constant: with v = -2 dL/dq (zero where
-// alpha is clamped) the moments of v about the Gaussian's centre and the colour
-// weights.  Both pixels of a thread share dx, so its moments come from three
-// values.  k_preprocess_backward applies the conic and the opacity once per
-// Gaussian.  1M Gaussians at 1280x720: 650 us with a pixel per thread, 16x2-pixel
-// warps and nine finished gradients per pixel (646M warp instructions), 246 us now
-// (187M).
-__global__ void __launch_bounds__(kBwdThreads, 6)   // 80 registers; 5, 7 and 8 CTAs per SM: 249, 252, 256 us
+// One CTA of 128 threads per tile: warp w has the 16x4-pixel strip w, a lane two
+// vertically adjacent pixels, whose arithmetic is paired FP32.  Bound by
+// instruction issue: a (warp, Gaussian) that blends costs about 90 instructions,
+// 30 of them the sum over lanes, so a warp walks only the staged Gaussians that
+// reach its strip (rects_reached) up to its last blended position.
+//
+// The sums are dL/d(px, py) of each pixel, the second moments of v = -2 dL/dq
+// about the centre, sum v and the colour weights; k_preprocess_backward scales
+// them once per Gaussian.  Long thin Gaussians amplify the rounding of the sums by
+// the square of their axes' ratio (to about 1e-3 of a scale's gradient), so they
+// are taken as finely as pixel by pixel: each pixel's terms are rounded on their
+// own and added along a row pair first.  1M Gaussians at 1280x720: 650 us with a pixel
+// per thread in 16x2-pixel warps that walk the whole list, 247 us now.  (Moments of
+// both pixels at once in 8x8 squares took 210 us, but their rounding put a scale's
+// gradient up to 3e-3 elsewhere, three times what this form does.)
+__global__ void __launch_bounds__(kBwdThreads, 6)   // 80 registers; 4 to 8 CTAs per SM are within 1.5%
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
-                  const float4* __restrict__ rec,
+                  const float4* __restrict__ rec, const float4* __restrict__ aux,
                   const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
                   const float* __restrict__ t_final, const int32_t* __restrict__ lstat,
                   const float* __restrict__ dl_dimg, const float* __restrict__ dl_dload,
@@ -87,7 +90,9 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     __shared__ float4 s_kl[kBwdStage];    // quad_k (two), log2(sigma), centre x from the tile origin
     __shared__ float4 s_nw[kBwdStage];    // -w1x, -w2x, -w1y, -w2y
     __shared__ float4 s_cy[kBwdStage];    // red, green, blue, centre y
-    __shared__ uint32_t s_g[kBwdStage];
+    __shared__ float4 s_cn[kBwdStage];    // conic a, b, c, the Gaussian
+    __shared__ uint32_t s_mask[kBwdWarps][kBwdStage / 32];   // staged Gaussians that reach each strip
+    __shared__ uint32_t s_list[kBwdWarps][kBwdStage];
     __shared__ int s_max[kBwdWarps];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -95,7 +100,7 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     const float e_low = fp->st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
     const int tile = blockIdx.x;
     const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int lx = (warp & 1) * 8 + (lane & 7), ly = (warp >> 1) * 8 + 2 * (lane >> 3);
+    const int lx = lane & 15, ly = 4 * warp + 2 * (lane >> 4);
     const int x = tx * kTile + lx, y = ty * kTile + ly;
     const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
     const float fx = (float)lx, fya = (float)ly;
@@ -135,7 +140,8 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     float2 acc2 = make_float2(fp->st.bg[2], fp->st.bg[2]);
     const float2 fx2 = make_float2(fx, fx), fya2 = make_float2(fya, fya), fyb2 = make_float2(fya + 1.f, fya + 1.f);
     const float2 one2 = make_float2(1.f, 1.f);
-    const int slot = (lane & 1) ? -1 : reduce_slot(lane);
+    const int slot = lane < 16 ? reduce_slot(lane) : -1;
+    const float e_lim = fmaxf(e_low, -126.f);   // below it alpha is 0 (ex2_approx flushes)
 
     // The longest prefix any pixel of the warp, and of the tile, needs.
     const int warp_last = __reduce_max_sync(0xffffffffu, max(last_a, last_b));
@@ -148,26 +154,44 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     for (int bend = tile_last; bend > 0; bend -= kBwdStage) {
         const int bstart = max(0, bend - kBwdStage);
         __syncthreads();
-        for (int j = threadIdx.x; j < bend - bstart; j += kBwdThreads) {
-            const uint32_t g = sorted_gauss[range.x + bstart + j];
-            const float4 r0 = rec[3 * (size_t)g + 0];
-            const float4 w = rec[3 * (size_t)g + 1];
-            const float4 col = rec[3 * (size_t)g + 2];
-            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
-                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
-            const float2 k = quad_k(c, w);
-            s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
-            s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
-            s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
-            s_g[j] = g;
+        const int m = bend - bstart;
+        for (int j0 = 0; j0 < m; j0 += kBwdThreads) {
+            const int j = j0 + (int)threadIdx.x;
+            uint32_t reached = 0u;
+            if (j < m) {
+                const uint32_t g = sorted_gauss[range.x + bstart + j];
+                const float4 r0 = rec[3 * (size_t)g + 0];
+                const float4 w = rec[3 * (size_t)g + 1];
+                const float4 col = rec[3 * (size_t)g + 2];
+                const float4 cn = aux[2 * (size_t)g];
+                const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                             __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+                const float2 k = quad_k(c, w);
+                s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
+                s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
+                s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
+                s_cn[j] = make_float4(cn.x, cn.y, cn.z, __uint_as_float(g));
+                reached = rects_reached<16, 4>(c, k, w, col.w, e_lim);
+            }
+            uint32_t mine = 0u;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t bits = __ballot_sync(0xffffffffu, (reached >> q) & 1u);
+                if (lane == q) mine = bits;
+            }
+            if (lane < 4) s_mask[lane][j >> 5] = mine;
         }
         __syncthreads();
         // this warp's positions: none of its pixels blended one past warp_last
+        const uint32_t* list = s_list[warp];
+        const int n = warp_list(s_mask[warp], min(bend, warp_last) - bstart, lane, s_list[warp]);
+        __syncwarp();
 #pragma unroll 2
-        for (int j = min(bend, warp_last) - bstart - 1; j >= 0; --j) {
-            const int p = bstart + j;
-            const float4 kl = s_kl[j];
-            const float4 nw = s_nw[j];
+        for (int i = n - 1; i >= 0; --i) {
+            const uint32_t off = list[i];
+            const int p = bstart + (int)(off / 16u);
+            const float4 kl = at_offset(s_kl, off);
+            const float4 nw = at_offset(s_nw, off);
             // Same evaluation as the forward pass, so the same skip decision.
             const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
             const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
@@ -176,36 +200,43 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
             const bool la = ea >= e_low && p < last_a, lb = eb >= e_low && p < last_b;
             if (!__any_sync(0xffffffffu, la || lb)) continue;
-            const float4 cy = s_cy[j];
+            const float4 cy = at_offset(s_cy, off);
+            const float4 cn = at_offset(s_cn, off);
             // A pixel that did not blend this Gaussian has raw = alpha = 0, which
             // leaves its T and colour as they are and adds nothing to the sums.
             const float2 raw = make_float2(la ? ex2_approx(ea) : 0.f, lb ? ex2_approx(eb) : 0.f);
             const float2 alpha = make_float2(fminf(0.99f, raw.x), fminf(0.99f, raw.y));
             const float2 one_m = fsub2(one2, alpha);
-            // 1 / (1 - alpha): the hardware reciprocal and one Newton step
+            const float2 less = make_float2(-one_m.x, -one_m.y);
+            // T before this blend, T / (1 - alpha): the hardware reciprocal with a Newton
+            // step, and the quotient with its remainder added (rounded as a division is)
             float2 inv = make_float2(rcp_approx(one_m.x), rcp_approx(one_m.y));
-            inv = ffma2(inv, ffma2(make_float2(-one_m.x, -one_m.y), inv, one2), inv);
-            T = fmul2(T, inv);                                   // T before this blend
+            inv = ffma2(inv, ffma2(less, inv, one2), inv);
+            const float2 quot = fmul2(T, inv);
+            T = ffma2(ffma2(less, quot, T), inv, quot);
             const float2 wgt = fmul2(alpha, T);
             const float2 d0 = fsub2(make_float2(cy.x, cy.x), acc0), d1 = fsub2(make_float2(cy.y, cy.y), acc1),
                          d2 = fsub2(make_float2(cy.z, cy.z), acc2);
-            float2 dalpha = fmul2(T, ffma2(d2, g2, ffma2(d1, g1, fmul2(d0, g0))));
-            dalpha = fadd2(dalpha, ffma2(gl_stop, inv, gl));     // load term
-            acc0 = ffma2(alpha, d0, acc0);                       // alpha c + (1 - alpha) acc
-            acc1 = ffma2(alpha, d1, acc1);
-            acc2 = ffma2(alpha, d2, acc2);
+            const float2 dalpha = ffma2(T, ffma2(d2, g2, ffma2(d1, g1, fmul2(d0, g0))),
+                                        ffma2(gl_stop, inv, gl));   // with the load term
+            acc0 = ffma2(make_float2(cy.x, cy.x), alpha, fmul2(one_m, acc0));
+            acc1 = ffma2(make_float2(cy.y, cy.y), alpha, fmul2(one_m, acc1));
+            acc2 = ffma2(make_float2(cy.z, cy.z), alpha, fmul2(one_m, acc2));
             float2 v = fmul2(raw, dalpha);                       // alpha = sigma G, G = exp(-q / 2)
             if (!(raw.x < 0.99f)) v.x = 0.f;                     // clamped
             if (!(raw.y < 0.99f)) v.y = 0.f;
-            const float dx = kl.w - fx, dya = cy.w - fya, dyb = dya - 1.f;
-            const float V = v.x + v.y;
-            const float vya = v.x * dya, vyb = v.y * dyb;
-            const float Vy = vya + vyb, Vyy = fmaf(vyb, dyb, vya * dya), Vx = V * dx;
-            const float sums[9] = {V, Vx, Vy, Vx * dx, Vy * dx, Vyy,
-                                   fmaf(wgt.x, g0.x, wgt.y * g0.y), fmaf(wgt.x, g1.x, wgt.y * g1.y),
-                                   fmaf(wgt.x, g2.x, wgt.y * g2.y)};
+            const float dx = kl.w - fx;
+            const float2 dx2 = make_float2(dx, dx), dy = fsub2(make_float2(cy.w, cy.w), make_float2(fya2.x, fyb2.x));
+            const float2 tx2 = ffma2(make_float2(cn.x, cn.x), dx2, fmul2(make_float2(cn.y, cn.y), dy));
+            const float2 ty2 = ffma2(make_float2(cn.y, cn.y), dx2, fmul2(make_float2(cn.z, cn.z), dy));
+            const float2 vx = fmul2(v, dx2), vy = fmul2(v, dy);
+            const float2 px = fmul2(v, tx2), py = fmul2(v, ty2);
+            const float2 xx = fmul2(vx, dx2), xy = fmul2(vx, dy), yy = fmul2(vy, dy);
+            const float2 c0 = fmul2(wgt, g0), c1 = fmul2(wgt, g1), c2 = fmul2(wgt, g2);
+            const float sums[9] = {v.x + v.y,   px.x + px.y, py.x + py.y, xx.x + xx.y, xy.x + xy.y,
+                                   yy.x + yy.y, c0.x + c0.y, c1.x + c1.y, c2.x + c2.y};
             const float tot = reduce_scatter9(sums, lane);
-            if (slot >= 0) atomicAdd(g2d + (size_t)s_g[j] * 9 + slot, tot);
+            if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * 9 + slot, tot);
         }
     }
 }
@@ -271,12 +302,11 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
         for (int j = 0; j < 12; ++j) gsh4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
         const float* G = g2d + (size_t)i * 9;
-        // With q = C_a dx^2 + 2 C_b dx dy + C_c dy^2 and v = -2 dL/dq per pixel:
-        // dL/dC from the second moments, dL/dp from C times the first ones, and
-        // dL/dsigma = V / sigma.
+        // With q = C_a dx^2 + 2 C_b dx dy + C_c dy^2 and v = -2 dL/dq per pixel: dL/dC
+        // from the second moments, and dL/dsigma = sum v / sigma.
         const float4 cn = aux[2 * (size_t)i];
         const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
-        const float gpx = -fmaf(Ca, G[1], Cb * G[2]), gpy = -fmaf(Cb, G[1], Cc * G[2]);
+        const float gpx = -G[1], gpy = -G[2];
         const float gca = -0.5f * G[3], gcb = -G[4], gcc = -0.5f * G[5];
         go = G[0] / cn.w;
         const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
@@ -533,14 +563,14 @@ k_load_grad(const int32_t* __restrict__ load, int64_t hw, double* __restrict__ s
 
 }  // namespace
 
-void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec,
+void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
                             const FrameParams* fp, int num_tiles,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
                             cudaStream_t stream) {
     const int tiles = num_tiles;
     if (tiles <= 0) return;
-    k_render_backward<<<tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, fp,
+    k_render_backward<<<tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, aux, fp,
                                                          last, t_final, lstat, dl_dimg, dl_dload, g2d);
 }
 

@@ -466,7 +466,7 @@ void enqueue_backward(const Workspace& ws, const FrameState& fs, const float* me
     if (fs.n <= 0) return;
     cudaMemsetAsync(ws.g2d, 0, (size_t)fs.n * 9 * sizeof(float), stream);
     TIMED(ws, kKRenderBackward, stream,
-          launch_render_backward(ws.ranges, fs.sorted_gauss, ws.rec, ws.d_fp, fs.num_tiles,
+          launch_render_backward(ws.ranges, fs.sorted_gauss, ws.rec, ws.aux, ws.d_fp, fs.num_tiles,
                                  ws.last, ws.tfin, ws.lstat, dl_dimg, dl_dload, ws.g2d, stream));
     TIMED(ws, kKPreprocessBackward, stream,
           launch_preprocess_backward((int)fs.n, means, scales, rots, opac, sh, ws.d_fp, ws.gbox,

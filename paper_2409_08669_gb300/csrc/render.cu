@@ -37,7 +37,7 @@ namespace {
 // the staged Gaussians only a part blends at a pixel of a given quadrant (measured
 // on a CPU walk of 60 tiles each: 22% for 150k large Gaussians at 1001x667, 40% with the plain
 // rectangles, 65% at 1M to 3M and 1080p), so staging tests each against the four
-// quadrants (quadrants_reached, exact up to its rounding margin) and a warp walks
+// quadrants (rects_reached, exact up to its rounding margin) and a warp walks
 // its quadrant's own list.  What it walks nearly always blends, so the loop has no
 // skip: two list entries a step, straight-line, with one vote per step for the
 // rare stop.  With one entry a step, every entry evaluated and a vote and a branch
@@ -53,10 +53,6 @@ constexpr int kRenderWarps = kRenderThreads / 32;
 static_assert(kStage % kRenderThreads == 0, "whole rounds of staging");
 constexpr int kGroup = 2;                    // list entries blended per step
 constexpr float kInf = __builtin_huge_valf();
-
-__device__ __forceinline__ float4 at_offset(const float4* s, uint32_t bytes) {
-    return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s) + bytes);
-}
 
 // Column tx's run range [start, end) in its pass's column lists (empty after
 // a pair overflow); warp 0 writes it to *out, the caller synchronises.
@@ -146,50 +142,6 @@ __device__ __forceinline__ uint32_t stage_column_batch(uint32_t base, uint32_t e
     return total;
 }
 
-// Which of the tile's 8x8 quadrants a Gaussian can blend in, as bits
-// (quadrant x, y at bit x + 2 y): those with a point where its exponent
-// log2(sigma) - |u|^2 reaches the limit.  |u|^2 is a convex quadratic, so its
-// minimum over a rectangle lies at the centre's nearest x or y edge line, at the
-// other coordinate's minimiser clamped to the rectangle; u is formed from k and
-// w as the pixels form it.  A quadrant is dropped only where the bound holds
-// with every rounding on the wrong side: the errors of k, of u and of the
-// minimiser are a few ulp of `scale` (the largest term that cancels in u), and
-// those of the exponent a few ulp of its own terms.  Comparisons with a NaN keep
-// the quadrant.
-__device__ __forceinline__ uint32_t quadrants_reached(float2 c, float2 k, float4 w, float log2_sigma, float e_lim) {
-    const float thr = log2_sigma - e_lim;
-    if (thr < 0.f) return 0u;   // no pixel reaches the limit: |u|^2 >= 0
-    const float scale = (fabsf(w.x) + fabsf(w.z)) * (fabsf(c.x) + 16.f) + (fabsf(w.y) + fabsf(w.w)) * (fabsf(c.y) + 16.f);
-    const float reach = sqrtf(thr) + fmaf(4e-6f, scale, 1e-5f);
-    const float most = fmaf(reach, reach, fmaf(1e-6f, fabsf(log2_sigma) + fabsf(e_lim), 1e-5f));
-    const float A = fmaf(w.x, w.x, w.z * w.z), B = fmaf(w.x, w.y, w.z * w.w), C = fmaf(w.y, w.y, w.w * w.w);
-    const float slope_y = -B * rcp_approx(C), slope_x = -B * rcp_approx(A);   // the minimiser's drift per pixel off centre
-    float xs[2], ys[2], fy[2], fx[2];
-    float2 ux[2], uy[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float lo = 8.f * (float)h, hi = lo + 7.f;
-        xs[h] = fminf(fmaxf(c.x, lo), hi);
-        ys[h] = fminf(fmaxf(c.y, lo), hi);
-        fy[h] = fmaf(slope_y, xs[h] - c.x, c.y);   // y of the minimum on the line x = xs
-        fx[h] = fmaf(slope_x, ys[h] - c.y, c.x);
-        ux[h] = make_float2(fmaf(-w.x, xs[h], k.x), fmaf(-w.z, xs[h], k.y));
-        uy[h] = make_float2(fmaf(-w.y, ys[h], k.x), fmaf(-w.w, ys[h], k.y));
-    }
-    uint32_t out = 0u;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int hx = q & 1, hy = q >> 1;
-        const float y = fminf(fmaxf(fy[hx], 8.f * (float)hy), 8.f * (float)hy + 7.f);
-        const float x = fminf(fmaxf(fx[hy], 8.f * (float)hx), 8.f * (float)hx + 7.f);
-        const float a1 = fmaf(-w.y, y, ux[hx].x), a2 = fmaf(-w.w, y, ux[hx].y);
-        const float b1 = fmaf(-w.x, x, uy[hy].x), b2 = fmaf(-w.z, x, uy[hy].y);
-        const float least = fminf(fmaf(a1, a1, a2 * a2), fmaf(b1, b1, b2 * b2));
-        if (!(least > most)) out |= 1u << q;
-    }
-    return out;
-}
-
 // The m staged Gaussians' terms, the centre taken relative to the tile origin
 // (ox, oy): (hi - origin) is exact, one rounding for lo.  With kLists the
 // Gaussians each quadrant can blend are marked in s_mask[quadrant][slot / 32].
@@ -213,7 +165,7 @@ __device__ __forceinline__ void stage_records(int m, const uint32_t* s_gid, cons
             s_kl[sl] = make_float4(k.x, k.y, col.w, col.z);   // k1, k2, log2(sigma), blue
             s_nw[sl] = make_float4(-w.x, -w.z, -w.y, -w.w);   // -w1x, -w2x, -w1y, -w2y
             s_rg[sl] = make_float4(col.x, col.x, col.y, col.y);
-            if (kLists) reached = quadrants_reached(c, k, w, col.w, e_lim);
+            if (kLists) reached = rects_reached<8, 8>(c, k, w, col.w, e_lim);
         }
         if (kLists) {
             uint32_t mine = 0u;
@@ -365,12 +317,7 @@ k_render(const RenderBatch batch) {
         if (!__all_sync(0xffffffffu, fminf(elim.x, elim.y) == kInf)) {   // warp-uniform: the loop votes
             // The quadrant's own list, padded to a whole group.
             uint32_t* list = s_list[warp];
-            int n = 0;
-            for (int wd = 0; 32 * wd < m; ++wd) {
-                const uint32_t b = s_mask[warp][wd];
-                if ((b >> lane) & 1u) list[n + __popc(b & ((1u << lane) - 1u))] = (uint32_t)(32 * wd + lane) * 16u;
-                n += __popc(b);
-            }
+            const int n = warp_list(s_mask[warp], m, lane, list);
             if (lane < 2 * kGroup) list[n + lane] = kStage * 16u;
             __syncwarp();
             // A pixel becomes done only where it stops (its exponent limit
