@@ -210,7 +210,7 @@ size_t workspace_bytes(int64_t max_gaussians, int64_t pair_capacity, int32_t max
     const size_t tiles = (size_t)((max_width + kTile - 1) / kTile) * ((max_height + kTile - 1) / kTile);
     const size_t lb = ((N + kSortChunk - 1) / kSortChunk + 2) * kRadix * 8;
     return N * (kRecFloat4 * 16 + kAuxFloat4 * 16 + 4 * 4 + 8 + 8 + 16 + 36 + 12) + P * 14 +
-           2 * (P / kSortChunk + 2) * 4 + tiles * 20 + pixels * 48 + lb +
+           2 * (P / kMarkRuns + 2) * 4 + tiles * 20 + pixels * 48 + lb +
            (size_t)kRadix * kMaxTileGrid * 4 + (kZeroWords + 2 * bin_map(max_gaussians).count) * 4 +
            2 * (N / kWindow + 2) * 4 + 8192;
 }
@@ -262,7 +262,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.pgauss, P * sizeof(uint32_t));
     ALLOC(w.tile_counts, (size_t)w.max_tiles * sizeof(uint32_t));
     ALLOC(w.tcounts, (size_t)kRadix * kMaxTileGrid * sizeof(uint32_t));
-    ALLOC(w.chunk_first, (P / kSortChunk + 2) * sizeof(uint32_t));
+    ALLOC(w.chunk_first, (P / kMarkRuns + 2) * sizeof(uint32_t));
     ALLOC(w.ranges, (size_t)w.max_tiles * sizeof(uint2));
     ALLOC(w.last, pixels * sizeof(int32_t));
     ALLOC(w.trav, pixels * sizeof(int32_t));
@@ -274,7 +274,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
         ALLOC(w.s_order, N * sizeof(uint32_t));
         ALLOC(w.s_box, N * sizeof(uint32_t));
         ALLOC(w.s_offsets, N * sizeof(uint32_t));
-        ALLOC(w.s_chunk_first, (P / kSortChunk + 2) * sizeof(uint32_t));
+        ALLOC(w.s_chunk_first, (P / kMarkRuns + 2) * sizeof(uint32_t));
         ALLOC(w.surv_cnt, 2 * kMaxTileGrid * sizeof(uint32_t));
         ALLOC(w.surv_flag, N);
         ALLOC(w.pst, pixels * sizeof(float4));

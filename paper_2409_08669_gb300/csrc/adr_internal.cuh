@@ -113,6 +113,7 @@ constexpr int kAuxFloat4 = 2;
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortChunk = kSortThreads * kSortItems;   // 4096 keys per chunk
+constexpr int kMarkRuns = 1024;                         // column runs per chunk_first entry
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kMaxPasses = 4;                           // up to 32 key bits
@@ -178,7 +179,7 @@ struct Workspace {
     uint32_t* ttotals = nullptr;           // [kTotalSets * kRadix] per-digit totals of the tile passes
                                            // (in the zeroed block, see kZeroWords)
     uint32_t* tile_counts = nullptr;       // [max_tiles] pairs per tile
-    uint32_t* chunk_first = nullptr;       // [capacity / kSortChunk + 2]
+    uint32_t* chunk_first = nullptr;       // [capacity / kMarkRuns + 2]
     uint2* ranges = nullptr;               // [max_tiles]
     int32_t* last = nullptr;               // [max pixels]
     int32_t* trav = nullptr;               // [max pixels]
@@ -206,7 +207,7 @@ struct Workspace {
     uint32_t* s_order = nullptr;           // [max_n] slice-1 Gaussians in depth order
     uint32_t* s_box = nullptr;             // [max_n] their packed rectangles
     uint32_t* s_offsets = nullptr;         // [max_n] their run offsets
-    uint32_t* s_chunk_first = nullptr;     // [capacity / kSortChunk + 2]
+    uint32_t* s_chunk_first = nullptr;     // [capacity / kMarkRuns + 2]
     uint32_t* s_win_lo = nullptr;          // [max_n / kWindow + 2] windows of slice 1
     uint32_t* surv_cnt = nullptr;          // [2 * kMaxTileGrid] per-CTA kept counts and runs
     uint8_t* surv_flag = nullptr;          // [max_n] kept flag per depth-order position
@@ -459,14 +460,15 @@ void launch_tile_count_columns(const PairSource& src, uint32_t* counts, uint32_t
 void launch_tile_scatter_columns(const PairSource& src, const uint32_t* starts, uint2* runs_out,
                                  uint16_t* rows_out, uint32_t* status, int grid, cudaStream_t stream);
 void launch_tile_count_rows(const uint2* runs, const uint32_t* counters, int64_t capacity,
-                            int tiles_x, int num_tiles, uint32_t* counts, uint32_t* totals,
+                            int tiles_x, int tiles_y, uint32_t* counts, uint32_t* totals,
                             uint32_t* tile_counts, uint32_t* status, int grid, cudaStream_t stream);
 void launch_tile_ranges(const uint32_t* tile_counts, int num_tiles, const uint32_t* counters,
                         int64_t capacity, uint2* ranges, cudaStream_t stream);
 void launch_tile_scatter_rows(const uint2* runs, const uint32_t* counters, int64_t capacity,
                               const uint32_t* starts, uint32_t* gauss_out, uint32_t* status,
                               int grid, int tiles_y, cudaStream_t stream);
-void launch_tile_count_scan(uint32_t* counts, const uint32_t* totals, int grid, cudaStream_t stream);
+void launch_tile_count_scan(uint32_t* counts, const uint32_t* totals, const uint32_t* counters, int64_t capacity,
+                            int digits, int grid, bool columns, cudaStream_t stream);
 
 // Packed tile rectangle: x0 | y0 << 8 | (w-1) << 16 | (h-1) << 24 (tile
 // coordinates and extents fit 8 bits because images are at most 4096 pixels
@@ -475,7 +477,7 @@ void launch_tile_count_scan(uint32_t* counts, const uint32_t* totals, int grid, 
 // rectangles in depth order (sorted_box, all ones = no tiles), with decoupled
 // lookback.  Also writes the run total, visible count and pair total to
 // counters (with the capacity flag), and chunk_first[c] = position of the
-// Gaussian holding run c * kSortChunk.
+// Gaussian holding run c * kMarkRuns.
 // A wait that gives up sets kErrLookback and counters[kCntScanFailed]; the
 // pair total then reads as saturated, so every later stage of the frame
 // skips its work exactly as after a capacity overflow.

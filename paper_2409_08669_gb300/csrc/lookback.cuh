@@ -70,15 +70,15 @@ __device__ __forceinline__ uint32_t warp_lookback(unsigned long long* lookback, 
     return e;
 }
 
-// The run chunks (of kSortChunk runs) that start inside the runs [run, run + t)
+// The run chunks (of kMarkRuns runs) that start inside the runs [run, run + t)
 // of the Gaussian at depth-order position i: each one's holder is i.
 __device__ __forceinline__ void mark_chunks(uint32_t run, uint32_t t, uint32_t i, int64_t capacity,
                                             uint32_t* __restrict__ chunk_first) {
     // run < 2^31 and t <= 256, so run + t does not wrap
-    uint32_t c = (run + (uint32_t)kSortChunk - 1u) / (uint32_t)kSortChunk;
-    if (t == 0u || c * (uint32_t)kSortChunk >= run + t || (int64_t)run >= capacity) return;
-    const uint32_t c_max = (uint32_t)((capacity - 1) / kSortChunk);
-    for (; c * (uint32_t)kSortChunk < run + t && c <= c_max; ++c) chunk_first[c] = i;
+    uint32_t c = (run + (uint32_t)kMarkRuns - 1u) / (uint32_t)kMarkRuns;
+    if (t == 0u || c * (uint32_t)kMarkRuns >= run + t || (int64_t)run >= capacity) return;
+    const uint32_t c_max = (uint32_t)((capacity - 1) / kMarkRuns);
+    for (; c * (uint32_t)kMarkRuns < run + t && c <= c_max; ++c) chunk_first[c] = i;
 }
 
 }  // namespace adr

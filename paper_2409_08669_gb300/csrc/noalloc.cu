@@ -53,7 +53,7 @@ constexpr size_t kOffPRuns = align256(kOffWinLo + (kNaMaxGaussians / kWindow + 2
 constexpr size_t kOffPRows = align256(kOffPRuns + kNaMaxPairs * 8);
 constexpr size_t kOffPGauss = align256(kOffPRows + (kNaMaxPairs + 8) * 2);
 constexpr size_t kOffChunkFirst = align256(kOffPGauss + kNaMaxPairs * 4);
-constexpr size_t kOffRanges = align256(kOffChunkFirst + (kNaMaxPairs / kSortChunk + 2) * 4);
+constexpr size_t kOffRanges = align256(kOffChunkFirst + (kNaMaxPairs / kMarkRuns + 2) * 4);
 constexpr size_t kOffLast = align256(kOffRanges + kNaMaxTiles * 8);
 constexpr size_t kOffTrav = align256(kOffLast + kPixels * 4);
 constexpr size_t kOffTfin = align256(kOffTrav + kPixels * 4);

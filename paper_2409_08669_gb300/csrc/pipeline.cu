@@ -195,11 +195,12 @@ static void enqueue_tile_pass2(const Workspace& ws, FrameState& fs, cudaStream_t
         // (kMaxTileGrid CTAs) that the hardware schedules as CTAs finish.
         const int G2 = kMaxTileGrid;
         TIMED(ws, kKTileCountRows, stream,
-              launch_tile_count_rows(ws.pruns, ws.counters, ws.capacity, fs.cam.tiles_x, fs.num_tiles,
+              launch_tile_count_rows(ws.pruns, ws.counters, ws.capacity, fs.cam.tiles_x, fs.cam.tiles_y,
                                      ws.tcounts, totals, ws.tile_counts, ws.status, G2,
                                      stream));
         TIMED(ws, kKTileCountScan, stream,
-              launch_tile_count_scan(ws.tcounts, totals, G2, stream));
+              launch_tile_count_scan(ws.tcounts, totals, ws.counters, ws.capacity, fs.cam.tiles_y, G2, false,
+                                     stream));
         TIMED(ws, kKTileScatterRows, stream,
               launch_tile_scatter_rows(ws.pruns, ws.counters, ws.capacity, ws.tcounts, ws.pgauss,
                                        ws.status, G2, fs.cam.tiles_y, stream));
@@ -221,7 +222,8 @@ static void enqueue_pass1(const Workspace& ws, FrameState& fs, const PairSource&
     if (fs.n > 0 && fs.order) {
         TIMED(ws, kKTileCountColumns, stream,
               launch_tile_count_columns(src, ws.tcounts, totals, ws.status, G, stream));
-        TIMED(ws, kKTileCountScan, stream, launch_tile_count_scan(ws.tcounts, totals, G, stream));
+        TIMED(ws, kKTileCountScan, stream,
+              launch_tile_count_scan(ws.tcounts, totals, src.counters, src.capacity, src.tiles_x, G, true, stream));
         TIMED(ws, kKTileScatterColumns, stream,
               launch_tile_scatter_columns(src, ws.tcounts, ws.pruns, ws.prows, ws.status, G, stream));
     }
@@ -374,7 +376,7 @@ static void slice1_runs(const Workspace& ws, FrameState& fs, cudaStream_t stream
         const int surv_grid = (int)std::min<int64_t>(kMaxTileGrid, std::max<int64_t>(ws.sort_grid, fs.n / 1024));
         TIMED(ws, kKSlice, stream,
               launch_survivors(fs.cam.tiles_x, ws.sat, ws.sorted_box, fs.order, ws.counters, surv_grid,
-                               ws.surv_cnt, ws.surv_flag, ws.max_n, ws.capacity / kSortChunk + 2, ws.s_order,
+                               ws.surv_cnt, ws.surv_flag, ws.max_n, ws.capacity / kMarkRuns + 2, ws.s_order,
                                ws.s_box, ws.s_offsets, ws.s_chunk_first, c1, ws.status, stream));
     }
     enqueue_pass1(ws, fs, pair_source(ws, fs, 1), kTotalsSlice1, stream);

@@ -297,8 +297,8 @@ k_surv_scatter(const uint32_t* __restrict__ sorted_box, const uint32_t* __restri
                 s_order[j] = order[i];
                 s_box[j] = box;
                 s_offsets[j] = o;
-                for (uint32_t c = (o + (uint32_t)kSortChunk - 1u) / (uint32_t)kSortChunk;
-                     (int64_t)c < chunk_max && c * (uint32_t)kSortChunk < o + w; ++c)
+                for (uint32_t c = (o + (uint32_t)kMarkRuns - 1u) / (uint32_t)kMarkRuns;
+                     (int64_t)c < chunk_max && c * (uint32_t)kMarkRuns < o + w; ++c)
                     s_chunk_first[c] = j;
             } else {
                 atomicOr(status, kErrRange);

@@ -229,7 +229,7 @@ void launch_depth_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
     const uint32_t* n_dev = first ? nullptr : kept;
     launch_pdl(k_digit_counts, grid, kSortThreads, 0, stream, keys_in, n, n_dev, first, shift, grid, counts,
                                                       totals, first ? kept : nullptr);
-    launch_tile_count_scan(counts, totals, grid, stream);
+    launch_tile_count_scan(counts, totals, nullptr, 0, kRadix, grid, false, stream);
     launch_pdl(k_digit_scatter, grid, kSortThreads, kSortSmem, stream, keys_in, vals_in, keys_out, vals_out, n,
                                                               n_dev, first, shift, counts, grid,
                                                               pay_in, pay_out, status);

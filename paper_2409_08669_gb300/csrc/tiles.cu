@@ -17,10 +17,11 @@
 // row ty) by one scan, with no boundary search.
 //
 // Each pass is range-partitioned (count, scan, scatter): CTA b of a grid of G
-// owns a contiguous run of 4096-item chunks,
+// owns a contiguous run of chunks (1024 or 4096 column runs in pass 1, 512 in
+// pass 2),
 //   1. counts its items per digit (pass 1 straight from the Gaussians'
 //      rectangles, pass 2 from the runs' row intervals, as difference arrays),
-//   2. the G x 256 counts become the global start of every (digit, CTA) run
+//   2. the G x digits counts become the global start of every (digit, CTA) run
 //      (per-digit totals are summed with atomics while counting),
 //   3. CTA b walks its chunks in order, ranks each chunk's items stably,
 //      groups them by digit in shared memory and writes every digit's run
@@ -88,19 +89,33 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-// The item count of a pass and the chunks [c0, c1) of CTA blockIdx.x.
+// The item count of a pass, its chunk size, the chunks [c0, c1) of a CTA, and the
+// CTAs that have any (the others leave without a trace: their counts are not read).
 struct Span {
     int64_t n;
-    uint32_t nchunks, c0, c1;
+    uint32_t chunk, nchunks, c0, c1, active;
 };
-__device__ __forceinline__ Span cta_span(int64_t n, int grid) {
+__device__ __forceinline__ Span cta_span(int64_t n, int chunk, int grid, uint32_t cta) {
     Span s;
     s.n = n;
-    s.nchunks = (uint32_t)((n + kSortChunk - 1) / kSortChunk);
+    s.chunk = (uint32_t)chunk;
+    s.nchunks = (uint32_t)((n + chunk - 1) / chunk);
     const uint32_t per = (s.nchunks + (uint32_t)grid - 1u) / (uint32_t)grid;
-    s.c0 = min(s.nchunks, per * blockIdx.x);
+    s.c0 = min(s.nchunks, per * cta);
     s.c1 = min(s.nchunks, s.c0 + per);
+    s.active = per ? (s.nchunks + per - 1u) / per : 0u;
     return s;
+}
+
+// Pass 1's chunks: 1024 runs (4 per thread) while a CTA then gets at most two, else
+// 4096.  A chunk's time is the latency of its chain (staging, one ranking round per
+// item, prefix, write-out), so a frame of few runs is spread over more CTAs with a
+// quarter of the rounds; with many, fewer chunks pay fewer prefixes.  k_scatter_columns
+// at 10k / 1M Gaussians (slices 0 and 1): 13.3 / 11.7 + 13.0 us in chunks of 4096,
+// 7.0 / 7.8 + 8.7 in chunks of 1024; frames of 1M at 1080p 344 -> 331 us, 3M 522 -> 510.
+// With the line at one chunk each 3M takes 516, at four 511.
+__device__ __forceinline__ int column_chunk(int64_t runs, int grid) {
+    return runs <= (int64_t)grid * (2 * kMarkRuns) ? kMarkRuns : kSortChunk;
 }
 
 // Items of the two passes: the column runs C, or none when the pairs
@@ -134,16 +149,27 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
     return base + x - v;
 }
 
-// In-place running maximum over map[0 .. kSortChunk) (u16 entries, 16 per
-// thread), so that every slot names the staged item holding it.
+// In-place running maximum over map[0 .. kItems * kSortThreads) (u16 entries, kItems
+// per thread), so that every slot names the staged item holding it.
+template <int kItems>
 __device__ __forceinline__ void map_running_max(uint16_t* map, uint32_t* wsum) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kWords = kItems / 2;
+    static_assert(kWords == 8 || kWords == 2, "two 16-byte or one 8-byte access");
+    uint32_t w32[kWords];
     uint4* m4 = reinterpret_cast<uint4*>(map) + 2 * tid;
-    const uint4 a = m4[0], b = m4[1];
-    const uint32_t w32[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint2* m2 = reinterpret_cast<uint2*>(map) + tid;
+    if constexpr (kWords == 8) {
+        const uint4 a = m4[0], b = m4[1];
+        w32[0] = a.x; w32[1] = a.y; w32[2] = a.z; w32[3] = a.w;
+        w32[4] = b.x; w32[5] = b.y; w32[6] = b.z; w32[7] = b.w;
+    } else {
+        const uint2 a = *m2;
+        w32[0] = a.x; w32[1] = a.y;
+    }
     uint32_t tmax = 0;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) tmax = max(tmax, max(w32[x] & 0xFFFFu, w32[x] >> 16));
+    for (int x = 0; x < kWords; ++x) tmax = max(tmax, max(w32[x] & 0xFFFFu, w32[x] >> 16));
     uint32_t incl = tmax;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -155,15 +181,19 @@ __device__ __forceinline__ void map_running_max(uint16_t* map, uint32_t* wsum) {
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
     for (int w = 0; w < warp; ++w) excl = max(excl, wsum[w]);
-    uint32_t run = excl, out[8];
+    uint32_t run = excl, out[kWords];
 #pragma unroll
-    for (int x = 0; x < 8; ++x) {
+    for (int x = 0; x < kWords; ++x) {
         const uint32_t lo = run = max(run, w32[x] & 0xFFFFu);
         const uint32_t hi = run = max(run, w32[x] >> 16);
         out[x] = lo | (hi << 16);
     }
-    m4[0] = make_uint4(out[0], out[1], out[2], out[3]);
-    m4[1] = make_uint4(out[4], out[5], out[6], out[7]);
+    if constexpr (kWords == 8) {
+        m4[0] = make_uint4(out[0], out[1], out[2], out[3]);
+        m4[1] = make_uint4(out[4], out[5], out[6], out[7]);
+    } else {
+        *m2 = make_uint2(out[0], out[1]);
+    }
     __syncthreads();
 }
 
@@ -172,12 +202,11 @@ __device__ __forceinline__ void map_running_max(uint16_t* map, uint32_t* wsum) {
 // item's position among the items of its digit in its warp; sm.local,
 // sm.warp_cnt (exclusive prefix over warps) and sm.dst are set and sm.run
 // advanced past the chunk.
-template <class Shared>
-__device__ __forceinline__ void rank_chunk(Shared& sm, const uint32_t (&dig)[kSortItems],
-                                           uint32_t (&rank)[kSortItems]) {
+template <int kItems, class Shared>
+__device__ __forceinline__ void rank_chunk(Shared& sm, const uint32_t (&dig)[kItems], uint32_t (&rank)[kItems]) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-    for (int q = 0; q < kSortItems; ++q) {
+    for (int q = 0; q < kItems; ++q) {
         const uint32_t d = dig[q];
         // The lanes with the same digit (0..kRadix): one ballot per bit of the
         // 9-bit value, every bit agreeing (match_any's result, without its
@@ -223,8 +252,9 @@ __device__ __forceinline__ bool gauss_span(const PairSource& src, const Span& sp
                                            uint32_t c1, uint32_t* status, uint32_t& i0,
                                            uint32_t& i1) {
     const uint32_t visible = src.counters[kCntVisible];
-    i0 = src.chunk_first[c0];
-    i1 = c1 < sp.nchunks ? src.chunk_first[c1] : visible - 1u;
+    const uint32_t marks = sp.chunk / (uint32_t)kMarkRuns;
+    i0 = src.chunk_first[c0 * marks];
+    i1 = c1 < sp.nchunks ? src.chunk_first[c1 * marks] : visible - 1u;
     if (visible == 0 || i0 >= visible || i1 < i0 || i1 >= visible) {
         if (threadIdx.x == 0) atomicOr(status, kErrRange);
         return false;
@@ -242,13 +272,15 @@ k_count_columns(PairSource src, int grid, uint32_t* __restrict__ counts, uint32_
     __shared__ int s_diff[kRadix + 1];
     __shared__ uint32_t s_wsum[kWarps];
     const int tid = threadIdx.x;
+    const int64_t n = run_count(src.counters, src.capacity);
+    const Span sp = cta_span(n, column_chunk(n, grid), grid, blockIdx.x);
+    if (sp.c0 >= sp.c1) return;
     for (int d = tid; d <= kRadix; d += kSortThreads) s_diff[d] = 0;
     __syncthreads();
-    const Span sp = cta_span(run_count(src.counters, src.capacity), grid);
     uint32_t i0, i1;
-    if (sp.c0 < sp.c1 && gauss_span(src, sp, sp.c0, sp.c1, status, i0, i1)) {
-        const int64_t A = (int64_t)sp.c0 * kSortChunk;
-        const int64_t B = min((int64_t)sp.c1 * kSortChunk, sp.n);
+    if (gauss_span(src, sp, sp.c0, sp.c1, status, i0, i1)) {
+        const int64_t A = (int64_t)sp.c0 * sp.chunk;
+        const int64_t B = min((int64_t)sp.c1 * sp.chunk, sp.n);
         for (uint32_t i = i0 + tid; i <= i1; i += kSortThreads) {
             const int64_t off = src.offsets[i];
             const uint32_t box = src.sorted_box[i];
@@ -266,6 +298,7 @@ k_count_columns(PairSource src, int grid, uint32_t* __restrict__ counts, uint32_
     uint32_t total;
     const int v = s_diff[tid];
     const uint32_t c = block_exclusive_scan((uint32_t)v, s_wsum, total) + (uint32_t)v;
+    if (tid >= src.tiles_x) return;   // no runs there
     counts[(size_t)tid * grid + blockIdx.x] = c;
     if (c) atomicAdd(totals + tid, c);
 }
@@ -273,27 +306,31 @@ k_count_columns(PairSource src, int grid, uint32_t* __restrict__ counts, uint32_
 // Generate the column runs of chunk `chunk` (items base .. base+count-1 of
 // the depth-ordered emission) into key (run record y) / val (Gaussian id) in
 // warp-striped order.
+template <int kItems>
 __device__ __forceinline__ void generate_runs(const PairSource& src, const Span& sp,
                                               ColumnShared& sm, uint32_t chunk, int64_t base,
                                               int count, uint32_t* status,
-                                              uint32_t (&key)[kSortItems],
-                                              uint32_t (&val)[kSortItems]) {
+                                              uint32_t (&key)[kItems],
+                                              uint32_t (&val)[kItems]) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kChunk = kItems * kSortThreads;
+    constexpr uint32_t kMost = kChunk + 1;   // every listed Gaussian has >= 1 run
+    constexpr uint32_t kMarks = kChunk / kMarkRuns;
     const uint32_t visible = src.counters[kCntVisible];
-    uint32_t i0 = src.chunk_first[chunk];
+    uint32_t i0 = src.chunk_first[chunk * kMarks];
     // Gaussians [i0, i1] hold this chunk's runs; the one holding the next
-    // chunk's first run closes the range (the last chunk: at most 4097 on).
-    uint32_t i1 = chunk + 1 < sp.nchunks ? src.chunk_first[chunk + 1]
-                                         : min(visible - 1u, i0 + (uint32_t)kMaxChunkGauss - 1u);
+    // chunk's first run closes the range (the last chunk: at most kMost on).
+    uint32_t i1 = chunk + 1 < sp.nchunks ? src.chunk_first[(chunk + 1) * kMarks]
+                                         : min(visible - 1u, i0 + kMost - 1u);
     if (visible == 0 || i0 >= visible || i1 < i0 || i1 >= visible ||
-        i1 - i0 + 1 > (uint32_t)kMaxChunkGauss) {
+        i1 - i0 + 1 > kMost) {
         if (tid == 0) atomicOr(status, kErrRange);   // inconsistent scan output: stay in bounds
         i0 = visible == 0 ? 0u : min(i0, visible - 1u);
-        i1 = visible == 0 ? i0 : min(visible - 1u, i0 + (uint32_t)kMaxChunkGauss - 1u);
+        i1 = visible == 0 ? i0 : min(visible - 1u, i0 + kMost - 1u);
     }
     const int G = (int)(i1 - i0 + 1);
     uint32_t* map32 = reinterpret_cast<uint32_t*>(sm.u.stage.map);
-    for (int x = tid; x < kSortChunk / 2; x += kSortThreads) map32[x] = 0u;
+    for (int x = tid; x < kChunk / 2; x += kSortThreads) map32[x] = 0u;
     for (int j = tid; j < G; j += kSortThreads) {   // coalesced staging
         const uint32_t i = i0 + j;
         sm.u.stage.off[j] = src.offsets[i];
@@ -308,10 +345,10 @@ __device__ __forceinline__ void generate_runs(const PairSource& src, const Span&
         if (slot > 0 && slot < count) sm.u.stage.map[slot] = (uint16_t)j;
     }
     __syncthreads();
-    map_running_max(sm.u.stage.map, sm.wsum);
-    const int wfirst = warp * (kSortItems * 32);
+    map_running_max<kItems>(sm.u.stage.map, sm.wsum);
+    const int wfirst = warp * (kItems * 32);
 #pragma unroll
-    for (int q = 0; q < kSortItems; ++q) {
+    for (int q = 0; q < kItems; ++q) {
         const int s = wfirst + q * 32 + lane;
         if (s < count) {
             const int jj = sm.u.stage.map[s];
@@ -327,33 +364,29 @@ __device__ __forceinline__ void generate_runs(const PairSource& src, const Span&
     }
 }
 
-__global__ void __launch_bounds__(kSortThreads, 3)
-k_scatter_columns(PairSource src, const uint32_t* __restrict__ starts, uint2* __restrict__ runs_out,
-                  uint16_t* __restrict__ rows_out,
-                  int grid, uint32_t* __restrict__ status) {
-    pdl_prologue();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    ColumnShared& sm = *reinterpret_cast<ColumnShared*>(smem_raw);
+// The CTA's chunks of kItems runs per thread.
+template <int kItems>
+__device__ __forceinline__ void scatter_chunks(const PairSource& src, const Span& sp, ColumnShared& sm,
+                                               uint2* __restrict__ runs_out, uint16_t* __restrict__ rows_out,
+                                               uint32_t* __restrict__ status) {
+    constexpr int kChunk = kItems * kSortThreads;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const Span sp = cta_span(run_count(src.counters, src.capacity), grid);
-    if (sp.c0 >= sp.c1) return;
     const int64_t n = sp.n;
-    sm.run[tid] = starts[(size_t)tid * grid + blockIdx.x];
     for (uint32_t chunk = sp.c0; chunk < sp.c1; ++chunk) {
         for (int d = lane; d <= kRadix; d += 32) sm.warp_cnt[warp][d] = 0;
-        const int64_t base = (int64_t)chunk * kSortChunk;
-        const int count = (int)min((int64_t)kSortChunk, n - base);
-        uint32_t key[kSortItems], val[kSortItems], dig[kSortItems], rank[kSortItems];
-        generate_runs(src, sp, sm, chunk, base, count, status, key, val);
+        const int64_t base = (int64_t)chunk * kChunk;
+        const int count = (int)min((int64_t)kChunk, n - base);
+        uint32_t key[kItems], val[kItems], dig[kItems], rank[kItems];
+        generate_runs<kItems>(src, sp, sm, chunk, base, count, status, key, val);
 #pragma unroll
-        for (int q = 0; q < kSortItems; ++q) {
-            const int s = warp * (kSortItems * 32) + q * 32 + lane;
+        for (int q = 0; q < kItems; ++q) {
+            const int s = warp * (kItems * 32) + q * 32 + lane;
             dig[q] = s < count ? min(run_tx(key[q]), (uint32_t)kRadix - 1u) : (uint32_t)kRadix;
         }
         __syncthreads();   // staging no longer read
-        rank_chunk(sm, dig, rank);
+        rank_chunk<kItems>(sm, dig, rank);
 #pragma unroll
-        for (int q = 0; q < kSortItems; ++q) {
+        for (int q = 0; q < kItems; ++q) {
             if (dig[q] < (uint32_t)kRadix) {
                 const uint32_t d = dig[q];
                 const uint32_t pos = sm.local[d] + sm.warp_cnt[warp][d] + rank[q];
@@ -376,6 +409,22 @@ k_scatter_columns(PairSource src, const uint32_t* __restrict__ starts, uint2* __
     }
 }
 
+__global__ void __launch_bounds__(kSortThreads, 3)
+k_scatter_columns(PairSource src, const uint32_t* __restrict__ starts, uint2* __restrict__ runs_out,
+                  uint16_t* __restrict__ rows_out,
+                  int grid, uint32_t* __restrict__ status) {
+    pdl_prologue();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ColumnShared& sm = *reinterpret_cast<ColumnShared*>(smem_raw);
+    const int tid = threadIdx.x;
+    const int64_t n = run_count(src.counters, src.capacity);
+    const Span sp = cta_span(n, column_chunk(n, grid), grid, blockIdx.x);
+    if (sp.c0 >= sp.c1) return;
+    sm.run[tid] = tid < src.tiles_x ? starts[(size_t)tid * grid + blockIdx.x] : 0u;
+    if (sp.chunk == (uint32_t)kMarkRuns) scatter_chunks<kMarkRuns / kSortThreads>(src, sp, sm, runs_out, rows_out, status);
+    else scatter_chunks<kSortItems>(src, sp, sm, runs_out, rows_out, status);
+}
+
 // ---------------------------------------------------------------------------
 // Pass 2: pairs grouped by ty.
 // ---------------------------------------------------------------------------
@@ -387,7 +436,7 @@ k_scatter_columns(PairSource src, const uint32_t* __restrict__ starts, uint2* __
 // with few runs) add to tile_counts directly.
 __global__ void __launch_bounds__(kSortThreads)
 k_count_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ counters, int64_t capacity,
-             int grid, int tiles_x, int num_tiles, uint32_t* __restrict__ counts,
+             int grid, int tiles_x, int tiles_y, uint32_t* __restrict__ counts,
              uint32_t* __restrict__ totals, uint32_t* __restrict__ tile_counts,
              uint32_t* __restrict__ status) {
     pdl_prologue();
@@ -395,14 +444,16 @@ k_count_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ counte
     __shared__ int s_col[kColSlots][kRadix + 1];
     __shared__ uint32_t s_wsum[kWarps];
     const int tid = threadIdx.x;
+    const int num_tiles = tiles_x * tiles_y;
+    const Span sp = cta_span(run_count(counters, capacity), kRunStage, grid, blockIdx.x);
+    if (sp.c0 >= sp.c1) return;
     for (int d = tid; d <= kRadix; d += kSortThreads) s_diff[d] = 0;
     for (int d = tid; d < kColSlots * (kRadix + 1); d += kSortThreads) (&s_col[0][0])[d] = 0;
     __syncthreads();
-    const Span sp = cta_span(run_count(counters, capacity), grid);
     uint32_t tx0 = 0;
-    if (sp.c0 < sp.c1) {
-        const int64_t A = (int64_t)sp.c0 * kSortChunk;
-        const int64_t B = min((int64_t)sp.c1 * kSortChunk, sp.n);
+    {
+        const int64_t A = (int64_t)sp.c0 * sp.chunk;
+        const int64_t B = min((int64_t)sp.c1 * sp.chunk, sp.n);
         tx0 = run_tx(runs[A].y);
         for (int64_t i = A + tid; i < B; i += kSortThreads) {
             const uint32_t y = runs[i].y;
@@ -430,10 +481,12 @@ k_count_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ counte
     uint32_t total;
     const int v = s_diff[tid];
     const uint32_t c = block_exclusive_scan((uint32_t)v, s_wsum, total) + (uint32_t)v;
-    counts[(size_t)tid * grid + blockIdx.x] = c;
-    if (c) atomicAdd(totals + tid, c);
+    if (tid < tiles_y) {
+        counts[(size_t)tid * grid + blockIdx.x] = c;
+        if (c) atomicAdd(totals + tid, c);
+    }
     // Tile counts of the on-chip columns: prefix over rows, one warp per column.
-    if (sp.c0 < sp.c1) {
+    {
         const int lane = tid & 31, warp = tid >> 5;
         const uint32_t tx = tx0 + (uint32_t)warp;
         if (warp < kColSlots && tx < (uint32_t)tiles_x) {
@@ -491,7 +544,9 @@ k_tile_ranges(const uint32_t* __restrict__ tile_counts, int num_tiles,
 // one and sweep each band's list 32 runs at a time: for every row ty of the band,
 // the lanes whose run covers ty (ballot) write their Gaussians to consecutive
 // positions of the row, in run order.  Each row's output is thus written front
-// to back with coalesced stores, and no pair is staged on chip.
+// to back with coalesced stores, and no pair is staged on chip. A CTA's
+// share is whole stagings of 512 runs: with shares of 4096 a frame of few runs kept
+// tens of CTAs busy (40k runs: 35 us, 7.3 now; 2.5M runs: 58 us, 25 now).
 __global__ void __launch_bounds__(kSortThreads, 8)   // 8 CTAs per SM: 32 registers, 22 KB shared
 k_scatter_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ counters,
                int64_t capacity, const uint32_t* __restrict__ starts, uint32_t* __restrict__ gauss_out,
@@ -499,14 +554,14 @@ k_scatter_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ coun
     pdl_prologue();
     __shared__ RowShared sm;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const Span sp = cta_span(run_count(counters, capacity), grid);
+    const Span sp = cta_span(run_count(counters, capacity), kRunStage, grid, blockIdx.x);
     if (sp.c0 >= sp.c1) return;
     const int64_t n_pairs = min((int64_t)counters[kCntPairs], capacity);
-    sm.pos[tid] = starts[(size_t)tid * grid + blockIdx.x];
-    const int64_t B = min((int64_t)sp.c1 * kSortChunk, sp.n);
+    sm.pos[tid] = tid < tiles_y ? starts[(size_t)tid * grid + blockIdx.x] : 0u;
+    const int64_t B = min((int64_t)sp.c1 * sp.chunk, sp.n);
     const uint32_t lt = lanemask_lt();
     const int band_h = (tiles_y + kBands - 1) / kBands;   // rows per band
-    for (int64_t r = (int64_t)sp.c0 * kSortChunk; r < B; r += kRunStage) {
+    for (int64_t r = (int64_t)sp.c0 * sp.chunk; r < B; r += kRunStage) {
         const int avail = (int)min((int64_t)kRunStage, B - r);
         __syncthreads();   // the previous staging is no longer read
         for (int j = tid; j < kRunStage; j += kSortThreads) {
@@ -579,7 +634,8 @@ k_scatter_rows(const uint2* __restrict__ runs, const uint32_t* __restrict__ coun
 }
 
 // ---------------------------------------------------------------------------
-// Global start of every (digit, CTA) run: counts [256][grid] in place.
+// Global start of every (digit, CTA) run: counts [digits][grid] in place, the CTAs
+// that had items.
 // CTA d: start of digit d = sum of the totals of the digits below it, then an
 // exclusive scan of its grid counts.
 // ---------------------------------------------------------------------------
@@ -588,8 +644,14 @@ constexpr int kScanPerThread = kMaxTileGrid / kScanCtaThreads;
 static_assert(kScanPerThread * kScanCtaThreads == kMaxTileGrid, "scan covers the largest grid");
 
 __global__ void __launch_bounds__(kScanCtaThreads)
-k_count_scan(uint32_t* __restrict__ counts, const uint32_t* __restrict__ totals, int grid) {
+k_count_scan(uint32_t* __restrict__ counts, const uint32_t* __restrict__ totals,
+             const uint32_t* __restrict__ counters, int64_t capacity, int grid, bool columns) {
     pdl_prologue();
+    int active = grid;   // depth passes: every CTA has counts
+    if (counters) {
+        const int64_t n = run_count(counters, capacity);
+        active = (int)cta_span(n, columns ? column_chunk(n, grid) : kRunStage, grid, 0u).active;
+    }
     __shared__ uint32_t s_w[kScanCtaThreads / 32];
     __shared__ uint32_t s_base;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -605,7 +667,7 @@ k_count_scan(uint32_t* __restrict__ counts, const uint32_t* __restrict__ totals,
 #pragma unroll
     for (int u = 0; u < kScanPerThread; ++u) {
         const int b = tid * kScanPerThread + u;
-        v[u] = b < grid ? row[b] : 0u;
+        v[u] = b < active ? row[b] : 0u;
         t += v[u];
     }
     uint32_t x = t;
@@ -621,7 +683,7 @@ k_count_scan(uint32_t* __restrict__ counts, const uint32_t* __restrict__ totals,
 #pragma unroll
     for (int u = 0; u < kScanPerThread; ++u) {
         const int b = tid * kScanPerThread + u;
-        if (b < grid) row[b] = run;
+        if (b < active) row[b] = run;
         run += v[u];
     }
 }
@@ -649,9 +711,9 @@ void launch_tile_scatter_columns(const PairSource& src, const uint32_t* starts, 
 }
 
 void launch_tile_count_rows(const uint2* runs, const uint32_t* counters, int64_t capacity,
-                            int tiles_x, int num_tiles, uint32_t* counts, uint32_t* totals,
+                            int tiles_x, int tiles_y, uint32_t* counts, uint32_t* totals,
                             uint32_t* tile_counts, uint32_t* status, int grid, cudaStream_t stream) {
-    launch_pdl(k_count_rows, grid, kSortThreads, 0, stream, runs, counters, capacity, grid, tiles_x, num_tiles,
+    launch_pdl(k_count_rows, grid, kSortThreads, 0, stream, runs, counters, capacity, grid, tiles_x, tiles_y,
                                                     counts, totals, tile_counts, status);
 }
 
@@ -668,8 +730,10 @@ void launch_tile_scatter_rows(const uint2* runs, const uint32_t* counters, int64
                                                       grid, tiles_y, status);
 }
 
-void launch_tile_count_scan(uint32_t* counts, const uint32_t* totals, int grid, cudaStream_t stream) {
-    launch_pdl(k_count_scan, kRadix, kScanCtaThreads, 0, stream, counts, totals, grid);
+void launch_tile_count_scan(uint32_t* counts, const uint32_t* totals, const uint32_t* counters, int64_t capacity,
+                            int digits, int grid, bool columns, cudaStream_t stream) {
+    if (digits <= 0) return;
+    launch_pdl(k_count_scan, digits, kScanCtaThreads, 0, stream, counts, totals, counters, capacity, grid, columns);
 }
 
 }  // namespace adr
