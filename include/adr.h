@@ -200,6 +200,10 @@ adr_status adr_sort(adr_ctx *ctx, void *stream);
  *   load [H,W] int32 Gaussians blended per pixel, l_i of Eq. 12 (may be NULL). */
 adr_status adr_render(adr_ctx *ctx, float *img, float *t_final, int32_t *load, void *stream);
 
+/* adr_render with the loads as floats (a differentiable consumer's type),
+ * load [H,W] = (float) l_i, instead of a conversion pass over them. */
+adr_status adr_render_float_load(adr_ctx *ctx, float *img, float *t_final, float *load, void *stream);
+
 /* Backward of the last adr_render (the differentiable path the paper trains
  * through, Sec. 4.4 total loss): given dL/dimg [3,H,W] and optionally
  * dL/dload [H,W] (may be NULL; it reaches the opacities through the reading
@@ -225,6 +229,11 @@ adr_status adr_render_backward(adr_ctx *ctx, const float *means, const float *sc
 adr_status adr_load_loss(adr_ctx *ctx, const int32_t *load, int64_t hw, float weight,
                          double *stats, float *dl_dload, void *stream);
 
+/* adr_load_loss of loads given as floats (adr_render_float_load), each rounded
+ * to the nearest integer; writes std (one device float) in place of stats. */
+adr_status adr_load_loss_float(adr_ctx *ctx, const float *load, int64_t hw, float weight,
+                               float *std_out, float *dl_dload, void *stream);
+
 /* Image loss of the training objective (Sec. 4.4 total loss: the L1 and SSIM
  * terms beside L_load).  img and ref: [channels, height, width] device fp32
  * (the render and its target).  SSIM follows Wang et al. 2004: per channel,
@@ -242,6 +251,13 @@ adr_status adr_load_loss(adr_ctx *ctx, const int32_t *load, int64_t hw, float we
 adr_status adr_image_loss(const float *img, const float *ref, int32_t channels, int32_t height,
                           int32_t width, float w_l1, float w_ssim, double *stats, float *dl_dimg,
                           float *scratch, void *stream);
+
+/* adr_image_loss that also writes the loss itself, (float) (w_l1 * stats[0] +
+ * w_ssim * (1 - stats[1])) formed in double, to the device float *loss. */
+adr_status adr_image_loss_value(const float *img, const float *ref, int32_t channels,
+                                int32_t height, int32_t width, double w_l1, double w_ssim,
+                                double *stats, float *loss, float *dl_dimg, float *scratch,
+                                void *stream);
 
 /* Waits for the context's last stream and returns the pair count P (the sum
  * of tiles over Gaussians, which may exceed pair_capacity).  Returns

@@ -69,6 +69,7 @@ _SIGNATURES = {
                               ctypes.POINTER(adr_settings), _P]),
     "adr_sort": (_I32, [_P, _P]),
     "adr_render": (_I32, [_P, _P, _P, _P, _P]),
+    "adr_render_float_load": (_I32, [_P, _P, _P, _P, _P]),
     "adr_num_pairs": (_I32, [_P, ctypes.POINTER(_I64)]),
     "adr_frame_counts": (_I32, [_P, _P, _I32]),
     "adr_read_pairs": (_I32, [_P, _P, _P, _I64, _P]),
@@ -85,6 +86,9 @@ _SIGNATURES = {
     "adr_load_loss": (_I32, [_P, _P, _I64, ctypes.c_float, _P, _P, _P]),
     "adr_image_loss": (_I32, [_P, _P, _I32, _I32, _I32, ctypes.c_float, ctypes.c_float, _P, _P,
                               _P, _P]),
+    "adr_load_loss_float": (_I32, [_P, _P, _I64, ctypes.c_float, _P, _P, _P]),
+    "adr_image_loss_value": (_I32, [_P, _P, _I32, _I32, _I32, ctypes.c_double, ctypes.c_double, _P,
+                                    _P, _P, _P, _P]),
     "adr_profile_enable": (_I32, [_P, _I32]),
     "adr_set_depth_slices": (_I32, [_P, _I32]),
     "adr_set_host_reads": (_I32, [_P, _I32]),
@@ -194,6 +198,10 @@ def adr_render(ctx, img, t_final, load_, stream):
     return check(load().adr_render(ctx, img, t_final, load_, stream), "adr_render")
 
 
+def adr_render_float_load(ctx, img, t_final, load_, stream):
+    return check(load().adr_render_float_load(ctx, img, t_final, load_, stream), "adr_render_float_load")
+
+
 def adr_num_pairs(ctx, raise_on_error=True):
     p = _I64(0)
     st = load().adr_num_pairs(ctx, ctypes.byref(p))
@@ -250,6 +258,17 @@ def adr_image_loss(img, ref, channels, height, width, w_l1, w_ssim, stats, dl_di
                    stream):
     return check(load().adr_image_loss(img, ref, channels, height, width, w_l1, w_ssim, stats,
                                        dl_dimg, scratch, stream), "adr_image_loss")
+
+
+def adr_load_loss_float(ctx, load_, hw, weight, std_out, dl_dload, stream):
+    return check(load().adr_load_loss_float(ctx, load_, hw, weight, std_out, dl_dload, stream),
+                 "adr_load_loss_float")
+
+
+def adr_image_loss_value(img, ref, channels, height, width, w_l1, w_ssim, stats, loss, dl_dimg, scratch,
+                         stream):
+    return check(load().adr_image_loss_value(img, ref, channels, height, width, w_l1, w_ssim, stats, loss,
+                                             dl_dimg, scratch, stream), "adr_image_loss_value")
 
 
 def adr_set_depth_slices(ctx, mode):

@@ -21,13 +21,13 @@ class AdrRasterize(torch.autograd.Function):
     @staticmethod
     def forward(ctx, means, scales, rots, opac, sh, rast: Rasterizer, camera, settings):
         params = tuple(t.contiguous() for t in (means, scales, rots, opac, sh))
-        img, t_final, load = rast.forward(params, camera, settings)
+        img, t_final, load = rast.forward(params, camera, settings, load_dtype=torch.float32)
         ctx.rast = rast
         ctx.frame = rast.frame
         ctx.save_for_backward(*params)
-        ctx.load_int = load
+        ctx.size = load.shape
         ctx.mark_non_differentiable(t_final)
-        return img, load.to(torch.float32), t_final
+        return img, load, t_final
 
     @staticmethod
     def backward(ctx, g_img, g_load, g_t):
@@ -36,7 +36,7 @@ class AdrRasterize(torch.autograd.Function):
             raise RuntimeError("the Rasterizer rendered another frame before this backward; "
                                "use one Rasterizer per frame in flight")
         if g_img is None:
-            g_img = torch.zeros((3,) + ctx.load_int.shape, device=params[0].device)
+            g_img = torch.zeros((3,) + ctx.size, device=params[0].device)
         grads = ctx.rast.backward(params, g_img, g_load)
         return (*grads, None, None, None)
 
@@ -46,10 +46,13 @@ class LoadBalanceLoss(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, load_f, rast: Rasterizer):
-        load_i = load_f.detach().round().to(torch.int32)
-        stats, grad = rast.load_loss(load_i, 1.0, want_grad=True)
+        if load_f.dtype == torch.float32 and load_f.is_contiguous():
+            std, grad = rast.load_loss_float(load_f.detach())
+        else:
+            stats, grad = rast.load_loss(load_f.detach().round().to(torch.int32), 1.0, want_grad=True)
+            std = stats[1].to(torch.float32)
         ctx.save_for_backward(grad)
-        return stats[1].to(torch.float32)
+        return std
 
     @staticmethod
     def backward(ctx, g):
@@ -60,10 +63,10 @@ class LoadBalanceLoss(torch.autograd.Function):
 class ImageLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, img, ref, w_l1, w_ssim):
-        stats, grad = image_loss(img.detach(), ref.detach(), w_l1, w_ssim, want_grad=True)
+        loss = torch.empty((), dtype=torch.float32, device=img.device)
+        ctx.stats, grad = image_loss(img.detach(), ref.detach(), w_l1, w_ssim, want_grad=True, value=loss)
         ctx.save_for_backward(grad)
-        ctx.stats = stats
-        return (w_l1 * stats[0] + w_ssim * (1.0 - stats[1])).to(torch.float32)
+        return loss
 
     @staticmethod
     def backward(ctx, g):

@@ -452,7 +452,8 @@ adr_status adr_sort(adr_ctx* c, void* stream) {
     return ok();
 }
 
-adr_status adr_render(adr_ctx* c, float* img, float* t_final, int32_t* load, void* stream) {
+static adr_status render_frame(adr_ctx* c, float* img, float* t_final, int32_t* load, bool load_float,
+                               void* stream) {
     NvtxRange range_("adr_render");
     if (!c) return fail(ADR_ERR_INVALID, "ctx is NULL");
     if (!c->have_sort) return fail(ADR_ERR_INVALID, "adr_render before adr_sort");
@@ -461,6 +462,7 @@ adr_status adr_render(adr_ctx* c, float* img, float* t_final, int32_t* load, voi
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     c->fs.split_last_slice = c->tile_split == ADR_TILE_SPLIT_LAST_SLICE;
+    c->fs.load_float = load_float;
     enqueue_render(c->ws, c->fs, img, t_final, load, strm);
     if (c->fs.sliced && !c->slice_probe) {
         // Runs of every Gaussian, of slice 0 and of slice 1, back to the host.
@@ -476,6 +478,14 @@ adr_status adr_render(adr_ctx* c, float* img, float* t_final, int32_t* load, voi
     if ((s = check_launch("adr_render")) != ADR_OK) return s;
     c->have_render = true;
     return ok();
+}
+
+adr_status adr_render(adr_ctx* c, float* img, float* t_final, int32_t* load, void* stream) {
+    return render_frame(c, img, t_final, load, false, stream);
+}
+
+adr_status adr_render_float_load(adr_ctx* c, float* img, float* t_final, float* load, void* stream) {
+    return render_frame(c, img, t_final, reinterpret_cast<int32_t*>(load), true, stream);
 }
 
 adr_status adr_sync_status(adr_ctx* c) {
@@ -611,21 +621,33 @@ adr_status adr_load_loss(adr_ctx* c, const int32_t* load, int64_t hw, float weig
     DeviceGuard guard(c->device);
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
-    launch_load_loss(load, hw, c->ws.load_sums, weight, dl_dload, c->ws.sm_count, strm);
+    launch_load_loss(load, hw, c->ws.load_sums, weight, nullptr, dl_dload, c->ws.sm_count, strm);
     ADR_CUDA(cudaMemcpyAsync(stats, c->ws.load_sums + 2, 2 * sizeof(double),
                              cudaMemcpyDeviceToDevice, strm));
     return check_launch("adr_load_loss") == ADR_OK ? ok() : ADR_ERR_CUDA;
 }
 
-adr_status adr_image_loss(const float* img, const float* ref, int32_t channels, int32_t height,
-                          int32_t width, float w_l1, float w_ssim, double* stats, float* dl_dimg,
-                          float* scratch, void* stream) {
+adr_status adr_load_loss_float(adr_ctx* c, const float* load, int64_t hw, float weight, float* std_out,
+                               float* dl_dload, void* stream) {
+    NvtxRange range_("adr_load_loss");
+    if (!c || !load || !std_out) return fail(ADR_ERR_INVALID, "NULL argument");
+    if (hw <= 0) return fail(ADR_ERR_INVALID, "hw must be positive");
+    DeviceGuard guard(c->device);
+    cudaStream_t strm = (cudaStream_t)stream;
+    c->last_stream = strm;
+    launch_load_loss(load, hw, c->ws.load_sums, weight, std_out, dl_dload, c->ws.sm_count, strm);
+    return check_launch("adr_load_loss_float") == ADR_OK ? ok() : ADR_ERR_CUDA;
+}
+
+static adr_status image_loss(const float* img, const float* ref, int32_t channels, int32_t height, int32_t width,
+                             double w_l1, double w_ssim, double* stats, float* loss, float* dl_dimg, float* scratch,
+                             void* stream) {
     NvtxRange range_("adr_image_loss");
     if (!img || !ref || !stats) return fail(ADR_ERR_INVALID, "NULL argument");
     if (channels <= 0 || height <= 0 || width <= 0 || (int64_t)channels * height * width > (1ll << 31))
         return fail(ADR_ERR_INVALID, "image size %d x %d x %d out of range", channels, height, width);
     if (dl_dimg && !scratch) return fail(ADR_ERR_INVALID, "scratch is required with dl_dimg");
-    if (!std::isfinite(w_l1) || !std::isfinite(w_ssim)) return fail(ADR_ERR_INVALID, "bad weight");
+    if (!std::isfinite((float)w_l1) || !std::isfinite((float)w_ssim)) return fail(ADR_ERR_INVALID, "bad weight");
     // Gaussian window of standard deviation 1.5 over 11 taps, normalised to sum 1.
     LossWindow win;
     double w[11], sum = 0.0;
@@ -635,9 +657,22 @@ adr_status adr_image_loss(const float* img, const float* ref, int32_t channels, 
         sum += w[k];
     }
     for (int k = 0; k < 11; ++k) win.w[k] = (float)(w[k] / sum);
-    launch_image_loss(img, ref, channels, height, width, win, w_l1, w_ssim, stats, dl_dimg,
-                      scratch, (cudaStream_t)stream);
+    launch_image_loss(img, ref, channels, height, width, win, w_l1, w_ssim, stats, loss,
+                      dl_dimg, scratch, (cudaStream_t)stream);
     return check_launch("adr_image_loss") == ADR_OK ? ok() : ADR_ERR_CUDA;
+}
+
+adr_status adr_image_loss(const float* img, const float* ref, int32_t channels, int32_t height,
+                          int32_t width, float w_l1, float w_ssim, double* stats, float* dl_dimg,
+                          float* scratch, void* stream) {
+    return image_loss(img, ref, channels, height, width, w_l1, w_ssim, stats, nullptr, dl_dimg, scratch, stream);
+}
+
+adr_status adr_image_loss_value(const float* img, const float* ref, int32_t channels, int32_t height, int32_t width,
+                                double w_l1, double w_ssim, double* stats, float* loss, float* dl_dimg,
+                                float* scratch, void* stream) {
+    if (!loss) return fail(ADR_ERR_INVALID, "NULL argument");
+    return image_loss(img, ref, channels, height, width, w_l1, w_ssim, stats, loss, dl_dimg, scratch, stream);
 }
 
 adr_status adr_set_tile_split(adr_ctx* c, int32_t mode) {

@@ -300,6 +300,7 @@ struct FrameState {
     int order_held = 0;                      // which of OrderHeld `order` and its boxes and offsets hold
     bool totals_used[kTotalSets] = {false, false, false};   // written since the frame's head zeroed them
     bool sliced = false;                     // the frame renders in two depth slices
+    bool load_float = false;      // Render writes the loads as floats
     bool split_last_slice = false;           // slice 1 renders tiles by pixel halves (f2)
     int runs_held = 0;                       // which Gaussians' column runs ws.pruns holds
     int lists = -1;                          // a ListKind; -1 before the first sort
@@ -524,6 +525,7 @@ struct RenderCam {
     float* img = nullptr;
     float* t_final = nullptr;
     int32_t* load = nullptr;
+    bool load_float = false;              // load holds floats
     int32_t* last = nullptr;
     int32_t* trav = nullptr;
     float* tfin = nullptr;
@@ -713,9 +715,12 @@ struct LossWindow {
     float w[11];
 };
 void launch_image_loss(const float* img, const float* ref, int channels, int H, int W,
-                       const LossWindow& win, float w_l1, float w_ssim, double* stats,
+                       const LossWindow& win, double w_l1, double w_ssim, double* stats, float* loss,
                        float* dl_dimg, float* scratch, cudaStream_t stream);
-void launch_load_loss(const int32_t* load, int64_t hw, double* sums, float weight, float* dl_dload,
+// The loads as int32 (std_out null: sums[2], sums[3] hold mean and std) or as
+// floats (std_out gets the std).
+template <typename T>
+void launch_load_loss(const T* load, int64_t hw, double* sums, float weight, float* std_out, float* dl_dload,
                       int sm_count, cudaStream_t stream);
 void enqueue_backward(const Workspace& ws, const FrameState& fs, const float* means,
                       const float* scales, const float* rots, const float* opac, const float* sh,

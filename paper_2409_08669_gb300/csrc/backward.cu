@@ -473,13 +473,25 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
 
 constexpr int kLoadSumWords = 4;   // the integer sums follow the four FP64 words
 
+// Loads as whole numbers, from int32 or from floats (rounded to the nearest).
+__device__ __forceinline__ int4 whole_loads(int4 v) { return v; }
+__device__ __forceinline__ int4 whole_loads(float4 v) {
+    return make_int4(__float2int_rn(v.x), __float2int_rn(v.y), __float2int_rn(v.z), __float2int_rn(v.w));
+}
+__device__ __forceinline__ int32_t whole_load(int32_t v) { return v; }
+__device__ __forceinline__ int32_t whole_load(float v) { return __float2int_rn(v); }
+template <typename T> struct Quad;
+template <> struct Quad<int32_t> { using type = int4; };
+template <> struct Quad<float> { using type = float4; };
+
 // The loads are whole numbers: their sums and the sums of their squares are
 // exact in 64-bit integers (the squares' low and high halves apart, so that no
 // sum overflows), where this chip does FP64 arithmetic at 1/64 of the FP32 rate.
 // Three atomics per CTA.  1280x720: 23 us with FP64 sums and an atomic pair per
 // warp, 5.4 us now (k_load_grad 23 us -> 7.1 us).
+template <typename T>
 __global__ void __launch_bounds__(256)
-k_load_moments(const int32_t* __restrict__ load, int64_t hw, unsigned long long* __restrict__ sums) {
+k_load_moments(const T* __restrict__ load, int64_t hw, unsigned long long* __restrict__ sums) {
     __shared__ unsigned long long s_w[3][8];
     unsigned long long s = 0, sq_lo = 0, sq_hi = 0;   // the sum in two's complement; squares in two halves
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -491,13 +503,13 @@ k_load_moments(const int32_t* __restrict__ load, int64_t hw, unsigned long long*
     };
     const int64_t quads = (reinterpret_cast<uintptr_t>(load) & 15) == 0 ? hw / 4 : 0;
     for (int64_t i = t; i < quads; i += stride) {
-        const int4 q = reinterpret_cast<const int4*>(load)[i];
+        const int4 q = whole_loads(reinterpret_cast<const typename Quad<T>::type*>(load)[i]);
         add(q.x);
         add(q.y);
         add(q.z);
         add(q.w);
     }
-    for (int64_t i = 4 * quads + t; i < hw; i += stride) add(load[i]);
+    for (int64_t i = 4 * quads + t; i < hw; i += stride) add(whole_load(load[i]));
     for (int o = 16; o > 0; o >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, o);
         sq_lo += __shfl_xor_sync(0xffffffffu, sq_lo, o);
@@ -518,9 +530,10 @@ k_load_moments(const int32_t* __restrict__ load, int64_t hw, unsigned long long*
 
 // The gradient weight * (l - mean) / (HW std): l - mean and the scale as float
 // pairs, so that their product is rounded once to FP32, as from FP64.
+template <typename T>
 __global__ void __launch_bounds__(256)
-k_load_grad(const int32_t* __restrict__ load, int64_t hw, double* __restrict__ sums,
-            float weight, float* __restrict__ dl_dload, int write_stats) {
+k_load_grad(const T* __restrict__ load, int64_t hw, double* __restrict__ sums,
+            float weight, float* __restrict__ std_out, float* __restrict__ dl_dload) {
     __shared__ float s_c[4];
     if (threadIdx.x == 0) {
         const unsigned long long* whole = reinterpret_cast<const unsigned long long*>(sums + kLoadSumWords);
@@ -533,9 +546,10 @@ k_load_grad(const int32_t* __restrict__ load, int64_t hw, double* __restrict__ s
         s_c[1] = (float)(mean - (double)s_c[0]);
         s_c[2] = (float)scale;
         s_c[3] = (float)(scale - (double)s_c[2]);
-        if (write_stats && blockIdx.x == 0) {
+        if (blockIdx.x == 0) {
             sums[2] = mean;
             sums[3] = sd;
+            if (std_out) *std_out = (float)sd;
         }
     }
     if (!dl_dload) return;
@@ -555,10 +569,10 @@ k_load_grad(const int32_t* __restrict__ load, int64_t hw, double* __restrict__ s
     const bool vec = ((reinterpret_cast<uintptr_t>(load) | reinterpret_cast<uintptr_t>(dl_dload)) & 15) == 0;
     const int64_t quads = vec ? hw / 4 : 0;
     for (int64_t i = t; i < quads; i += stride) {
-        const int4 q = reinterpret_cast<const int4*>(load)[i];
+        const int4 q = whole_loads(reinterpret_cast<const typename Quad<T>::type*>(load)[i]);
         reinterpret_cast<float4*>(dl_dload)[i] = make_float4(grad(q.x), grad(q.y), grad(q.z), grad(q.w));
     }
-    for (int64_t i = 4 * quads + t; i < hw; i += stride) dl_dload[i] = grad(load[i]);
+    for (int64_t i = 4 * quads + t; i < hw; i += stride) dl_dload[i] = grad(whole_load(load[i]));
 }
 
 }  // namespace
@@ -585,7 +599,8 @@ void launch_preprocess_backward(int n, const float* means, const float* scales, 
                                                                g_scales, g_rots, g_opac, g_sh);
 }
 
-void launch_load_loss(const int32_t* load, int64_t hw, double* sums, float weight, float* dl_dload,
+template <typename T>
+void launch_load_loss(const T* load, int64_t hw, double* sums, float weight, float* std_out, float* dl_dload,
                       int sm_count, cudaStream_t stream) {
     if (hw <= 0) return;
     cudaMemsetAsync(sums, 0, 8 * sizeof(double), stream);
@@ -593,7 +608,9 @@ void launch_load_loss(const int32_t* load, int64_t hw, double* sums, float weigh
     const int64_t most = (hw + 1023) / 1024, full = (int64_t)sm_count * 4;
     const unsigned grid = (unsigned)(most < full ? most : full);
     k_load_moments<<<grid, 256, 0, stream>>>(load, hw, reinterpret_cast<unsigned long long*>(sums + kLoadSumWords));
-    k_load_grad<<<grid, 256, 0, stream>>>(load, hw, sums, weight, dl_dload, 1);
+    k_load_grad<<<grid, 256, 0, stream>>>(load, hw, sums, weight, std_out, dl_dload);
 }
+template void launch_load_loss<int32_t>(const int32_t*, int64_t, double*, float, float*, float*, int, cudaStream_t);
+template void launch_load_loss<float>(const float*, int64_t, double*, float, float*, float*, int, cudaStream_t);
 
 }  // namespace adr

@@ -332,15 +332,19 @@ k_ssim_backward(const float* __restrict__ img, const float* __restrict__ ref, in
     }
 }
 
-__global__ void k_loss_finalize(double* stats, double count) {
-    stats[0] /= count;
-    stats[1] /= count;
+// The means and, where asked for, the loss: formed here, as one more launch over
+// one value costs a caller as much as a pass over a small image.
+__global__ void k_loss_finalize(double* stats, double count, double w_l1, double w_ssim, float* loss) {
+    const double l1 = stats[0] / count, ssim = stats[1] / count;
+    stats[0] = l1;
+    stats[1] = ssim;
+    if (loss) *loss = (float)__dadd_rn(__dmul_rn(w_l1, l1), __dmul_rn(w_ssim, 1.0 - ssim));
 }
 
 }  // namespace
 
 void launch_image_loss(const float* img, const float* ref, int channels, int H, int W,
-                       const LossWindow& win, float w_l1, float w_ssim, double* stats,
+                       const LossWindow& win, double w_l1, double w_ssim, double* stats, float* loss,
                        float* dl_dimg, float* scratch, cudaStream_t stream) {
     const dim3 grid((W + kLW - 1) / kLW, (H + kLTall - 1) / kLTall, channels);
     const double count = (double)channels * H * W;
@@ -353,12 +357,12 @@ void launch_image_loss(const float* img, const float* ref, int channels, int H, 
     cudaFuncSetAttribute(k_ssim_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BackwardShared));
     cudaMemsetAsync(stats, 0, 2 * sizeof(double), stream);
     // loss = w_l1 * mean|x - y| + w_ssim * (1 - mean S): d loss / dS = -w_ssim / count
-    k_ssim_forward<<<grid, kLThreads, sizeof(ForwardShared), stream>>>(img, ref, H, W, win, (float)(-w_ssim / count),
+    k_ssim_forward<<<grid, kLThreads, sizeof(ForwardShared), stream>>>(img, ref, H, W, win, (float)(-(float)w_ssim / count),
                                                    g_mu, g_xx, g_xy, stats);
     if (dl_dimg)
         k_ssim_backward<<<grid, kLThreads, sizeof(BackwardShared), stream>>>(img, ref, H, W, win, g_mu, g_xx, g_xy,
-                                                        (float)(w_l1 / count), dl_dimg);
-    k_loss_finalize<<<1, 1, 0, stream>>>(stats, count);
+                                                        (float)((float)w_l1 / count), dl_dimg);
+    k_loss_finalize<<<1, 1, 0, stream>>>(stats, count, w_l1, w_ssim, loss);
 }
 
 }  // namespace adr

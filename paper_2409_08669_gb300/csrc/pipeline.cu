@@ -295,6 +295,7 @@ static RenderCam render_cam(const Workspace& ws, const FrameState& fs, float* im
     rc.img = img;
     rc.t_final = t_final;
     rc.load = load;
+    rc.load_float = fs.load_float;
     rc.last = ws.last;
     rc.trav = ws.trav;
     rc.tfin = ws.tfin;

@@ -449,7 +449,7 @@ k_render(const RenderBatch batch) {
         rc.img[hw + pixa] = C1.x + T.x * bg1;
         rc.img[2 * hw + pixa] = C2.x + T.x * bg2;
         if (rc.t_final) rc.t_final[pixa] = T.x;
-        if (rc.load) rc.load[pixa] = cnt_a;
+        if (rc.load) rc.load[pixa] = rc.load_float ? __float_as_int((float)cnt_a) : cnt_a;
         if (rc.last) rc.last[pixa] = last_a;
         if (rc.trav) rc.trav[pixa] = trav_a;
         if (rc.tfin) rc.tfin[pixa] = T.x;
@@ -460,7 +460,7 @@ k_render(const RenderBatch batch) {
         rc.img[hw + pixb] = C1.y + T.y * bg1;
         rc.img[2 * hw + pixb] = C2.y + T.y * bg2;
         if (rc.t_final) rc.t_final[pixb] = T.y;
-        if (rc.load) rc.load[pixb] = cnt_b;
+        if (rc.load) rc.load[pixb] = rc.load_float ? __float_as_int((float)cnt_b) : cnt_b;
         if (rc.last) rc.last[pixb] = last_b;
         if (rc.trav) rc.trav[pixb] = trav_b;
         if (rc.tfin) rc.tfin[pixb] = T.y;
@@ -577,7 +577,7 @@ k_render_half(const RenderBatch batch) {
         rc.img[hw + pix] = C1 + T * st.bg[1];
         rc.img[2 * hw + pix] = C2 + T * st.bg[2];
         if (rc.t_final) rc.t_final[pix] = T;
-        if (rc.load) rc.load[pix] = cnt;
+        if (rc.load) rc.load[pix] = rc.load_float ? __float_as_int((float)cnt) : cnt;
         if (rc.last) rc.last[pix] = last;
         if (rc.trav) rc.trav[pix] = trav;
         if (rc.tfin) rc.tfin[pix] = T;

@@ -65,10 +65,11 @@ def check_params(params, device=None):
     return n
 
 
-def image_loss(img, ref, w_l1=1.0, w_ssim=0.0, want_grad=True, stream=None, scratch=None):
+def image_loss(img, ref, w_l1=1.0, w_ssim=0.0, want_grad=True, stream=None, scratch=None, value=None):
     """(stats, grad): stats = device float64 [mean |img - ref|, mean SSIM] and
     grad = d(w_l1 * L1 + w_ssim * (1 - SSIM)) / d img (None unless want_grad),
-    computed by adr_image_loss.  img, ref: [C, H, W] float32 on one device."""
+    computed by adr_image_loss.  img, ref: [C, H, W] float32 on one device.
+    `value` (a device float32, optional) gets w_l1 * L1 + w_ssim * (1 - SSIM)."""
     img, ref = img.contiguous(), ref.contiguous()
     if img.dim() != 3:
         raise ValueError(f"img must be [C, H, W], got shape {tuple(img.shape)}")
@@ -86,8 +87,13 @@ def image_loss(img, ref, w_l1=1.0, w_ssim=0.0, want_grad=True, stream=None, scra
         if scratch is None or scratch.numel() < 3 * img.numel():
             scratch = torch.empty(3 * img.numel(), dtype=torch.float32, device=img.device)
     with torch.cuda.device(img.device):
-        _lib.adr_image_loss(_ptr(img), _ptr(ref), c, h, w, float(w_l1), float(w_ssim), _ptr(stats),
-                            _ptr(grad), _ptr(scratch) if want_grad else 0, _stream(stream))
+        args = (_ptr(img), _ptr(ref), c, h, w, float(w_l1), float(w_ssim), _ptr(stats))
+        rest = (_ptr(grad), _ptr(scratch) if want_grad else 0, _stream(stream))
+        if value is None:
+            _lib.adr_image_loss(*args, *rest)
+        else:
+            check_tensor("value", value, 1, device=img.device.index)
+            _lib.adr_image_loss_value(*args, _ptr(value), *rest)
     return stats, grad
 
 
@@ -129,7 +135,11 @@ class Rasterizer:
     def sort(self, stream=None):
         _lib.adr_sort(self.ctx, _stream(stream))
 
-    def render(self, img=None, t_final=None, load=None, stream=None, want_aux=True):
+    def render(self, img=None, t_final=None, load=None, stream=None, want_aux=True,
+               load_dtype=torch.int32):
+        """`load_dtype`: torch.int32, or torch.float32 for the loads as floats."""
+        if load_dtype not in (torch.int32, torch.float32):
+            raise ValueError(f"load_dtype must be torch.int32 or torch.float32, got {load_dtype}")
         h, w = self.camera.height, self.camera.width
         dev = f"cuda:{self.device}"
         if img is None:
@@ -137,13 +147,14 @@ class Rasterizer:
         if want_aux and t_final is None:
             t_final = torch.empty((h, w), dtype=torch.float32, device=dev)
         if want_aux and load is None:
-            load = torch.empty((h, w), dtype=torch.int32, device=dev)
+            load = torch.empty((h, w), dtype=load_dtype, device=dev)
         check_tensor("img", img, 3 * h * w, device=self.device)
         if t_final is not None:
             check_tensor("t_final", t_final, h * w, device=self.device)
         if load is not None:
-            check_tensor("load", load, h * w, dtype=torch.int32, device=self.device)
-        _lib.adr_render(self.ctx, _ptr(img), _ptr(t_final), _ptr(load), _stream(stream))
+            check_tensor("load", load, h * w, dtype=load_dtype, device=self.device)
+        call = _lib.adr_render if load_dtype == torch.int32 else _lib.adr_render_float_load
+        call(self.ctx, _ptr(img), _ptr(t_final), _ptr(load), _stream(stream))
         return img, t_final, load
 
     def forward(self, params, camera, settings, stream=None, **kw):
@@ -187,6 +198,15 @@ class Rasterizer:
         _lib.adr_load_loss(self.ctx, _ptr(load), load.numel(), float(weight), _ptr(stats), _ptr(grad),
                            _stream(stream))
         return stats, grad
+
+    def load_loss_float(self, load, weight=1.0, stream=None):
+        """(std, weight * dL_load/dl) of loads given as floats (rounded to whole numbers)."""
+        check_tensor("load", load, load.numel(), device=self.device)
+        std = torch.empty((), dtype=torch.float32, device=load.device)
+        grad = torch.empty_like(load)
+        _lib.adr_load_loss_float(self.ctx, _ptr(load), load.numel(), float(weight), _ptr(std), _ptr(grad),
+                                 _stream(stream))
+        return std, grad
 
     # -- inspection -------------------------------------------------------------
     def num_pairs(self, raise_on_error=True):
