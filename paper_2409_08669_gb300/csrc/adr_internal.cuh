@@ -710,6 +710,57 @@ __device__ __forceinline__ int warp_list(const uint32_t* mask, int m, int lane, 
     return n;
 }
 
+// A warp's SH rows (32 Gaussians of 12 float4 each, 6 KB) in shared memory, padded
+// by 16 bytes so that 32 lanes reading or writing one float4 each of their own row
+// use distinct banks.  They move to and from memory as consecutive 16-byte pieces
+// of consecutive lanes: a lane reading its own row from memory touches 32 cache
+// lines an instruction, and twelve of those take the L1 longer than DRAM takes for
+// their bytes (k_preprocess_backward, 1M Gaussians: 122 -> 88 us; frames of 1M from
+// host memory 757 -> 651 us).
+constexpr int kShQuads = 12, kShStride = kShQuads + 1;
+using ShRows = float4[32 * kShStride];
+
+__device__ __forceinline__ void async_quad(float4* to, const float4* from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+// Starts copying the first `quads` (1, 3, 7 or 12) float4 of the rows `wanted` of
+// the 32 to their places; from(r) is where row r (0 <= r < 32) lies, called by all
+// lanes.  async_rows_wait() ends it for the whole warp.
+template <int kQuads, class From>
+__device__ __forceinline__ void async_rows_of(uint32_t wanted, int lane, ShRows& rows, From from) {
+    if constexpr (kQuads == kShQuads) {   // two rows an instruction, lane 12 r + c its row's piece c
+        const int second = lane >= kShQuads ? 1 : 0, col = lane - second * kShQuads;
+        const uint32_t mine = lane < 2 * kShQuads ? wanted >> second : 0u;
+        float4* to = rows + second * kShStride + col;
+#pragma unroll
+        for (int r = 0; r < 32; r += 2) {
+            const float4* row = from(r + second);
+            if ((mine >> r) & 1u) async_quad(to + r * kShStride, row + col);
+        }
+    } else {   // the pieces in order, 32 an instruction
+#pragma unroll
+        for (int j = 0; j < kQuads; ++j) {
+            const int f = 32 * j + lane, r = f / kQuads, col = f % kQuads;
+            const float4* row = from(r);
+            if ((wanted >> r) & 1u) async_quad(rows + r * kShStride + col, row + col);
+        }
+    }
+}
+template <class From>
+__device__ __forceinline__ void async_rows(uint32_t wanted, int quads, int lane, ShRows& rows, From from) {
+    if (quads == 12) async_rows_of<12>(wanted, lane, rows, from);
+    else if (quads == 7) async_rows_of<7>(wanted, lane, rows, from);
+    else if (quads == 3) async_rows_of<3>(wanted, lane, rows, from);
+    else async_rows_of<1>(wanted, lane, rows, from);
+}
+__device__ __forceinline__ void async_rows_wait() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+}
+// The float4 of a row that SH degree `degree` reads: of 1, 4, 9 or 16 coefficients.
+__device__ __forceinline__ int sh_quads(int degree) { return degree >= 3 ? 12 : degree == 2 ? 7 : degree == 1 ? 3 : 1; }
+
 // 1-D taps of the SSIM window (the 2-D window is their outer product).
 struct LossWindow {
     float w[11];

@@ -26,17 +26,8 @@ constexpr float kY3c = 0.45704579946446572f;   // sqrt(21/(32 pi))
 constexpr float kY3d = 0.37317633259011540f;   // sqrt(7/(16 pi))
 constexpr float kY3e = 1.4453057213202769f;    // sqrt(105/(16 pi))
 
-__device__ __forceinline__ float3 sh_to_rgb(const float* __restrict__ sh, int degree, float x,
-                                            float y, float z) {
-    // sh: 16 coefficients x 3 channels, 16-byte aligned (192 bytes per Gaussian).
-    const float4* s4 = reinterpret_cast<const float4*>(sh);
-    float c[48];
-    const int nload = degree >= 3 ? 12 : (degree == 2 ? 7 : (degree == 1 ? 3 : 1));
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        float4 v = k < nload ? __ldg(s4 + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-        c[4 * k + 0] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
-    }
+// row: 16 coefficients x 3 channels as 12 float4, of which sh_quads(degree) are read.
+__device__ __forceinline__ float3 sh_to_rgb(const float4* row, int degree, float x, float y, float z) {
     float w[16];
     w[0] = kY00;
     w[1] = -kY1 * y; w[2] = kY1 * z; w[3] = -kY1 * x;
@@ -53,16 +44,26 @@ __device__ __forceinline__ float3 sh_to_rgb(const float* __restrict__ sh, int de
     w[13] = -kY3c * x * (4.f * zz - xx - yy);
     w[14] = kY3e * z * (xx - yy);
     w[15] = -kY3a * x * (xx - 3.f * yy);
-    const int nb = (degree + 1) * (degree + 1);
-    float r = 0.f, g = 0.f, b = 0.f;
+    float rgb[3] = {0.f, 0.f, 0.f};
+    auto add = [&](int j, int nb) {
+        const float4 q = row[j];
+        const float v[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        if (k < nb) {
-            r = fmaf(c[3 * k + 0], w[k], r);
-            g = fmaf(c[3 * k + 1], w[k], g);
-            b = fmaf(c[3 * k + 2], w[k], b);
+        for (int u = 0; u < 4; ++u) {
+            const int e = 4 * j + u, k = e / 3, c = e % 3;
+            if (k < nb) rgb[c] = fmaf(v[u], w[k], rgb[c]);
         }
+    };
+    if (degree >= 3) {   // no test per coefficient
+#pragma unroll
+        for (int j = 0; j < kShQuads; ++j) add(j, 16);
+    } else {
+        const int nb = (degree + 1) * (degree + 1), quads = sh_quads(degree);
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+            if (j < quads) add(j, nb);
     }
+    const float r = rgb[0], g = rgb[1], b = rgb[2];
     return make_float3(fmaxf(r + 0.5f, 0.f), fmaxf(g + 0.5f, 0.f), fmaxf(b + 0.5f, 0.f));
 }
 
@@ -94,16 +95,6 @@ __device__ __forceinline__ ff ff_add_f(ff a, float b) {
     ff s = ff_two_sum(a.hi, b);
     return ff_norm(s.hi, __fadd_rn(s.lo, a.lo));
 }
-__device__ __forceinline__ ff ff_mul_f(ff a, float b) {
-    ff p = ff_two_prod(a.hi, b);
-    return ff_norm(p.hi, __fmaf_rn(a.lo, b, p.lo));
-}
-__device__ __forceinline__ ff ff_div(ff a, ff b) {
-    const float q1 = __fdiv_rn(a.hi, b.hi);
-    ff r = ff_add(a, ff_mul_f(b, -q1));
-    const float q2 = __fdiv_rn(r.hi, b.hi);
-    return ff_norm(q1, q2);
-}
 // sum_k v[k] * x[k] + t, accumulated in float-float.
 __device__ __forceinline__ ff ff_dot3_plus(float v0, float v1, float v2, float t, float x0,
                                            float x1, float x2) {
@@ -111,6 +102,48 @@ __device__ __forceinline__ ff ff_dot3_plus(float v0, float v1, float v2, float t
     acc = ff_add(acc, ff_two_prod(v1, x1));
     acc = ff_add(acc, ff_two_prod(v2, x2));
     return ff_add_f(acc, t);
+}
+// The same on two values at once, paired FP32 operations: x and y of the view.
+struct ff2 { float2 hi, lo; };
+
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ ff2 ff2_two_prod(float2 a, float2 b) {
+    const float2 p = fmul2(a, b);
+    return {p, ffma2(a, b, neg2(p))};
+}
+__device__ __forceinline__ ff2 ff2_two_sum(float2 a, float2 b) {
+    const float2 s = fadd2(a, b);
+    const float2 bb = fsub2(s, a);
+    return {s, fadd2(fsub2(a, fsub2(s, bb)), fsub2(b, bb))};
+}
+__device__ __forceinline__ ff2 ff2_norm(float2 hi, float2 lo) {
+    const float2 s = fadd2(hi, lo);
+    return {s, fsub2(lo, fsub2(s, hi))};
+}
+__device__ __forceinline__ ff2 ff2_add(ff2 a, ff2 b) {
+    const ff2 s = ff2_two_sum(a.hi, b.hi);
+    return ff2_norm(s.hi, fadd2(s.lo, fadd2(a.lo, b.lo)));
+}
+__device__ __forceinline__ ff2 ff2_add_f(ff2 a, float2 b) {
+    const ff2 s = ff2_two_sum(a.hi, b);
+    return ff2_norm(s.hi, fadd2(s.lo, a.lo));
+}
+__device__ __forceinline__ ff2 ff2_mul_f(ff2 a, float2 b) {
+    const ff2 p = ff2_two_prod(a.hi, b);
+    return ff2_norm(p.hi, ffma2(a.lo, b, p.lo));
+}
+__device__ __forceinline__ ff2 ff2_div(ff2 a, ff b) {   // both halves by one divisor
+    const float2 q1 = make_float2(__fdiv_rn(a.hi.x, b.hi), __fdiv_rn(a.hi.y, b.hi));
+    const ff2 r = ff2_add(a, ff2_mul_f({dup2(b.hi), dup2(b.lo)}, neg2(q1)));
+    const float2 q2 = make_float2(__fdiv_rn(r.hi.x, b.hi), __fdiv_rn(r.hi.y, b.hi));
+    return ff2_norm(q1, q2);
+}
+__device__ __forceinline__ ff2 ff2_dot3_plus(float2 v0, float2 v1, float2 v2, float2 t, float x0, float x1, float x2) {
+    ff2 acc = ff2_two_prod(v0, dup2(x0));
+    acc = ff2_add(acc, ff2_two_prod(v1, dup2(x1)));
+    acc = ff2_add(acc, ff2_two_prod(v2, dup2(x2)));
+    return ff2_add_f(acc, t);
 }
 // a*d - b*c with one rounding error (Kahan's fused form).
 __device__ __forceinline__ float det2(float a, float b, float c, float d) {
@@ -158,9 +191,18 @@ constexpr float kHalfLog2e = 0.84932180028801907f;
 // Gaussians of chunk k / count for camera k % count, so the blocks of one
 // chunk run side by side and every camera after the first reads the chunk's
 // parameters from L2 rather than DRAM.
-constexpr int kPreThreads = 256;
-constexpr int kPreCtasPerSm = 3;
-__global__ void __launch_bounds__(kPreThreads, kPreCtasPerSm)   // <= 80 registers
+//
+// Bound by instruction issue (about 1240 a warp: float-float centres, IEEE divisions
+// and roots, culls, colour; 70% of the slots) with the memory's latency behind it.
+// The view's x and y and their quotients go through paired FP32 operations, which
+// round as the single ones do; the SH rows arrive in shared memory by coalesced
+// asynchronous copies while the records are written (async_rows), so no 48
+// coefficients are held in registers: 7 CTAs of 128 threads per SM (72 registers)
+// instead of 3 of 256 (80).  1390 -> 1240 instructions a warp; frames of 3M Gaussians
+// at 1080p 508 -> 479 us, at 4K 969 -> 935; 6 CTAs 479, 5 490, 8 489.
+constexpr int kPreThreads = 128;
+constexpr int kPreCtasPerSm = 7;
+__global__ void __launch_bounds__(kPreThreads, kPreCtasPerSm)
 k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ scales,
              const float* __restrict__ rots, const float* __restrict__ opac,
              const float* __restrict__ sh, PreprocessBatch batch, int64_t ahead) {
@@ -182,7 +224,10 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], 128;" ::"l"(opac + g) : "memory");
         }
     }
-    if (i >= n) return;
+    __shared__ ShRows s_rows[kPreThreads / 32];
+    const int lane = threadIdx.x & 31;
+    if (i - lane >= n) return;   // no lane of the warp has a Gaussian
+    const bool mine = i < n;
     const CamDev cam = out.fp->cam;
     const SetDev st = out.fp->st;
     float4* __restrict__ rec = out.rec;
@@ -191,7 +236,8 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
     uint32_t* __restrict__ gbox = out.gbox;
     uint32_t rank = kNoRank;   // arrival rank in the depth bin
 
-    const float mx = means[3 * i + 0], my = means[3 * i + 1], mz = means[3 * i + 2];
+    const float mx = mine ? means[3 * i + 0] : 0.f, my = mine ? means[3 * i + 1] : 0.f,
+                mz = mine ? means[3 * i + 2] : 0.f;
     // Sort depth: fixed evaluation order, each operation rounded separately.
     float depth = __fmul_rn(cam.v[8], mx);
     depth = __fadd_rn(depth, __fmul_rn(cam.v[9], my));
@@ -204,14 +250,15 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
     float4 r0 = zero4, r1 = zero4, r2 = zero4, a0 = zero4;
     float4 a1 = make_float4(0.f, 0.f, depth, 0.f);
 
-    if (depth > cam.near_z) {
+    if (mine && depth > cam.near_z) {
         // View-space position in float-float; the pixel centre px = fx x/z + cx
         // keeps ~1e-9 px accuracy at any image size.
-        const ff xv = ff_dot3_plus(cam.v[0], cam.v[1], cam.v[2], cam.v[3], mx, my, mz);
-        const ff yv = ff_dot3_plus(cam.v[4], cam.v[5], cam.v[6], cam.v[7], mx, my, mz);
+        const ff2 xy = ff2_dot3_plus(make_float2(cam.v[0], cam.v[4]), make_float2(cam.v[1], cam.v[5]),
+                                     make_float2(cam.v[2], cam.v[6]), make_float2(cam.v[3], cam.v[7]), mx, my, mz);
         const ff zv = ff_dot3_plus(cam.v[8], cam.v[9], cam.v[10], cam.v[11], mx, my, mz);
-        const ff pxf = ff_add_f(ff_mul_f(ff_div(xv, zv), cam.fx), cam.cx);
-        const ff pyf = ff_add_f(ff_mul_f(ff_div(yv, zv), cam.fy), cam.cy);
+        const ff2 centre = ff2_add_f(ff2_mul_f(ff2_div(xy, zv), make_float2(cam.fx, cam.fy)),
+                                     make_float2(cam.cx, cam.cy));
+        const ff pxf = {centre.hi.x, centre.lo.x}, pyf = {centre.hi.y, centre.lo.y};
         const float pz_v = zv.hi;
 
         // Rotation of the normalised quaternion and M = R diag(s): Sigma = M M^T (Eq. 1).
@@ -227,8 +274,8 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
         // EWA: Sigma' = T Sigma T^T + lowpass I with T = J W, so Sigma' - lowpass I = U U^T, U = T M.
         const float inv_z = 1.f / pz_v;
         const float limx = st.jac_clamp * cam.tan_fovx, limy = st.jac_clamp * cam.tan_fovy;
-        const float txz = fminf(limx, fmaxf(-limx, xv.hi * inv_z)) * pz_v;
-        const float tyz = fminf(limy, fmaxf(-limy, yv.hi * inv_z)) * pz_v;
+        const float txz = fminf(limx, fmaxf(-limx, xy.hi.x * inv_z)) * pz_v;
+        const float tyz = fminf(limy, fmaxf(-limy, xy.hi.y * inv_z)) * pz_v;
         const float j00 = cam.fx * inv_z, j02 = -cam.fx * txz * inv_z * inv_z;
         const float j11 = cam.fy * inv_z, j12 = -cam.fy * tyz * inv_z * inv_z;
         float T0[3], T1[3];
@@ -300,17 +347,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
                 // The depth histogram (bins.cu); the count comes back while the
                 // SH coefficients are on their way.
                 if (batch.map.count) rank = atomicAdd(out.bins + bin_of(key, bin_base(cam.near_z), batch.map), 1u);
-                // SH colour, d = normalise(X0 - cam_pos); with sh == nullptr
-                // (deferred colours) k_colors fills .xyz in for the Gaussians
-                // a Render launch blends.
-                float3 rgb = make_float3(0.f, 0.f, 0.f);
-                if (sh) {
-                    float dx = mx - cam.cam_pos[0], dy = my - cam.cam_pos[1], dz = mz - cam.cam_pos[2];
-                    const float dn = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-                    dx *= dn; dy *= dn; dz *= dn;
-                    rgb = sh_to_rgb(sh + (size_t)i * 48, st.sh_degree, dx, dy, dz);
-                }
-                r2 = make_float4(rgb.x, rgb.y, rgb.z, log2f(sigma));
+                r2.w = log2f(sigma);
             }
             r0 = make_float4(px, py, pxf.lo, pyf.lo);
             r1 = make_float4(s1 * e1x, s1 * e1y, -s2 * e1y, s2 * e1x);
@@ -318,21 +355,44 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
             a1 = make_float4(rx, ry, depth, lam);
         }
     }
+    // The SH rows of the Gaussians with tiles, on their way while the records are
+    // written.
+    ShRows& rows = s_rows[threadIdx.x >> 5];
+    const float4* sh4 = reinterpret_cast<const float4*>(sh) + (size_t)(i - lane) * kShQuads;
+    if (sh)
+        async_rows(__ballot_sync(0xffffffffu, ntiles != 0u), sh_quads(st.sh_degree), lane, rows,
+                   [&](int r) { return sh4 + r * kShQuads; });
     // Render and the backward read the records of Gaussians with tiles only;
     // the others keep just a1 (radii, depth) for inspection.
     if (ntiles) {
         rec[3 * i + 0] = r0;
         rec[3 * i + 1] = r1;
-        rec[3 * i + 2] = r2;
         aux[2 * i + 0] = a0;
     }
-    out.rank[i] = rank;
-    aux[2 * i + 1] = a1;
-    depth_key[i] = key;
-    // packed rectangle x0 | y0 << 8 | (w-1) << 16 | (h-1) << 24, all ones if no tiles
-    gbox[i] = ntiles ? (uint32_t)rc.x | ((uint32_t)rc.y << 8) | ((uint32_t)(rc.z - rc.x - 1) << 16) |
-                           ((uint32_t)(rc.w - rc.y - 1) << 24)
-                     : 0xFFFFFFFFu;
+    if (mine) {
+        out.rank[i] = rank;
+        aux[2 * i + 1] = a1;
+        depth_key[i] = key;
+        // packed rectangle x0 | y0 << 8 | (w-1) << 16 | (h-1) << 24, all ones if no tiles
+        gbox[i] = ntiles ? (uint32_t)rc.x | ((uint32_t)rc.y << 8) | ((uint32_t)(rc.z - rc.x - 1) << 16) |
+                               ((uint32_t)(rc.w - rc.y - 1) << 24)
+                         : 0xFFFFFFFFu;
+    }
+    // SH colour, d = normalise(X0 - cam_pos); with sh == nullptr (deferred colours)
+    // k_colors fills .xyz in for the Gaussians a Render launch blends.
+    if (sh) async_rows_wait();
+    if (ntiles) {
+        if (sh) {
+            float dx = mx - cam.cam_pos[0], dy = my - cam.cam_pos[1], dz = mz - cam.cam_pos[2];
+            const float dn = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+            dx *= dn; dy *= dn; dz *= dn;
+            const float3 rgb = sh_to_rgb(rows + lane * kShStride, st.sh_degree, dx, dy, dz);
+            r2.x = rgb.x;
+            r2.y = rgb.y;
+            r2.z = rgb.z;
+        }
+        rec[3 * i + 2] = r2;
+    }
     // The frame's pairs and column runs, a warp's lanes together (whichever of
     // them are here together: the sums add up), over kSumSlots addresses.
     const unsigned lanes = __activemask();
@@ -348,27 +408,41 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
 // Stage 1's view-dependent colour, rgb = max(0, sum_k sh_k Y_k(d) + 0.5) with
 // d = normalise(X0 - cam_pos), for the Gaussians ids[0 .. *count) (one per
 // thread, grid-stride): written into .xyz of their third render record.
-constexpr int kColorThreads = 256;
-__global__ void __launch_bounds__(kColorThreads)
+constexpr int kColorThreads = 128;
+__global__ void __launch_bounds__(kColorThreads, 8)   // as many as their rows fit in shared memory
 k_colors(const uint32_t* __restrict__ ids, const uint32_t* __restrict__ count,
          const float* __restrict__ means, const float* __restrict__ sh,
          const FrameParams* __restrict__ fp, float4* __restrict__ rec) {
     pdl_prologue();
+    __shared__ ShRows s_rows[kColorThreads / 32];
+    ShRows& rows = s_rows[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
     const uint32_t m = *count;
     const CamDev cam = fp->cam;
-    const int degree = fp->st.sh_degree;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-        const uint32_t i = ids[k];
-        const float mx = means[3 * (size_t)i + 0], my = means[3 * (size_t)i + 1], mz = means[3 * (size_t)i + 2];
-        float dx = mx - cam.cam_pos[0], dy = my - cam.cam_pos[1], dz = mz - cam.cam_pos[2];
-        const float dn = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
-        dx *= dn; dy *= dn; dz *= dn;
-        const float3 rgb = sh_to_rgb(sh + (size_t)i * 48, degree, dx, dy, dz);
-        float4 r2 = rec[3 * (size_t)i + 2];
-        r2.x = rgb.x;
-        r2.y = rgb.y;
-        r2.z = rgb.z;
-        rec[3 * (size_t)i + 2] = r2;
+    const int degree = fp->st.sh_degree, quads = sh_quads(degree);
+    for (uint32_t k0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); k0 < m; k0 += gridDim.x * blockDim.x) {
+        const bool mine = k0 + (uint32_t)lane < m;
+        const uint32_t i = mine ? ids[k0 + lane] : 0u;
+        // row r's Gaussian is lane r's
+        async_rows(__ballot_sync(0xffffffffu, mine), quads, lane, rows, [&](int r) {
+            return reinterpret_cast<const float4*>(sh) + (size_t)__shfl_sync(0xffffffffu, i, r) * kShQuads;
+        });
+        float4 r2 = make_float4(0.f, 0.f, 0.f, 0.f);
+        float dx = 0.f, dy = 0.f, dz = 0.f;
+        if (mine) {
+            dx = means[3 * (size_t)i + 0] - cam.cam_pos[0];
+            dy = means[3 * (size_t)i + 1] - cam.cam_pos[1];
+            dz = means[3 * (size_t)i + 2] - cam.cam_pos[2];
+            r2 = rec[3 * (size_t)i + 2];
+        }
+        async_rows_wait();
+        if (mine) {
+            const float dn = rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+            dx *= dn; dy *= dn; dz *= dn;
+            const float3 rgb = sh_to_rgb(rows + lane * kShStride, degree, dx, dy, dz);
+            rec[3 * (size_t)i + 2] = make_float4(rgb.x, rgb.y, rgb.z, r2.w);
+        }
+        __syncwarp();   // the rows are no longer read
     }
 }
 
