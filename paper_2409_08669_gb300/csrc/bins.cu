@@ -19,9 +19,10 @@
 // The radix sort's four passes are twelve launches whose time is the latency
 // of one 4096-key chunk's chain (load, sixteen ranking rounds, prefix,
 // write-out) several times over, whatever the number of keys; here a key is
-// moved once through memory and once through shared memory.  Measured with the
-// run scan that both need, us per frame (10k / 300k / 1.5M Gaussians with
-// tiles): see the table at kWindow.
+// moved once through memory and once through shared memory.  With the run scan
+// that both need: 88 us by the passes at 10k Gaussians (of a 155 us frame) and 100 at
+// 1M, 21 and 25 us by these three kernels (at 1M of depth slice 0), each 5 to 10 us
+// of latency.
 #include <cooperative_groups.h>
 
 #include "lookback.cuh"

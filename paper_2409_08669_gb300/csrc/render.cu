@@ -8,9 +8,10 @@
 // column runs of its column of tiles (kRuns) -- or its own list.  Each batch
 // reads up to 2048 runs (16 per thread), keeps those whose rows hold the
 // tile's row, compacts the first 256 kept ones stably into shared memory with
-// their records, and every pixel blends them.  Pixels stop early (transmittance below t_min), so a tile
-// usually reads only the front of its list; the CTA leaves as soon as every
-// pixel has terminated (__syncthreads_count).  Pixel offsets are taken
+// their records, and every warp blends those that reach its 8x8 quadrant.
+// Pixels stop early (transmittance below t_min), so a tile usually reads only the
+// front of its list; the CTA leaves as soon as every pixel has terminated
+// (__syncthreads_count).  Pixel offsets are taken
 // relative to the tile origin so the float-float centre collapses to one
 // well-conditioned float per Gaussian per tile.
 //
@@ -43,7 +44,7 @@ namespace {
 // rare stop.  With one entry a step, every entry evaluated and a vote and a branch
 // for the skip and the stop each, a step was a chain of about 200 clocks where a
 // tile's warp is alone on its scheduler.  Frames before -> after: 150k 1001x667
-// 316 -> 182 us, 600k plain 720p 262 -> 195, 3M 1080p 579 -> 516, 3M 4K 1087 -> 969,
+// 316 -> 182 us, 600k plain 720p 262 -> 195, 3M 1080p 583 -> 516, 3M 4K 1087 -> 969,
 // 2k 64x48 160 -> 137.  Four entries a step: fewer instructions, but 72 registers
 // and more steps with a stop in them (3M 4K 974, 16 served frames 3305 against
 // 3140).  Staging 128 at a time: 3M 1080p 534.
