@@ -158,6 +158,7 @@ struct adr_ctx {
     // half of all runs, and every kSliceProbe-th frame slices to measure again.
     cudaEvent_t slice_ev = nullptr;
     bool slice_probe = false;        // a readback is in flight
+    bool last_backward = false;      // the last frame had a backward
     bool slices_pay = true;
     uint32_t frames = 0;
     uint32_t radix_probe_in = kRadixProbe;   // see next_depth_sort
@@ -432,8 +433,11 @@ static bool next_frame_slices(adr_ctx* c) {
             cudaGetLastError();   // not an error: clear it
         }
     }
-    return c->slice_mode == ADR_SLICES_ALWAYS ||
-           (c->slice_mode == ADR_SLICES_ADAPTIVE && (c->slices_pay || (c->frames % kSliceProbe) == 0));
+    if (c->slice_mode != ADR_SLICES_ADAPTIVE) return c->slice_mode == ADR_SLICES_ALWAYS;
+    // A backward needs every Gaussian's runs: where one followed the last frame, this
+    // one's are built at once rather than in two slices and then again (training step
+    // of 1M Gaussians at 1280x720: 815 -> 708 us).
+    return !c->last_backward && (c->slices_pay || (c->frames % kSliceProbe) == 0);
 }
 
 adr_status adr_sort(adr_ctx* c, void* stream) {
@@ -444,6 +448,7 @@ adr_status adr_sort(adr_ctx* c, void* stream) {
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     c->fs.allow_slices = next_frame_slices(c);
+    c->last_backward = false;
     ++c->frames;
     enqueue_sort(c->ws, c->fs, c->epoch, strm);
     adr_status s;
@@ -608,6 +613,7 @@ adr_status adr_render_backward(adr_ctx* c, const float* means, const float* scal
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     enqueue_tile_lists(c->ws, c->fs, strm);   // the backward walks per-tile lists
+    c->last_backward = true;
     enqueue_backward(c->ws, c->fs, means, scales, rots, opac, sh, dl_dimg, dl_dload, g_means,
                      g_scales, g_rots, g_opac, g_sh, strm);
     return check_launch("adr_render_backward") == ADR_OK ? ok() : ADR_ERR_CUDA;

@@ -37,6 +37,30 @@ def test_render_writes_the_loads_as_floats(slices, split):
         rast.close()
 
 
+def test_a_frame_after_a_backward_is_not_sliced():
+    from paper_2409_08669_gb300.raster import upload
+    rast = _rast()
+    try:
+        params = upload(S.tiny_scene(3, n=2000))
+        cam, st = S.look_at((0, 0.2, -2.5), width=130, height=75), S.Settings()
+        frames, sliced = [], []
+        for backward in (True, True, False, False):
+            img, t_final, load = rast.forward(params, cam, st)
+            frames.append((img, t_final, load))
+            sliced.append(rast.frame_counts()["sliced"])
+            if backward:
+                rast.backward(params, torch.ones_like(img))
+        assert sliced[:3] == [1, 0, 0]      # the first frame measures, two follow a backward
+        rast.set_depth_slices(rast.SLICES_ALWAYS)
+        rast.backward(params, torch.ones_like(img))
+        frames.append(rast.forward(params, cam, st))
+        assert rast.frame_counts()["sliced"] == 1
+        for frame in frames[1:]:
+            assert all(torch.equal(a, b) for a, b in zip(frame, frames[0]))
+    finally:
+        rast.close()
+
+
 @pytest.mark.parametrize("hw,offset", [(1, 0), (3, 0), (1023, 1), (4096, 2), (921_601, 3)])
 def test_load_loss_of_floats_is_that_of_the_rounded_loads(hw, offset):
     rast = _rast()
