@@ -178,16 +178,17 @@ k_ssim_forward(const float* __restrict__ img, const float* __restrict__ ref, int
         const float vx = mm[o].x - mx * mx, vy = mm[o].y - my * my, cxy = p[o] - mx * my;
         const float A1 = 2.f * mx * my + kC1, A2 = 2.f * cxy + kC2;
         const float B1 = mx * mx + my * my + kC1, B2 = vx + vy + kC2;
-        const float R = 1.f / (B1 * B2), S = A1 * A2 * R;
+        const float S = (A1 * A2) / (B1 * B2);
         const float2 xy = sm.xy[(r + kLR) * kPairStride + lane + kLR];
         pair_add(ssim_sum, S);
         pair_add(l1_sum, fabsf(xy.x - xy.y));
         if (g_mu) {
             // dS/dmu_x, dS/dE[x^2], dS/dE[xy] at this pixel, times d loss / dS.
-            // S / A1, S / A2 and S / B2 share the one division.
-            const float d_mu = 2.f * (my * (A2 - A1) - mx * S * (B2 - B1)) * R;
-            const float d_xx = -S * B1 * R;
-            const float d_xy = 2.f * A1 * R;
+            // A quotient each: their sums cancel in the gradient, and one shared
+            // reciprocal put it up to 1e-6 further from FP64.
+            const float d_mu = S * (2.f * my / A1 - 2.f * my / A2 - 2.f * mx / B1 + 2.f * mx / B2);
+            const float d_xx = -S / B2;
+            const float d_xy = 2.f * S / A2;
             const uint32_t at = channel + (uint32_t)(gy * W + gx);
             g_mu[at] = g_scale * d_mu;
             g_xx[at] = g_scale * d_xx;
