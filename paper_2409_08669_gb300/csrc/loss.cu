@@ -24,7 +24,8 @@
 // store phase into distinct banks.  Sums over pixels run in float pairs (two-sum)
 // and only the tiles' totals in FP64, of which this chip has 1/64 of the FP32
 // rate.  1920x1080x3, forward / backward: 118 / 85 us with one output per thread
-// and step and FP64 sums, 66 / 44 us now (FMA pipe 53 / 43% busy, 3 CTAs per SM).
+// and step and FP64 sums, 75 / 42 us now (3 CTAs per SM; 66 forward with one shared
+// reciprocal instead of seven quotients a pixel).
 #include "adr_internal.cuh"
 
 namespace adr {
