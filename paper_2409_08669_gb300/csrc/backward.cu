@@ -7,8 +7,8 @@
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
 //                         and accumulates, with v = alpha dL/dalpha, sum v, dL/d(px,
 //                         py), the second moments of v about the Gaussian's centre
-//                         and its colour gradient; warp-reduced, then atomicAdd
-//                         into 9 floats per Gaussian.
+//                         and its colour gradient; reduced over the tile, then
+//                         atomicAdd into 9 floats per Gaussian.
 //   k_preprocess_backward dL/d(conic, sigma) from the moments, and the chain rule
 //                         to means, scales, rotations, opacities and SH
 //                         coefficients.
@@ -22,7 +22,8 @@ namespace {
 
 constexpr int kBwdThreads = kTilePixels / 2;   // two vertically adjacent pixels per thread
 constexpr int kBwdWarps = kBwdThreads / 32;
-constexpr int kBwdStage = 256;                 // list positions staged at a time
+constexpr int kBwdStage = 128;                 // list positions staged at a time
+constexpr int kSums = 9;                       // per Gaussian
 
 // Sum over the warp of nine per-lane values, as a reduce-scatter by recursive
 // halving: at distance 8, 4, 2 and 1 the lanes whose bit is clear keep the first
@@ -80,6 +81,10 @@ __device__ __forceinline__ int reduce_slot(int lane) {
 // per thread in 16x2-pixel warps that walk the whole list, 247 us now.  (Moments of
 // both pixels at once in 8x8 squares took 210 us, but their rounding put a scale's
 // gradient up to 3e-3 elsewhere, three times what this form does.)
+// A Gaussian's sums over the four strips are added on chip, so that a tile makes one
+// addition to memory per value: a Gaussian of thousands of tiles rounds its total
+// that much less often (a step's time is 1% more; with four, its SH gradients lay
+// further from FP64 than with a sum per 16x2 warp on some frames).
 __global__ void __launch_bounds__(kBwdThreads, 6)   // 80 registers; 4 to 8 CTAs per SM are within 1.5%
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
                   const float4* __restrict__ rec, const float4* __restrict__ aux,
@@ -93,6 +98,7 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     __shared__ float4 s_cn[kBwdStage];    // conic a, b, c, the Gaussian
     __shared__ uint32_t s_mask[kBwdWarps][kBwdStage / 32];   // staged Gaussians that reach each strip
     __shared__ uint32_t s_list[kBwdWarps][kBwdStage];
+    __shared__ alignas(16) float s_sum[kBwdWarps][kBwdStage * kSums];   // each warp's sums
     __shared__ int s_max[kBwdWarps];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -181,6 +187,8 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             }
             if (lane < 4) s_mask[lane][j >> 5] = mine;
         }
+        for (int v = threadIdx.x; v < kBwdWarps * kBwdStage * kSums / 4; v += kBwdThreads)
+            reinterpret_cast<float4*>(&s_sum[0][0])[v] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
         // this warp's positions: none of its pixels blended one past warp_last
         const uint32_t* list = s_list[warp];
@@ -236,7 +244,14 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             const float sums[9] = {v.x + v.y,   px.x + px.y, py.x + py.y, xx.x + xx.y, xy.x + xy.y,
                                    yy.x + yy.y, c0.x + c0.y, c1.x + c1.y, c2.x + c2.y};
             const float tot = reduce_scatter9(sums, lane);
-            if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * 9 + slot, tot);
+            if (slot >= 0) s_sum[warp][(off / 16u) * kSums + slot] = tot;
+        }
+        __syncthreads();
+        // The tile's sums: one addition to memory per Gaussian and value.
+        for (int v = threadIdx.x; v < m * kSums; v += kBwdThreads) {
+            const float t = (s_sum[0][v] + s_sum[1][v]) + (s_sum[2][v] + s_sum[3][v]);
+            const int j = v / kSums;
+            if (t != 0.f) atomicAdd(g2d + (size_t)__float_as_uint(s_cn[j].w) * kSums + (v - j * kSums), t);
         }
     }
 }
