@@ -213,7 +213,7 @@ adr_status adr_render_float_load(adr_ctx *ctx, float *img, float *t_final, float
  * above sh_degree get 0).  The parameter arrays must be the ones passed to
  * adr_preprocess for this frame, unchanged.  Gradient buffers are overwritten.
  * Per tile, each pixel walks its blended Gaussians back to front recovering
- * T_k = T_{k+1}/(1-alpha_k); contributions are reduced per tile and then added to
+ * T_k = T_{k+1}/(1-alpha_k); contributions are warp-reduced and then added to
  * per-Gaussian accumulators with atomics (summation order varies run to run). */
 adr_status adr_render_backward(adr_ctx *ctx, const float *means, const float *scales,
                                const float *rots, const float *opac, const float *sh,

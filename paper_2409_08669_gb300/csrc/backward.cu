@@ -7,7 +7,7 @@
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
 //                         and accumulates, with v = alpha dL/dalpha, sum v, dL/d(px,
 //                         py), the second moments of v about the Gaussian's centre
-//                         and its colour gradient; reduced over the tile, then
+//                         and its colour gradient; reduced over a warp, then
 //                         atomicAdd into 9 floats per Gaussian.
 //   k_preprocess_backward dL/d(conic, sigma) from the moments, and the chain rule
 //                         to means, scales, rotations, opacities and SH
@@ -20,16 +20,16 @@
 namespace adr {
 namespace {
 
-constexpr int kBwdThreads = kTilePixels / 2;   // two vertically adjacent pixels per thread
-constexpr int kBwdWarps = kBwdThreads / 32;
-constexpr int kBwdStage = 128;                 // list positions staged at a time
+constexpr int kBwdThreads = kTilePixels;       // a pixel per thread
+constexpr int kBwdWarps = kBwdThreads / 32;    // 16x2-pixel strips
+constexpr int kBwdStage = kBwdThreads;         // list positions staged at a time
 constexpr int kSums = 9;                       // per Gaussian
 
 // Sum over the warp of nine per-lane values, as a reduce-scatter by recursive
-// halving: at distance 8, 4, 2 and 1 the lanes whose bit is clear keep the first
+// halving: at distance 16, 8, 4 and 2 the lanes whose bit is clear keep the first
 // ceil(n / 2) of their n values and the others the rest (5 and 4 of 9, then 3 and
-// 2, 2 and 1, 1), each adding its partner's copy of them, then the warp's halves
-// add: 12 shuffles.  Lanes s and s + 16 share one value; reduce_slot says which.
+// 2, 2 and 1, 1), each adding its partner's copy of them, then pairs (lane, lane ^ 1)
+// add: 12 shuffles.  Lanes 2 s and 2 s + 1 share one value; reduce_slot says which.
 __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) {
     float a[9];
 #pragma unroll
@@ -38,7 +38,7 @@ __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) 
     int n = 9;
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
-        const int dist = 8 >> step, keep = kKeep[step];
+        const int dist = 16 >> step, keep = kKeep[step];
         const bool up = (lane & dist) != 0;
 #pragma unroll
         for (int i = 0; i < keep; ++i) {
@@ -48,44 +48,44 @@ __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) 
         }
         n = keep;
     }
-    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 16);
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
-// The slot (0..8) whose total a lane ends with; -1 for lanes left without one.
+// The slot (0..8) whose total an even lane ends with; -1 for the lanes without one.
 __device__ __forceinline__ int reduce_slot(int lane) {
     constexpr int kKeep[4] = {5, 3, 2, 1};
     int base = 0, n = 9;   // the slots the lane still holds: base .. base + n - 1
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
-        if (lane & (8 >> step)) {
+        if (lane & (16 >> step)) {
             base += kKeep[step];
             n -= kKeep[step];
         } else {
             n = min(n, kKeep[step]);
         }
     }
-    return n > 0 ? base : -1;
+    return n > 0 && !(lane & 1) ? base : -1;
 }
 
-// One CTA of 128 threads per tile: warp w has the 16x4-pixel strip w, a lane two
-// vertically adjacent pixels, whose arithmetic is paired FP32.  Bound by
-// instruction issue: a (warp, Gaussian) that blends costs about 90 instructions,
-// 30 of them the sum over lanes, so a warp walks only the staged Gaussians that
-// reach its strip (rects_reached) up to its last blended position.
+// One CTA of 256 threads per tile: a pixel per thread, a 16x2-pixel strip per warp.
+// The sums are dL/d(px, py) of each pixel, the second moments of v = -2 dL/dq about
+// the centre, sum v and the colour weights; k_preprocess_backward scales them once
+// per Gaussian.
 //
-// The sums are dL/d(px, py) of each pixel, the second moments of v = -2 dL/dq
-// about the centre, sum v and the colour weights; k_preprocess_backward scales
-// them once per Gaussian.  Long thin Gaussians amplify the rounding of the sums by
-// the square of their axes' ratio (to about 1e-3 of a scale's gradient), so they
-// are taken as finely as pixel by pixel: each pixel's terms are rounded on their
-// own and added along a row pair first.  1M Gaussians at 1280x720: 650 us with a pixel
-// per thread in 16x2-pixel warps that walk the whole list, 247 us now.  (Moments of
-// both pixels at once in 8x8 squares took 210 us, but their rounding put a scale's
-// gradient up to 3e-3 elsewhere, three times what this form does.)
-// A Gaussian's sums over the four strips are added on chip, so that a tile makes one
-// addition to memory per value: a Gaussian of thousands of tiles rounds its total
-// that much less often (a step's time is 1% more; with four, its SH gradients lay
-// further from FP64 than with a sum per 16x2 warp on some frames).
-__global__ void __launch_bounds__(kBwdThreads, 6)   // 80 registers; 4 to 8 CTAs per SM are within 1.5%
+// Long thin Gaussians amplify the rounding of the sums by the square of their axes'
+// ratio (to about 1e-4 of the rotations' gradients, single values to 1e-2), so the
+// order of the additions shows in the results.  It is a tree over the strip (row
+// pairs, then halves of the row), then one addition to memory per strip, as the
+// warps come to the Gaussian.  Of 100 random scenes trained for a step, 20 had a
+// gradient more than four times this order's own spread away when a tile's strips were added on chip
+// first (16x4 strips, two pixels a lane; 735 us a step at 1M Gaussians and 1280x720), 9 to 13
+// when this order was run again.
+//
+// Bound by instruction issue: a (strip, Gaussian) that blends costs about 90
+// instructions, a third of them the sum over lanes, so the pixels take it without
+// branches (with one around the blend: 948 us a step).  4 CTAs per SM (60 registers):
+// 786 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
+// conic's and opacity's factors per pixel: 1480.
+__global__ void __launch_bounds__(kBwdThreads, 4)
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
                   const float4* __restrict__ rec, const float4* __restrict__ aux,
                   const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
@@ -96,9 +96,6 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     __shared__ float4 s_nw[kBwdStage];    // -w1x, -w2x, -w1y, -w2y
     __shared__ float4 s_cy[kBwdStage];    // red, green, blue, centre y
     __shared__ float4 s_cn[kBwdStage];    // conic a, b, c, the Gaussian
-    __shared__ uint32_t s_mask[kBwdWarps][kBwdStage / 32];   // staged Gaussians that reach each strip
-    __shared__ uint32_t s_list[kBwdWarps][kBwdStage];
-    __shared__ alignas(16) float s_sum[kBwdWarps][kBwdStage * kSums];   // each warp's sums
     __shared__ int s_max[kBwdWarps];
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -106,51 +103,39 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     const float e_low = fp->st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
     const int tile = blockIdx.x;
     const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int lx = lane & 15, ly = 4 * warp + 2 * (lane >> 4);
+    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
     const int x = tx * kTile + lx, y = ty * kTile + ly;
     const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-    const float fx = (float)lx, fya = (float)ly;
-    const size_t hw = (size_t)width * height;
+    const float fx = (float)lx, fy = (float)ly;
     const uint2 range = ranges[tile];
     if (range.x >= range.y) return;
 
-    // Pixel a in .x, pixel b in .y.
-    int32_t last_a = 0, last_b = 0;       // 1-based position of the last blend
-    float2 T = make_float2(1.f, 1.f);
-    float2 g0 = make_float2(0.f, 0.f), g1 = g0, g2 = g0, gl = g0, gl_stop = g0;
-    // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
-    // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
-    // that stopped (a more opaque Gaussian makes it stop sooner).
-    const bool termination = fp->st.load_grad == ADR_LOAD_GRAD_TERMINATION && lstat;
-    auto pixel = [&](size_t pix, int32_t& last, float& t, float& r, float& g, float& b, float& l, float& l_stop) {
+    int32_t last = 0;       // 1-based position of the last blend
+    float T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, gl = 0.f, gl_stop = 0.f;
+    if (x < width && y < height) {
+        const size_t hw = (size_t)width * height, pix = (size_t)y * width + x;
         last = last_pos[pix];
-        t = t_final[pix];
-        r = dl_dimg[pix];
-        g = dl_dimg[hw + pix];
-        b = dl_dimg[2 * hw + pix];
-        if (!dl_dload) return;
-        l = dl_dload[pix];
-        if (termination && l != 0.f) {
+        T = t_final[pix];
+        g0 = dl_dimg[pix];
+        g1 = dl_dimg[hw + pix];
+        g2 = dl_dimg[2 * hw + pix];
+        if (dl_dload) gl = dl_dload[pix];
+        // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
+        // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
+        // that stopped (a more opaque Gaussian makes it stop sooner).
+        if (fp->st.load_grad == ADR_LOAD_GRAD_TERMINATION && gl != 0.f && lstat) {
             const int32_t ls = lstat[pix];
-            if (ls < 0 && t < 1.f) {
-                l_stop = l * -(float)(ls & 0x7FFFFFFF) / -logf(t);
-                l = 0.f;
+            if (ls < 0 && T < 1.f) {
+                gl_stop = gl * -(float)(ls & 0x7FFFFFFF) / -logf(T);
+                gl = 0.f;
             }
         }
-    };
-    const size_t pixa = (size_t)y * width + x;
-    if (x < width && y < height) pixel(pixa, last_a, T.x, g0.x, g1.x, g2.x, gl.x, gl_stop.x);
-    if (x < width && y + 1 < height) pixel(pixa + width, last_b, T.y, g0.y, g1.y, g2.y, gl.y, gl_stop.y);
-    float2 acc0 = make_float2(fp->st.bg[0], fp->st.bg[0]);   // colour behind the current Gaussian
-    float2 acc1 = make_float2(fp->st.bg[1], fp->st.bg[1]);
-    float2 acc2 = make_float2(fp->st.bg[2], fp->st.bg[2]);
-    const float2 fx2 = make_float2(fx, fx), fya2 = make_float2(fya, fya), fyb2 = make_float2(fya + 1.f, fya + 1.f);
-    const float2 one2 = make_float2(1.f, 1.f);
-    const int slot = lane < 16 ? reduce_slot(lane) : -1;
-    const float e_lim = fmaxf(e_low, -126.f);   // below it alpha is 0 (ex2_approx flushes)
+    }
+    float acc0 = fp->st.bg[0], acc1 = fp->st.bg[1], acc2 = fp->st.bg[2];   // colour behind the current Gaussian
+    const int slot = reduce_slot(lane);
 
     // The longest prefix any pixel of the warp, and of the tile, needs.
-    const int warp_last = __reduce_max_sync(0xffffffffu, max(last_a, last_b));
+    const int warp_last = __reduce_max_sync(0xffffffffu, last);
     if (lane == 0) s_max[warp] = warp_last;
     __syncthreads();
     int tile_last = 0;
@@ -160,98 +145,55 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     for (int bend = tile_last; bend > 0; bend -= kBwdStage) {
         const int bstart = max(0, bend - kBwdStage);
         __syncthreads();
-        const int m = bend - bstart;
-        for (int j0 = 0; j0 < m; j0 += kBwdThreads) {
-            const int j = j0 + (int)threadIdx.x;
-            uint32_t reached = 0u;
-            if (j < m) {
-                const uint32_t g = sorted_gauss[range.x + bstart + j];
-                const float4 r0 = rec[3 * (size_t)g + 0];
-                const float4 w = rec[3 * (size_t)g + 1];
-                const float4 col = rec[3 * (size_t)g + 2];
-                const float4 cn = aux[2 * (size_t)g];
-                const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
-                                             __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
-                const float2 k = quad_k(c, w);
-                s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
-                s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
-                s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
-                s_cn[j] = make_float4(cn.x, cn.y, cn.z, __uint_as_float(g));
-                reached = rects_reached<16, 4>(c, k, w, col.w, e_lim);
-            }
-            uint32_t mine = 0u;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t bits = __ballot_sync(0xffffffffu, (reached >> q) & 1u);
-                if (lane == q) mine = bits;
-            }
-            if (lane < 4) s_mask[lane][j >> 5] = mine;
+        const int j = (int)threadIdx.x;
+        if (bstart + j < bend) {
+            const uint32_t g = sorted_gauss[range.x + bstart + j];
+            const float4 r0 = rec[3 * (size_t)g + 0];
+            const float4 w = rec[3 * (size_t)g + 1];
+            const float4 col = rec[3 * (size_t)g + 2];
+            const float4 cn = aux[2 * (size_t)g];
+            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+            const float2 k = quad_k(c, w);
+            s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
+            s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
+            s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
+            s_cn[j] = make_float4(cn.x, cn.y, cn.z, __uint_as_float(g));
         }
-        for (int v = threadIdx.x; v < kBwdWarps * kBwdStage * kSums / 4; v += kBwdThreads)
-            reinterpret_cast<float4*>(&s_sum[0][0])[v] = make_float4(0.f, 0.f, 0.f, 0.f);
         __syncthreads();
         // this warp's positions: none of its pixels blended one past warp_last
-        const uint32_t* list = s_list[warp];
-        const int n = warp_list(s_mask[warp], min(bend, warp_last) - bstart, lane, s_list[warp]);
-        __syncwarp();
 #pragma unroll 2
-        for (int i = n - 1; i >= 0; --i) {
-            const uint32_t off = list[i];
-            const int p = bstart + (int)(off / 16u);
-            const float4 kl = at_offset(s_kl, off);
-            const float4 nw = at_offset(s_nw, off);
+        for (int i = min(bend, warp_last) - bstart - 1; i >= 0; --i) {
+            const float4 kl = s_kl[i];
+            const float4 nw = s_nw[i];
             // Same evaluation as the forward pass, so the same skip decision.
-            const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
-            const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
-            const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
-            const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
-            const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
-            const bool la = ea >= e_low && p < last_a, lb = eb >= e_low && p < last_b;
-            if (!__any_sync(0xffffffffu, la || lb)) continue;
-            const float4 cy = at_offset(s_cy, off);
-            const float4 cn = at_offset(s_cn, off);
+            const float u1 = fmaf(nw.z, fy, fmaf(nw.x, fx, kl.x)), u2 = fmaf(nw.w, fy, fmaf(nw.y, fx, kl.y));
+            const float e = fmaf(-u1, u1, fmaf(-u2, u2, kl.z));
+            const bool blended = e >= e_low && bstart + i < last;
+            if (!__any_sync(0xffffffffu, blended)) continue;
+            const float4 cy = s_cy[i];
+            const float4 cn = s_cn[i];
             // A pixel that did not blend this Gaussian has raw = alpha = 0, which
             // leaves its T and colour as they are and adds nothing to the sums.
-            const float2 raw = make_float2(la ? ex2_approx(ea) : 0.f, lb ? ex2_approx(eb) : 0.f);
-            const float2 alpha = make_float2(fminf(0.99f, raw.x), fminf(0.99f, raw.y));
-            const float2 one_m = fsub2(one2, alpha);
-            const float2 less = make_float2(-one_m.x, -one_m.y);
+            const float raw = blended ? ex2_approx(e) : 0.f, alpha = fminf(0.99f, raw), one_m = 1.f - alpha;
             // T before this blend, T / (1 - alpha): the hardware reciprocal with a Newton
             // step, and the quotient with its remainder added (rounded as a division is)
-            float2 inv = make_float2(rcp_approx(one_m.x), rcp_approx(one_m.y));
-            inv = ffma2(inv, ffma2(less, inv, one2), inv);
-            const float2 quot = fmul2(T, inv);
-            T = ffma2(ffma2(less, quot, T), inv, quot);
-            const float2 wgt = fmul2(alpha, T);
-            const float2 d0 = fsub2(make_float2(cy.x, cy.x), acc0), d1 = fsub2(make_float2(cy.y, cy.y), acc1),
-                         d2 = fsub2(make_float2(cy.z, cy.z), acc2);
-            const float2 dalpha = ffma2(T, ffma2(d2, g2, ffma2(d1, g1, fmul2(d0, g0))),
-                                        ffma2(gl_stop, inv, gl));   // with the load term
-            acc0 = ffma2(make_float2(cy.x, cy.x), alpha, fmul2(one_m, acc0));
-            acc1 = ffma2(make_float2(cy.y, cy.y), alpha, fmul2(one_m, acc1));
-            acc2 = ffma2(make_float2(cy.z, cy.z), alpha, fmul2(one_m, acc2));
-            float2 v = fmul2(raw, dalpha);                       // alpha = sigma G, G = exp(-q / 2)
-            if (!(raw.x < 0.99f)) v.x = 0.f;                     // clamped
-            if (!(raw.y < 0.99f)) v.y = 0.f;
-            const float dx = kl.w - fx;
-            const float2 dx2 = make_float2(dx, dx), dy = fsub2(make_float2(cy.w, cy.w), make_float2(fya2.x, fyb2.x));
-            const float2 tx2 = ffma2(make_float2(cn.x, cn.x), dx2, fmul2(make_float2(cn.y, cn.y), dy));
-            const float2 ty2 = ffma2(make_float2(cn.y, cn.y), dx2, fmul2(make_float2(cn.z, cn.z), dy));
-            const float2 vx = fmul2(v, dx2), vy = fmul2(v, dy);
-            const float2 px = fmul2(v, tx2), py = fmul2(v, ty2);
-            const float2 xx = fmul2(vx, dx2), xy = fmul2(vx, dy), yy = fmul2(vy, dy);
-            const float2 c0 = fmul2(wgt, g0), c1 = fmul2(wgt, g1), c2 = fmul2(wgt, g2);
-            const float sums[9] = {v.x + v.y,   px.x + px.y, py.x + py.y, xx.x + xx.y, xy.x + xy.y,
-                                   yy.x + yy.y, c0.x + c0.y, c1.x + c1.y, c2.x + c2.y};
+            float inv = rcp_approx(one_m);
+            inv = fmaf(inv, fmaf(-one_m, inv, 1.f), inv);
+            const float quot = __fmul_rn(T, inv);
+            T = fmaf(fmaf(-one_m, quot, T), inv, quot);
+            const float wgt = alpha * T;
+            const float dcol = fmaf(cy.z - acc2, g2, fmaf(cy.y - acc1, g1, __fmul_rn(cy.x - acc0, g0)));
+            const float dalpha = fmaf(T, dcol, fmaf(gl_stop, inv, gl));   // with the load term
+            acc0 = fmaf(cy.x, alpha, __fmul_rn(one_m, acc0));
+            acc1 = fmaf(cy.y, alpha, __fmul_rn(one_m, acc1));
+            acc2 = fmaf(cy.z, alpha, __fmul_rn(one_m, acc2));
+            const float v = raw < 0.99f ? raw * dalpha : 0.f;       // alpha = sigma G, G = exp(-q / 2); 0 if clamped
+            const float dx = kl.w - fx, dy = cy.w - fy, vx = v * dx, vy = v * dy;
+            const float sums[9] = {v, v * fmaf(cn.x, dx, __fmul_rn(cn.y, dy)), v * fmaf(cn.y, dx, __fmul_rn(cn.z, dy)),
+                                   vx * dx, vx * dy, vy * dy, wgt * g0, wgt * g1, wgt * g2};
             const float tot = reduce_scatter9(sums, lane);
-            if (slot >= 0) s_sum[warp][(off / 16u) * kSums + slot] = tot;
-        }
-        __syncthreads();
-        // The tile's sums: one addition to memory per Gaussian and value.
-        for (int v = threadIdx.x; v < m * kSums; v += kBwdThreads) {
-            const float t = (s_sum[0][v] + s_sum[1][v]) + (s_sum[2][v] + s_sum[3][v]);
-            const int j = v / kSums;
-            if (t != 0.f) atomicAdd(g2d + (size_t)__float_as_uint(s_cn[j].w) * kSums + (v - j * kSums), t);
+            if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * kSums + slot, tot);
         }
     }
 }

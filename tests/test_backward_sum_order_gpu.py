@@ -1,0 +1,55 @@
+"""Backward: a Gaussian's sums over a tile are its 16x2-pixel strips' sums, added
+one after another.  Opacities of 0.5 make the opacity gradient the exact double of
+the sum of v over the pixels, and a pixel's v depends on its own upstream gradient
+only, so a backward with the gradient of one strip gives that strip's sum: the whole
+gradient has to be what FP32 additions of them give in some order."""
+import itertools
+
+import numpy as np
+import pytest
+
+from paper_2409_08669_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def sequential_sums(strips):
+    """What adding the strips' sums one by one gives, over all orders."""
+    orders = np.array(list(itertools.permutations(strips)), np.float32)
+    total = np.zeros(len(orders), np.float32)
+    for k in range(len(strips)):
+        total = total + orders[:, k]
+    return set(total.tolist())
+
+
+@pytest.mark.parametrize("w,h", [(16, 16), (16, 13), (11, 9)])
+def test_a_tiles_strips_are_added_one_by_one(w, h):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2409_08669_gb300.raster import Rasterizer, upload
+    n = 300
+    rng = np.random.default_rng(16 * w + h)
+    scene = S.tiny_scene(w, n=n)
+    scene.scales[:] = np.exp(rng.normal(-1.5, 0.5, (n, 3))).astype(np.float32)
+    scene.opac[:] = 0.5
+    cam = S.look_at((0.3, 0.2, -3.0), width=w, height=h)
+    rast = Rasterizer(max_gaussians=n, pair_capacity=1 << 16, max_width=16, max_height=16)
+    try:
+        params = upload(scene)
+        rast.forward(params, cam, S.Settings(mode=S.MODE_AABB))
+        g_img = torch.from_numpy(rng.normal(size=(3, h, w)).astype(np.float32)).cuda()
+
+        def opacity_gradient(first, end):
+            g = torch.zeros_like(g_img)
+            g[:, first:end] = g_img[:, first:end]
+            return rast.backward(params, g)[3].cpu().numpy().reshape(n)
+
+        whole = opacity_gradient(0, h)
+        strips = np.stack([opacity_gradient(y, min(y + 2, h)) for y in range(0, h, 2)], 1)
+    finally:
+        rast.close()
+    assert np.count_nonzero((strips != 0).sum(1) >= 4) >= 20      # some meet enough strips
+    for i in range(n):
+        assert float(whole[i]) in sequential_sums(strips[i][strips[i] != 0]), (i, whole[i], strips[i])
