@@ -83,8 +83,8 @@ __device__ __forceinline__ int reduce_slot(int lane) {
 // Bound by instruction issue: a (strip, Gaussian) that blends costs about 90
 // instructions, a third of them the sum over lanes, so the pixels take it without
 // branches (with one around the blend: 948 us a step).  4 CTAs per SM (60 registers):
-// 786 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
-// conic's and opacity's factors per pixel: 1480.
+// 790 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
+// conic's and opacity's factors per pixel: 1040.
 __global__ void __launch_bounds__(kBwdThreads, 4)
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
                   const float4* __restrict__ rec, const float4* __restrict__ aux,
@@ -173,8 +173,9 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             if (!__any_sync(0xffffffffu, blended)) continue;
             const float4 cy = s_cy[i];
             const float4 cn = s_cn[i];
-            // A pixel that did not blend this Gaussian has raw = alpha = 0, which
-            // leaves its T and colour as they are and adds nothing to the sums.
+            // A pixel that did not blend this Gaussian has raw = alpha = 0, which leaves its
+            // T as it is; its colour and its terms are selected, as 0 times an infinite
+            // gradient or colour would not be 0.
             const float raw = blended ? ex2_approx(e) : 0.f, alpha = fminf(0.99f, raw), one_m = 1.f - alpha;
             // T before this blend, T / (1 - alpha): the hardware reciprocal with a Newton
             // step, and the quotient with its remainder added (rounded as a division is)
@@ -185,13 +186,13 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             const float wgt = alpha * T;
             const float dcol = fmaf(cy.z - acc2, g2, fmaf(cy.y - acc1, g1, __fmul_rn(cy.x - acc0, g0)));
             const float dalpha = fmaf(T, dcol, fmaf(gl_stop, inv, gl));   // with the load term
-            acc0 = fmaf(cy.x, alpha, __fmul_rn(one_m, acc0));
-            acc1 = fmaf(cy.y, alpha, __fmul_rn(one_m, acc1));
-            acc2 = fmaf(cy.z, alpha, __fmul_rn(one_m, acc2));
-            const float v = raw < 0.99f ? raw * dalpha : 0.f;       // alpha = sigma G, G = exp(-q / 2); 0 if clamped
+            acc0 = blended ? fmaf(cy.x, alpha, __fmul_rn(one_m, acc0)) : acc0;
+            acc1 = blended ? fmaf(cy.y, alpha, __fmul_rn(one_m, acc1)) : acc1;
+            acc2 = blended ? fmaf(cy.z, alpha, __fmul_rn(one_m, acc2)) : acc2;
+            const float v = blended && raw < 0.99f ? raw * dalpha : 0.f;       // alpha = sigma G, G = exp(-q / 2); 0 if clamped
             const float dx = kl.w - fx, dy = cy.w - fy, vx = v * dx, vy = v * dy;
             const float sums[9] = {v, v * fmaf(cn.x, dx, __fmul_rn(cn.y, dy)), v * fmaf(cn.y, dx, __fmul_rn(cn.z, dy)),
-                                   vx * dx, vx * dy, vy * dy, wgt * g0, wgt * g1, wgt * g2};
+                                   vx * dx, vx * dy, vy * dy, blended ? wgt * g0 : 0.f, blended ? wgt * g1 : 0.f, blended ? wgt * g2 : 0.f};
             const float tot = reduce_scatter9(sums, lane);
             if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * kSums + slot, tot);
         }

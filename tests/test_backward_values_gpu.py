@@ -1,0 +1,54 @@
+"""Backward: values at the ends of the range.  A pixel adds nothing to a Gaussian
+that it did not blend, whatever its upstream gradient."""
+import numpy as np
+import pytest
+
+from paper_2409_08669_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture
+def rast():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2409_08669_gb300.raster import Rasterizer
+    r = Rasterizer(max_gaussians=1024, pair_capacity=1 << 16, max_width=64, max_height=64)
+    yield r
+    r.close()
+
+
+def _scene(n, seed):
+    rng = np.random.default_rng(seed)
+    scene = S.tiny_scene(seed, n=n)
+    scene.scales[:] = np.exp(rng.normal(-2.0, 0.5, (n, 3))).astype(np.float32)
+    scene.opac[:] = rng.uniform(0.1, 0.5, n).astype(np.float32)
+    return scene
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+@pytest.mark.parametrize("which", ["image", "load"])
+def test_a_pixels_infinite_gradient_reaches_only_what_it_blended(rast, value, which):
+    from paper_2409_08669_gb300.raster import upload
+    n, w, h, y, x = 400, 21, 18, 9, 12
+    params = upload(_scene(n, 3))
+    rast.forward(params, S.look_at((0.3, 0.2, -3.0), width=w, height=h), S.Settings(mode=S.MODE_AABB))
+    rng = np.random.default_rng(4)
+    g_img = torch.from_numpy(rng.normal(size=(3, h, w)).astype(np.float32)).cuda()
+    g_load = torch.from_numpy((0.01 * rng.normal(size=(h, w))).astype(np.float32)).cuda()
+    at_pixel = torch.zeros_like(g_load)
+    at_pixel[y, x] = 1.0
+    alone = rast.backward(params, at_pixel.expand(3, h, w), at_pixel)
+    blended = (alone[3] != 0) | (alone[4].reshape(n, -1) != 0).any(1)
+    assert 3 <= int(blended.sum()) <= n // 2
+    (g_img[1] if which == "image" else g_load)[y, x] = 0.0
+    finite = rast.backward(params, g_img, g_load)
+    (g_img[1] if which == "image" else g_load)[y, x] = value
+    grads = rast.backward(params, g_img, g_load)
+    assert not torch.isfinite(grads[3][blended]).all()
+    for g, f in zip(grads, finite):
+        g, f = g.reshape(n, -1)[~blended], f.reshape(n, -1)[~blended]
+        assert torch.isfinite(g).all()
+        assert (g - f).abs().max() <= 1e-3 * f.abs().max()     # two orders of the same additions
