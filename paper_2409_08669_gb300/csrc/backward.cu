@@ -83,7 +83,7 @@ __device__ __forceinline__ int reduce_slot(int lane) {
 // Bound by instruction issue: a (strip, Gaussian) that blends costs about 90
 // instructions, a third of them the sum over lanes, so the pixels take it without
 // branches (with one around the blend: 948 us a step).  4 CTAs per SM (60 registers):
-// 790 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
+// 806 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
 // conic's and opacity's factors per pixel: 1040.
 __global__ void __launch_bounds__(kBwdThreads, 4)
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
@@ -133,6 +133,7 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     }
     float acc0 = fp->st.bg[0], acc1 = fp->st.bg[1], acc2 = fp->st.bg[2];   // colour behind the current Gaussian
     const int slot = reduce_slot(lane);
+    const bool termination = __any_sync(0xffffffffu, gl_stop != 0.f);
 
     // The longest prefix any pixel of the warp, and of the tile, needs.
     const int warp_last = __reduce_max_sync(0xffffffffu, last);
@@ -177,15 +178,12 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
             // T as it is; its colour and its terms are selected, as 0 times an infinite
             // gradient or colour would not be 0.
             const float raw = blended ? ex2_approx(e) : 0.f, alpha = fminf(0.99f, raw), one_m = 1.f - alpha;
-            // T before this blend, T / (1 - alpha): the hardware reciprocal with a Newton
-            // step, and the quotient with its remainder added (rounded as a division is)
-            float inv = rcp_approx(one_m);
-            inv = fmaf(inv, fmaf(-one_m, inv, 1.f), inv);
-            const float quot = __fmul_rn(T, inv);
-            T = fmaf(fmaf(-one_m, quot, T), inv, quot);
+            T = __fdiv_rn(T, one_m);   // before this blend
             const float wgt = alpha * T;
+            float term = gl;   // the load's; dividing a zero is the division's slow path (1M: 950 us a step)
+            if (termination) term += __fdiv_rn(gl_stop, one_m);
             const float dcol = fmaf(cy.z - acc2, g2, fmaf(cy.y - acc1, g1, __fmul_rn(cy.x - acc0, g0)));
-            const float dalpha = fmaf(T, dcol, fmaf(gl_stop, inv, gl));   // with the load term
+            const float dalpha = fmaf(T, dcol, term);
             acc0 = blended ? fmaf(cy.x, alpha, __fmul_rn(one_m, acc0)) : acc0;
             acc1 = blended ? fmaf(cy.y, alpha, __fmul_rn(one_m, acc1)) : acc1;
             acc2 = blended ? fmaf(cy.z, alpha, __fmul_rn(one_m, acc2)) : acc2;

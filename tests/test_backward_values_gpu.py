@@ -52,3 +52,27 @@ def test_a_pixels_infinite_gradient_reaches_only_what_it_blended(rast, value, wh
         g, f = g.reshape(n, -1)[~blended], f.reshape(n, -1)[~blended]
         assert torch.isfinite(g).all()
         assert (g - f).abs().max() <= 1e-3 * f.abs().max()     # two orders of the same additions
+
+
+def test_the_load_gradients_quotient_is_a_division(rast):
+    """One pixel that blends one Gaussian and stops before the next, in the termination reading and without an image
+    gradient: dL/dsigma = alpha (dl / (1 - alpha)) / sigma, each step rounded to FP32.  Of alpha >= 1/2, 1 - alpha = T_final
+    is exact, so alpha is known."""
+    from paper_2409_08669_gb300.raster import upload
+    cam = S.look_at((0.0, 0.0, -3.0), width=1, height=1)
+    st = S.Settings(mode=S.MODE_AABB, t_min=0.4, load_grad=S.LOAD_GRAD_TERMINATION)
+    scene = S.tiny_scene(0, n=2)
+    scene.means[:] = [[0.0, 0.0, 0.0], [0.0, 0.0, 1.0]]
+    scene.scales[:] = 1.0
+    zero = torch.zeros(3, 1, 1, device="cuda")
+    rng = np.random.default_rng(0)
+    for sigma in rng.uniform(0.53, 0.59, 100).astype(np.float32):
+        scene.opac[:] = sigma
+        params = upload(scene)
+        t_final, load = rast.forward(params, cam, st)[1:]
+        assert int(load) == 1 and 0.4 <= float(t_final) < 0.5
+        g_load = torch.full((1, 1), float(rng.uniform(0.5, 2.0)), device="cuda")
+        got = rast.backward(params, zero, g_load)[3].cpu().numpy().reshape(2)
+        T, stop = t_final.cpu().numpy()[0, 0], ((g_load * -1.0) / -torch.log(t_final)).cpu().numpy()[0, 0]
+        alpha = np.float32(1.0) - T
+        assert got[0] == np.float32(alpha * np.float32(stop / T)) / sigma and got[1] == 0.0, (sigma, got)
