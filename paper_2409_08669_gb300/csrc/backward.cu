@@ -275,7 +275,7 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
         const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
         const float gpx = -G[1], gpy = -G[2];
         const float gca = -0.5f * G[3], gcb = -G[4], gcc = -0.5f * G[5];
-        go = G[0] / cn.w;
+        go = G[0] != 0.f ? G[0] / cn.w : 0.f;   // sigma may be 0 in the plain mode: it blends nothing
         const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
         // --- colour: rgb = max(0, sum_k sh_k Y_k(d) + 0.5), d = (X0 - cam) / |X0 - cam|
         float vx = mx - cam.cam_pos[0], vy = my - cam.cam_pos[1], vz = mz - cam.cam_pos[2];

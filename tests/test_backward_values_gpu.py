@@ -76,3 +76,20 @@ def test_the_load_gradients_quotient_is_a_division(rast):
         T, stop = t_final.cpu().numpy()[0, 0], ((g_load * -1.0) / -torch.log(t_final)).cpu().numpy()[0, 0]
         alpha = np.float32(1.0) - T
         assert got[0] == np.float32(alpha * np.float32(stop / T)) / sigma and got[1] == 0.0, (sigma, got)
+
+
+@pytest.mark.parametrize("mode", [S.MODE_PLAIN, S.MODE_AABB])
+def test_an_opacity_of_zero_has_no_gradient(rast, mode):
+    from paper_2409_08669_gb300.raster import upload
+    n, w, h = 400, 30, 22
+    scene = _scene(n, 5)
+    scene.opac[::7] = 0.0
+    scene.opac[3::7] = 1e-30
+    params = upload(scene)
+    rast.forward(params, S.look_at((0.3, 0.2, -3.0), width=w, height=h), S.Settings(mode=mode))
+    grads = rast.backward(params, torch.ones(3, h, w, device="cuda"), torch.ones(h, w, device="cuda"))
+    assert all(torch.isfinite(g).all() for g in grads)
+    assert bool((grads[3] != 0).any())
+    for g in grads:
+        g = g.reshape(n, -1)
+        assert not g[::7].any() and not g[3::7].any()
