@@ -161,7 +161,7 @@ struct adr_ctx {
     bool last_backward = false;      // the last frame had a backward
     bool slices_pay = true;
     uint32_t frames = 0;
-    uint32_t radix_probe_in = kRadixProbe;   // see next_depth_sort
+    DepthSortChoice depth_sort;
     int32_t slice_mode = ADR_SLICES_ADAPTIVE;
     int32_t host_reads = ADR_HOST_READ_MAPPED;   // adr_render_host: read mapped host buffers in place
     bool defer_colors = false;   // the next adr_preprocess leaves the SH colours to adr_render
@@ -408,9 +408,9 @@ adr_status adr_preprocess(adr_ctx* c, const float* means, const float* scales, c
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     fill_frame_state(c->fs, n, cam, st);
-    // The host word is written by the device and read without waiting.
-    c->fs.depth_sort = next_depth_sort(*static_cast<volatile uint32_t*>(c->host_words + kHostLargestBin),
-                                       c->radix_probe_in);
+    // The host word is written by the device (frames with a histogram) and read without waiting.
+    c->depth_sort.largest_bin = *static_cast<volatile uint32_t*>(c->host_words + kHostLargestBin);
+    c->fs.depth_sort = c->depth_sort.next();
     enqueue_preprocess(c->ws, c->fs, c->epoch, means, scales, rots, opac, sh, strm, true,
                        c->defer_colors);
     if ((s = check_launch("adr_preprocess")) != ADR_OK) return s;

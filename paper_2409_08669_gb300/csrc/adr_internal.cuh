@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "adr.h"
+#include "depth_sort.h"
 #include "status_bits.h"   // device-side error word bits and their adr_status
 
 namespace adr {
@@ -247,32 +248,12 @@ __device__ __forceinline__ uint32_t bin_of(uint32_t key, uint32_t base, const Bi
 }
 // Gaussians of a window of the window sort, not counting what its last bin adds.
 constexpr int kWindow = 1024;
-constexpr uint32_t kRadixBin = 8192;
-constexpr uint32_t kRadixProbe = 64;   // a histogram every 64th radix frame
 
 // hist layout: 4 x 256 per-digit totals of the depth passes.
 constexpr int kHistWords = kMaxPasses * kRadix;
 
 // Contents of the column-run buffer: every Gaussian's runs, or a slice's.
 enum RunsHeld : int { kRunsAll = 0, kRunsSlice0 = 1, kRunsSlice1 = 2 };
-
-// How a frame orders its Gaussians by depth: by bins (bins.cu), or by the
-// radix sort (sort.cu), with or without a depth histogram beside it.  Both give
-// the same order; the radix sort is the faster one when one bin holds more than
-// kRadixBin Gaussians (very many at nearly one depth: the bin is sorted by one
-// CTA and counted by atomics on one address).  A caller learns the last frame's
-// largest bin and picks: next_depth_sort.
-enum DepthSort : int { kSortBins = 0, kSortRadix = 1, kSortRadixProbe = 2 };
-// `probe_in`: radix frames until the next one with a histogram.
-inline DepthSort next_depth_sort(uint32_t largest_bin, uint32_t& probe_in) {
-    if (largest_bin <= kRadixBin) {
-        probe_in = kRadixProbe;
-        return kSortBins;
-    }
-    if (--probe_in > 0) return kSortRadix;
-    probe_in = kRadixProbe;
-    return kSortRadixProbe;
-}
 
 // Gaussians whose depth order a frame has built so far (a mask).  A sliced frame
 // of the binned order needs slice 0's only.

@@ -76,7 +76,7 @@ struct DeviceState {
     unsigned char* base = nullptr;   // device address of g_na_scratch on this device
     Workspace ws;                    // buffers inside the array
     std::atomic<uint32_t> epoch{0};
-    uint32_t largest_bin = 0, radix_probe_in = kRadixProbe;   // see next_depth_sort
+    DepthSortChoice depth_sort;
 };
 
 std::mutex g_setup_mutex;
@@ -181,7 +181,7 @@ extern "C" adr_status adr_render_frame_noalloc(const float* means, const float* 
     cudaStream_t strm = static_cast<cudaStream_t>(stream);
     FrameState fs;
     fill_frame_state(fs, n, cam, st);
-    fs.depth_sort = next_depth_sort(ds->largest_bin, ds->radix_probe_in);
+    fs.depth_sort = ds->depth_sort.next();
     enqueue_preprocess(ws, fs, ds->epoch, means, scales, rots, opac, sh, strm);
     enqueue_sort(ws, fs, ds->epoch, strm);
     enqueue_render(ws, fs, img, t_final, load, strm);
@@ -197,7 +197,7 @@ extern "C" adr_status adr_render_frame_noalloc(const float* means, const float* 
     // A wait that gave up skips the frame and reads its pair count as
     // saturated, so it is reported before the capacity check.
     const StatusReport r = status_from_bits(words[kCntSlots], (int64_t)words[kCntPairs], kNaMaxPairs);
-    if (n > 0 && fs.depth_sort != kSortRadix) ds->largest_bin = words[kCntLargestBin];
+    if (n > 0) ds->depth_sort.completed(fs.depth_sort, words[kCntLargestBin]);
     if (r.status == ADR_ERR_CAPACITY)
         return report_error(ADR_ERR_CAPACITY,
                             "adr_render_frame_noalloc: more than 1048576 Gaussian-tile pairs "

@@ -48,8 +48,7 @@ struct Scene {
     int64_t n;
     SetDev st;
     double pairs_per_pixel = -1.0;   // learned; < 0 = unknown
-    uint32_t largest_bin = 0;        // of the last completed frame with a depth histogram
-    uint32_t radix_probe_in = kRadixProbe;   // see next_depth_sort
+    DepthSortChoice depth_sort;
 };
 
 enum ReqState { kQueued, kRunning, kDone };
@@ -180,7 +179,7 @@ adr_status run_batch(adr_server* s, Group& g) {
     Scene& sc = s->scenes[g.reqs[0]->scene];
     const int k = (int)g.reqs.size();
     cudaStream_t strm = g.stream;
-    const DepthSort depth_sort = next_depth_sort(sc.largest_bin, sc.radix_probe_in);
+    const DepthSort depth_sort = sc.depth_sort.next();
     for (int b = 0; b < k; ++b) {
         Slot& sl = *g.slots[b];
         fill_frame_state(sl.fs, sc.n, g.reqs[b]->cam, sc.st);
@@ -234,8 +233,8 @@ adr_status run_batch(adr_server* s, Group& g) {
 
 #undef SERVE_CUDA
 
-void finish_request(adr_server* s, Request* r, const uint32_t* host_words, cudaError_t q) {
-    const uint32_t bits = host_words[0], pairs = host_words[1];
+void finish_request(adr_server* s, Request* r, const Slot& sl, cudaError_t q) {
+    const uint32_t bits = sl.host_words[0], pairs = sl.host_words[1];
     r->t_done = now_ms();
     if (q != cudaSuccess) {
         r->result = ADR_ERR_CUDA;
@@ -247,7 +246,7 @@ void finish_request(adr_server* s, Request* r, const uint32_t* host_words, cudaE
         if (rep.status == ADR_ERR_CUDA) snprintf(s->error, sizeof(s->error), "%s", rep.message);
     }
     Scene& sc = s->scenes[r->scene];
-    if (q == cudaSuccess) sc.largest_bin = host_words[2];
+    if (q == cudaSuccess) sc.depth_sort.completed(sl.fs.depth_sort, sl.host_words[2]);
     if (q == cudaSuccess && !(bits & kErrLookback)) {   // a skipped frame's pair count is not a measurement
         const double ppp = (double)pairs / ((double)r->cam.width * r->cam.height);
         sc.pairs_per_pixel = sc.pairs_per_pixel < 0 ? ppp
@@ -272,7 +271,7 @@ void scheduler(adr_server* s) {
             const cudaError_t q = cudaEventQuery(g->done);
             if (q == cudaErrorNotReady) continue;
             for (size_t b = 0; b < g->reqs.size(); ++b)
-                finish_request(s, g->reqs[b], g->slots[b]->host_words, q);
+                finish_request(s, g->reqs[b], *g->slots[b], q);
             g->reqs.clear();
             progressed = true;
         }
