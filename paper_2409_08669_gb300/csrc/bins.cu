@@ -451,23 +451,29 @@ __device__ const uint2* sort_large(WindowShared& sm, uint4* recs, uint32_t m) {
     return src;
 }
 
-// The parts of k_window_sort for a window that does not fit on chip: its order,
-// boxes and run total, and its run offsets.
-__device__ __noinline__ void order_large(WindowShared& sm, uint4* recs, uint32_t m, const uint32_t* gbox,
-                                         uint32_t* order, uint32_t* sorted_box) {
-    const uint2* sorted = sort_large(sm, recs, m);
+// The parts of k_window_sort for a window that does not fit on chip: its run total
+// (of the unsorted records: the windows behind it wait for this, not for the sort),
+// its order and boxes, and its run offsets.
+__device__ __noinline__ void total_large(WindowShared& sm, const uint4* recs, uint32_t m) {
     if (threadIdx.x == 0) sm.sum = 0ull;
     __syncthreads();
     unsigned long long runs = 0;
-    for (uint32_t s = threadIdx.x; s < m; s += kWinThreads) {
-        const uint32_t i = sorted[s].y, box = gbox[i];
-        order[s] = i;
-        sorted_box[s] = box;
-        runs += box_runs(box);
-    }
+#pragma unroll 4
+    for (uint32_t s = threadIdx.x; s < m; s += kWinThreads) runs += box_runs(recs[s].z);
     atomicAdd(&sm.sum, runs);
     __syncthreads();
     if (threadIdx.x == 0) sm.total = (uint32_t)min(sm.sum, (unsigned long long)kSat);
+}
+
+__device__ __noinline__ void order_large(WindowShared& sm, uint4* recs, uint32_t m, const uint32_t* gbox,
+                                         uint32_t* order, uint32_t* sorted_box) {
+    const uint2* sorted = sort_large(sm, recs, m);
+    for (uint32_t s = threadIdx.x; s < m; s += kWinThreads) {
+        const uint32_t i = sorted[s].y;
+        order[s] = i;
+        sorted_box[s] = gbox[i];
+    }
+    __syncthreads();   // offsets_large reads the boxes
 }
 
 __device__ __noinline__ void offsets_large(WindowShared& sm, uint32_t lo, uint32_t m, const uint32_t* sorted_box,
@@ -526,7 +532,7 @@ k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* 
             o4[1] = make_uint4(before + off[4], before + off[5], before + off[6], before + off[7]);
             if (tid == 0) sm.total = total;
         } else {
-            order_large(sm, recs + lo, m, gbox, order + lo, sorted_box + lo);
+            total_large(sm, recs + lo, m);
         }
         __syncthreads();
         if (warp == 0) {
@@ -555,6 +561,7 @@ k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* 
                 mark_chunks(run, box_runs(sm.u.out.box[s]), lo + s, capacity, chunk_first);
             }
         } else {
+            order_large(sm, recs + lo, m, gbox, order + lo, sorted_box + lo);
             offsets_large(sm, lo, m, sorted_box, sm.prefix, capacity, offsets, chunk_first);
         }
         __syncthreads();   // the window is no longer read

@@ -1,0 +1,57 @@
+"""The depth order of scenes at nearly one depth, after frames of ordinary ones (the
+choice of the sort goes by earlier frames, so this frame's bins hold them all)."""
+import numpy as np
+import pytest
+
+from paper_2409_08669_gb300 import scenes as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _scene(depth, seed=1):
+    n = len(depth)
+    scene = S.tiny_scene(seed, n=n)
+    scene.means[:] = np.stack([np.zeros(n), np.zeros(n), depth], axis=1).astype(np.float32)
+    scene.scales[:] = (0.05 * np.asarray(depth)[:, None]).astype(np.float32)     # a few pixels at any depth
+    scene.opac[:] = 0.5
+    return scene
+
+
+def _frames(n):
+    """An ordinary scene's parameters and depths of n Gaussians, and the camera that sees their order in one tile."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    cam = S.look_at((0, 0, 0), target=(0, 0, 1), width=16, height=16, near=1e-3)
+    return _scene(np.random.default_rng(n).uniform(0.5, 8.0, n)), cam
+
+
+@pytest.fixture
+def expiry():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2409_08669_gb300 import _lib
+    yield _lib.adr_test_lookback_expiry
+    _lib.adr_test_lookback_expiry(-1)
+
+
+def test_windows_do_not_wait_for_the_sort_of_a_large_one(expiry):
+    """300k Gaussians in one bin: its sort takes a few ms, its run total a few percent of that, and the windows behind it
+    wait for the total only (1500 polls are under 1.5 ms; no chunk is withheld)."""
+    from paper_2409_08669_gb300.raster import Rasterizer, upload
+    n = 300_000
+    ordinary, cam = _frames(n)
+    flat = _scene(np.full(n, 3.0))
+    st = S.Settings(t_min=0.0)
+    rast = Rasterizer(max_gaussians=n, pair_capacity=n, max_width=16, max_height=16)
+    try:
+        for _ in range(2):
+            rast.forward(upload(ordinary), cam, st)
+            assert rast.sync_status() == 0
+        expiry(1 << 20, 1500)
+        rast.forward(upload(flat), cam, st)
+        assert rast.sync_status() == 0
+        assert np.array_equal(rast.read_pairs()[1], np.arange(n))
+    finally:
+        rast.close()
