@@ -40,6 +40,9 @@ constexpr int kLargeItems = 4;           // per thread and round of the large wi
 constexpr int kSubBits = 12;
 constexpr int kSub = 1 << kSubBits;      // sub-bins of a window's key range
 constexpr int kWinWarps = kWinThreads / 32;
+// Most members of a sub-bin that are placed by comparing each with all: 8 a thread at 20 ns each are 20 us,
+// what the radix sort of a window takes (2000 Gaussians at one depth, whole frame: 438 us -> 81).
+constexpr uint32_t kCrowded = 128;
 
 // ---------------------------------------------------------------------------
 // Bin starts and window starts.  Warp w of CTA r holds the 128 kQuads bins from
@@ -265,8 +268,9 @@ __device__ __forceinline__ uint32_t win_scan(uint32_t v, uint32_t* s_w, uint32_t
 // Window [lo, lo + m), m <= kWinCap, into sm.u.out in depth order.  Its key
 // range is cut into at most kSub sub-bins, filled with shared-memory atomics; a
 // Gaussian's place is its sub-bin's start plus the members before it (a window
-// has about kSub / 4 Gaussians, so most are alone in their sub-bin).
-__device__ __forceinline__ void sort_on_chip(WindowShared& sm, const uint4* __restrict__ recs, uint32_t lo,
+// has about kSub / 4 Gaussians, so most are alone in their sub-bin).  False, and
+// nothing done, if a sub-bin has more than kCrowded members (many equal depths).
+__device__ __forceinline__ bool sort_on_chip(WindowShared& sm, const uint4* __restrict__ recs, uint32_t lo,
                                              int m) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint4 rec[kWinItems];   // key, index, box, then the place
@@ -308,12 +312,17 @@ __device__ __forceinline__ void sort_on_chip(WindowShared& sm, const uint4* __re
         }
     }
     __syncthreads();
+    bool crowded;
     {
         uint4 a = c4[0], b = c4[1];
         uint32_t* v[8] = {&a.x, &a.y, &a.z, &a.w, &b.x, &b.y, &b.z, &b.w};
-        uint32_t sum = 0;
+        uint32_t sum = 0, most = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) sum += (*v[j] & 0xFFFFu) + (*v[j] >> 16);
+        for (int j = 0; j < 8; ++j) {
+            sum += (*v[j] & 0xFFFFu) + (*v[j] >> 16);
+            most = max(most, max(*v[j] & 0xFFFFu, *v[j] >> 16));
+        }
+        crowded = most > kCrowded;
         uint32_t total;
         uint32_t run = win_scan(sum, sm.w0, total);
 #pragma unroll
@@ -326,7 +335,7 @@ __device__ __forceinline__ void sort_on_chip(WindowShared& sm, const uint4* __re
         c4[1] = b;
         if (tid == 0) sm.c.pair[kSub / 2] = (uint32_t)m;
     }
-    __syncthreads();
+    if (__syncthreads_or(crowded)) return false;
     const uint16_t* start = reinterpret_cast<const uint16_t*>(sm.c.pair);
 #pragma unroll
     for (int q = 0; q < kWinItems; ++q) {
@@ -360,10 +369,11 @@ __device__ __forceinline__ void sort_on_chip(WindowShared& sm, const uint4* __re
         }
     }
     __syncthreads();
+    return true;
 }
 
 // A window of more than kWinCap Gaussians (one bin that large: very many
-// Gaussians at nearly one depth): a least-significant-digit radix sort by
+// Gaussians at nearly one depth) or a crowded one: a least-significant-digit radix sort by
 // (key, index) of the CTA alone, skipping the digits that all its Gaussians
 // share.  The window's 16-byte records make room for two buffers of (key, index).
 // Returns the one holding the result.
@@ -451,7 +461,7 @@ __device__ const uint2* sort_large(WindowShared& sm, uint4* recs, uint32_t m) {
     return src;
 }
 
-// The parts of k_window_sort for a window that does not fit on chip: its run total
+// The parts of k_window_sort for a window that is not sorted on chip: its run total
 // (of the unsorted records: the windows behind it wait for this, not for the sort),
 // its order and boxes, and its run offsets.
 __device__ __noinline__ void total_large(WindowShared& sm, const uint4* recs, uint32_t m) {
@@ -511,9 +521,8 @@ k_window_sort(uint4* recs, const uint32_t* __restrict__ win_lo, const uint32_t* 
         const uint32_t w = sm.ticket;
         if (w >= windows) return;
         const uint32_t lo = min(win_lo[w], V), hi = min(max(win_lo[w + 1], lo), V), m = hi - lo;
-        const bool on_chip = m <= (uint32_t)kWinCap;
+        const bool on_chip = m <= (uint32_t)kWinCap && sort_on_chip(sm, recs, lo, (int)m);
         if (on_chip) {
-            sort_on_chip(sm, recs, lo, (int)m);
             // Thread t's eight consecutive Gaussians: their run offsets from the
             // window's first run.
             uint32_t runs = 0, off[kWinItems];

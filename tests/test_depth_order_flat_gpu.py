@@ -55,3 +55,42 @@ def test_windows_do_not_wait_for_the_sort_of_a_large_one(expiry):
         assert np.array_equal(rast.read_pairs()[1], np.arange(n))
     finally:
         rast.close()
+
+
+def _order_is_right(rast, params, depth, cam, st):
+    rast.forward(params, cam, st)
+    vals = rast.read_pairs()[1].astype(np.int64)
+    assert rast.sync_status() == 0
+    return np.array_equal(vals, np.lexsort((np.arange(len(depth)), depth.astype(np.float32).view(np.uint32))))
+
+
+@pytest.mark.parametrize("n,equal", [(2000, 2000), (1025, 130), (1500, 127), (2040, 1000)])
+def test_equal_depths_in_a_window(n, equal):
+    """Windows that fit on chip, `equal` of whose Gaussians have one depth (the others a few octaves about it): ordered by
+    index, and in no more than three times an ordinary frame's time (comparing each with all took 3.5 times at 2000)."""
+    from paper_2409_08669_gb300.raster import Rasterizer, upload
+    ordinary, cam = _frames(n)
+    depth = np.random.default_rng(equal).uniform(0.5, 8.0, n)
+    depth[np.random.default_rng(n).permutation(n)[:equal]] = 3.0
+    st = S.Settings(t_min=0.0)
+    rast = Rasterizer(max_gaussians=n, pair_capacity=1 << 16, max_width=16, max_height=16)
+    try:
+        same, spread = upload(_scene(depth)), upload(ordinary)
+        us = {}
+        for name, params in (("spread", spread), ("same", same)):
+            for _ in range(5):
+                rast.forward(params, cam, st)
+            best = []
+            for _ in range(5):
+                e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                e[0].record()
+                for _ in range(10):
+                    rast.forward(params, cam, st)
+                e[1].record()
+                torch.cuda.synchronize()
+                best.append(e[0].elapsed_time(e[1]) * 100)
+            us[name] = min(best)
+        assert _order_is_right(rast, same, depth, cam, st)
+        assert us["same"] <= 3 * us["spread"], us
+    finally:
+        rast.close()
