@@ -254,7 +254,7 @@ adr_status alloc_workspace(Workspace& w, int64_t max_gaussians, int64_t pair_cap
     ALLOC(w.offsets, N * sizeof(uint32_t));
     ALLOC(w.gbox, N * sizeof(uint32_t));
     ALLOC(w.sorted_box, N * sizeof(uint32_t));
-    ALLOC(w.sortbuf, N * sizeof(uint4));
+    ALLOC(w.sortbuf, sortbuf_quads(max_gaussians) * sizeof(uint4));
     ALLOC(w.order, N * sizeof(uint32_t));
     ALLOC(w.rank, N * sizeof(uint32_t));
     ALLOC(w.win_lo, (N / kWindow + 2) * sizeof(uint32_t));

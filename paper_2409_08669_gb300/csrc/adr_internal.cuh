@@ -169,8 +169,8 @@ struct Workspace {
     uint32_t* offsets = nullptr;           // [max_n]
     uint32_t* gbox = nullptr;              // [max_n] packed tile rectangle per Gaussian (all ones: none)
     uint32_t* sorted_box = nullptr;        // [max_n] the same per depth-order position
-    uint4* sortbuf = nullptr;              // [max_n] (key, index, box) records of the window sort; the
-                                           // radix sort's two buffers of max_n keys and max_n values
+    uint4* sortbuf = nullptr;              // [sortbuf_quads(max_n)] (key, index, box) records of the window
+                                           // sort; the radix sort's two buffers of keys and values
     uint32_t* order = nullptr;             // [max_n] Gaussians by depth
     uint32_t* win_lo = nullptr;            // [max_n / kWindow + 2] first position of each window
     uint2* pruns = nullptr;                // [capacity] column runs grouped by tile column
@@ -218,6 +218,10 @@ struct Workspace {
     int32_t* tile_fbase = nullptr;         // [max_tiles]
     uint32_t* sat = nullptr;               // [(tiles_x + 1) * (tiles_y + 1)] at the largest image
 };
+
+// The sort buffer in 16-byte records: of n, or four arrays of n words that each
+// start on 16 bytes.
+constexpr size_t sortbuf_quads(int64_t n) { return ((size_t)n + 3) & ~(size_t)3; }
 
 // Words that start a frame at zero, one block: counters, the counters of the
 // two depth slices, the tile passes' totals, Preprocess's sums, then the depth

@@ -46,7 +46,7 @@ constexpr size_t kOffOffsets = align256(kOffDepth + kNaMaxGaussians * 4);
 constexpr size_t kOffGBox = align256(kOffOffsets + kNaMaxGaussians * 4);
 constexpr size_t kOffSortedBox = align256(kOffGBox + kNaMaxGaussians * 4);
 constexpr size_t kOffSortBuf = align256(kOffSortedBox + kNaMaxGaussians * 4);
-constexpr size_t kOffOrder = align256(kOffSortBuf + kNaMaxGaussians * 16);
+constexpr size_t kOffOrder = align256(kOffSortBuf + sortbuf_quads(kNaMaxGaussians) * 16);
 constexpr size_t kOffRank = align256(kOffOrder + kNaMaxGaussians * 4);
 constexpr size_t kOffWinLo = align256(kOffRank + kNaMaxGaussians * 4);
 constexpr size_t kOffPRuns = align256(kOffWinLo + (kNaMaxGaussians / kWindow + 2) * 4);

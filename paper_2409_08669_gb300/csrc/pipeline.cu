@@ -139,8 +139,9 @@ static void preprocess_tail(const Workspace& ws, FrameState& fs, cudaStream_t st
     const uint32_t* kin = ws.depth_key;
     const uint32_t* vin = nullptr;
     for (int p = 0; p < kMaxPasses; ++p) {
-        uint32_t* keys = reinterpret_cast<uint32_t*>(ws.sortbuf) + (size_t)(p & 1) * 2 * ws.max_n;
-        uint32_t* vals = p + 1 == kMaxPasses ? ws.order : keys + ws.max_n;
+        const size_t quarter = sortbuf_quads(ws.max_n);   // words: the passes read 16 bytes at a time
+        uint32_t* keys = reinterpret_cast<uint32_t*>(ws.sortbuf) + (size_t)(p & 1) * 2 * quarter;
+        uint32_t* vals = p + 1 == kMaxPasses ? ws.order : keys + quarter;
         TIMED(ws, kKDepthPass, stream,
               launch_depth_pass(kin, vin, keys, vals, n, ws.counters + kCntDepthKept, p == 0, 8 * p, ws.tcounts,
                                 ws.hist + p * kRadix, p + 1 == kMaxPasses ? ws.gbox : nullptr,

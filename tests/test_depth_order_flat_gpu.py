@@ -94,3 +94,19 @@ def test_equal_depths_in_a_window(n, equal):
         assert us["same"] <= 3 * us["spread"], us
     finally:
         rast.close()
+
+
+@pytest.mark.parametrize("n", [20_001, 20_002, 20_003, 20_004])
+def test_radix_frames_of_odd_sizes(n):
+    """The radix passes' buffers in a workspace of any number of Gaussians (they are read 16 bytes at a time)."""
+    from paper_2409_08669_gb300.raster import Rasterizer, upload
+    _, cam = _frames(n)
+    depth = np.full(n, 3.0)
+    depth[::5] = np.random.default_rng(n).uniform(0.5, 8.0, len(depth[::5]))
+    rast = Rasterizer(max_gaussians=n, pair_capacity=n, max_width=16, max_height=16)
+    try:
+        params = upload(_scene(depth))
+        for _ in range(3):
+            assert _order_is_right(rast, params, depth, cam, S.Settings(t_min=0.0))
+    finally:
+        rast.close()
