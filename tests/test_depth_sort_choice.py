@@ -51,3 +51,10 @@ def test_a_flat_scene_keeps_the_radix_sort_beside_an_ordinary_one(choices):
     assert ordinary[1:] == [BINS] * 199
     assert BINS not in flat[1:]
     assert [k for k, c in enumerate(flat[1:], 1) if c == PROBE] == [64, 128, 192]
+
+
+@pytest.mark.parametrize("largest,sort", [(50, BINS), (1000, BINS), (1500, BINS), (2300, RADIX), (5000, RADIX), (1_000_000, RADIX)])
+def test_the_faster_sort_by_the_largest_bin(choices, largest, sort):
+    """The line lies where the two sorts were measured to cross (1500 to 2200 Gaussians in a bin)."""
+    got = choices([(0, largest)] * 10)
+    assert got[2:] == [sort] * 8
