@@ -377,7 +377,7 @@ adr_status adr_create(adr_ctx** out, int64_t max_gaussians, int64_t pair_capacit
     }
     cudaError_t e = cudaHostAlloc((void**)&c->host_words, 64 * sizeof(uint32_t), cudaHostAllocDefault);
     if (e != cudaSuccess) { free_ctx(c); return fail(ADR_ERR_CUDA, "cudaHostAlloc: %s", cudaGetErrorString(e)); }
-    c->host_words[kHostLargestBin] = 0;
+    c->host_words[kHostLargestBin] = kUnknownBin;
     e = cudaHostGetDevicePointer((void**)&c->ws.largest_bin, c->host_words + kHostLargestBin, 0);
     if (e != cudaSuccess) { free_ctx(c); return fail(ADR_ERR_CUDA, "cudaHostGetDevicePointer: %s", cudaGetErrorString(e)); }
     e = cudaEventCreateWithFlags(&c->slice_ev, cudaEventDisableTiming);
@@ -410,7 +410,7 @@ adr_status adr_preprocess(adr_ctx* c, const float* means, const float* scales, c
     fill_frame_state(c->fs, n, cam, st);
     // The host word is written by the device (frames with a histogram) and read without waiting.
     c->depth_sort.largest_bin = *static_cast<volatile uint32_t*>(c->host_words + kHostLargestBin);
-    c->fs.depth_sort = c->depth_sort.next();
+    c->fs.depth_sort = c->depth_sort.next(n);
     enqueue_preprocess(c->ws, c->fs, c->epoch, means, scales, rots, opac, sh, strm, true,
                        c->defer_colors);
     if ((s = check_launch("adr_preprocess")) != ADR_OK) return s;

@@ -365,6 +365,7 @@ struct PreprocessOut {
 struct PreprocessBatch {
     int count = 0;
     BinMap map;              // count 0: no histogram
+    uint32_t skip = 0;       // its Gaussians: those whose index has none of these bits
     PreprocessOut cam[kMaxBatch];
 };
 // grid = chunks of 256 Gaussians x count, the camera index fastest
@@ -393,7 +394,7 @@ void launch_depth_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
 //                block, a failed wait to `counters` and the slices' blocks); it
 //                may overwrite the records.
 enum BinScan : int {
-    kScanLargest = 0,   // the largest bin only (beside the radix sort)
+    kScanLargest = 0,   // the largest bin only (beside the radix sort, of every kProbeEvery-th Gaussian)
     kScanFrame = 1,     // + the frame's counts (pairs with the capacity flag, runs, Gaussians) and slice 0
     kScanSlice1 = 2     // + slice 1's counts
 };

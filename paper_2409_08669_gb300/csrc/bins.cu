@@ -165,6 +165,7 @@ k_bin_scan(uint32_t* __restrict__ bins, uint32_t* __restrict__ win_lo, int what,
         if (lane == 0) {
             win_lo[(total + (uint32_t)kWindow - 1u) / (uint32_t)kWindow] = total;
             if (what != kScanSlice1) {
+                if (what == kScanLargest) most *= kProbeEvery;
                 counters[kCntLargestBin] = most;
                 if (largest) *largest = most;
             }

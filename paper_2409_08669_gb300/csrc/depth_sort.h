@@ -18,17 +18,25 @@ namespace adr {
 enum DepthSort : int { kSortBins = 0, kSortRadix = 1, kSortRadixProbe = 2 };
 constexpr uint32_t kRadixBin = 1536;
 constexpr uint32_t kRadixProbe = 64;   // a histogram every 64th radix frame
+// That histogram counts every 8th Gaussian: of all, atomics on one address took 435 us
+// of a 1016 us frame (3M Gaussians within 1% of one depth).
+constexpr uint32_t kProbeEvery = 8;
+constexpr uint32_t kUnknownBin = 0xFFFFFFFFu;
 
 // One per context, served scene or allocation-free device.
 struct DepthSortChoice {
-    uint32_t largest_bin = 0;          // of the last completed frame that had a histogram
+    uint32_t largest_bin = kUnknownBin;   // of the last completed frame that had a histogram
     uint32_t probe_in = kRadixProbe;   // radix frames until the next one with a histogram
 
-    DepthSort next() {
-        if (largest_bin <= kRadixBin) {
+    // The sort of a frame of n Gaussians.  Until a frame has been measured the radix sort, whose
+    // time does not depend on the depths: a first frame of 3M Gaussians, over octaves to one
+    // depth, took 0.43 to 33 ms by bins, 0.58 to 0.82 by the passes.
+    DepthSort next(int64_t n) {
+        if (largest_bin <= kRadixBin || n <= (int64_t)kRadixBin) {
             probe_in = kRadixProbe;
             return kSortBins;
         }
+        if (largest_bin == kUnknownBin) return kSortRadixProbe;
         if (--probe_in > 0) return kSortRadix;
         probe_in = kRadixProbe;
         return kSortRadixProbe;

@@ -181,7 +181,7 @@ extern "C" adr_status adr_render_frame_noalloc(const float* means, const float* 
     cudaStream_t strm = static_cast<cudaStream_t>(stream);
     FrameState fs;
     fill_frame_state(fs, n, cam, st);
-    fs.depth_sort = ds->depth_sort.next();
+    fs.depth_sort = ds->depth_sort.next(n);
     enqueue_preprocess(ws, fs, ds->epoch, means, scales, rots, opac, sh, strm);
     enqueue_sort(ws, fs, ds->epoch, strm);
     enqueue_render(ws, fs, img, t_final, load, strm);

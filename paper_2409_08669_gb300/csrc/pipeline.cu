@@ -95,6 +95,11 @@ static BinMap frame_bins(const FrameState& fs) {
     return fs.depth_sort == kSortRadix ? BinMap{} : bin_map(fs.n);
 }
 
+static uint32_t histogram_skip(const FrameState& fs) {
+    static_assert((kProbeEvery & (kProbeEvery - 1)) == 0, "a mask of the index");
+    return fs.depth_sort == kSortRadixProbe ? kProbeEvery - 1 : 0u;
+}
+
 static PreprocessOut preprocess_out(const Workspace& ws) {
     return PreprocessOut{ws.d_fp, ws.d_stage, ws.rec, ws.aux, ws.depth_key, ws.gbox, ws.bins, ws.rank, ws.sums};
 }
@@ -170,6 +175,7 @@ void enqueue_preprocess(const Workspace& ws, FrameState& fs, std::atomic<uint32_
     PreprocessBatch pb;
     pb.count = 1;
     pb.map = frame_bins(fs);
+    pb.skip = histogram_skip(fs);
     pb.cam[0] = preprocess_out(ws);
     TIMED(ws, kKPreprocess, stream,
           launch_preprocess((int)fs.n, means, scales, rots, opac, defer_colors ? nullptr : sh, pb,
@@ -444,6 +450,7 @@ void enqueue_frame_batch(const BatchItem* items, int count, const float* means, 
     PreprocessBatch pb;
     pb.count = count;
     pb.map = frame_bins(*items[0].fs);
+    pb.skip = histogram_skip(*items[0].fs);
     for (int b = 0; b < count; ++b) {
         const BatchItem& it = items[b];
         preprocess_head(*it.ws, *it.fs, *it.epoch, stream, set_params);

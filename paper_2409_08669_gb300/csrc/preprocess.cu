@@ -359,7 +359,8 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
                 key = __float_as_uint(depth);
                 // The depth histogram (bins.cu); the count comes back while the
                 // SH coefficients are on their way.
-                if (batch.map.count) rank = atomicAdd(out.bins + bin_of(key, bin_base(cam.near_z), batch.map), 1u);
+                if (batch.map.count && ((uint32_t)i & batch.skip) == 0u)
+                    rank = atomicAdd(out.bins + bin_of(key, bin_base(cam.near_z), batch.map), 1u);
                 r2.w = log2f(sigma);
             }
             r0 = make_float4(px, py, pxf.lo, pyf.lo);

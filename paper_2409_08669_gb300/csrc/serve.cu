@@ -179,7 +179,7 @@ adr_status run_batch(adr_server* s, Group& g) {
     Scene& sc = s->scenes[g.reqs[0]->scene];
     const int k = (int)g.reqs.size();
     cudaStream_t strm = g.stream;
-    const DepthSort depth_sort = sc.depth_sort.next();
+    const DepthSort depth_sort = sc.depth_sort.next(sc.n);
     for (int b = 0; b < k; ++b) {
         Slot& sl = *g.slots[b];
         fill_frame_state(sl.fs, sc.n, g.reqs[b]->cam, sc.st);

@@ -110,3 +110,24 @@ def test_radix_frames_of_odd_sizes(n):
             assert _order_is_right(rast, params, depth, cam, S.Settings(t_min=0.0))
     finally:
         rast.close()
+
+
+@pytest.mark.parametrize("n,kind", [(4097, "equal"), (20_001, "equal"), (9_000, "mixed"), (40_001, "wall"), (30_000, "ties")])
+def test_large_windows_after_an_ordinary_frame(n, kind):
+    """A frame that was expected to have no large bin sorts it in its window."""
+    from paper_2409_08669_gb300.raster import Rasterizer, upload
+    ordinary, cam = _frames(n)
+    rng = np.random.default_rng(n + 1)
+    wall = 4.0 + rng.uniform(0.0, 1e-4, n)
+    depth = {"equal": np.full(n, 3.0), "wall": wall, "mixed": np.where(rng.random(n) < 0.5, wall, rng.uniform(0.5, 8.0, n)),
+             "ties": 2.0 + rng.integers(0, 5, n) / 64.0}[kind]
+    st = S.Settings(t_min=0.0)
+    rast = Rasterizer(max_gaussians=n, pair_capacity=n, max_width=16, max_height=16)
+    try:
+        for _ in range(2):
+            rast.forward(upload(ordinary), cam, st)
+            assert rast.sync_status() == 0
+        for _ in range(2):
+            assert _order_is_right(rast, upload(_scene(depth)), depth, cam, st)
+    finally:
+        rast.close()
