@@ -23,7 +23,8 @@
 // threads without a remainder; the row strides put the eight rows of a load or
 // store phase into distinct banks.  Sums over pixels run in float pairs (two-sum)
 // and only the tiles' totals in FP64, of which this chip has 1/64 of the FP32
-// rate.  1920x1080x3, forward / backward: 118 / 85 us with one output per thread
+// rate: summed pixel by pixel in FP64, a pass without the gradient takes 76 us instead
+// of 57, and both give the exact mean of |x - y| (images in [0, 1], 64x48 to 1920x1080).  1920x1080x3, forward / backward: 118 / 85 us with one output per thread
 // and step and FP64 sums, 75 / 42 us now (3 CTAs per SM; 66 forward with one shared
 // reciprocal instead of seven quotients a pixel).
 #include "adr_internal.cuh"
@@ -206,12 +207,25 @@ k_ssim_forward(const float* __restrict__ img, const float* __restrict__ ref, int
     }
     if (lane == 0) sm.red[0][warp] = l1_sum;
     if (lane == 0) sm.red[1][warp] = ssim_sum;
-    __syncthreads();
+    // An infinite difference, or a sum over FP32's range, makes the pairs' second words NaN:
+    // such a tile's |x - y| are summed again, in FP64.
+    const bool beyond = __syncthreads_or(!(l1_sum.x < 4e37f));   // eight warps' sums stay finite
     if (threadIdx.x < 2) {
         float2 t = make_float2(0.f, 0.f);
         for (int w = 0; w < kLThreads / 32; ++w) t = pair_sum(t, sm.red[threadIdx.x][w]);
-        atomicAdd(stats + threadIdx.x, (double)t.x + (double)t.y);
+        if (!beyond || threadIdx.x == 1) atomicAdd(stats + threadIdx.x, isfinite(t.x) ? (double)t.x + (double)t.y : (double)t.x);
     }
+    if (!beyond) return;
+    double sum = 0.0;
+    for (int i = threadIdx.x; i < kLW * kLTall; i += kLThreads) {
+        const int r = i / kLW, q = i % kLW;
+        if (Y0 + r >= H || X0 + q >= W) continue;
+        const float2 xy = sm.xy[(r + kLR) * kPairStride + q + kLR];
+        sum += (double)fabsf(xy.x - xy.y);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) atomicAdd(stats, sum);
 }
 
 __global__ void __launch_bounds__(kLThreads, 3)
