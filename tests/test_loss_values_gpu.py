@@ -43,3 +43,21 @@ def test_the_mean_difference_has_64_bits(c, h, w):
     exact = math.fsum(img.reshape(-1).astype(np.float64)) / img.size
     tiles = c * -(-h // 54) * -(-w // 32)
     assert abs(_stats(img, ref)[0][0] - exact) <= (20 + tiles + 1) * 2.0 ** -53 * exact
+
+
+@pytest.mark.parametrize("hw,top", [(136 * 120, 60), (300 * 200 + 1, 300), (1280 * 720, 2000)])
+def test_the_load_gradient_is_the_rounded_64_bit_one(hw, top):
+    """Its float pairs keep 48 bits before the one rounding to FP32: of the loads of frames (whole numbers to a few
+    thousand) no value lies near enough to a rounding's middle to fall on the other side."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2409_08669_gb300.raster import Rasterizer
+    load = np.minimum(np.random.default_rng(hw).gamma(2.0, top / 6, hw), top).astype(np.int32)
+    rast = Rasterizer(max_gaussians=16, pair_capacity=16, max_width=16, max_height=16)
+    try:
+        stats, grad = rast.load_loss(torch.from_numpy(load).cuda(), weight=1.0)
+        mean, std = stats.cpu().numpy()
+        grad = grad.cpu().numpy()
+    finally:
+        rast.close()
+    assert np.array_equal(grad, ((load.astype(np.float64) - mean) * (1.0 / (hw * std))).astype(np.float32))
