@@ -185,12 +185,18 @@ adr_status adr_set_tile_split(adr_ctx *ctx, int32_t mode);
  * still blending (a pixel's blend stops once its transmittance falls below
  * t_min, so the others cannot change a pixel).  A context slices a frame when
  * the last sliced frame's two slices held fewer than half of all runs (read
- * back without waiting), and every 16th frame to measure again; otherwise, and
- * after a frame that had a backward, it builds every Gaussian's runs at once.  Either way the image is the same.
+ * back without waiting), and every 16th frame to measure again; otherwise it
+ * builds every Gaussian's runs at once.  Either way the image is the same.
  * adr_render_backward, adr_read_pairs and adr_read_ranges first build every
  * Gaussian's runs and expand them into per-tile lists and ranges (a second,
  * stable pass by tile row), enqueued on their own stream. */
 adr_status adr_sort(adr_ctx *ctx, void *stream);
+
+/* adr_sort of a frame that adr_render_backward will follow: with
+ * ADR_SLICES_ADAPTIVE it builds every Gaussian's runs at once, which the
+ * backward needs, rather than in two slices and then again.  The results are
+ * the same, and a backward may follow either. */
+adr_status adr_sort_for_backward(adr_ctx *ctx, void *stream);
 
 /* Stage 6: per-tile front-to-back alpha blending (Eq. 2-3) of the sorted
  * Gaussians; pairs with alpha < alpha_low are skipped and a pixel stops

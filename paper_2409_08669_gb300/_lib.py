@@ -68,6 +68,7 @@ _SIGNATURES = {
     "adr_preprocess": (_I32, [_P, _P, _P, _P, _P, _P, _I64, ctypes.POINTER(adr_camera),
                               ctypes.POINTER(adr_settings), _P]),
     "adr_sort": (_I32, [_P, _P]),
+    "adr_sort_for_backward": (_I32, [_P, _P]),
     "adr_render": (_I32, [_P, _P, _P, _P, _P]),
     "adr_render_float_load": (_I32, [_P, _P, _P, _P, _P]),
     "adr_num_pairs": (_I32, [_P, ctypes.POINTER(_I64)]),
@@ -192,6 +193,10 @@ def adr_preprocess(ctx, means, scales, rots, opac, sh, n, camera, settings, stre
 
 def adr_sort(ctx, stream):
     return check(load().adr_sort(ctx, stream), "adr_sort")
+
+
+def adr_sort_for_backward(ctx, stream):
+    return check(load().adr_sort_for_backward(ctx, stream), "adr_sort_for_backward")
 
 
 def adr_render(ctx, img, t_final, load_, stream):

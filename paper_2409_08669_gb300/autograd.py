@@ -19,9 +19,10 @@ from .raster import Rasterizer, image_loss
 
 class AdrRasterize(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, means, scales, rots, opac, sh, rast: Rasterizer, camera, settings):
+    def forward(ctx, means, scales, rots, opac, sh, rast: Rasterizer, camera, settings, for_backward=True):
         params = tuple(t.contiguous() for t in (means, scales, rots, opac, sh))
-        img, t_final, load = rast.forward(params, camera, settings, load_dtype=torch.float32)
+        img, t_final, load = rast.forward(params, camera, settings, for_backward=for_backward,
+                                          load_dtype=torch.float32)
         ctx.rast = rast
         ctx.frame = rast.frame
         ctx.save_for_backward(*params)
@@ -38,7 +39,7 @@ class AdrRasterize(torch.autograd.Function):
         if g_img is None:
             g_img = torch.zeros((3,) + ctx.size, device=params[0].device)
         grads = ctx.rast.backward(params, g_img, g_load)
-        return (*grads, None, None, None)
+        return (*grads, None, None, None, None)
 
 
 class LoadBalanceLoss(torch.autograd.Function):
@@ -76,7 +77,8 @@ class ImageLoss(torch.autograd.Function):
 
 def rasterize(params, rast: Rasterizer, camera, settings):
     """(img [3,H,W], load [H,W] float, t_final [H,W]) differentiable w.r.t. params."""
-    return AdrRasterize.apply(*params, rast, camera, settings)
+    for_backward = torch.is_grad_enabled() and any(p.requires_grad for p in params)
+    return AdrRasterize.apply(*params, rast, camera, settings, for_backward)
 
 
 def load_balance_loss(load_f, rast: Rasterizer):

@@ -158,7 +158,6 @@ struct adr_ctx {
     // half of all runs, and every kSliceProbe-th frame slices to measure again.
     cudaEvent_t slice_ev = nullptr;
     bool slice_probe = false;        // a readback is in flight
-    bool last_backward = false;      // the last frame had a backward
     bool slices_pay = true;
     uint32_t frames = 0;
     DepthSortChoice depth_sort;
@@ -422,7 +421,9 @@ adr_status adr_preprocess(adr_ctx* c, const float* means, const float* scales, c
 // Whether the context's next adr_sort builds depth slices: always, never, or
 // (adaptive) when the last sliced frame's run counts, read back without
 // waiting, showed they pay, and every kSliceProbe-th frame to measure again.
-static bool next_frame_slices(adr_ctx* c) {
+// A backward needs every Gaussian's runs: adaptively, a frame that will have one
+// is built whole (training step of 1M Gaussians at 1280x720: 815 -> 708 us).
+static bool next_frame_slices(adr_ctx* c, bool for_backward) {
     if (c->slice_probe) {   // the last sliced frame's run counts, if they are back
         const cudaError_t q = cudaEventQuery(c->slice_ev);
         if (q == cudaSuccess) {
@@ -434,21 +435,17 @@ static bool next_frame_slices(adr_ctx* c) {
         }
     }
     if (c->slice_mode != ADR_SLICES_ADAPTIVE) return c->slice_mode == ADR_SLICES_ALWAYS;
-    // A backward needs every Gaussian's runs: where one followed the last frame, this
-    // one's are built at once rather than in two slices and then again (training step
-    // of 1M Gaussians at 1280x720: 815 -> 708 us).
-    return !c->last_backward && (c->slices_pay || (c->frames % kSliceProbe) == 0);
+    return !for_backward && (c->slices_pay || (c->frames % kSliceProbe) == 0);
 }
 
-adr_status adr_sort(adr_ctx* c, void* stream) {
+static adr_status sort_frame(adr_ctx* c, bool for_backward, void* stream) {
     NvtxRange range_("adr_sort");
     if (!c) return fail(ADR_ERR_INVALID, "ctx is NULL");
     if (!c->have_frame) return fail(ADR_ERR_INVALID, "adr_sort before adr_preprocess");
     DeviceGuard guard(c->device);
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
-    c->fs.allow_slices = next_frame_slices(c);
-    c->last_backward = false;
+    c->fs.allow_slices = next_frame_slices(c, for_backward);
     ++c->frames;
     enqueue_sort(c->ws, c->fs, c->epoch, strm);
     adr_status s;
@@ -456,6 +453,10 @@ adr_status adr_sort(adr_ctx* c, void* stream) {
     c->have_sort = true;
     return ok();
 }
+
+adr_status adr_sort(adr_ctx* c, void* stream) { return sort_frame(c, false, stream); }
+
+adr_status adr_sort_for_backward(adr_ctx* c, void* stream) { return sort_frame(c, true, stream); }
 
 static adr_status render_frame(adr_ctx* c, float* img, float* t_final, int32_t* load, bool load_float,
                                void* stream) {
@@ -613,7 +614,6 @@ adr_status adr_render_backward(adr_ctx* c, const float* means, const float* scal
     cudaStream_t strm = (cudaStream_t)stream;
     c->last_stream = strm;
     enqueue_tile_lists(c->ws, c->fs, strm);   // the backward walks per-tile lists
-    c->last_backward = true;
     enqueue_backward(c->ws, c->fs, means, scales, rots, opac, sh, dl_dimg, dl_dload, g_means,
                      g_scales, g_rots, g_opac, g_sh, strm);
     return check_launch("adr_render_backward") == ADR_OK ? ok() : ADR_ERR_CUDA;
@@ -821,7 +821,7 @@ adr_status adr_render_host(adr_ctx* c, const float* means, const float* scales, 
             // only those of the Gaussians each Render phase blends; an
             // unsliced frame blends every Gaussian with tiles and reads them
             // in Preprocess, in index order.
-            c->defer_colors = next_frame_slices(c);
+            c->defer_colors = next_frame_slices(c, false);
             adr_status s = adr_preprocess(c, dm, ds, dr, dop, dsh, n, camera, settings, stream);
             c->defer_colors = false;
             if (s != ADR_OK) return s;

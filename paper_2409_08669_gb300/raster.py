@@ -132,8 +132,9 @@ class Rasterizer:
                             n, _lib.make_camera(camera), _lib.make_settings(settings),
                             _stream(stream))
 
-    def sort(self, stream=None):
-        _lib.adr_sort(self.ctx, _stream(stream))
+    def sort(self, stream=None, for_backward=False):
+        """`for_backward`: a backward of this frame will follow (the same results, in less time)."""
+        (_lib.adr_sort_for_backward if for_backward else _lib.adr_sort)(self.ctx, _stream(stream))
 
     def render(self, img=None, t_final=None, load=None, stream=None, want_aux=True,
                load_dtype=torch.int32):
@@ -157,9 +158,9 @@ class Rasterizer:
         call(self.ctx, _ptr(img), _ptr(t_final), _ptr(load), _stream(stream))
         return img, t_final, load
 
-    def forward(self, params, camera, settings, stream=None, **kw):
+    def forward(self, params, camera, settings, stream=None, for_backward=False, **kw):
         self.preprocess(params, camera, settings, stream)
-        self.sort(stream)
+        self.sort(stream, for_backward)
         return self.render(stream=stream, **kw)
 
     SLICES_NEVER, SLICES_ALWAYS, SLICES_ADAPTIVE = 0, 1, 2
