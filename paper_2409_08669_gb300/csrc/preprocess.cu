@@ -205,7 +205,7 @@ constexpr int kPreCtasPerSm = 7;
 __global__ void __launch_bounds__(kPreThreads, kPreCtasPerSm)
 k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ scales,
              const float* __restrict__ rots, const float* __restrict__ opac,
-             const float* __restrict__ sh, PreprocessBatch batch, int64_t ahead) {
+             const float* __restrict__ sh, PreprocessBatch batch, int64_t ahead, bool early) {
     pdl_prologue();
     const int b = (int)(blockIdx.x % (unsigned)batch.count);
     const int i = (int)(blockIdx.x / (unsigned)batch.count) * blockDim.x + threadIdx.x;
@@ -214,7 +214,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
     // Lane 0 of each warp asks L2 for the parameters (44 B per Gaussian) of
     // the warp that runs one wave of CTAs later (`ahead` Gaussians on), so
     // that warp's first loads hit L2 instead of waiting on DRAM.  Bulk
-    // prefetches: 16-byte aligned, sizes multiples of 16.
+    // prefetches: 16-byte aligned (the launch looks at the arrays), sizes multiples of 16.
     if ((threadIdx.x & 31) == 0 && b == 0 && ahead > 0) {
         const int64_t g = (int64_t)i + ahead;
         if (g + 32 <= n) {
@@ -240,8 +240,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
                 mz = mine ? means[3 * i + 2] : 0.f;
     // Device memory: the other parameters at once with the means (all are on their way
     // to L2 anyway; frames of 1M at 1080p 330 -> 323 us, 3M 477 -> 466, 16 served 3090 ->
-    // 3058).  Host memory: only those in front of the camera cross the link.
-    const bool early = ahead > 0;
+    // 3058).  Host memory (not early): only those in front of the camera cross the link.
     float4 rot = make_float4(0.f, 0.f, 0.f, 0.f);
     float sx = 0.f, sy = 0.f, sz = 0.f, sigma = 0.f;
     auto load_rest = [&] {
@@ -479,9 +478,13 @@ void launch_preprocess(int n, const float* means, const float* scales, const flo
     const cudaError_t pe = cudaPointerGetAttributes(&pa, means);
     if (pe != cudaSuccess) (void)cudaGetLastError();   // this query's own error only
     const bool on_device = pe == cudaSuccess && pa.type == cudaMemoryTypeDevice;
-    const int64_t ahead = on_device ? ((int64_t)sms * kPreCtasPerSm * threads / batch.count) & ~(int64_t)31 : 0;
+    // Arrays of 4-byte alignment (a slice of a larger one) are read without it too.
+    const bool aligned = ((reinterpret_cast<uintptr_t>(means) | reinterpret_cast<uintptr_t>(scales) |
+                           reinterpret_cast<uintptr_t>(rots) | reinterpret_cast<uintptr_t>(opac)) & 15) == 0;
+    const int64_t ahead =
+        on_device && aligned ? ((int64_t)sms * kPreCtasPerSm * threads / batch.count) & ~(int64_t)31 : 0;
     launch_pdl(k_preprocess, chunks * (unsigned)batch.count, threads, 0, stream, n, means, scales, rots,
-               opac, sh, batch, ahead);
+               opac, sh, batch, ahead, on_device);
 }
 
 void launch_colors(const uint32_t* ids, const uint32_t* count, const float* means, const float* sh,
