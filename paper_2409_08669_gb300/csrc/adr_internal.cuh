@@ -284,6 +284,7 @@ struct FrameState {
     bool slice1_bins_used = false;           // slice 1's bins are no longer zero
     int order_held = 0;                      // which of OrderHeld `order` and its boxes and offsets hold
     bool totals_used[kTotalSets] = {false, false, false};   // written since the frame's head zeroed them
+    unsigned long long head_capture = 0;     // the graph capture that holds the frame's head (0: none)
     bool sliced = false;                     // the frame renders in two depth slices
     bool load_float = false;      // Render writes the loads as floats
     bool split_last_slice = false;           // slice 1 renders tiles by pixel halves (f2)

@@ -80,6 +80,19 @@ void fill_frame_state(FrameState& fs, int64_t n, const CamDev& cam, const SetDev
     fs.sorted_gauss = nullptr;
 }
 
+// The graph capture that `stream` is in, 0 if none.  What the frame's head zeroes is
+// zero again in every replay only of a graph that holds the head; a stage captured
+// without it (adr_sort or adr_render_backward alone) clears its words itself.
+static unsigned long long capture_of(cudaStream_t stream) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess) {
+        (void)cudaGetLastError();   // this query's own error only
+        return 0;
+    }
+    return status == cudaStreamCaptureStatusActive ? id : 0;
+}
+
 // Before Preprocess: the stage tag, the frame parameters and the zeroed words.
 static void preprocess_head(const Workspace& ws, FrameState& fs, std::atomic<uint32_t>& epoch,
                             cudaStream_t stream, bool set_params) {
@@ -89,6 +102,7 @@ static void preprocess_head(const Workspace& ws, FrameState& fs, std::atomic<uin
     for (bool& used : fs.totals_used) used = false;
     fs.order_held = 0;
     fs.slice1_bins_used = false;
+    fs.head_capture = capture_of(stream);
 }
 
 static BinMap frame_bins(const FrameState& fs) {
@@ -184,10 +198,11 @@ void enqueue_preprocess(const Workspace& ws, FrameState& fs, std::atomic<uint32_
 }
 
 // One of the tile passes' total sets, zero: as the frame's head left it, or
-// cleared again for a second pass of the frame.
+// cleared again for a second pass of the frame or in a graph without the head.
 static uint32_t* fresh_totals(const Workspace& ws, FrameState& fs, TotalSet which, cudaStream_t stream) {
     uint32_t* totals = ws.ttotals + (int)which * kRadix;
-    if (fs.totals_used[which]) cudaMemsetAsync(totals, 0, kRadix * sizeof(uint32_t), stream);
+    if (fs.totals_used[which] || capture_of(stream) != fs.head_capture)
+        cudaMemsetAsync(totals, 0, kRadix * sizeof(uint32_t), stream);
     fs.totals_used[which] = true;
     return totals;
 }
@@ -359,7 +374,7 @@ static void slice1_runs(const Workspace& ws, FrameState& fs, cudaStream_t stream
         uint32_t* bins = ws.bins + map.count;
         uint32_t* rank = ws.s_offsets;   // last read before the run offsets are written
         const EpochRef ep{ws.d_stage, (uint32_t)(kMaxPasses + 2)};
-        if (fs.slice1_bins_used) {   // a second render of the frame
+        if (fs.slice1_bins_used || capture_of(stream) != fs.head_capture) {   // a second render of the frame
             cudaMemsetAsync(bins, 0, map.count * sizeof(uint32_t), stream);
             cudaMemsetAsync(c1, 0, kCntSlots * sizeof(uint32_t), stream);
         }
