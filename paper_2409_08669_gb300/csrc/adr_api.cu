@@ -566,7 +566,7 @@ adr_status adr_read_gaussians(adr_ctx* c, float* geom, int32_t* rect, int32_t* t
     if (geom && c->fs.defer_colors && c->fs.sh && c->fs.order && c->fs.n > 0) {
         enqueue_order_all(c->ws, c->fs, (cudaStream_t)stream);
         launch_colors(c->fs.order, c->ws.counters + kCntVisible, c->fs.means, c->fs.sh, c->ws.d_fp,
-                      c->ws.rec, c->ws.sm_count, (cudaStream_t)stream);
+                      c->ws.rec, infinite_colour(c->ws.sums), c->ws.sm_count, (cudaStream_t)stream);
     }
     launch_read_gaussians(c->ws.rec, c->ws.aux, c->ws.gbox, (int)c->fs.n, geom, rect,
                           tiles, (cudaStream_t)stream);

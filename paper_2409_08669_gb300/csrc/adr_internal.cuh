@@ -227,7 +227,8 @@ constexpr size_t sortbuf_quads(int64_t n) { return ((size_t)n + 3) & ~(size_t)3;
 // two depth slices, the tile passes' totals, Preprocess's sums, then the depth
 // bins of the frame and (with depth slices) those of slice 1's Gaussians.
 enum TotalSet : int { kTotalsFirst = 0, kTotalsSlice1 = 1, kTotalsRows = 2, kTotalSets = 3 };
-constexpr int kSumSlots = 64;    // Preprocess's pair and run sums: 64-bit words 0 and 1 of each slot
+constexpr int kSumSlots = 64;    // Preprocess's pair and run sums: 64-bit words 0 and 1 of each slot;
+                                 // word 2 of the first: not 0 if a colour of the frame is infinite
 constexpr int kSumStride = 4;    // 64-bit words (32 bytes) a slot
 constexpr int kZeroWords = 3 * kCntSlots + kTotalSets * kRadix + 2 * kSumSlots * kSumStride;   // + the bins
 static_assert(kZeroWords % 4 == 0 && (3 * kCntSlots + kTotalSets * kRadix) % 4 == 0,
@@ -252,6 +253,11 @@ __device__ __forceinline__ uint32_t bin_of(uint32_t key, uint32_t base, const Bi
 }
 // Gaussians of a window of the window sort, not counting what its last bin adds.
 constexpr int kWindow = 1024;
+
+// Where a kernel that forms colours leaves that one is infinite (no colour is negative).
+__device__ __host__ __forceinline__ uint32_t* infinite_colour(unsigned long long* sums) {
+    return reinterpret_cast<uint32_t*>(sums + 2);
+}
 
 // hist layout: 4 x 256 per-digit totals of the depth passes.
 constexpr int kHistWords = kMaxPasses * kRadix;
@@ -417,7 +423,7 @@ void launch_window_sort(uint4* recs, const uint32_t* win_lo, const uint32_t* gbo
 // a frame with deferred colours computes them only for the Gaussians a Render
 // launch blends.
 void launch_colors(const uint32_t* ids, const uint32_t* count, const float* means, const float* sh,
-                   const FrameParams* fp, float4* rec, int sm_count, cudaStream_t stream);
+                   const FrameParams* fp, float4* rec, uint32_t* infinite, int sm_count, cudaStream_t stream);
 
 // Inputs of the tile passes.
 struct PairSource {
@@ -513,6 +519,7 @@ struct RenderCam {
     float* t_final = nullptr;
     int32_t* load = nullptr;
     bool load_float = false;              // load holds floats
+    const uint32_t* infinite = nullptr;   // not 0: a colour is (infinite_colour)
     int32_t* last = nullptr;
     int32_t* trav = nullptr;
     float* tfin = nullptr;

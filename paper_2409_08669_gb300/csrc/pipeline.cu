@@ -318,6 +318,7 @@ static RenderCam render_cam(const Workspace& ws, const FrameState& fs, float* im
     rc.t_final = t_final;
     rc.load = load;
     rc.load_float = fs.load_float;
+    rc.infinite = infinite_colour(ws.sums);
     rc.last = ws.last;
     rc.trav = ws.trav;
     rc.tfin = ws.tfin;
@@ -346,7 +347,7 @@ static void enqueue_colors(const Workspace& ws, const FrameState& fs, int phase,
                             : phase == 1 ? ws.slice_counters + kCntVisible
                                          : ws.slice_counters + kCntSlots + kCntVisible;
     TIMED(ws, kKColors, stream,
-          launch_colors(ids, count, fs.means, fs.sh, ws.d_fp, ws.rec, ws.sm_count, stream));
+          launch_colors(ids, count, fs.means, fs.sh, ws.d_fp, ws.rec, infinite_colour(ws.sums), ws.sm_count, stream));
 }
 
 // One Render launch over the items' cameras (all of the same list kind).

@@ -403,6 +403,7 @@ k_preprocess(int n, const float* __restrict__ means, const float* __restrict__ s
             r2.x = rgb.x;
             r2.y = rgb.y;
             r2.z = rgb.z;
+            if (!(rgb.x + rgb.y + rgb.z < INFINITY)) *infinite_colour(out.sums) = 1u;
         }
         rec[3 * i + 2] = r2;
     }
@@ -425,7 +426,7 @@ constexpr int kColorThreads = 128;
 __global__ void __launch_bounds__(kColorThreads, 8)   // as many as their rows fit in shared memory
 k_colors(const uint32_t* __restrict__ ids, const uint32_t* __restrict__ count,
          const float* __restrict__ means, const float* __restrict__ sh,
-         const FrameParams* __restrict__ fp, float4* __restrict__ rec) {
+         const FrameParams* __restrict__ fp, float4* __restrict__ rec, uint32_t* __restrict__ infinite) {
     pdl_prologue();
     __shared__ ShRows s_rows[kColorThreads / 32];
     ShRows& rows = s_rows[threadIdx.x >> 5];
@@ -454,6 +455,7 @@ k_colors(const uint32_t* __restrict__ ids, const uint32_t* __restrict__ count,
             dx *= dn; dy *= dn; dz *= dn;
             const float3 rgb = sh_to_rgb(rows + lane * kShStride, degree, dx, dy, dz);
             rec[3 * (size_t)i + 2] = make_float4(rgb.x, rgb.y, rgb.z, r2.w);
+            if (!(rgb.x + rgb.y + rgb.z < INFINITY)) *infinite = 1u;
         }
         __syncwarp();   // the rows are no longer read
     }
@@ -488,9 +490,9 @@ void launch_preprocess(int n, const float* means, const float* scales, const flo
 }
 
 void launch_colors(const uint32_t* ids, const uint32_t* count, const float* means, const float* sh,
-                   const FrameParams* fp, float4* rec, int sm_count, cudaStream_t stream) {
+                   const FrameParams* fp, float4* rec, uint32_t* infinite, int sm_count, cudaStream_t stream) {
     launch_pdl(k_colors, (sm_count > 0 ? sm_count : 1) * 8, kColorThreads, 0, stream, ids, count,
-               means, sh, fp, rec);
+               means, sh, fp, rec, infinite);
 }
 
 }  // namespace adr

@@ -188,7 +188,122 @@ __device__ __forceinline__ void stage_records(int m, const uint32_t* s_gid, cons
 // only its own state in registers.
 struct TileInfo {
     int width, height, tiles_x, tiles_y, tx, ty;
+    uint32_t infinite;   // a colour of the frame is
 };
+
+// Per-pixel blend state: pixel a in .x, pixel b in .y.  elim is each pixel's limit on
+// the exponent: a Gaussian reaches it iff e >= limit.
+struct BlendState {
+    float2 T, C0, C1, C2, elim;
+    int32_t cnt_a, cnt_b, last_a, last_b;
+};
+
+// A warp's blend of its quadrant's list.  A pixel becomes done only where it stops
+// (its exponent limit then becomes +inf, so no later Gaussian reaches it), and the
+// loop leaves there once every pixel of the warp is done.  The list goes in
+// windows of 32 entries: bit k of bits_a / bits_b records that
+// pixel a / b blended entry i0 + k, and each window's bits are
+// folded into l_i (their count) and the last blended position
+// (their highest bit) when the window ends.
+// kVotes (a frame with an infinite colour): a Gaussian that no pixel of the warp
+// blends is left out, as 0 times its colour would not be 0.  With that vote in every
+// loop 3M Gaussians at 4K take 943 us instead of 928, in a function of its own 930.
+template <bool kVotes>
+__device__ __forceinline__ void walk_list(BlendState& st, const uint32_t* list, int n, const float4* s_kl,
+                                          const float4* s_nw, const float4* s_rg, int2* s_stop, float2 fx2,
+                                          float2 fya2, float2 fyb2, float t_min, int32_t fbase) {
+    bool warp_done = false;
+    uint2 ahead = *reinterpret_cast<const uint2*>(list);   // the next group's entries
+#pragma unroll 1
+    for (int i0 = 0; i0 < n && !warp_done; i0 += 32) {
+        const int len = min(32, n - i0);
+        uint32_t bits_a = 0u, bits_b = 0u;
+#pragma unroll 1
+        for (int k = 0; k < len && !warp_done; k += kGroup) {
+            const uint32_t off[kGroup] = {ahead.x, ahead.y};
+            ahead = *reinterpret_cast<const uint2*>(list + i0 + k + kGroup);
+            float2 alpha[kGroup], wgt[kGroup], now = st.T;
+            float blue[kGroup];
+            uint32_t na = 0u, nb = 0u;
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q) {
+                const float4 kl = at_offset(s_kl, off[q]);
+                const float4 nw = at_offset(s_nw, off[q]);
+                blue[q] = kl.w;
+                // u = (k - w_x fx) - w_y fy, the fx-term shared, as quad_exponent
+                const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
+                const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
+                const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
+                // e = log2(sigma) - q log2(e) / 2; alpha = min(0.99, 2^e) (Eq. 2)
+                // reaches alpha_low iff e >= e_low
+                const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
+                const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
+                const bool la = ea >= st.elim.x, lb = eb >= st.elim.y;
+                // A pixel that skips has alpha 0, so T and C stay as they are.
+                alpha[q] = make_float2(la ? fminf(0.99f, ex2_approx(ea)) : 0.f,
+                                       lb ? fminf(0.99f, ex2_approx(eb)) : 0.f);
+                if (la) na |= 1u << q;
+                if (lb) nb |= 1u << q;
+            }
+            // Front-to-back steps (Eq. 3), both pixels at once: T (1 - alpha) = T - alpha T
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q) {
+                wgt[q] = fmul2(alpha[q], now);
+                now = fsub2(now, wgt[q]);
+            }
+            bool used[kGroup] = {};
+            if (kVotes) {
+#pragma unroll
+                for (int q = 0; q < kGroup; ++q) used[q] = __any_sync(0xffffffffu, ((na | nb) >> q) & 1u);
+            }
+            // T never grows, and a done pixel keeps T >= t_min: some pixel stops
+            // in this group iff its last T is below t_min.
+            if (__any_sync(0xffffffffu, fminf(now.x, now.y) < t_min)) {
+                // The steps again, each pixel up to the Gaussian it stops before,
+                // which it does not blend.
+                now = st.T;
+#pragma unroll
+                for (int q = 0; q < kGroup; ++q) {
+                    const int32_t pos = fbase + (int32_t)(off[q] / 16u) + 1;
+                    if (st.elim.x == kInf) alpha[q].x = 0.f;
+                    if (st.elim.y == kInf) alpha[q].y = 0.f;
+                    if (kVotes) used[q] = __any_sync(0xffffffffu, alpha[q].x > 0.f || alpha[q].y > 0.f);
+                    wgt[q] = fmul2(alpha[q], now);
+                    float2 t = fsub2(now, wgt[q]);
+                    if (t.x < t_min) { wgt[q].x = 0.f; t.x = now.x; s_stop[threadIdx.x].x = pos; st.elim.x = kInf; na &= (1u << q) - 1u; }
+                    if (t.y < t_min) { wgt[q].y = 0.f; t.y = now.y; s_stop[threadIdx.x].y = pos; st.elim.y = kInf; nb &= (1u << q) - 1u; }
+                    now = t;
+                    // the last pixel stopped: nothing blends this Gaussian
+                    if (kVotes && __all_sync(0xffffffffu, fminf(st.elim.x, st.elim.y) == kInf)) used[q] = false;
+                }
+                warp_done = __all_sync(0xffffffffu, fminf(st.elim.x, st.elim.y) == kInf);
+            }
+            st.T = now;
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q) {
+                if (kVotes && !used[q]) continue;
+                const float4 rg = at_offset(s_rg, off[q]);
+                st.C0 = ffma2(make_float2(rg.x, rg.y), wgt[q], st.C0);
+                st.C1 = ffma2(make_float2(rg.z, rg.w), wgt[q], st.C1);
+                st.C2 = ffma2(make_float2(blue[q], blue[q]), wgt[q], st.C2);
+            }
+            bits_a |= na << k;
+            bits_b |= nb << k;
+        }
+        st.cnt_a += __popc(bits_a);
+        st.cnt_b += __popc(bits_b);
+        // 1-based position of the highest bit's Gaussian
+        if (bits_a) st.last_a = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_a)] / 16u);
+        if (bits_b) st.last_b = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_b)] / 16u);
+    }
+}
+__device__ __noinline__ void walk_list_votes(BlendState* s, const uint32_t* list, int n, const float4* s_kl,
+                                             const float4* s_nw, const float4* s_rg, int2* s_stop, float2 fx2,
+                                             float2 fya2, float2 fyb2, float t_min, int32_t fbase) {
+    BlendState st = *s;
+    walk_list<true>(st, list, n, s_kl, s_nw, s_rg, s_stop, fx2, fya2, fyb2, t_min, fbase);
+    *s = st;
+}
 
 // CTAs per SM: 64 registers, no spills.  Frame at 4K, 3M Gaussians: 8 CTAs 969 us,
 // 9 (56 registers, small spills) 976, 7 982.
@@ -227,7 +342,7 @@ k_render(const RenderBatch batch) {
     // a few columns' run lists and Gaussian records in L2.
     const int ty0 = tile_index % cam.tiles_y, tx0 = tile_index / cam.tiles_y;
     if (threadIdx.x == 0) {
-        s_ti = TileInfo{cam.width, cam.height, cam.tiles_x, cam.tiles_y, tx0, ty0};
+        s_ti = TileInfo{cam.width, cam.height, cam.tiles_x, cam.tiles_y, tx0, ty0, *batch.cam[cb].infinite};
         if (batch.cam[cb].trace) {
             uint32_t t;
             asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(t));
@@ -321,88 +436,16 @@ k_render(const RenderBatch batch) {
             const int n = warp_list(s_mask[warp], m, lane, list);
             if (lane < 2 * kGroup) list[n + lane] = kStage * 16u;
             __syncwarp();
-            // A pixel becomes done only where it stops (its exponent limit
-            // then becomes +inf, so no later Gaussian reaches it), and the
-            // loop leaves there once every pixel of the warp is done.  The list goes in
-            // windows of 32 entries: bit k of bits_a / bits_b records that
-            // pixel a / b blended entry i0 + k, and each window's bits are
-            // folded into l_i (their count) and the last blended position
-            // (their highest bit) when the window ends.
-            bool warp_done = false;
-            uint2 ahead = *reinterpret_cast<const uint2*>(list);   // the next group's entries
-#pragma unroll 1
-            for (int i0 = 0; i0 < n && !warp_done; i0 += 32) {
-                const int len = min(32, n - i0);
-                uint32_t bits_a = 0u, bits_b = 0u;
-#pragma unroll 1
-                for (int k = 0; k < len && !warp_done; k += kGroup) {
-                    const uint32_t off[kGroup] = {ahead.x, ahead.y};
-                    ahead = *reinterpret_cast<const uint2*>(list + i0 + k + kGroup);
-                    float2 alpha[kGroup], wgt[kGroup], now = T;
-                    float blue[kGroup];
-                    uint32_t na = 0u, nb = 0u;
-#pragma unroll
-                    for (int q = 0; q < kGroup; ++q) {
-                        const float4 kl = at_offset(s_kl, off[q]);
-                        const float4 nw = at_offset(s_nw, off[q]);
-                        blue[q] = kl.w;
-                        // u = (k - w_x fx) - w_y fy, the fx-term shared, as quad_exponent
-                        const float2 in = ffma2(make_float2(nw.x, nw.y), fx2, make_float2(kl.x, kl.y));
-                        const float2 ua = ffma2(make_float2(nw.z, nw.w), fya2, in);
-                        const float2 ub = ffma2(make_float2(nw.z, nw.w), fyb2, in);
-                        // e = log2(sigma) - q log2(e) / 2; alpha = min(0.99, 2^e) (Eq. 2)
-                        // reaches alpha_low iff e >= e_low
-                        const float ea = fmaf(-ua.x, ua.x, fmaf(-ua.y, ua.y, kl.z));
-                        const float eb = fmaf(-ub.x, ub.x, fmaf(-ub.y, ub.y, kl.z));
-                        const bool la = ea >= elim.x, lb = eb >= elim.y;
-                        // A pixel that skips has alpha 0, so T and C stay as they are.
-                        alpha[q] = make_float2(la ? fminf(0.99f, ex2_approx(ea)) : 0.f,
-                                               lb ? fminf(0.99f, ex2_approx(eb)) : 0.f);
-                        if (la) na |= 1u << q;
-                        if (lb) nb |= 1u << q;
-                    }
-                    // Front-to-back steps (Eq. 3), both pixels at once: T (1 - alpha) = T - alpha T
-#pragma unroll
-                    for (int q = 0; q < kGroup; ++q) {
-                        wgt[q] = fmul2(alpha[q], now);
-                        now = fsub2(now, wgt[q]);
-                    }
-                    // T never grows, and a done pixel keeps T >= t_min: some pixel stops
-                    // in this group iff its last T is below t_min.
-                    if (__any_sync(0xffffffffu, fminf(now.x, now.y) < t_min)) {
-                        // The steps again, each pixel up to the Gaussian it stops before,
-                        // which it does not blend.
-                        now = T;
-#pragma unroll
-                        for (int q = 0; q < kGroup; ++q) {
-                            const int32_t pos = fbase + (int32_t)(off[q] / 16u) + 1;
-                            if (elim.x == kInf) alpha[q].x = 0.f;
-                            if (elim.y == kInf) alpha[q].y = 0.f;
-                            wgt[q] = fmul2(alpha[q], now);
-                            float2 t = fsub2(now, wgt[q]);
-                            if (t.x < t_min) { wgt[q].x = 0.f; t.x = now.x; s_stop[threadIdx.x].x = pos; elim.x = kInf; na &= (1u << q) - 1u; }
-                            if (t.y < t_min) { wgt[q].y = 0.f; t.y = now.y; s_stop[threadIdx.x].y = pos; elim.y = kInf; nb &= (1u << q) - 1u; }
-                            now = t;
-                        }
-                        warp_done = __all_sync(0xffffffffu, fminf(elim.x, elim.y) == kInf);
-                    }
-                    T = now;
-#pragma unroll
-                    for (int q = 0; q < kGroup; ++q) {
-                        const float4 rg = at_offset(s_rg, off[q]);
-                        C0 = ffma2(make_float2(rg.x, rg.y), wgt[q], C0);
-                        C1 = ffma2(make_float2(rg.z, rg.w), wgt[q], C1);
-                        C2 = ffma2(make_float2(blue[q], blue[q]), wgt[q], C2);
-                    }
-                    bits_a |= na << k;
-                    bits_b |= nb << k;
-                }
-                cnt_a += __popc(bits_a);
-                cnt_b += __popc(bits_b);
-                // 1-based position of the highest bit's Gaussian
-                if (bits_a) last_a = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_a)] / 16u);
-                if (bits_b) last_b = fbase + 1 + (int32_t)(list[i0 + 31 - __clz(bits_b)] / 16u);
+            BlendState st{T, C0, C1, C2, elim, cnt_a, cnt_b, last_a, last_b};
+            if (s_ti.infinite) {
+                BlendState copy = st;
+                walk_list_votes(&copy, list, n, s_kl, s_nw, s_rg, s_stop, fx2, fya2, fyb2, t_min, fbase);
+                st = copy;
+            } else {
+                walk_list<false>(st, list, n, s_kl, s_nw, s_rg, s_stop, fx2, fya2, fyb2, t_min, fbase);
             }
+            T = st.T; C0 = st.C0; C1 = st.C1; C2 = st.C2; elim = st.elim;
+            cnt_a = st.cnt_a; cnt_b = st.cnt_b; last_a = st.last_a; last_b = st.last_b;
         }
         fbase += m;
         base = next;
