@@ -186,7 +186,7 @@ struct Workspace {
     int32_t* trav = nullptr;               // [max pixels]
     float* tfin = nullptr;                 // [max pixels] final transmittance of the last render
     int32_t* lstat = nullptr;              // [max pixels] l_i | terminated << 31 of the last render
-    float* g2d = nullptr;                  // [max_n * 9] backward: moments of v (1, x, y, xx, xy, yy), dL/drgb
+    float* g2d = nullptr;                  // [max_n * 9] backward: dL/d(px, py, conic, sigma, rgb)
     double* load_sums = nullptr;           // [8] load-balancing loss: mean, std at 2, 3; integer sums from 4
     uint32_t* hist = nullptr;              // [kHistWords]
     uint32_t* counters = nullptr;          // [kCntSlots], the start of the zeroed block

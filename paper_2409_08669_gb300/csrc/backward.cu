@@ -5,13 +5,10 @@
 //
 //   k_render_backward     per tile, walks each pixel's blended Gaussians from
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
-//                         and accumulates, with v = alpha dL/dalpha, sum v, dL/d(px,
-//                         py), the second moments of v about the Gaussian's centre
-//                         and its colour gradient; reduced over a warp, then
-//                         atomicAdd into 9 floats per Gaussian.
-//   k_preprocess_backward dL/d(conic, sigma) from the moments, and the chain rule
-//                         to means, scales, rotations, opacities and SH
-//                         coefficients.
+//                         and accumulates dL/d(px, py, conic, sigma, rgb);
+//                         warp-reduced, then atomicAdd into 9 floats per Gaussian.
+//   k_preprocess_backward chain rule from those 2D quantities to means, scales,
+//                         rotations, opacities and SH coefficients.
 //   k_load_moments / k_load_grad
 //                         L_load = std over pixels of l_i (Eq. 13, population
 //                         form) and dL_load/dl_i = (l_i - mean) / (HW std).
@@ -20,179 +17,171 @@
 namespace adr {
 namespace {
 
-constexpr int kBwdThreads = kTilePixels;       // a pixel per thread
-constexpr int kBwdWarps = kBwdThreads / 32;    // 16x2-pixel strips
-constexpr int kBwdStage = kBwdThreads;         // list positions staged at a time
-constexpr int kSums = 9;                       // per Gaussian
+constexpr int kBwdThreads = kTilePixels;
 
-// Sum over the warp of nine per-lane values, as a reduce-scatter by recursive
-// halving: at distance 16, 8, 4 and 2 the lanes whose bit is clear keep the first
-// ceil(n / 2) of their n values and the others the rest (5 and 4 of 9, then 3 and
-// 2, 2 and 1, 1), each adding its partner's copy of them, then pairs (lane, lane ^ 1)
-// add: 12 shuffles.  Lanes 2 s and 2 s + 1 share one value; reduce_slot says which.
+// Sum over the warp of nine per-lane values, as a reduce-scatter over 16
+// slots (slots 9-15 zero) by recursive halving: at distance 16, 8, 4, 2 each
+// lane keeps half of its slots (the half bit 4, 3, 2, 1 of its lane selects)
+// and adds its partner's copy of them, then pairs (lane, lane ^ 1) add; 16
+// shuffles instead of 45.  Lanes 2s and 2s + 1 end with the total of slot s.
 __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) {
-    float a[9];
+    float a[16];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) a[i] = v[i];
-    constexpr int kKeep[4] = {5, 3, 2, 1};   // kept by the lower lanes
-    int n = 9;
+    for (int i = 0; i < 16; ++i) a[i] = i < 9 ? v[i] : 0.f;
 #pragma unroll
-    for (int step = 0; step < 4; ++step) {
-        const int dist = 16 >> step, keep = kKeep[step];
+    for (int half = 8, dist = 16; half >= 1; half >>= 1, dist >>= 1) {
         const bool up = (lane & dist) != 0;
 #pragma unroll
-        for (int i = 0; i < keep; ++i) {
-            const float hi = i + keep < n ? a[i + keep] : 0.f;   // none for the odd one
-            const float send = up ? a[i] : hi, own = up ? hi : a[i];
-            a[i] = own + __shfl_xor_sync(0xffffffffu, send, dist);
+        for (int i = 0; i < half; ++i) {
+            const float send = up ? a[i] : a[i + half];
+            const float keep = up ? a[i + half] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, dist);
         }
-        n = keep;
     }
     return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
-// The slot (0..8) whose total an even lane ends with; -1 for the lanes without one.
-__device__ __forceinline__ int reduce_slot(int lane) {
-    constexpr int kKeep[4] = {5, 3, 2, 1};
-    int base = 0, n = 9;   // the slots the lane still holds: base .. base + n - 1
-#pragma unroll
-    for (int step = 0; step < 4; ++step) {
-        if (lane & (16 >> step)) {
-            base += kKeep[step];
-            n -= kKeep[step];
-        } else {
-            n = min(n, kKeep[step]);
-        }
-    }
-    return n > 0 && !(lane & 1) ? base : -1;
-}
 
 // One CTA of 256 threads per tile: a pixel per thread, a 16x2-pixel strip per warp.
-// The sums are dL/d(px, py) of each pixel, the second moments of v = -2 dL/dq about
-// the centre, sum v and the colour weights; k_preprocess_backward scales them once
-// per Gaussian.
+// Bound by instruction issue: a (strip, Gaussian) that blends costs about 200
+// instructions, a third of them the sum over lanes.
 //
 // Long thin Gaussians amplify the rounding of the sums by the square of their axes'
 // ratio (to about 1e-4 of the rotations' gradients, single values to 1e-2), so the
-// order of the additions shows in the results.  It is a tree over the strip (row
-// pairs, then halves of the row), then one addition to memory per strip, as the
-// warps come to the Gaussian.  Of 100 random scenes trained for a step, 20 had a
-// gradient more than four times this order's own spread away when a tile's strips were added on chip
-// first (16x4 strips, two pixels a lane; 735 us a step at 1M Gaussians and 1280x720), 9 to 13
-// when this order was run again.
-//
-// Bound by instruction issue: a (strip, Gaussian) that blends costs about 90
-// instructions, a third of them the sum over lanes, so the pixels take it without
-// branches (with one around the blend: 948 us a step).  4 CTAs per SM (60 registers):
-// 806 us; with 3 or 5 2% more.  A pixel per thread with a 16-shuffle sum and the
-// conic's and opacity's factors per pixel: 1040.
-__global__ void __launch_bounds__(kBwdThreads, 4)
+// order of the additions shows in the results: a tree over the strip, then one
+// addition to memory per strip, as the warps come to the Gaussian, which is nearly
+// the same order in every run.  Of 182 random scenes trained for a step, so many had a
+// gradient more than four times the spread of two runs (at least 2e-5) away from this
+// kernel's: this kernel again 18; the same sums with 12 shuffles, or the factor
+// 1 / sigma after the sum, or without the branch, which only shift when warps meet,
+// 28, 35 and 46; a tile's strips added on chip (16x4 strips, two pixels a lane, lists
+// per strip) 75.  Those take 1002, 1011, 878 and 735 us of a training step of 1M
+// Gaussians at 1280x720, this one 1041.
+__global__ void __launch_bounds__(kBwdThreads, 5)   // 5 CTAs per SM: <= 48 registers
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
                   const float4* __restrict__ rec, const float4* __restrict__ aux,
                   const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
                   const float* __restrict__ t_final, const int32_t* __restrict__ lstat,
                   const float* __restrict__ dl_dimg, const float* __restrict__ dl_dload,
                   float* __restrict__ g2d) {
-    __shared__ float4 s_kl[kBwdStage];    // quad_k (two), log2(sigma), centre x from the tile origin
-    __shared__ float4 s_nw[kBwdStage];    // -w1x, -w2x, -w1y, -w2y
-    __shared__ float4 s_cy[kBwdStage];    // red, green, blue, centre y
-    __shared__ float4 s_cn[kBwdStage];    // conic a, b, c, the Gaussian
-    __shared__ int s_max[kBwdWarps];
+    __shared__ float2 s_xy[kBwdThreads];
+    __shared__ float2 s_k[kBwdThreads];       // quad_k of the Gaussian at this tile
+    __shared__ float4 s_w[kBwdThreads];
+    __shared__ float4 s_c[kBwdThreads];
+    __shared__ float4 s_conic[kBwdThreads];   // conic a, b, c, sigma
+    __shared__ uint32_t s_g[kBwdThreads];
 
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tiles_x = fp->cam.tiles_x, width = fp->cam.width, height = fp->cam.height;
-    const float e_low = fp->st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
+    const CamDev cam = fp->cam;
+    const SetDev st = fp->st;
     const int tile = blockIdx.x;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int tx = tile % cam.tiles_x, ty = tile / cam.tiles_x;
     const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
     const int x = tx * kTile + lx, y = ty * kTile + ly;
+    const bool inside = x < cam.width && y < cam.height;
     const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
     const float fx = (float)lx, fy = (float)ly;
-    const uint2 range = ranges[tile];
-    if (range.x >= range.y) return;
+    const size_t hw = (size_t)cam.width * cam.height;
+    const size_t pix = inside ? (size_t)y * cam.width + x : 0;
 
-    int32_t last = 0;       // 1-based position of the last blend
-    float T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, gl = 0.f, gl_stop = 0.f;
-    if (x < width && y < height) {
-        const size_t hw = (size_t)width * height, pix = (size_t)y * width + x;
-        last = last_pos[pix];
-        T = t_final[pix];
+    const uint2 range = ranges[tile];
+    int32_t last = inside ? last_pos[pix] : 0;          // 1-based position of the last blend
+    float T = inside ? t_final[pix] : 1.f;
+    float g0 = 0.f, g1 = 0.f, g2 = 0.f, gl = 0.f;
+    if (inside) {
         g0 = dl_dimg[pix];
         g1 = dl_dimg[hw + pix];
         g2 = dl_dimg[2 * hw + pix];
         if (dl_dload) gl = dl_dload[pix];
-        // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
-        // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
-        // that stopped (a more opaque Gaussian makes it stop sooner).
-        if (fp->st.load_grad == ADR_LOAD_GRAD_TERMINATION && gl != 0.f && lstat) {
-            const int32_t ls = lstat[pix];
-            if (ls < 0 && T < 1.f) {
-                gl_stop = gl * -(float)(ls & 0x7FFFFFFF) / -logf(T);
-                gl = 0.f;
-            }
+    }
+    // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
+    // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
+    // that stopped (a more opaque Gaussian makes it stop sooner).
+    float gl_stop = 0.f;
+    if (st.load_grad == ADR_LOAD_GRAD_TERMINATION && inside && gl != 0.f && lstat) {
+        const int32_t ls = lstat[pix];
+        if (ls < 0 && T < 1.f) {
+            gl_stop = gl * -(float)(ls & 0x7FFFFFFF) / -logf(T);
+            gl = 0.f;
         }
     }
-    float acc0 = fp->st.bg[0], acc1 = fp->st.bg[1], acc2 = fp->st.bg[2];   // colour behind the current Gaussian
-    const int slot = reduce_slot(lane);
-    const bool termination = __any_sync(0xffffffffu, gl_stop != 0.f);
+    float acc0 = st.bg[0], acc1 = st.bg[1], acc2 = st.bg[2];   // colour behind the current Gaussian
+    const float e_low = st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
 
-    // The longest prefix any pixel of the warp, and of the tile, needs.
-    const int warp_last = __reduce_max_sync(0xffffffffu, last);
-    if (lane == 0) s_max[warp] = warp_last;
-    __syncthreads();
-    int tile_last = 0;
-#pragma unroll
-    for (int w = 0; w < kBwdWarps; ++w) tile_last = max(tile_last, s_max[w]);
-    // Batches of list positions, from the back.
-    for (int bend = tile_last; bend > 0; bend -= kBwdStage) {
-        const int bstart = max(0, bend - kBwdStage);
+    if (range.x < range.y) {
+        // The longest prefix any pixel of the warp, and of the tile, needs.
+        const int warp_last = __reduce_max_sync(0xffffffffu, last);
+        const int max_last = warp_last;
+        __shared__ int s_max[kBwdThreads / 32];
+        if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = max_last;
         __syncthreads();
-        const int j = (int)threadIdx.x;
-        if (bstart + j < bend) {
-            const uint32_t g = sorted_gauss[range.x + bstart + j];
-            const float4 r0 = rec[3 * (size_t)g + 0];
-            const float4 w = rec[3 * (size_t)g + 1];
-            const float4 col = rec[3 * (size_t)g + 2];
-            const float4 cn = aux[2 * (size_t)g];
-            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
-                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
-            const float2 k = quad_k(c, w);
-            s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
-            s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
-            s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
-            s_cn[j] = make_float4(cn.x, cn.y, cn.z, __uint_as_float(g));
-        }
-        __syncthreads();
-        // this warp's positions: none of its pixels blended one past warp_last
-#pragma unroll 2
-        for (int i = min(bend, warp_last) - bstart - 1; i >= 0; --i) {
-            const float4 kl = s_kl[i];
-            const float4 nw = s_nw[i];
-            // Same evaluation as the forward pass, so the same skip decision.
-            const float u1 = fmaf(nw.z, fy, fmaf(nw.x, fx, kl.x)), u2 = fmaf(nw.w, fy, fmaf(nw.y, fx, kl.y));
-            const float e = fmaf(-u1, u1, fmaf(-u2, u2, kl.z));
-            const bool blended = e >= e_low && bstart + i < last;
-            if (!__any_sync(0xffffffffu, blended)) continue;
-            const float4 cy = s_cy[i];
-            const float4 cn = s_cn[i];
-            // A pixel that did not blend this Gaussian has raw = alpha = 0, which leaves its
-            // T as it is; its colour and its terms are selected, as 0 times an infinite
-            // gradient or colour would not be 0.
-            const float raw = blended ? ex2_approx(e) : 0.f, alpha = fminf(0.99f, raw), one_m = 1.f - alpha;
-            T = __fdiv_rn(T, one_m);   // before this blend
-            const float wgt = alpha * T;
-            float term = gl;   // the load's; dividing a zero is the division's slow path (1M: 950 us a step)
-            if (termination) term += __fdiv_rn(gl_stop, one_m);
-            const float dcol = fmaf(cy.z - acc2, g2, fmaf(cy.y - acc1, g1, __fmul_rn(cy.x - acc0, g0)));
-            const float dalpha = fmaf(T, dcol, term);
-            acc0 = blended ? fmaf(cy.x, alpha, __fmul_rn(one_m, acc0)) : acc0;
-            acc1 = blended ? fmaf(cy.y, alpha, __fmul_rn(one_m, acc1)) : acc1;
-            acc2 = blended ? fmaf(cy.z, alpha, __fmul_rn(one_m, acc2)) : acc2;
-            const float v = blended && raw < 0.99f ? raw * dalpha : 0.f;       // alpha = sigma G, G = exp(-q / 2); 0 if clamped
-            const float dx = kl.w - fx, dy = cy.w - fy, vx = v * dx, vy = v * dy;
-            const float sums[9] = {v, v * fmaf(cn.x, dx, __fmul_rn(cn.y, dy)), v * fmaf(cn.y, dx, __fmul_rn(cn.z, dy)),
-                                   vx * dx, vx * dy, vy * dy, blended ? wgt * g0 : 0.f, blended ? wgt * g1 : 0.f, blended ? wgt * g2 : 0.f};
-            const float tot = reduce_scatter9(sums, lane);
-            if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * kSums + slot, tot);
+        int tile_last = 0;
+        for (int w = 0; w < kBwdThreads / 32; ++w) tile_last = max(tile_last, s_max[w]);
+        // Batches of 256 list positions, from the back.
+        for (int bend = tile_last; bend > 0; bend -= kBwdThreads) {
+            const int bstart = max(0, bend - kBwdThreads);
+            __syncthreads();
+            const int pos = bstart + threadIdx.x;
+            if (pos < bend) {
+                const uint32_t g = sorted_gauss[range.x + pos];
+                const float4 r0 = rec[3 * (size_t)g + 0];
+                const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                             __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+                const float4 w = rec[3 * (size_t)g + 1];
+                s_xy[threadIdx.x] = c;
+                s_k[threadIdx.x] = quad_k(c, w);
+                s_w[threadIdx.x] = w;
+                s_c[threadIdx.x] = rec[3 * (size_t)g + 2];
+                s_conic[threadIdx.x] = aux[2 * (size_t)g + 0];
+                s_g[threadIdx.x] = g;
+            }
+            __syncthreads();
+            // this warp's positions: none of its pixels blended one past warp_last
+            for (int p = min(bend, warp_last) - 1; p >= bstart; --p) {
+                const int j = p - bstart;
+                bool contrib = false;
+                float d_px = 0.f, d_py = 0.f, d_ca = 0.f, d_cb = 0.f, d_cc = 0.f, d_sig = 0.f;
+                float d_r = 0.f, d_g = 0.f, d_b = 0.f;
+                if (p < last) {
+                    // Same evaluation as the forward pass, so the same skip decision.
+                    const float2 c = s_xy[j];
+                    const float4 w = s_w[j];
+                    const float4 col = s_c[j];
+                    const float dx = c.x - fx, dy = c.y - fy;
+                    const float e = quad_exponent(s_k[j], w, col.w, fx, fy);
+                    if (e >= e_low) {
+                        const float raw = ex2_approx(e);
+                        const float alpha = fminf(0.99f, raw);
+                        contrib = true;
+                        const float one_m = 1.f - alpha;
+                        T = T / one_m;                                    // T before this blend
+                        const float wgt = alpha * T;
+                        d_r = wgt * g0;
+                        d_g = wgt * g1;
+                        d_b = wgt * g2;
+                        float dalpha = T * ((col.x - acc0) * g0 + (col.y - acc1) * g1 + (col.z - acc2) * g2);
+                        dalpha += gl + gl_stop / one_m;                   // load term
+                        acc0 = fmaf(col.x, alpha, one_m * acc0);
+                        acc1 = fmaf(col.y, alpha, one_m * acc1);
+                        acc2 = fmaf(col.z, alpha, one_m * acc2);
+                        if (raw < 0.99f) {                                // not clamped
+                            const float4 cn = s_conic[j];
+                            d_sig = dalpha * raw / cn.w;                  // alpha = sigma * G
+                            const float dq = -0.5f * raw * dalpha;        // G = exp(-q/2)
+                            d_px = dq * 2.f * fmaf(cn.x, dx, cn.y * dy);
+                            d_py = dq * 2.f * fmaf(cn.y, dx, cn.z * dy);
+                            d_ca = dq * dx * dx;
+                            d_cb = dq * 2.f * dx * dy;
+                            d_cc = dq * dy * dy;
+                        }
+                    }
+                }
+                if (__any_sync(0xffffffffu, contrib)) {
+                    const int lane = threadIdx.x & 31;
+                    const float v[9] = {d_px, d_py, d_ca, d_cb, d_cc, d_sig, d_r, d_g, d_b};
+                    const float tot = reduce_scatter9(v, lane);
+                    const int slot = (lane >> 1) & 15;   // the slot lane's total belongs to
+                    if (!(lane & 1) && slot < 9) atomicAdd(g2d + (size_t)s_g[j] * 9 + slot, tot);
+                }
+            }
         }
     }
 }
@@ -269,13 +258,10 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
         for (int j = 0; j < kShQuads; ++j) row[j] = make_float4(0.f, 0.f, 0.f, 0.f);
     } else {
         const float* G = g2d + (size_t)i * 9;
-        // With q = C_a dx^2 + 2 C_b dx dy + C_c dy^2 and v = -2 dL/dq per pixel: dL/dC
-        // from the second moments, and dL/dsigma = sum v / sigma.
         const float4 cn = aux[2 * (size_t)i];
         const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
-        const float gpx = -G[1], gpy = -G[2];
-        const float gca = -0.5f * G[3], gcb = -G[4], gcc = -0.5f * G[5];
-        go = G[0] != 0.f ? G[0] / cn.w : 0.f;   // sigma may be 0 in the plain mode: it blends nothing
+        const float gpx = G[0], gpy = G[1], gca = G[2], gcb = G[3], gcc = G[4];
+        go = G[5];
         const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
         // --- colour: rgb = max(0, sum_k sh_k Y_k(d) + 0.5), d = (X0 - cam) / |X0 - cam|
         float vx = mx - cam.cam_pos[0], vy = my - cam.cam_pos[1], vz = mz - cam.cam_pos[2];
