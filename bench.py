@@ -58,7 +58,13 @@ def select_workload(name):
     kind, n, w, h, cap = WORKLOADS[name]
     WORKLOAD, N_GAUSS, WIDTH, HEIGHT, PAIR_CAPACITY = name, n, w, h, cap
     return kind
-EVAL_FP32_OPS = 15        # FP32 lane operations per Gaussian-pixel evaluation in Render
+# FP32 lane operations per Gaussian-pixel evaluation in Render.  Evaluations are counted
+# as the list positions that the pixels traverse; Render's quadrant lists leave out those
+# that no pixel of an 8x8 quadrant can blend, so the rate is an equivalent, not that of
+# the operations executed.
+EVAL_FP32_OPS = 15
+EVAL_WORK = (f"{EVAL_FP32_OPS} FP32 ops per list position a pixel traverses (an equivalent: positions that a "
+             "quadrant's list leaves out count as evaluated)")
 # Kernels of one sliced forward frame: frame head 1, preprocess 1, depth order of
 # slice 0 (bin scan, bin scatter, window sort with the run scan) 3, tile pass 1 (count, count scan, scatter) 3, render slice 0 1,
 # unfinished-tile table (rows, columns) 2, depth order of slice 1 (its selection
@@ -831,7 +837,7 @@ def run_ours(args):
         achieved = u_mean["evals"] * EVAL_FP32_OPS / (dk["ms_per_frame"] / 1e3) / 1e12
         roofline = {"kernel": dominant, "bound": "alu", "achieved": achieved, "peak": alu_peak,
                     "unit": "T FP32 lane-ops/s", "frac": achieved / alu_peak, "traffic": traffic,
-                    "peak_source": f"{sm_count} SMs x 128 FP32 lanes x {clk_mhz:.0f} MHz"}
+                    "peak_source": f"{sm_count} SMs x 128 FP32 lanes x {clk_mhz:.0f} MHz", "work": EVAL_WORK}
     else:
         roofline = {"kernel": dominant, "bound": "hbm", "achieved": dk["gbs"], "peak": hbm_gbs,
                     "unit": "GB/s", "frac": dk["gbs"] / hbm_gbs, "traffic": traffic,
@@ -896,7 +902,7 @@ def run_ours(args):
         "kernels": ktable,
         "render_roofline": {"alu": {"achieved": render_alu, "peak": alu_peak,
                                     "unit": "T FP32 lane-ops/s", "frac": render_alu / alu_peak,
-                                    "work": f"{EVAL_FP32_OPS} FP32 ops per Gaussian-pixel evaluation"},
+                                    "work": EVAL_WORK},
                             "hbm": {"achieved_gbs": render["gbs"] if render else None,
                                     "peak_gbs": hbm_gbs,
                                     "frac": (render["gbs"] / hbm_gbs) if render else None}},

@@ -438,7 +438,7 @@ struct PairSource {
 
 // Tile sort (tiles.cu): two range-partitioned counting passes, over the
 // column runs by tx, then over the pairs by ty; `grid` CTAs, each owning a
-// contiguous run of 4096-item chunks; counts holds kRadix x grid words, totals
+// contiguous run of chunks (1024 or 4096 runs, then 512); counts holds kRadix x grid words, totals
 // kRadix words (zeroed before the count kernel that sums into them).
 //   count_columns:   per-CTA tx counts of the runs, from the Gaussians' rectangles;
 //   scatter_columns: runs generated on chip from the depth-ordered Gaussians,

@@ -8,7 +8,7 @@
 //   * the pair total P = sum of w h (64-bit atomics, published by a one-thread
 //     kernel after the scan) and the capacity check;
 //   * chunk_first[c] = depth-order position of the Gaussian that holds run
-//     c * 4096, so the tile sort can generate each chunk's runs on chip;
+//     c * kMarkRuns, so the tile sort can generate each chunk's runs on chip;
 // It reads the packed rectangles in depth order, which the last depth-sort
 // pass carries along.  Plus small helpers for the tile ranges.
 #include "lookback.cuh"

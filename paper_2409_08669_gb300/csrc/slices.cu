@@ -254,8 +254,8 @@ k_surv_scan(uint32_t* __restrict__ cnt, int grid, const uint32_t* __restrict__ c
 }
 
 // Writes the kept Gaussians in depth order with their packed rectangles, run
-// offsets (exclusive prefix of their widths) and, for every 4096-run chunk
-// that starts inside a Gaussian's runs, that Gaussian's position.
+// offsets (exclusive prefix of their widths) and, for every kMarkRuns-th run
+// that lies inside a Gaussian's runs, that Gaussian's position.
 __global__ void __launch_bounds__(kSurvThreads)
 k_surv_scatter(const uint32_t* __restrict__ sorted_box, const uint32_t* __restrict__ order,
                const uint32_t* __restrict__ counters, const uint8_t* __restrict__ keep_flag,
