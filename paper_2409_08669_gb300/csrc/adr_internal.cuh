@@ -554,15 +554,16 @@ void launch_survivor_bins(const uint32_t* keys, const uint32_t* boxes, int64_t n
                           const uint32_t* counters, uint32_t* bins, uint32_t* rank, cudaStream_t stream);
 
 // Backward (backward.cu).
-void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
-                            const FrameParams* fp, int num_tiles,
+// True if sigma is still to divide the sums of dL/dsigma (large images).
+bool launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
+                            const FrameParams* fp, int num_tiles, int sm_count,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
                             cudaStream_t stream);
 void launch_preprocess_backward(int n, const float* means, const float* scales, const float* rots,
                                 const float* opac, const float* sh, const FrameParams* fp,
                                 const uint32_t* gbox, const float4* aux,
-                                const float* g2d, float* g_means, float* g_scales, float* g_rots,
+                                const float* g2d, bool over_sigma, float* g_means, float* g_scales, float* g_rots,
                                 float* g_opac, float* g_sh, cudaStream_t stream);
 // 2^x with the hardware's approximate base-2 exponential (PTX ex2.approx.ftz:
 // relative error ~2^-22, results below 2^-126 flushed to zero).  Render and its

@@ -6,7 +6,8 @@
 //   k_render_backward     per tile, walks each pixel's blended Gaussians from
 //                         back to front, recovering T_k = T_{k+1} / (1 - alpha_k),
 //                         and accumulates dL/d(px, py, conic, sigma, rgb);
-//                         warp-reduced, then atomicAdd into 9 floats per Gaussian.
+//                         warp-reduced, then atomicAdd into 9 floats per Gaussian
+//                         (k_render_backward_many: images of many tiles).
 //   k_preprocess_backward chain rule from those 2D quantities to means, scales,
 //                         rotations, opacities and SH coefficients.
 //   k_load_moments / k_load_grad
@@ -18,6 +19,9 @@ namespace adr {
 namespace {
 
 constexpr int kBwdThreads = kTilePixels;
+constexpr int kBwdWarps = kBwdThreads / 32;    // 16x2-pixel strips
+constexpr int kBwdStage = kBwdThreads;         // list positions staged at a time
+constexpr int kBwdCtas = 5;                    // per SM, k_render_backward
 
 // Sum over the warp of nine per-lane values, as a reduce-scatter over 16
 // slots (slots 9-15 zero) by recursive halving: at distance 16, 8, 4, 2 each
@@ -42,21 +46,21 @@ __device__ __forceinline__ float reduce_scatter9(const float (&v)[9], int lane) 
 }
 
 // One CTA of 256 threads per tile: a pixel per thread, a 16x2-pixel strip per warp.
-// Bound by instruction issue: a (strip, Gaussian) that blends costs about 200
-// instructions, a third of them the sum over lanes.
+// Both kernels are bound by instruction issue (0.89 of the slots).
 //
 // Long thin Gaussians amplify the rounding of the sums by the square of their axes'
 // ratio (to about 1e-4 of the rotations' gradients, single values to 1e-2), so the
 // order of the additions shows in the results: a tree over the strip, then one
-// addition to memory per strip, as the warps come to the Gaussian, which is nearly
-// the same order in every run.  Of 182 random scenes trained for a step, so many had a
-// gradient more than four times the spread of two runs (at least 2e-5) away from this
-// kernel's: this kernel again 18; the same sums with 12 shuffles, or the factor
-// 1 / sigma after the sum, or without the branch, which only shift when warps meet,
-// 28, 35 and 46; a tile's strips added on chip (16x4 strips, two pixels a lane, lists
-// per strip) 75.  Those take 1002, 1011, 878 and 735 us of a training step of 1M
-// Gaussians at 1280x720, this one 1041.
-__global__ void __launch_bounds__(kBwdThreads, 5)   // 5 CTAs per SM: <= 48 registers
+// addition to memory per strip, as the warps come to the Gaussian.  While all tiles
+// of an image are on the chip at once that is nearly the same order in every run, and
+// what changes the warps' speed changes it: of 182 random scenes of up to 1170 tiles,
+// trained for a step, 18 had a gradient more than four times the spread of two runs
+// (at least 2e-5) away when this kernel ran again, 28 with the sum in 12 shuffles, 35
+// with the factor 1 / sigma after the sum, 46 without the branch.  So images of one
+// wave of CTAs keep it.  Larger ones are scheduled anew in every run (of 186 of more
+// than 760 tiles: 14 and 17 with this kernel again, 22 with k_render_backward_many).
+// Adding a tile's strips on chip (16x4 strips, two pixels a lane) had 75 of the 182.
+__global__ void __launch_bounds__(kBwdThreads, kBwdCtas)   // <= 48 registers
 k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
                   const float4* __restrict__ rec, const float4* __restrict__ aux,
                   const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
@@ -186,6 +190,163 @@ k_render_backward(const uint2* __restrict__ ranges, const uint32_t* __restrict__
     }
 }
 
+// The same sums (bit for bit) in 12 shuffles: at distance 16, 8, 4 and 2 the lanes
+// whose bit is clear keep the first ceil(n / 2) of their n values and the others the
+// rest (5 and 4 of 9, then 3 and 2, 2 and 1, 1), each adding its partner's copy of
+// them, then pairs (lane, lane ^ 1) add.  Lanes 2 s and 2 s + 1 share one value; sum_slot says which.
+__device__ __forceinline__ float sum_over_lanes(const float (&v)[9], int lane) {
+    float a[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) a[i] = v[i];
+    constexpr int kKeep[4] = {5, 3, 2, 1};   // kept by the lower lanes
+    int n = 9;
+#pragma unroll
+    for (int step = 0; step < 4; ++step) {
+        const int dist = 16 >> step, keep = kKeep[step];
+        const bool up = (lane & dist) != 0;
+#pragma unroll
+        for (int i = 0; i < keep; ++i) {
+            const float hi = i + keep < n ? a[i + keep] : 0.f;   // none for the odd one
+            const float send = up ? a[i] : hi, own = up ? hi : a[i];
+            a[i] = own + __shfl_xor_sync(0xffffffffu, send, dist);
+        }
+        n = keep;
+    }
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+}
+// The slot (0..8) whose total an even lane ends with; -1 for the lanes without one.
+__device__ __forceinline__ int sum_slot(int lane) {
+    constexpr int kKeep[4] = {5, 3, 2, 1};
+    int base = 0, n = 9;   // the slots the lane still holds: base .. base + n - 1
+#pragma unroll
+    for (int step = 0; step < 4; ++step) {
+        if (lane & (16 >> step)) {
+            base += kKeep[step];
+            n -= kKeep[step];
+        } else {
+            n = min(n, kKeep[step]);
+        }
+    }
+    return n > 0 && !(lane & 1) ? base : -1;
+}
+
+// Images of more than one wave of CTAs.  A (strip, Gaussian) that blends costs about 95
+// instructions instead of 200: the pixels take it without a branch, the lanes' sums
+// take 12 shuffles, and sigma divides the whole sum (k_preprocess_backward).  4 CTAs per SM, 60 registers; with 3 or
+// 5 2% more.  1M Gaussians at 1280x720: 647 -> 351 us.
+__global__ void __launch_bounds__(kBwdThreads, 4)
+k_render_backward_many(const uint2* __restrict__ ranges, const uint32_t* __restrict__ sorted_gauss,
+                       const float4* __restrict__ rec, const float4* __restrict__ aux,
+                       const FrameParams* __restrict__ fp, const int32_t* __restrict__ last_pos,
+                       const float* __restrict__ t_final, const int32_t* __restrict__ lstat,
+                       const float* __restrict__ dl_dimg, const float* __restrict__ dl_dload,
+                       float* __restrict__ g2d) {
+    __shared__ float4 s_kl[kBwdStage];    // quad_k (two), log2(sigma), centre x from the tile origin
+    __shared__ float4 s_nw[kBwdStage];    // -w1x, -w2x, -w1y, -w2y
+    __shared__ float4 s_cy[kBwdStage];    // red, green, blue, centre y
+    __shared__ float4 s_cn[kBwdStage];    // conic a, b, c, the Gaussian
+    __shared__ int s_max[kBwdWarps];
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tiles_x = fp->cam.tiles_x, width = fp->cam.width, height = fp->cam.height;
+    const float e_low = fp->st.e_low;   // alpha >= alpha_low as 2^e >= alpha_low, decided on e
+    const int tile = blockIdx.x;
+    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int lx = threadIdx.x % kTile, ly = threadIdx.x / kTile;
+    const int x = tx * kTile + lx, y = ty * kTile + ly;
+    const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
+    const float fx = (float)lx, fy = (float)ly;
+    const uint2 range = ranges[tile];
+    if (range.x >= range.y) return;
+
+    int32_t last = 0;       // 1-based position of the last blend
+    float T = 1.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, gl = 0.f, gl_stop = 0.f;
+    if (x < width && y < height) {
+        const size_t hw = (size_t)width * height, pix = (size_t)y * width + x;
+        last = last_pos[pix];
+        T = t_final[pix];
+        g0 = dl_dimg[pix];
+        g1 = dl_dimg[hw + pix];
+        g2 = dl_dimg[2 * hw + pix];
+        if (dl_dload) gl = dl_dload[pix];
+        // d l_i / d alpha_k per blended Gaussian k: 1 (straight-through), or, with
+        // the termination reading, -l_i / (-ln T_final) / (1 - alpha_k) for a pixel
+        // that stopped (a more opaque Gaussian makes it stop sooner).
+        if (fp->st.load_grad == ADR_LOAD_GRAD_TERMINATION && gl != 0.f && lstat) {
+            const int32_t ls = lstat[pix];
+            if (ls < 0 && T < 1.f) {
+                gl_stop = gl * -(float)(ls & 0x7FFFFFFF) / -logf(T);
+                gl = 0.f;
+            }
+        }
+    }
+    float acc0 = fp->st.bg[0], acc1 = fp->st.bg[1], acc2 = fp->st.bg[2];   // colour behind the current Gaussian
+    const int slot = sum_slot(lane);
+    const bool termination = __any_sync(0xffffffffu, gl_stop != 0.f);
+
+    // The longest prefix any pixel of the warp, and of the tile, needs.
+    const int warp_last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) s_max[warp] = warp_last;
+    __syncthreads();
+    int tile_last = 0;
+#pragma unroll
+    for (int w = 0; w < kBwdWarps; ++w) tile_last = max(tile_last, s_max[w]);
+    // Batches of list positions, from the back.
+    for (int bend = tile_last; bend > 0; bend -= kBwdStage) {
+        const int bstart = max(0, bend - kBwdStage);
+        __syncthreads();
+        const int j = (int)threadIdx.x;
+        if (bstart + j < bend) {
+            const uint32_t g = sorted_gauss[range.x + bstart + j];
+            const float4 r0 = rec[3 * (size_t)g + 0];
+            const float4 w = rec[3 * (size_t)g + 1];
+            const float4 col = rec[3 * (size_t)g + 2];
+            const float4 cn = aux[2 * (size_t)g];
+            const float2 c = make_float2(__fadd_rn(__fsub_rn(r0.x, ox), r0.z),
+                                         __fadd_rn(__fsub_rn(r0.y, oy), r0.w));
+            const float2 k = quad_k(c, w);
+            s_kl[j] = make_float4(k.x, k.y, col.w, c.x);
+            s_nw[j] = make_float4(-w.x, -w.z, -w.y, -w.w);
+            s_cy[j] = make_float4(col.x, col.y, col.z, c.y);
+            s_cn[j] = make_float4(cn.x, cn.y, cn.z, __uint_as_float(g));
+        }
+        __syncthreads();
+        // this warp's positions: none of its pixels blended one past warp_last
+#pragma unroll 2
+        for (int i = min(bend, warp_last) - bstart - 1; i >= 0; --i) {
+            const float4 kl = s_kl[i];
+            const float4 nw = s_nw[i];
+            // Same evaluation as the forward pass, so the same skip decision.
+            const float u1 = fmaf(nw.z, fy, fmaf(nw.x, fx, kl.x)), u2 = fmaf(nw.w, fy, fmaf(nw.y, fx, kl.y));
+            const float e = fmaf(-u1, u1, fmaf(-u2, u2, kl.z));
+            const bool blended = e >= e_low && bstart + i < last;
+            if (!__any_sync(0xffffffffu, blended)) continue;
+            const float4 cy = s_cy[i];
+            const float4 cn = s_cn[i];
+            // A pixel that did not blend this Gaussian has raw = alpha = 0, which leaves its
+            // T as it is; its colour and its terms are selected, as 0 times an infinite
+            // gradient or colour would not be 0.
+            const float raw = blended ? ex2_approx(e) : 0.f, alpha = fminf(0.99f, raw), one_m = 1.f - alpha;
+            T = __fdiv_rn(T, one_m);   // before this blend
+            const float wgt = alpha * T;
+            float term = gl;   // the load's; dividing a zero is the division's slow path (1M: 950 us a step)
+            if (termination) term += __fdiv_rn(gl_stop, one_m);
+            const float dcol = fmaf(cy.z - acc2, g2, fmaf(cy.y - acc1, g1, __fmul_rn(cy.x - acc0, g0)));
+            const float dalpha = fmaf(T, dcol, term);
+            acc0 = blended ? fmaf(cy.x, alpha, __fmul_rn(one_m, acc0)) : acc0;
+            acc1 = blended ? fmaf(cy.y, alpha, __fmul_rn(one_m, acc1)) : acc1;
+            acc2 = blended ? fmaf(cy.z, alpha, __fmul_rn(one_m, acc2)) : acc2;
+            const float v = blended && raw < 0.99f ? raw * dalpha : 0.f;       // alpha = sigma G, G = exp(-q / 2); 0 if clamped
+            const float dq = -0.5f * v, dx = kl.w - fx, dy = cy.w - fy;
+            const float sums[9] = {-v * fmaf(cn.x, dx, __fmul_rn(cn.y, dy)), -v * fmaf(cn.y, dx, __fmul_rn(cn.z, dy)),
+                                   dq * dx * dx, -v * dx * dy, dq * dy * dy, v,
+                                   blended ? wgt * g0 : 0.f, blended ? wgt * g1 : 0.f, blended ? wgt * g2 : 0.f};
+            const float tot = sum_over_lanes(sums, lane);
+            if (slot >= 0) atomicAdd(g2d + (size_t)__float_as_uint(cn.w) * 9 + slot, tot);
+        }
+    }
+}
+
 // SH basis gradient: dY_k/d(x, y, z) of the degree-3 real polynomials used in
 // the forward pass (Condon-Shortley phase).
 constexpr float kY1 = 0.48860251190291992f, kY2a = 1.0925484305920792f,
@@ -234,7 +395,7 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
                       const float* __restrict__ rots, const float* __restrict__ opac,
                       const float* __restrict__ sh, const FrameParams* __restrict__ fp,
                       const uint32_t* __restrict__ gbox, const float4* __restrict__ aux,
-                      const float* __restrict__ g2d, float* __restrict__ g_means,
+                      const float* __restrict__ g2d, bool over_sigma, float* __restrict__ g_means,
                       float* __restrict__ g_scales, float* __restrict__ g_rots,
                       float* __restrict__ g_opac, float* __restrict__ g_sh) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -261,7 +422,7 @@ k_preprocess_backward(int n, const float* __restrict__ means, const float* __res
         const float4 cn = aux[2 * (size_t)i];
         const float Ca = cn.x, Cb = cn.y, Cc = cn.z;
         const float gpx = G[0], gpy = G[1], gca = G[2], gcb = G[3], gcc = G[4];
-        go = G[5];
+        go = !over_sigma ? G[5] : G[5] != 0.f ? G[5] / cn.w : 0.f;   // an opacity of 0 blends nothing
         const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
         // --- colour: rgb = max(0, sum_k sh_k Y_k(d) + 0.5), d = (X0 - cam) / |X0 - cam|
         float vx = mx - cam.cam_pos[0], vy = my - cam.cam_pos[1], vz = mz - cam.cam_pos[2];
@@ -542,25 +703,27 @@ k_load_grad(const T* __restrict__ load, int64_t hw, double* __restrict__ sums,
 
 }  // namespace
 
-void launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
-                            const FrameParams* fp, int num_tiles,
+bool launch_render_backward(const uint2* ranges, const uint32_t* sorted_gauss, const float4* rec, const float4* aux,
+                            const FrameParams* fp, int num_tiles, int sm_count,
                             const int32_t* last, const float* t_final, const int32_t* lstat,
                             const float* dl_dimg, const float* dl_dload, float* g2d,
                             cudaStream_t stream) {
-    const int tiles = num_tiles;
-    if (tiles <= 0) return;
-    k_render_backward<<<tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, aux, fp,
-                                                         last, t_final, lstat, dl_dimg, dl_dload, g2d);
+    if (num_tiles <= 0) return false;
+    const bool many = num_tiles > kBwdCtas * sm_count;
+    auto* kernel = many ? k_render_backward_many : k_render_backward;
+    kernel<<<num_tiles, kBwdThreads, 0, stream>>>(ranges, sorted_gauss, rec, aux, fp, last, t_final, lstat, dl_dimg,
+                                                  dl_dload, g2d);
+    return many;
 }
 
 void launch_preprocess_backward(int n, const float* means, const float* scales, const float* rots,
                                 const float* opac, const float* sh, const FrameParams* fp,
                                 const uint32_t* gbox, const float4* aux,
-                                const float* g2d, float* g_means, float* g_scales, float* g_rots,
+                                const float* g2d, bool over_sigma, float* g_means, float* g_scales, float* g_rots,
                                 float* g_opac, float* g_sh, cudaStream_t stream) {
     if (n <= 0) return;
     k_preprocess_backward<<<(n + kPreBwdThreads - 1) / kPreBwdThreads, kPreBwdThreads, 0, stream>>>(n, means, scales, rots, opac, sh, fp,
-                                                               gbox, aux, g2d, g_means,
+                                                               gbox, aux, g2d, over_sigma, g_means,
                                                                g_scales, g_rots, g_opac, g_sh);
 }
 

@@ -492,12 +492,14 @@ void enqueue_backward(const Workspace& ws, const FrameState& fs, const float* me
                       float* g_rots, float* g_opac, float* g_sh, cudaStream_t stream) {
     if (fs.n <= 0) return;
     cudaMemsetAsync(ws.g2d, 0, (size_t)fs.n * 9 * sizeof(float), stream);
+    bool over_sigma = false;
     TIMED(ws, kKRenderBackward, stream,
-          launch_render_backward(ws.ranges, fs.sorted_gauss, ws.rec, ws.aux, ws.d_fp, fs.num_tiles,
-                                 ws.last, ws.tfin, ws.lstat, dl_dimg, dl_dload, ws.g2d, stream));
+          over_sigma = launch_render_backward(ws.ranges, fs.sorted_gauss, ws.rec, ws.aux, ws.d_fp, fs.num_tiles,
+                                              ws.sm_count, ws.last, ws.tfin, ws.lstat, dl_dimg, dl_dload, ws.g2d,
+                                              stream));
     TIMED(ws, kKPreprocessBackward, stream,
           launch_preprocess_backward((int)fs.n, means, scales, rots, opac, sh, ws.d_fp, ws.gbox,
-                                     ws.aux, ws.g2d, g_means, g_scales, g_rots, g_opac, g_sh,
+                                     ws.aux, ws.g2d, over_sigma, g_means, g_scales, g_rots, g_opac, g_sh,
                                      stream));
 }
 

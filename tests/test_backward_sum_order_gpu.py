@@ -24,32 +24,34 @@ def sequential_sums(strips):
     return set(total.tolist())
 
 
-@pytest.mark.parametrize("w,h", [(16, 16), (16, 13), (11, 9)])
-def test_a_tiles_strips_are_added_one_by_one(w, h):
+@pytest.mark.parametrize("w,h,n,log_scale", [(16, 16, 300, -1.5), (16, 13, 300, -1.5), (11, 9, 300, -1.5),
+                                             (256, 1024, 6000, -3.6)])      # the last: more than a wave of CTAs
+def test_a_tiles_strips_are_added_one_by_one(w, h, n, log_scale):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2409_08669_gb300.raster import Rasterizer, upload
-    n = 300
     rng = np.random.default_rng(16 * w + h)
     scene = S.tiny_scene(w, n=n)
-    scene.scales[:] = np.exp(rng.normal(-1.5, 0.5, (n, 3))).astype(np.float32)
+    scene.scales[:] = np.exp(rng.normal(log_scale, 0.5, (n, 3))).astype(np.float32)
     scene.opac[:] = 0.5
     cam = S.look_at((0.3, 0.2, -3.0), width=w, height=h)
-    rast = Rasterizer(max_gaussians=n, pair_capacity=1 << 16, max_width=16, max_height=16)
+    rast = Rasterizer(max_gaussians=n, pair_capacity=1 << 18, max_width=w, max_height=h)
     try:
         params = upload(scene)
         rast.forward(params, cam, S.Settings(mode=S.MODE_AABB))
         g_img = torch.from_numpy(rng.normal(size=(3, h, w)).astype(np.float32)).cuda()
 
-        def opacity_gradient(first, end):
+        def opacity_gradient(rows):          # of those rows of every tile
             g = torch.zeros_like(g_img)
-            g[:, first:end] = g_img[:, first:end]
+            for y in rows:
+                g[:, y::16] = g_img[:, y::16]
             return rast.backward(params, g)[3].cpu().numpy().reshape(n)
 
-        whole = opacity_gradient(0, h)
-        strips = np.stack([opacity_gradient(y, min(y + 2, h)) for y in range(0, h, 2)], 1)
+        in_one = rast.read_gaussians()[2] == 1         # Gaussians of one tile
+        whole = opacity_gradient(range(16))[in_one]
+        strips = np.stack([opacity_gradient((y, y + 1)) for y in range(0, 16, 2)], 1)[in_one]
     finally:
         rast.close()
     assert np.count_nonzero((strips != 0).sum(1) >= 4) >= 20      # some meet enough strips
-    for i in range(n):
+    for i in range(len(whole)):
         assert float(whole[i]) in sequential_sums(strips[i][strips[i] != 0]), (i, whole[i], strips[i])

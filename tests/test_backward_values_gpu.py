@@ -15,7 +15,7 @@ def rast():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2409_08669_gb300.raster import Rasterizer
-    r = Rasterizer(max_gaussians=1024, pair_capacity=1 << 16, max_width=64, max_height=64)
+    r = Rasterizer(max_gaussians=1024, pair_capacity=1 << 20, max_width=512, max_height=640)
     yield r
     r.close()
 
@@ -30,9 +30,10 @@ def _scene(n, seed):
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
 @pytest.mark.parametrize("which", ["image", "load"])
-def test_a_pixels_infinite_gradient_reaches_only_what_it_blended(rast, value, which):
+@pytest.mark.parametrize("w,h", [(21, 18), (400, 600)])      # a wave of CTAs, and more
+def test_a_pixels_infinite_gradient_reaches_only_what_it_blended(rast, value, which, w, h):
     from paper_2409_08669_gb300.raster import upload
-    n, w, h, y, x = 400, 21, 18, 9, 12
+    n, y, x = 400, h // 2, w // 2 + 2
     params = upload(_scene(n, 3))
     rast.forward(params, S.look_at((0.3, 0.2, -3.0), width=w, height=h), S.Settings(mode=S.MODE_AABB))
     rng = np.random.default_rng(4)
@@ -54,34 +55,38 @@ def test_a_pixels_infinite_gradient_reaches_only_what_it_blended(rast, value, wh
         assert (g - f).abs().max() <= 1e-3 * f.abs().max()     # two orders of the same additions
 
 
-def test_the_load_gradients_quotient_is_a_division(rast):
+@pytest.mark.parametrize("w,h", [(1, 1), (400, 600)])
+def test_the_load_gradients_quotient_is_a_division(rast, w, h):
     """One pixel that blends one Gaussian and stops before the next, in the termination reading and without an image
     gradient: dL/dsigma = alpha (dl / (1 - alpha)) / sigma, each step rounded to FP32.  Of alpha >= 1/2, 1 - alpha = T_final
     is exact, so alpha is known."""
     from paper_2409_08669_gb300.raster import upload
-    cam = S.look_at((0.0, 0.0, -3.0), width=1, height=1)
+    cam, at = S.look_at((0.0, 0.0, -3.0), width=w, height=h), (h // 2, w // 2)
     st = S.Settings(mode=S.MODE_AABB, t_min=0.4, load_grad=S.LOAD_GRAD_TERMINATION)
     scene = S.tiny_scene(0, n=2)
     scene.means[:] = [[0.0, 0.0, 0.0], [0.0, 0.0, 1.0]]
     scene.scales[:] = 1.0
-    zero = torch.zeros(3, 1, 1, device="cuda")
+    zero = torch.zeros(3, h, w, device="cuda")
     rng = np.random.default_rng(0)
     for sigma in rng.uniform(0.53, 0.59, 100).astype(np.float32):
         scene.opac[:] = sigma
         params = upload(scene)
         t_final, load = rast.forward(params, cam, st)[1:]
-        assert int(load) == 1 and 0.4 <= float(t_final) < 0.5
-        g_load = torch.full((1, 1), float(rng.uniform(0.5, 2.0)), device="cuda")
+        t_final = t_final[at]
+        assert int(load[at]) == 1 and 0.4 <= float(t_final) < 0.5
+        g_load = torch.zeros(h, w, device="cuda")
+        g_load[at] = float(rng.uniform(0.5, 2.0))
         got = rast.backward(params, zero, g_load)[3].cpu().numpy().reshape(2)
-        T, stop = t_final.cpu().numpy()[0, 0], ((g_load * -1.0) / -torch.log(t_final)).cpu().numpy()[0, 0]
+        T, stop = t_final.cpu().numpy(), ((g_load[at] * -1.0) / -torch.log(t_final)).cpu().numpy()
         alpha = np.float32(1.0) - T
         assert got[0] == np.float32(alpha * np.float32(stop / T)) / sigma and got[1] == 0.0, (sigma, got)
 
 
+@pytest.mark.parametrize("w,h", [(30, 22), (400, 600)])
 @pytest.mark.parametrize("mode", [S.MODE_PLAIN, S.MODE_AABB])
-def test_an_opacity_of_zero_has_no_gradient(rast, mode):
+def test_an_opacity_of_zero_has_no_gradient(rast, mode, w, h):
     from paper_2409_08669_gb300.raster import upload
-    n, w, h = 400, 30, 22
+    n = 400
     scene = _scene(n, 5)
     scene.opac[::7] = 0.0
     scene.opac[3::7] = 1e-30
