@@ -639,19 +639,17 @@ __device__ __forceinline__ float quad_exponent(float2 k, float4 w, float log2_si
     return fmaf(-u1, u1, fmaf(-u2, u2, log2_sigma));
 }
 
-// Which of the four kW x kH pixel rectangles of a tile (row by row) a Gaussian can
+// Which of the four 8x8 quadrants of a tile (row by row) a Gaussian can
 // blend in, as bits: those with a point where its exponent log2(sigma) - |u|^2
-// reaches the limit.  |u|^2 is a convex quadratic, so its minimum over a rectangle
+// reaches the limit.  |u|^2 is a convex quadratic, so its minimum over a quadrant
 // lies at the centre's nearest x or y edge line, at the other coordinate's
-// minimiser clamped to the rectangle; u is formed from k and w as the pixels form
-// it.  A rectangle is dropped only where the bound holds with every rounding on
+// minimiser clamped to the quadrant; u is formed from k and w as the pixels form
+// it.  A quadrant is dropped only where the bound holds with every rounding on
 // the wrong side: the errors of k, of u and of the minimiser are a few ulp of
 // `scale` (the largest term that cancels in u), and those of the exponent a few
-// ulp of its own terms.  Comparisons with a NaN keep the rectangle.
-template <int kW, int kH>
-__device__ __forceinline__ uint32_t rects_reached(float2 c, float2 k, float4 w, float log2_sigma, float e_lim) {
-    constexpr int kNx = kTile / kW, kNy = kTile / kH;
-    static_assert(kNx * kNy == 4 && kNx * kW == kTile && kNy * kH == kTile, "four rectangles cover the tile");
+// ulp of its own terms.  Comparisons with a NaN keep the quadrant.
+__device__ __forceinline__ uint32_t quadrants_reached(float2 c, float2 k, float4 w, float log2_sigma, float e_lim) {
+    constexpr int kN = 2, kW = kTile / kN;   // a side's quadrants, their pixels
     const float thr = log2_sigma - e_lim;
     if (thr < 0.f) return 0u;   // no pixel reaches the limit: |u|^2 >= 0
     const float scale = (fabsf(w.x) + fabsf(w.z)) * (fabsf(c.x) + 16.f) + (fabsf(w.y) + fabsf(w.w)) * (fabsf(c.y) + 16.f);
@@ -659,25 +657,25 @@ __device__ __forceinline__ uint32_t rects_reached(float2 c, float2 k, float4 w, 
     const float most = fmaf(reach, reach, fmaf(1e-6f, fabsf(log2_sigma) + fabsf(e_lim), 1e-5f));
     const float A = fmaf(w.x, w.x, w.z * w.z), B = fmaf(w.x, w.y, w.z * w.w), C = fmaf(w.y, w.y, w.w * w.w);
     const float slope_y = -B * rcp_approx(C), slope_x = -B * rcp_approx(A);   // the minimiser's drift per pixel off centre
-    float2 ux[kNx], uy[kNy];
-    float fy[kNx], fx[kNy];
+    float2 ux[kN], uy[kN];
+    float fy[kN], fx[kN];
 #pragma unroll
-    for (int i = 0; i < kNx; ++i) {
+    for (int i = 0; i < kN; ++i) {
         const float xs = fminf(fmaxf(c.x, (float)(kW * i)), (float)(kW * i + kW - 1));
         fy[i] = fmaf(slope_y, xs - c.x, c.y);   // y of the minimum on the line x = xs
         ux[i] = make_float2(fmaf(-w.x, xs, k.x), fmaf(-w.z, xs, k.y));
     }
 #pragma unroll
-    for (int i = 0; i < kNy; ++i) {
-        const float ys = fminf(fmaxf(c.y, (float)(kH * i)), (float)(kH * i + kH - 1));
+    for (int i = 0; i < kN; ++i) {
+        const float ys = fminf(fmaxf(c.y, (float)(kW * i)), (float)(kW * i + kW - 1));
         fx[i] = fmaf(slope_x, ys - c.y, c.x);
         uy[i] = make_float2(fmaf(-w.y, ys, k.x), fmaf(-w.w, ys, k.y));
     }
     uint32_t out = 0u;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int hx = q % kNx, hy = q / kNx;
-        const float y = fminf(fmaxf(fy[hx], (float)(kH * hy)), (float)(kH * hy + kH - 1));
+        const int hx = q % kN, hy = q / kN;
+        const float y = fminf(fmaxf(fy[hx], (float)(kW * hy)), (float)(kW * hy + kW - 1));
         const float x = fminf(fmaxf(fx[hy], (float)(kW * hx)), (float)(kW * hx + kW - 1));
         const float a1 = fmaf(-w.y, y, ux[hx].x), a2 = fmaf(-w.w, y, ux[hx].y);
         const float b1 = fmaf(-w.x, x, uy[hy].x), b2 = fmaf(-w.z, x, uy[hy].y);

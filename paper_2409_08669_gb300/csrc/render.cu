@@ -38,7 +38,7 @@ namespace {
 // the staged Gaussians only a part blends at a pixel of a given quadrant (measured
 // on a CPU walk of 60 tiles each: 22% for 150k large Gaussians at 1001x667, 40% with the plain
 // rectangles, 65% at 1M to 3M and 1080p), so staging tests each against the four
-// quadrants (rects_reached, exact up to its rounding margin) and a warp walks
+// quadrants (quadrants_reached, exact up to its rounding margin) and a warp walks
 // its quadrant's own list.  What it walks nearly always blends, so the loop has no
 // skip: two list entries a step, straight-line, with one vote per step for the
 // rare stop.  With one entry a step, every entry evaluated and a vote and a branch
@@ -166,7 +166,7 @@ __device__ __forceinline__ void stage_records(int m, const uint32_t* s_gid, cons
             s_kl[sl] = make_float4(k.x, k.y, col.w, col.z);   // k1, k2, log2(sigma), blue
             s_nw[sl] = make_float4(-w.x, -w.z, -w.y, -w.w);   // -w1x, -w2x, -w1y, -w2y
             s_rg[sl] = make_float4(col.x, col.x, col.y, col.y);
-            if (kLists) reached = rects_reached<8, 8>(c, k, w, col.w, e_lim);
+            if (kLists) reached = quadrants_reached(c, k, w, col.w, e_lim);
         }
         if (kLists) {
             uint32_t mine = 0u;
