@@ -73,10 +73,10 @@ EVAL_WORK = (f"{EVAL_FP32_OPS} FP32 ops per list position a pixel traverses (an 
 KERNELS_PER_FRAME = 19
 # DRAM bytes (read + write) of one launch from one-pass ncu captures at the
 # heavy 3M-Gaussian 1080p frame: Render (profiles/render_heavy-3M-1080p_traffic.md,
-# its two launches of one frame, 54.8 MB) and the per-tile list pass
+# its two launches of one frame, 53.4 MB) and the per-tile list pass
 # (profiles/tile_scatter_rows_heavy-3M-1080p_traffic.md, 128.34 + 576.92 MB over
 # P = 1.5958e8 pairs, scaled by the measured P).
-TRAFFIC_BYTES_PER_FRAME = {"render": (10479616 + 8927232) + (35350528 + 17920)}
+TRAFFIC_BYTES_PER_FRAME = {"render": (10485504 + 7260672) + (35361024 + 271360)}
 TRAFFIC_BYTES_PER_PAIR = {"tile_scatter_rows": (128.34e6 + 576.92e6) / 1.5958e8}
 
 
